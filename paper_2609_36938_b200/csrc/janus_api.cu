@@ -28,6 +28,11 @@ int launch_sparse_attn_generic(const void* q, int M, int H_q, int d_qk, const vo
                                int page_size, const int32_t* page_table, int64_t n_logical_pages, const int64_t* table_offsets,
                                float softmax_scale, void* out, float* lse, int32_t* dev_status, cudaStream_t stream);
 
+bool sparse_attn_heads_supported(int d_qk, int d_v);
+int launch_sparse_attn_heads(const void* q, int M, int H_q, int d_qk, const void* k_pool, const void* v_pool, int64_t page_stride,
+                             int64_t tok_stride, int64_t head_stride, int n_kv_heads, int d_v, const int32_t* idx, int k, int page_size,
+                             const int32_t* page_table, int64_t n_logical_pages, const int64_t* table_offsets, float softmax_scale, void* out,
+                             float* lse, int32_t* dev_status, cudaStream_t stream);
 bool sparse_attn_latent_tc_supported(int M, int H_q, int d_qk, const void* k_pool, const void* v_pool, int64_t page_stride,
                                      int64_t tok_stride, int n_kv_heads, int d_v, int k);
 int launch_sparse_attn_latent_tc(const void* q, int M, const void* pool, int64_t page_stride, int64_t tok_stride, const int32_t* idx, int k,
@@ -134,6 +139,9 @@ static int sparse_attn_dispatch(const void* q, int M, int H_q, int d_qk, const v
         sparse_attn_latent_tc_supported(M, H_q, d_qk, k_pool, v_pool, page_stride, tok_stride, n_kv_heads, d_v, k))
         return launch_sparse_attn_latent_tc(q, M, k_pool, page_stride, tok_stride, idx, k, page_size, page_table, n_logical_pages,
                                             table_offsets, softmax_scale, out, lse, dev_status, stream);
+    if (sparse_attn_heads_supported(d_qk, d_v))
+        return launch_sparse_attn_heads(q, M, H_q, d_qk, k_pool, v_pool, page_stride, tok_stride, head_stride, n_kv_heads, d_v, idx, k,
+                                        page_size, page_table, n_logical_pages, table_offsets, softmax_scale, out, lse, dev_status, stream);
     return launch_sparse_attn_generic(q, M, H_q, d_qk, k_pool, v_pool, page_stride, tok_stride, head_stride, n_kv_heads, d_v, idx, k,
                                       page_size, page_table, n_logical_pages, table_offsets, softmax_scale, out, lse, dev_status, stream);
 }

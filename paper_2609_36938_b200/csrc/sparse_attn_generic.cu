@@ -2,8 +2,8 @@
 // One CTA handles one query token and a group of G query heads that share a kv head.  Selected rows are
 // gathered through the page table with 16-byte loads into padded shared-memory tiles of 32 keys; the
 // softmax is the usual online form (running max and sum in fp32, accumulators rescaled when the max moves).
-// Serves multi-head layouts (a single query head per kv head is a matrix-vector problem with nothing for
-// tensor cores to do) and any shape the latent tensor-core kernel does not take.
+// Serves the dims that neither the latent kernel (128 heads, 576 / 512) nor the multi-head kernel (keys of 64, 128 or 192
+// dims, values of 64 or 128) takes.
 #include "janus_common.cuh"
 
 namespace janus {
