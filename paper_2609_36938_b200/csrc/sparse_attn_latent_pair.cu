@@ -40,6 +40,8 @@
 // cluster still meet at the final cluster barrier.
 #include <cuda_fp16.h>
 
+#include <mutex>
+
 #include "janus_common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -82,6 +84,14 @@ struct LpShared {
     uint32_t start_abort[2];
 };
 
+// Keys of one token split over several pairs of a cluster (few query rows): what a pair leaves for the merge.  Its fp32 output
+// goes where its key ring was, [column / 4][head][4]; reference maximum (log2 domain) and row sum of every head beside it.
+constexpr int LP_MAX_SPLIT = 8;
+struct LpSplitStats {
+    float m[LP_HEADS], l[LP_HEADS];
+};
+static_assert(LP_DVH * LP_HEADS * 4 <= LP_BUFS * LP_TILE_BYTES && sizeof(LpSplitStats) <= 2 * LP_XBUF_BYTES, "merge buffers reuse the ring and the exchange buffers");
+
 struct LpParams {
     const uint16_t* q;
     const uint16_t* pool;
@@ -113,7 +123,66 @@ __device__ __forceinline__ uint32_t lp_pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LP_THREADS, 1)
+__device__ __forceinline__ float lp_ld_cluster(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ float4 lp_ld_cluster4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+    return v;
+}
+
+// Output of token t from the `n_split` pairs' unnormalised outputs: CTA (s, c) takes every n_split-th block of 16 columns of value
+// half c, a thread one block of one head at a time.
+__device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s, int n_split, uint32_t c, uint32_t o_addr, uint32_t stats_addr) {
+    const int h = threadIdx.x & (LP_HEADS - 1);
+    float f[LP_MAX_SPLIT];
+    float m_all = __int_as_float(0xff800000), l_all = 0.f;
+#pragma unroll
+    for (int r = 0; r < LP_MAX_SPLIT; ++r) {
+        f[r] = r < n_split ? lp_ld_cluster(mapa_shared(stats_addr + 4 * h, 2 * r + c)) : __int_as_float(0xff800000);
+        m_all = fmaxf(m_all, f[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < LP_MAX_SPLIT; ++r) {
+        f[r] = m_all == __int_as_float(0xff800000) ? 0.f : lp_exp2(f[r] - m_all);
+        if (r < n_split) l_all += f[r] * lp_ld_cluster(mapa_shared(stats_addr + 4 * (LP_HEADS + h), 2 * r + c));
+    }
+    const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+    for (int blk = s + n_split * (threadIdx.x / LP_HEADS); blk < LP_DVH / 16; blk += n_split * (LP_THREADS / LP_HEADS)) {
+        float4 acc[4] = {};
+#pragma unroll
+        for (int r = 0; r < LP_MAX_SPLIT; ++r) {
+            if (r < n_split && f[r] != 0.f) {
+                const uint32_t src = mapa_shared(o_addr + static_cast<uint32_t>((blk * 4 * LP_HEADS + h) * 16), 2 * r + c);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const float4 x = lp_ld_cluster4(src + v * LP_HEADS * 16);
+                    acc[v].x = fmaf(f[r], x.x, acc[v].x); acc[v].y = fmaf(f[r], x.y, acc[v].y);
+                    acc[v].z = fmaf(f[r], x.z, acc[v].z); acc[v].w = fmaf(f[r], x.w, acc[v].w);
+                }
+            }
+        }
+        uint4* dst = reinterpret_cast<uint4*>(p.out + (static_cast<int64_t>(t) * LP_HEADS + h) * LP_DV + c * LP_DVH + blk * 16);
+        uint32_t w[8];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            w[2 * v] = lp_pack_bf16x2(acc[v].x * inv, acc[v].y * inv);
+            w[2 * v + 1] = lp_pack_bf16x2(acc[v].z * inv, acc[v].w * inv);
+        }
+        dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+    if (p.lse != nullptr && c == 0u && s == 0 && threadIdx.x < LP_HEADS)
+        p.lse[static_cast<int64_t>(t) * LP_HEADS + h] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : __int_as_float(0xff800000);
+}
+
+// SPLIT = false: clusters of two CTAs, persistent over tokens.  SPLIT = true: a cluster of 2 n CTAs takes one token, pair s of it
+// the tiles [s, s + 1) * n_tiles / n, and the pairs' outputs are merged through distributed shared memory at the end.
+template <bool SPLIT>
+__global__ void __launch_bounds__(LP_THREADS, 1)
 sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const LpParams p) {
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* k_smem = smem;                                              // 3 tiles x 5 atoms x [64 keys x 128 B]
@@ -122,15 +191,19 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     LpShared* sh = reinterpret_cast<LpShared*>(q_smem + LP_QS_BYTES);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t c = cluster_ctarank();          // 0 or 1: which bytes of the rows this CTA owns
-    const uint32_t peer = c ^ 1u;
+    const uint32_t rank = cluster_ctarank();
+    const uint32_t c = rank & 1u;                  // 0 or 1: which bytes of the rows this CTA owns
+    const uint32_t peer = rank ^ 1u;
     // persistent: cluster `cid` handles tokens cid, cid + n_clusters, ...; the key ring, the logit buffers and every barrier
     // phase run on across tokens (tiles are counted globally), so the next token's rows are gathered, and its queries
     // loaded, while the current token's last tiles and output are still in flight
-    const int cid = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-    const int n_my = cid < p.M ? (p.M - cid + n_clusters - 1) / n_clusters : 0;
+    const int n_split = SPLIT ? static_cast<int>(cluster_nctarank() >> 1) : 1;
+    const int cid = blockIdx.x / (2 * n_split), n_clusters = gridDim.x / (2 * n_split);
+    const int n_my = cid < p.M ? (p.M - cid + n_clusters - 1) / n_clusters : 0;     // SPLIT: one cluster per token, so 1
     const int n_atoms = 4 + static_cast<int>(c);
-    const int n_tiles = (p.k + LP_TILE - 1) / LP_TILE;
+    const int all_tiles = (p.k + LP_TILE - 1) / LP_TILE;
+    const int tile0 = SPLIT ? static_cast<int>(rank >> 1) * all_tiles / n_split : 0;
+    const int n_tiles = SPLIT ? (static_cast<int>(rank >> 1) + 1) * all_tiles / n_split - tile0 : all_tiles;
     const int n_half = 2 * n_tiles;
 
     if (threadIdx.x == 0) {
@@ -264,7 +337,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
         auto load_raw = [&](int gh) -> int {                   // lane r owns row r of global half-tile gh
             if (gh >= total_half) return -1;
             const int it = gh / n_half;
-            const int slot = (gh - it * n_half) * LP_HALF + lane;
+            const int slot = (2 * tile0 + gh - it * n_half) * LP_HALF + lane;
             const int64_t t_row = cid + it * n_clusters;
             if (p.table_offsets != nullptr) {                  // every query row has a page table of its own (a batch of sessions)
                 tbl_nxt = __ldg(p.table_offsets + t_row);
@@ -426,6 +499,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
         const float neg_inf = __int_as_float(0xff800000);
         const bool out_al32 = (reinterpret_cast<uint64_t>(p.out) & 31u) == 0u;
         bool ok = true;
+        bool merged = false;        // SPLIT: the output was left for the merge
         const uint32_t peer_xempty = mapa_shared(smem_u32(&sh->x_empty[0]), peer);
         int gi = 0;                 // tiles done so far, over all tokens
         for (int it = 0; it < n_my && ok; ++it) {
@@ -552,8 +626,30 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
-        const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
         const bool have_o = __any_sync(0xffffffffu, l_sum > 0.f);   // some P.V of this token has written O
+        if constexpr (SPLIT) {
+            // this pair's last P.V is complete, so nothing reads the ring or the exchange buffer any more: leave O for the merge
+            float* mo = reinterpret_cast<float*>(k_smem);
+            LpSplitStats* stats = reinterpret_cast<LpSplitStats*>(xbuf);
+            stats->m[h] = m_ref;
+            stats->l[h] = l_sum;
+#pragma unroll 1
+            for (int cc = 0; cc < LP_DVH / 32; ++cc) {
+                uint32_t o[32];
+                if (have_o) {
+                    tmem_ld32_wait(lane_addr + LP_COL_O + cc * 32, o);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) o[j] = 0u;
+                }
+#pragma unroll
+                for (int v = 0; v < 8; ++v)
+                    *reinterpret_cast<uint4*>(mo + ((cc * 8 + v) * LP_HEADS + h) * 4) = make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
+            }
+            merged = true;
+            break;
+        }
+        const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
         uint16_t* orow = p.out + (static_cast<int64_t>(t) * LP_HEADS + h) * LP_DV + c * LP_DVH;
 #pragma unroll 1
         for (int cc = 0; cc < LP_DVH / 32; ++cc) {
@@ -580,12 +676,21 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
             p.lse[static_cast<int64_t>(t) * LP_HEADS + h] = l_sum > 0.f ? (m_ref + log2f(l_sum)) * 0.6931471805599453f : neg_inf;
         }
         if (!ok && lane == 0) report(p.dev_status, JANUS_DEV_WAIT_TIMEOUT);
+        if (SPLIT && !merged) {     // gave up: the merge below reads zeros instead of leftovers
+            LpSplitStats* stats = reinterpret_cast<LpSplitStats*>(xbuf);
+            stats->m[h] = neg_inf;
+            stats->l[h] = 0.f;
+        }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
+    }
+    if constexpr (SPLIT) {
+        cluster_sync_all();         // every pair's output lies in its shared memory
+        if (!start_abort && n_my > 0) lp_merge_splits(p, cid, static_cast<int>(rank >> 1), n_split, c, smem_u32(k_smem), smem_u32(xbuf));
     }
     cluster_sync_all();   // neither CTA leaves while the other may still write into its shared memory or arrive on its barriers
 }
@@ -596,6 +701,53 @@ bool sparse_attn_latent_tc_supported(int M, int H_q, int d_qk, const void* k_poo
     if ((page_stride % 8) != 0 || (tok_stride % 8) != 0 || tok_stride < LP_DQK) return false;
     if (M > (1 << 30) / LP_HEADS || k <= 0) return false;
     return true;
+}
+
+static cudaLaunchConfig_t lp_launch_config(int cluster_size, int n_clusters, size_t smem, cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(cluster_size) * n_clusters);
+    cfg.blockDim = dim3(LP_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = cluster_size;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// n[s] = clusters of 2 s CTAs the device keeps resident at once (one CTA per SM), 0 where it takes none.  A property of the
+// device, asked for on its first call; so are the kernels' attributes.
+static int lp_resident_clusters(int dev, size_t smem, int (&n)[LP_MAX_SPLIT + 1]) {
+    constexpr int MAX_DEVICES = 64;
+    static std::mutex mu;
+    static int known[MAX_DEVICES][LP_MAX_SPLIT + 1] = {};
+    if (dev < 0 || dev >= MAX_DEVICES) return JANUS_ERR_UNSUPPORTED;
+    std::lock_guard<std::mutex> lock(mu);
+    int (&k)[LP_MAX_SPLIT + 1] = known[dev];
+    if (k[1] == 0) {
+        JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        for (int s = LP_MAX_SPLIT; s >= 1; --s) {
+            cudaLaunchAttribute attr;
+            const cudaLaunchConfig_t cfg = lp_launch_config(2 * s, 148, smem, &attr);
+            const cudaError_t e = s > 1 ? cudaOccupancyMaxActiveClusters(&k[s], sparse_attn_latent_pair_kernel<true>, &cfg)
+                                        : cudaOccupancyMaxActiveClusters(&k[s], sparse_attn_latent_pair_kernel<false>, &cfg);
+            if (e != cudaSuccess) {
+                (void)cudaGetLastError();
+                k[s] = 0;
+            }
+        }
+        if (k[1] <= 0) {
+            int sms = 0;
+            JANUS_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+            k[1] = sms > 2 ? sms / 2 : 1;
+        }
+    }
+    for (int s = 0; s <= LP_MAX_SPLIT; ++s) n[s] = k[s];
+    return JANUS_OK;
 }
 
 int launch_sparse_attn_latent_tc(const void* q, int M, const void* pool, int64_t page_stride, int64_t tok_stride, const int32_t* idx, int k,
@@ -627,36 +779,30 @@ int launch_sparse_attn_latent_tc(const void* q, int M, const void* pool, int64_t
         return JANUS_ERR_CUDA;
     const size_t smem = LP_BUFS * LP_TILE_BYTES + 2 * LP_XBUF_BYTES + LP_QS_BYTES + sizeof(LpShared) + 16;
     static_assert(LP_BUFS * LP_TILE_BYTES + 2 * LP_XBUF_BYTES + LP_QS_BYTES + sizeof(LpShared) + 16 <= 227 * 1024, "shared memory");
-    JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_latent_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    // persistent launch: as many 2-CTA clusters as the device keeps resident at once (one CTA per SM), each looping over tokens
-    static int resident_clusters[64] = {};
     int dev = 0;
     JANUS_CUDA_CHECK(cudaGetDevice(&dev));
-    int n_clusters = (dev >= 0 && dev < 64) ? resident_clusters[dev] : 0;
-    if (n_clusters <= 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2 * 148);
-        cfg.blockDim = dim3(LP_THREADS);
-        cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&n_clusters, sparse_attn_latent_pair_kernel, &cfg) != cudaSuccess || n_clusters <= 0) {
-            (void)cudaGetLastError();
-            int sms = 0;
-            JANUS_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-            n_clusters = sms / 2;
-        }
-        if (n_clusters <= 0) n_clusters = 1;
-        if (dev >= 0 && dev < 64) resident_clusters[dev] = n_clusters;
+    int n_resident[LP_MAX_SPLIT + 1];
+    const int rc = lp_resident_clusters(dev, smem, n_resident);
+    if (rc != JANUS_OK) return rc;
+    // A pair takes 1.16 us per tile of 64 keys and 8.7 us around them.  While the tokens are few, clusters of 2 n CTAs share a
+    // token's tiles; the merge, whose 112 KB per CTA cross the SM-to-SM network, makes that 12 + 0.6 n us.  The n with the least
+    // waves x time is taken.  Measured at 2048 keys: 1 token 45.8 us with one pair, 31.4 / 26.1 / 24.2 / 21.5 with 2 / 3 / 4 / 8;
+    // 19 tokens 47.6, 32.9 and 28.4 with 1, 2 and 3 (22 clusters of six CTAs are resident at once), 49.0 with 4 (two waves);
+    // 512 keys: 18.0 with one pair, 17.5 and 16.7 with 2 and 3.
+    const int all_tiles = (k + LP_TILE - 1) / LP_TILE;
+    int split = 1;
+    double best = 0.;
+    for (int n = 1; n <= LP_MAX_SPLIT && n <= all_tiles; ++n) {
+        if (n_resident[n] <= 0) break;
+        const double t = ((M + n_resident[n] - 1) / n_resident[n]) * (((all_tiles + n - 1) / n) * 1.16 + (n > 1 ? 12. + 0.6 * n : 8.7));
+        if (n == 1 || t < best) { best = t; split = n; }
     }
-    if (n_clusters > M) n_clusters = M;
-    sparse_attn_latent_pair_kernel<<<2 * n_clusters, LP_THREADS, smem, stream>>>(tq, p);   // clusters of 2 CTAs (compile-time cluster dims)
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    const int n_clusters = split > 1 ? M : (M < n_resident[1] ? M : n_resident[1]);     // one pair per cluster: persistent over tokens
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = lp_launch_config(2 * split, n_clusters, smem, &attr);
+    cfg.stream = stream;
+    if (split > 1) JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sparse_attn_latent_pair_kernel<true>, tq, p));
+    else JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sparse_attn_latent_pair_kernel<false>, tq, p));
     return JANUS_OK;
 }
 
