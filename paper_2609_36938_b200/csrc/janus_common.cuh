@@ -6,6 +6,8 @@
 #include <cuda_fp8.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/janus.h"
 
 namespace janus {
@@ -21,6 +23,26 @@ void set_last_cuda_error(cudaError_t e);
             return JANUS_ERR_CUDA;                     \
         }                                              \
     } while (0)
+
+// Runs a function once on every device (kernel attributes: they stay set, and setting them on each call costs a microsecond).
+class once_per_device {
+  public:
+    template <class F>
+    cudaError_t run(F&& f) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 0 || dev >= 64) return f();
+        const uint64_t bit = uint64_t(1) << dev;
+        if ((done_.load(std::memory_order_acquire) & bit) != 0) return cudaSuccess;
+        e = f();
+        if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_release);
+        return e;
+    }
+
+  private:
+    std::atomic<uint64_t> done_{0};
+};
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -75,45 +97,6 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int* 
     __syncthreads();
     *total = warp_sums[32];
     return warp_sums[warp] + incl - v;
-}
-
-// The same for three ints per thread at once (one set of barriers instead of three).  `warp_sums` holds 3 x 33 ints.
-template <int THREADS>
-__device__ __forceinline__ void block_exclusive_scan3(int (&v)[3], int* warp_sums, int (&excl)[3], int (&total)[3]) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl[3] = {v[0], v[1], v[2]};
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const int y = __shfl_up_sync(0xffffffffu, incl[q], d);
-            if (lane >= d) incl[q] += y;
-        }
-    }
-    __syncthreads();  // protect warp_sums from a previous use
-    if (lane == 31) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) warp_sums[33 * q + warp] = incl[q];
-    }
-    __syncthreads();
-    if (warp < 3) {   // warp q scans the warp totals of value q
-        const int q = warp;
-        const int sv = (lane < THREADS / 32) ? warp_sums[33 * q + lane] : 0;
-        int si = sv;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, si, d);
-            if (lane >= d) si += y;
-        }
-        if (lane < THREADS / 32) warp_sums[33 * q + lane] = si - sv;
-        if (lane == 31) warp_sums[33 * q + 32] = si;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        total[q] = warp_sums[33 * q + 32];
-        excl[q] = warp_sums[33 * q + warp] + incl[q] - v[q];
-    }
 }
 
 }  // namespace janus

@@ -2,269 +2,422 @@
 // maximal runs of adjacent physical pages, and the miss set "exact minus predicted"
 // (union of selections: Sec. 2.2; corrective reads: Sec. 4.2; read packing: Sec. 4.3).
 //
-// Kernel 1 (mark) streams the index block with 16-byte loads and sets page bits.  When the bitmap
-// fits in shared memory each CTA ORs into a private copy first and only touches a global word once
-// per CTA; bits are tested before the atomic so a saturated union costs no atomics at all.
-// Kernel 2 (lists) is one CTA that turns a bitmap into ordered lists with block-wide scans.
+// Latency bounds all of it: a few hundred kilobytes in, a few kilobytes out, but several dependent steps.  Up to a million
+// indices one launch of one cluster does everything (page_demand_kernel): every CTA marks its share of the indices in a private
+// bitmap in shared memory, the cluster ORs the bitmaps slice by slice through distributed shared memory, and each CTA
+// turns its slice of the set into its part of the lists, offsets coming from one exchange of the CTAs' counts.  Larger blocks of
+// indices are marked by the whole chip first (page_mark_kernel, one bitmap of *logical* pages per CTA, so that an index costs
+// one shared-memory test and the page table is read once per page and CTA), and the same kernel then only makes the lists.
 #include "janus_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace janus {
 
-constexpr int MARK_THREADS = 256;
-constexpr int MARK_SMEM_WORDS = 8192;  // 32 KB: bitmaps up to 262144 pages stay in shared memory
-constexpr int LIST_THREADS = 1024;
+using namespace ptx;
 
-__device__ __forceinline__ void mark_one(int s, int64_t demand_limit, int page_size, int page_shift,
-                                         const int32_t* __restrict__ page_table, int64_t n_logical_pages,
-                                         int64_t n_phys_pages, uint32_t* bm, int32_t* dev_status) {
-    if (s < 0 || static_cast<int64_t>(s) >= demand_limit) return;
-    const int64_t lp = page_shift >= 0 ? (s >> page_shift) : (s / page_size);
-    if (lp >= n_logical_pages) { report(dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE); return; }
-    const int32_t p = __ldg(page_table + lp);
-    if (p < 0 || static_cast<int64_t>(p) >= n_phys_pages) { report(dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE); return; }
+constexpr int PD_THREADS = 1024;
+constexpr int PD_MAX_CLUSTER = 16;
+constexpr int PD_SMEM_WORDS = PD_MAX_CLUSTER * PD_THREADS;      // private bitmap of a CTA: up to 64 KB, half a million pages
+constexpr int MARK_THREADS = 1024;
+constexpr int MARK_SMEM_WORDS = 24576;             // bitmaps of logical and physical pages of a marking CTA together: 96 KB, two CTAs per SM
+
+enum { PD_LISTS = 0, PD_MARK = 1, PD_MARK_ROWS = 2 };      // what page_demand_kernel does before the lists
+
+struct PdParams {
+    const int32_t* idx;
+    int64_t n_idx;
+    int k;
+    int64_t demand_limit;                 // PD_MARK
+    const int64_t* demand_limits;         // PD_MARK_ROWS: per row
+    int page_size, page_shift;
+    const int32_t* page_table;
+    int64_t n_logical_pages;              // PD_MARK
+    const int64_t* table_offsets;         // PD_MARK_ROWS: row r uses page_table[table_offsets[r] .. table_offsets[r + 1])
+    int64_t n_phys_pages;
+    int n_words;
+    const uint32_t* predicted;            // may be NULL
+    uint32_t* bitmap;
+    int32_t *pages, *n_pages, *runs, *n_runs, *miss_pages, *n_miss, *miss_runs, *n_miss_runs;
+    int64_t capacity;
+    int32_t* dev_status;
+};
+
+struct PageDiv {      // token -> logical page
+    int size, shift;
+    __device__ __forceinline__ int64_t operator()(int s) const { return shift >= 0 ? (s >> shift) : (s / size); }
+};
+
+// Sets bit p of a bitmap in shared memory; tested first, because most pages are already there.
+__device__ __forceinline__ void set_bit_shared(uint32_t* bm, int p) {
     const uint32_t bit = 1u << (p & 31);
-    uint32_t* wp = bm + (p >> 5);
-    if ((*reinterpret_cast<volatile uint32_t*>(wp) & bit) == 0u) atomicOr(wp, bit);
+    uint32_t* w = bm + (p >> 5);
+    if ((*reinterpret_cast<volatile uint32_t*>(w) & bit) == 0u) atomicOr(w, bit);
 }
 
-template <bool USE_SMEM>
+// ---- marking by the whole chip ----------------------------------------------------------------------------------------------
+// A CTA's tokens become bits of its own bitmap of logical pages; at the end its set pages go through the page table into a
+// bitmap of physical pages, whose words are ORed into the global one (page by page they would be a contended atomic each:
+// 109 us).
+// Whole call at 4096 x 2048 indices: 35 us when every index went through the page table, 25.9 now; 8192 x 2048: 65.8 and 36.9.
 __global__ void __launch_bounds__(MARK_THREADS)
-page_mark_kernel(const int32_t* __restrict__ idx, int64_t n_idx, int64_t demand_limit, int page_size, int page_shift,
-                 const int32_t* __restrict__ page_table, int64_t n_logical_pages, int64_t n_phys_pages,
-                 uint32_t* __restrict__ bitmap, int n_words, int32_t* dev_status) {
-    __shared__ uint32_t sbm[USE_SMEM ? MARK_SMEM_WORDS : 1];
-    uint32_t* bm = bitmap;
-    if (USE_SMEM) {
-        for (int i = threadIdx.x; i < n_words; i += MARK_THREADS) sbm[i] = 0u;
-        __syncthreads();
-        bm = sbm;
-    }
-    const int64_t n_vec = n_idx >> 2;  // idx is 16-byte aligned
-    const int4* idx4 = reinterpret_cast<const int4*>(idx);
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * MARK_THREADS;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * MARK_THREADS + threadIdx.x; i < n_vec; i += stride) {
-        const int4 v = __ldg(idx4 + i);
-        mark_one(v.x, demand_limit, page_size, page_shift, page_table, n_logical_pages, n_phys_pages, bm, dev_status);
-        mark_one(v.y, demand_limit, page_size, page_shift, page_table, n_logical_pages, n_phys_pages, bm, dev_status);
-        mark_one(v.z, demand_limit, page_size, page_shift, page_table, n_logical_pages, n_phys_pages, bm, dev_status);
-        mark_one(v.w, demand_limit, page_size, page_shift, page_table, n_logical_pages, n_phys_pages, bm, dev_status);
-    }
-    if (blockIdx.x == 0) {
-        for (int64_t i = (n_vec << 2) + threadIdx.x; i < n_idx; i += MARK_THREADS)
-            mark_one(idx[i], demand_limit, page_size, page_shift, page_table, n_logical_pages, n_phys_pages, bm, dev_status);
-    }
-    if (USE_SMEM) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < n_words; i += MARK_THREADS) {
-            const uint32_t v = sbm[i];
-            if (v != 0u && (__ldcg(bitmap + i) & v) != v) atomicOr(bitmap + i, v);
+page_mark_kernel(const PdParams p, int n_log_words) {
+    extern __shared__ uint32_t lbm[];
+    uint32_t* pbm = lbm + n_log_words;
+    for (int i = threadIdx.x; i < n_log_words + p.n_words; i += MARK_THREADS) lbm[i] = 0u;
+    __syncthreads();
+    const PageDiv page{p.page_size, p.page_shift};
+    bool bad = false;
+    // four tokens at a time: their words are read together, and a bit is set only where it is not there yet
+    auto mark4 = [&](const int4& v) {
+        const int s[4] = {v.x, v.y, v.z, v.w};
+        int lp[4];
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            lp[e] = -1;
+            if (s[e] >= 0 && s[e] < p.demand_limit) {
+                const int64_t l = page(s[e]);
+                if (l >= p.n_logical_pages) bad = true;
+                else lp[e] = static_cast<int>(l);
+            }
+            w[e] = lp[e] >= 0 ? lbm[lp[e] >> 5] : 0xffffffffu;
         }
-    }
-}
-
-// Turns one bitmap (optionally "a AND NOT b") into: ascending ids, maximal runs, counts.
-// Single CTA; words are consumed LIST_THREADS at a time, one word per thread.
-__device__ void bitmap_to_lists(const uint32_t* __restrict__ a, const uint32_t* __restrict__ not_b, int n_words,
-                                int64_t n_bits, int32_t* __restrict__ ids, int32_t* __restrict__ n_ids,
-                                int32_t* __restrict__ runs, int32_t* __restrict__ n_runs, int64_t capacity,
-                                int32_t* dev_status, int* scan_scratch) {
-    int id_base = 0, run_base = 0, end_base = 0;
-    auto word_at = [&](int i) -> uint32_t {
-        if (i < 0 || i >= n_words) return 0u;
-        uint32_t v = a[i];
-        if (not_b != nullptr) v &= ~not_b[i];
-        if (i == n_words - 1 && (n_bits & 31)) v &= (1u << (n_bits & 31)) - 1u;  // ignore bits past the last page
-        return v;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (((w[e] >> (lp[e] & 31)) & 1u) == 0u) atomicOr(lbm + (lp[e] >> 5), 1u << (lp[e] & 31));
     };
-    for (int base = 0; base < n_words; base += LIST_THREADS) {
-        const int i = base + threadIdx.x;
-        const uint32_t v = word_at(i);
-        const uint32_t prev_top = word_at(i - 1) >> 31;
-        const uint32_t next_bot = word_at(i + 1) & 1u;
-        const uint32_t starts = v & ~((v << 1) | prev_top);          // set, and the page below is not
-        const uint32_t ends = v & ~((v >> 1) | (next_bot << 31));    // set, and the page above is not
-        int tot_ids, tot_starts, tot_ends;
-        int o_id = block_exclusive_scan<LIST_THREADS>(__popc(v), scan_scratch, &tot_ids) + id_base;
-        int o_st = block_exclusive_scan<LIST_THREADS>(__popc(starts), scan_scratch, &tot_starts) + run_base;
-        int o_en = block_exclusive_scan<LIST_THREADS>(__popc(ends), scan_scratch, &tot_ends) + end_base;
-        uint32_t m = v;
-        while (m) {
-            const int b = __ffs(m) - 1;
-            m &= m - 1;
-            if (o_id < capacity) ids[o_id] = i * 32 + b;
-            ++o_id;
-        }
-        m = starts;
-        while (m) {
-            const int b = __ffs(m) - 1;
-            m &= m - 1;
-            if (o_st < capacity) runs[2 * o_st] = i * 32 + b;
-            ++o_st;
-        }
-        m = ends;
-        while (m) {  // the j-th end closes the j-th start; store end+1, converted to a length below
-            const int b = __ffs(m) - 1;
-            m &= m - 1;
-            if (o_en < capacity) runs[2 * o_en + 1] = i * 32 + b + 1;
-            ++o_en;
-        }
-        id_base += tot_ids;
-        run_base += tot_starts;
-        end_base += tot_ends;
+    const int4* idx4 = reinterpret_cast<const int4*>(p.idx);      // 16-byte aligned
+    const int64_t n_vec = p.n_idx >> 2, stride = static_cast<int64_t>(gridDim.x) * MARK_THREADS;
+    int64_t i = static_cast<int64_t>(blockIdx.x) * MARK_THREADS + threadIdx.x;
+    for (; i + 3 * stride < n_vec; i += 4 * stride) {
+        int4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(idx4 + i + u * stride);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) mark4(v[u]);
+    }
+    for (; i < n_vec; i += stride) mark4(__ldg(idx4 + i));
+    if (blockIdx.x == 0 && threadIdx.x < (p.n_idx & 3)) mark4(make_int4(p.idx[(n_vec << 2) + threadIdx.x], -1, -1, -1));
+    __syncthreads();
+    for (int lp = threadIdx.x; lp < n_log_words * 32; lp += MARK_THREADS) {
+        if (((lbm[lp >> 5] >> (lp & 31)) & 1u) == 0u) continue;
+        const int32_t q = __ldg(p.page_table + lp);
+        if (q < 0 || q >= p.n_phys_pages) bad = true;
+        else atomicOr(pbm + (q >> 5), 1u << (q & 31));
     }
     __syncthreads();
-    const int n_r = run_base < capacity ? run_base : static_cast<int>(capacity);
-    for (int j = threadIdx.x; j < n_r; j += LIST_THREADS) runs[2 * j + 1] -= runs[2 * j];
-    if (threadIdx.x == 0) {
-        *n_ids = id_base;
-        *n_runs = run_base;
-        if (id_base > capacity || run_base > capacity) report(dev_status, JANUS_DEV_CAPACITY_EXCEEDED);
+    for (int w = threadIdx.x; w < p.n_words; w += MARK_THREADS) {
+        const uint32_t v = pbm[w];
+        if (v != 0u && (__ldcg(p.bitmap + w) & v) != v) atomicOr(p.bitmap + w, v);
+    }
+    if (bad) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
+}
+
+// Physical page of a token, -1 for none (padding, past the limit) and after reporting what is out of range.
+__device__ __forceinline__ int32_t page_of_token(int s, int64_t limit, const PageDiv& page, const int32_t* __restrict__ table, int64_t n_logical,
+                                                 int64_t n_phys, bool& bad) {
+    if (s < 0 || s >= limit) return -1;
+    const int64_t lp = page(s);
+    const int32_t q = lp < n_logical ? __ldg(table + lp) : -1;
+    if (q < 0 || q >= n_phys) { bad = true; return -1; }
+    return q;
+}
+
+// Tables or pools whose bitmaps do not fit shared memory: straight into the global bitmap.
+template <int MODE>
+__global__ void __launch_bounds__(256)
+page_mark_global_kernel(const PdParams p) {
+    const PageDiv page{p.page_size, p.page_shift};
+    bool bad = false;
+    for (int64_t e = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; e < p.n_idx; e += static_cast<int64_t>(gridDim.x) * 256) {
+        const int32_t* table = p.page_table;
+        int64_t n_log = p.n_logical_pages, limit = p.demand_limit;
+        if (MODE == PD_MARK_ROWS) {
+            const int64_t r = e / p.k, off = __ldg(p.table_offsets + r);
+            n_log = off < 0 ? 0 : __ldg(p.table_offsets + r + 1) - off;       // a table that starts before the array has no pages
+            table += off < 0 ? 0 : off;
+            limit = __ldg(p.demand_limits + r);
+        }
+        const int32_t q = page_of_token(__ldg(p.idx + e), limit, page, table, n_log, p.n_phys_pages, bad);
+        if (q < 0) continue;
+        const uint32_t bit = 1u << (q & 31);
+        if ((__ldcg(p.bitmap + (q >> 5)) & bit) == 0u) atomicOr(p.bitmap + (q >> 5), bit);
+    }
+    if (bad) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
+}
+
+// ---- one cluster: marking (optional) and the lists -----------------------------------------------------------------------------
+// Counts of a set up to some place, both in one 64-bit word so that they are scanned together: ids in the high half, run
+// starts in the low half.  The run ends before a word are the starts before it less the run that reaches into it.
+struct PdShared {
+    uint64_t warp_sums[2][33];
+    uint64_t totals[2];                       // this CTA's slice: the set, the miss set
+    uint64_t at[2][PD_THREADS];               // counts before each word of a chunk
+    uint32_t word[2][PD_THREADS + 2];         // the words of a chunk and one neighbour on either side
+};
+
+__device__ __forceinline__ void block_scan2_u64(uint64_t (&v)[2], uint64_t (*warp_sums)[33], uint64_t (&excl)[2], uint64_t (&total)[2]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint64_t incl[2] = {v[0], v[1]};
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const uint64_t y = __shfl_up_sync(0xffffffffu, incl[q], d);
+            if (lane >= d) incl[q] += y;
+        }
+    }
+    __syncthreads();                  // warp_sums is free again
+    if (lane == 31) { warp_sums[0][warp] = incl[0]; warp_sums[1][warp] = incl[1]; }
+    __syncthreads();
+    if (warp < 2) {                   // warp q scans the 32 warp totals of value q
+        const uint64_t sv = warp_sums[warp][lane];
+        uint64_t si = sv;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t y = __shfl_up_sync(0xffffffffu, si, d);
+            if (lane >= d) si += y;
+        }
+        warp_sums[warp][lane] = si - sv;
+        if (lane == 31) warp_sums[warp][32] = si;
     }
     __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        total[q] = warp_sums[q][32];
+        excl[q] = warp_sums[q][warp] + incl[q] - v[q];
+    }
 }
 
-__global__ void __launch_bounds__(LIST_THREADS)
-page_lists_kernel(const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ predicted, int n_words, int64_t n_phys_pages,
-                  int32_t* pages, int32_t* n_pages, int32_t* runs, int32_t* n_runs,
-                  int32_t* miss_pages, int32_t* n_miss, int32_t* miss_runs, int32_t* n_miss_runs,
-                  int64_t capacity, int32_t* dev_status) {
-    __shared__ int scan_scratch[40];
-    bitmap_to_lists(bitmap, nullptr, n_words, n_phys_pages, pages, n_pages, runs, n_runs, capacity, dev_status, scan_scratch);
-    if (miss_pages != nullptr)
-        bitmap_to_lists(bitmap, predicted, n_words, n_phys_pages, miss_pages, n_miss, miss_runs, n_miss_runs, capacity,
-                        dev_status, scan_scratch);
-}
+template <int MODE>
+__global__ void __launch_bounds__(PD_THREADS)
+page_demand_kernel(const PdParams p) {
+    extern __shared__ uint32_t bm[];      // private bitmap (marking modes)
+    __shared__ PdShared sh;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = static_cast<int>(cluster_ctarank()), n_cta = static_cast<int>(cluster_nctarank());
+    const int wps = (p.n_words + n_cta - 1) / n_cta;        // words of a slice; at most one chunk of PD_THREADS in the marking modes
+    const int w0 = min(p.n_words, rank * wps), w1 = min(p.n_words, w0 + wps);
 
-// Large pools (a decode batch addresses the whole KV pool: 10^5 pages and more): the same lists built by one CTA per
-// 1024-word chunk.  A CTA first counts the ids / run starts / run ends of all words before its chunk (a few KB of bitmap
-// for the sizes this path is used for), then writes its part exactly like the single-CTA kernel; run lengths need every
-// start and end, so a small second kernel turns (start, end+1) into (start, length).  blockIdx.y = 0: the set itself,
-// 1: the miss set (bitmap AND NOT predicted).
-constexpr int LIST_MAX_CHUNKS = 64;
+    if constexpr (MODE != PD_LISTS) {
+        for (int i = tid; i < p.n_words; i += PD_THREADS) bm[i] = 0u;
+        __syncthreads();
+        const PageDiv page{p.page_size, p.page_shift};
+        bool bad = false;
+        constexpr int U = 8;              // indices, then table entries, in flight per thread
+        const int stride = n_cta * PD_THREADS, n_idx = static_cast<int>(p.n_idx);
+        for (int base = rank * PD_THREADS + tid; base < n_idx; base += U * stride) {
+            int s[U];
+            int32_t q[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) s[u] = base + u * stride < n_idx ? __ldg(p.idx + base + u * stride) : -1;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int32_t* table = p.page_table;
+                int64_t n_log = p.n_logical_pages, limit = p.demand_limit;
+                if (MODE == PD_MARK_ROWS && s[u] >= 0) {
+                    const int r = (base + u * stride) / p.k;
+                    const int64_t off = __ldg(p.table_offsets + r);
+                    n_log = off < 0 ? 0 : __ldg(p.table_offsets + r + 1) - off;       // a table that starts before the array has no pages
+                    table += off < 0 ? 0 : off;
+                    limit = __ldg(p.demand_limits + r);
+                }
+                q[u] = page_of_token(s[u], limit, page, table, n_log, p.n_phys_pages, bad);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (q[u] >= 0) set_bit_shared(bm, q[u]);
+        }
+        if (bad) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
+        cluster_sync_all();               // every private bitmap is complete
+    }
 
-__global__ void __launch_bounds__(LIST_THREADS)
-page_lists_chunk_kernel(const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ predicted, int n_words, int64_t n_phys_pages,
-                        int32_t* pages, int32_t* n_pages, int32_t* runs, int32_t* n_runs, int32_t* miss_pages, int32_t* n_miss,
-                        int32_t* miss_runs, int32_t* n_miss_runs, int64_t capacity, int32_t* dev_status) {
-    __shared__ int scan_scratch[3 * 33];
-    const bool miss = blockIdx.y == 1;
-    const uint32_t* a = bitmap;
-    const uint32_t* not_b = miss ? predicted : nullptr;
-    int32_t* ids = miss ? miss_pages : pages;
-    int32_t* n_ids = miss ? n_miss : n_pages;
-    int32_t* out_runs = miss ? miss_runs : runs;
-    int32_t* out_n_runs = miss ? n_miss_runs : n_runs;
-    auto word_at = [&](int i) -> uint32_t {
-        if (i < 0 || i >= n_words) return 0u;
-        uint32_t v = a[i];
-        if (not_b != nullptr) v &= ~not_b[i];
-        if (i == n_words - 1 && (n_phys_pages & 31)) v &= (1u << (n_phys_pages & 31)) - 1u;
-        return v;
+    // ---- lists of this CTA's slice, a chunk of words at a time
+    const bool want_miss = p.miss_pages != nullptr;
+    // word i of the set: ORed over the CTAs' bitmaps, or as page_mark_kernel left it
+    auto union_word = [&](int i) -> uint32_t {
+        if (i < 0 || i >= p.n_words) return 0u;
+        if constexpr (MODE == PD_LISTS) {
+            return __ldcg(p.bitmap + i);
+        } else {
+            const uint32_t addr = smem_u32(bm + i);
+            uint32_t v = 0u;
+#pragma unroll
+            for (int r = 0; r < PD_MAX_CLUSTER; ++r)
+                if (r < n_cta) v |= ld_cluster_u32(mapa_shared(addr, r));
+            return v;
+        }
     };
-    auto starts_of = [&](int i, uint32_t v) { return v & ~((v << 1) | (word_at(i - 1) >> 31)); };
-    auto ends_of = [&](int i, uint32_t v) { return v & ~((v >> 1) | ((word_at(i + 1) & 1u) << 31)); };
-    const int base = blockIdx.x * LIST_THREADS;
-    // ---- everything before this chunk
-    int c_id = 0, c_st = 0, c_en = 0;
-    for (int i = threadIdx.x; i < base; i += LIST_THREADS) {
-        const uint32_t v = word_at(i);
-        c_id += __popc(v);
-        c_st += __popc(starts_of(i, v));
-        c_en += __popc(ends_of(i, v));
+    auto load_chunk = [&](int c0) {       // words c0 - 1 .. c0 + PD_THREADS, cut off at the slice's end + 1
+        __syncthreads();
+        for (int j = tid; j < PD_THREADS + 2; j += PD_THREADS) {
+            const int i = c0 - 1 + j;
+            const uint32_t v = i <= w1 ? union_word(i) : 0u;
+            sh.word[0][j] = v;
+            if (want_miss) sh.word[1][j] = v == 0u || p.predicted == nullptr ? v : v & ~__ldcg(p.predicted + i);
+            if (MODE != PD_LISTS && i >= w0 && i < w1) p.bitmap[i] = v;
+        }
+        __syncthreads();
+    };
+    auto count_chunk = [&](int c0, uint64_t (&mine)[2]) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            mine[q] = 0;
+            if (c0 + tid < w1 && (q == 0 || want_miss)) {
+                const uint32_t v = sh.word[q][tid + 1];
+                mine[q] = static_cast<uint64_t>(__popc(v)) << 32 | static_cast<uint64_t>(__popc(v & ~((v << 1) | (sh.word[q][tid] >> 31))));
+            }
+        }
+    };
+    const bool one_chunk = wps <= PD_THREADS;
+    uint64_t excl[2] = {0, 0}, sum[2] = {0, 0};
+    if (one_chunk) {                      // the scan of the only chunk gives the slice's counts as well
+        uint64_t mine[2];
+        load_chunk(w0);
+        count_chunk(w0, mine);
+        block_scan2_u64(mine, sh.warp_sums, excl, sum);
+    } else {
+        uint64_t mine[2] = {0, 0};
+        for (int c0 = w0; c0 < w1; c0 += PD_THREADS) {
+            uint64_t part[2];
+            load_chunk(c0);
+            count_chunk(c0, part);
+            mine[0] += part[0];
+            mine[1] += part[1];
+        }
+        block_scan2_u64(mine, sh.warp_sums, excl, sum);
     }
-    // ids, run starts and run ends are scanned together: one set of block barriers per scan instead of three
-    int before[3] = {c_id, c_st, c_en}, skip[3], bases[3];
-    block_exclusive_scan3<LIST_THREADS>(before, scan_scratch, skip, bases);
-    const int id_base = bases[0], run_base = bases[1], end_base = bases[2];
-    // ---- this chunk
-    const int i = base + threadIdx.x;
-    const uint32_t v = word_at(i);
-    const uint32_t starts = starts_of(i, v), ends = ends_of(i, v);
-    int mine[3] = {__popc(v), __popc(starts), __popc(ends)}, offs[3], tots[3];
-    block_exclusive_scan3<LIST_THREADS>(mine, scan_scratch, offs, tots);
-    const int tot_ids = tots[0], tot_starts = tots[1];
-    int o_id = offs[0] + id_base, o_st = offs[1] + run_base, o_en = offs[2] + end_base;
-    uint32_t m = v;
-    while (m) {
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        if (o_id < capacity) ids[o_id] = i * 32 + b;
-        ++o_id;
+    if (tid == 0) { sh.totals[0] = sum[0]; sh.totals[1] = sum[1]; }
+    cluster_sync_all();                   // counts are there; nobody reads the private bitmaps any more
+    uint64_t base[2] = {0, 0}, all[2] = {0, 0};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const uint32_t addr = smem_u32(&sh.totals[q]);
+#pragma unroll
+        for (int r = 0; r < PD_MAX_CLUSTER; ++r) {
+            if (r < n_cta) {
+                const uint64_t x = ld_cluster_u64(mapa_shared(addr, r));
+                all[q] += x;
+                if (r < rank) base[q] += x;
+            }
+        }
     }
-    m = starts;
-    while (m) {
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        if (o_st < capacity) out_runs[2 * o_st] = i * 32 + b;
-        ++o_st;
+    for (int c0 = w0; c0 < w1; c0 += PD_THREADS) {
+        if (!one_chunk) {
+            uint64_t mine[2];
+            load_chunk(c0);
+            count_chunk(c0, mine);
+            block_scan2_u64(mine, sh.warp_sums, excl, sum);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) sh.at[q][tid] = base[q] + excl[q];
+        __syncthreads();
+        // a warp writes one word's entries at a time, a lane per page: neighbouring entries leave in one store
+        const int n_in = min(PD_THREADS, w1 - c0);
+        for (int jq = warp; jq < (want_miss ? 2 * n_in : n_in); jq += PD_THREADS / 32) {
+            const int q = jq >= n_in ? 1 : 0, j = jq - q * n_in;
+            const uint32_t w = sh.word[q][j + 1];
+            if (w == 0u) continue;
+            int32_t* ids = q ? p.miss_pages : p.pages;
+            int32_t* runs = q ? p.miss_runs : p.runs;
+            const uint32_t b = sh.word[q][j] >> 31, a = sh.word[q][j + 2] & 1u;
+            const uint64_t o = sh.at[q][j];
+            const uint32_t starts = w & ~((w << 1) | b), ends = w & ~((w >> 1) | (a << 31)), below = (1u << lane) - 1u;
+            const int64_t o_id = static_cast<int64_t>(o >> 32) + __popc(w & below);
+            const int64_t o_st = static_cast<int64_t>(o & 0xffffffffu) + __popc(starts & below);
+            const int64_t o_en = static_cast<int64_t>(o & 0xffffffffu) - (b & w & 1u) + __popc(ends & below);
+            const int32_t page = (c0 + j) * 32 + lane;
+            if (((w >> lane) & 1u) && o_id < p.capacity) ids[o_id] = page;
+            if (((starts >> lane) & 1u) && o_st < p.capacity) runs[2 * o_st] = page;
+            if (((ends >> lane) & 1u) && o_en < p.capacity) runs[2 * o_en + 1] = page + 1;     // becomes a length below
+        }
+        base[0] += sum[0];
+        base[1] += sum[1];
     }
-    m = ends;
-    while (m) {  // the j-th end closes the j-th start; end+1 is stored and turned into a length by the second kernel
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        if (o_en < capacity) out_runs[2 * o_en + 1] = i * 32 + b + 1;
-        ++o_en;
+    cluster_sync_all();                   // every start and end is written (and every CTA has read the counts)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        if (q == 1 && !want_miss) break;
+        int32_t* runs = q ? p.miss_runs : p.runs;
+        const int64_t n_runs = static_cast<int64_t>(all[q] & 0xffffffffu), n_ids = static_cast<int64_t>(all[q] >> 32);
+        const int64_t n = n_runs < p.capacity ? n_runs : p.capacity;
+        for (int64_t j = static_cast<int64_t>(rank) * PD_THREADS + tid; j < n; j += static_cast<int64_t>(n_cta) * PD_THREADS)
+            runs[2 * j + 1] = __ldcg(runs + 2 * j + 1) - __ldcg(runs + 2 * j);
+        if (rank == 0 && tid == 0) {
+            *(q ? p.n_miss : p.n_pages) = static_cast<int32_t>(n_ids);
+            *(q ? p.n_miss_runs : p.n_runs) = static_cast<int32_t>(n_runs);
+            if (n_ids > p.capacity || n_runs > p.capacity) report(p.dev_status, JANUS_DEV_CAPACITY_EXCEEDED);
+        }
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        const int total_ids = id_base + tot_ids, total_runs = run_base + tot_starts;
-        *n_ids = total_ids;
-        *out_n_runs = total_runs;
-        if (total_ids > capacity || total_runs > capacity) report(dev_status, JANUS_DEV_CAPACITY_EXCEEDED);
-    }
-}
-
-__global__ void page_run_lengths_kernel(int32_t* runs, const int32_t* n_runs, int32_t* miss_runs, const int32_t* n_miss_runs, int64_t capacity) {
-    int32_t* r = blockIdx.y == 1 ? miss_runs : runs;
-    int64_t n = blockIdx.y == 1 ? *n_miss_runs : *n_runs;
-    if (n > capacity) n = capacity;
-    for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < n; j += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        r[2 * j + 1] -= r[2 * j];
-}
-
-// Chooses between the one-CTA list kernel (small bitmaps: one launch, no second pass) and the chunked pair.
-static int launch_page_lists(const uint32_t* bitmap, const uint32_t* predicted, int n_words, int64_t n_phys_pages, int32_t* pages,
-                             int32_t* n_pages, int32_t* runs, int32_t* n_runs, int32_t* miss_pages, int32_t* n_miss, int32_t* miss_runs,
-                             int32_t* n_miss_runs, int64_t capacity, int32_t* dev_status, cudaStream_t stream);
-
-// Batch form (decode over many sessions): row r of idx belongs to a session with its own page table
-// page_tables[table_offsets[r] .. table_offsets[r+1]) and its own history length demand_limits[r]; physical page ids are
-// global, so all rows mark one bitmap.  Sizes are small (rows x k indices), so this is the plain one-index-per-thread form.
-__global__ void __launch_bounds__(MARK_THREADS)
-page_mark_rows_kernel(const int32_t* __restrict__ idx, int64_t n_rows, int k, const int64_t* __restrict__ demand_limits, int page_size,
-                      int page_shift, const int32_t* __restrict__ page_tables, const int64_t* __restrict__ table_offsets,
-                      int64_t n_phys_pages, uint32_t* __restrict__ bitmap, int32_t* dev_status) {
-    const int64_t n_idx = n_rows * k;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * MARK_THREADS;
-    for (int64_t e = static_cast<int64_t>(blockIdx.x) * MARK_THREADS + threadIdx.x; e < n_idx; e += stride) {
-        const int64_t r = e / k;
-        const int64_t off = __ldg(table_offsets + r);
-        // a table that starts before the array has no pages: its selected tokens are reported and skipped
-        mark_one(__ldg(idx + e), __ldg(demand_limits + r), page_size, page_shift, page_tables + (off < 0 ? 0 : off),
-                 off < 0 ? 0 : __ldg(table_offsets + r + 1) - off, n_phys_pages, bitmap, dev_status);
-    }
-}
-
-static int launch_page_lists(const uint32_t* bitmap, const uint32_t* predicted, int n_words, int64_t n_phys_pages, int32_t* pages,
-                             int32_t* n_pages, int32_t* runs, int32_t* n_runs, int32_t* miss_pages, int32_t* n_miss, int32_t* miss_runs,
-                             int32_t* n_miss_runs, int64_t capacity, int32_t* dev_status, cudaStream_t stream) {
-    const int n_chunks = (n_words + LIST_THREADS - 1) / LIST_THREADS;
-    if (n_chunks >= 2 && n_chunks <= LIST_MAX_CHUNKS) {
-        const dim3 grid(n_chunks, miss_pages != nullptr ? 2 : 1);
-        page_lists_chunk_kernel<<<grid, LIST_THREADS, 0, stream>>>(bitmap, predicted, n_words, n_phys_pages, pages, n_pages, runs, n_runs, miss_pages,
-                                                                   n_miss, miss_runs, n_miss_runs, capacity, dev_status);
-        JANUS_CUDA_CHECK(cudaGetLastError());
-        page_run_lengths_kernel<<<dim3(64, grid.y), 256, 0, stream>>>(runs, n_runs, miss_runs, n_miss_runs, capacity);
-        JANUS_CUDA_CHECK(cudaGetLastError());
-        return JANUS_OK;
-    }
-    page_lists_kernel<<<1, LIST_THREADS, 0, stream>>>(bitmap, predicted, n_words, n_phys_pages, pages, n_pages, runs, n_runs, miss_pages, n_miss,
-                                                     miss_runs, n_miss_runs, capacity, dev_status);
-    JANUS_CUDA_CHECK(cudaGetLastError());
-    return JANUS_OK;
 }
 
 __global__ void page_union_kernel(uint32_t* __restrict__ dst, const uint32_t* __restrict__ src, int n_words) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_words; i += gridDim.x * blockDim.x) dst[i] |= src[i];
+}
+
+template <int MODE>
+static int launch_page_demand(const PdParams& p, int cluster, cudaStream_t stream) {
+    const size_t smem = MODE == PD_LISTS ? 0 : sizeof(uint32_t) * static_cast<size_t>(p.n_words);
+    static once_per_device attributes;
+    JANUS_CUDA_CHECK(attributes.run([] {
+        cudaError_t e = cudaFuncSetAttribute(page_demand_kernel<MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess && MODE != PD_LISTS)
+            e = cudaFuncSetAttribute(page_demand_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PD_SMEM_WORDS * static_cast<int>(sizeof(uint32_t)));
+        return e;
+    }));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(PD_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = cluster;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, page_demand_kernel<MODE>, p));
+    return JANUS_OK;
+}
+
+// One launch of one cluster while it reads the indices as fast as memset, chip-wide marking and lists would (14.4 us up to 512 K
+// indices): 128 K indices in 13 us, 256 K in 15.  Four CTAs up to 4 K indices (9.1 us, 9.6 with eight, 11.8 with sixteen), eight
+// up to 64 K (10.9 against 12.6 and 11.8 with four and sixteen at 256 x 256), sixteen beyond (64 rows of a 131136-page pool: 25.3
+// against 35.5 with eight and 27.5 for the three launches).  Memset, marking and one-CTA lists took 14.6, 18.5 and 36.6 us
+// for these three.
+constexpr int64_t PD_ONE_LAUNCH_INDICES = 1 << 17;
+
+template <int MODE>
+static int run_page_demand(const PdParams& p, cudaStream_t stream) {
+    if (p.n_idx <= PD_ONE_LAUNCH_INDICES && p.n_words <= PD_SMEM_WORDS) {
+        int cluster = p.n_idx <= 4096 ? 4 : p.n_idx <= 65536 ? 8 : 16;
+        while (p.n_words > cluster * PD_THREADS) cluster *= 2;      // a slice is one chunk
+        return launch_page_demand<MODE>(p, cluster, stream);
+    }
+    JANUS_CUDA_CHECK(cudaMemsetAsync(p.bitmap, 0, sizeof(uint32_t) * p.n_words, stream));
+    const int64_t n_log_words = (p.n_logical_pages + 31) / 32;
+    if (MODE == PD_MARK && n_log_words + p.n_words <= MARK_SMEM_WORDS) {
+        static once_per_device attributes;
+        JANUS_CUDA_CHECK(attributes.run([] {
+            return cudaFuncSetAttribute(page_mark_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MARK_SMEM_WORDS * static_cast<int>(sizeof(uint32_t)));
+        }));
+        const int64_t want = ((p.n_idx >> 2) + MARK_THREADS - 1) / MARK_THREADS;
+        const unsigned grid = static_cast<unsigned>(want < 1 ? 1 : want < 148 * 2 ? want : 148 * 2);
+        page_mark_kernel<<<grid, MARK_THREADS, sizeof(uint32_t) * (n_log_words + p.n_words), stream>>>(p, static_cast<int>(n_log_words));
+    } else if (p.n_idx > 0) {
+        const int64_t want = (p.n_idx + 1023) / 1024;
+        page_mark_global_kernel<MODE><<<static_cast<unsigned>(want < 148 * 8 ? want : 148 * 8), 256, 0, stream>>>(p);
+    }
+    JANUS_CUDA_CHECK(cudaGetLastError());
+    return launch_page_demand<PD_LISTS>(p, p.n_words <= 8 * PD_THREADS ? 8 : 16, stream);     // 131136 pages: 27.5 us with 16, 32.7 with 8; 2112 pages: 14.4 with 8, 16.5 with 16
+}
+
+static int page_shift_of(int page_size) {
+    if ((page_size & (page_size - 1)) != 0) return -1;
+    int shift = 0;
+    while ((1 << shift) < page_size) ++shift;
+    return shift;
 }
 
 }  // namespace janus
@@ -299,28 +452,17 @@ extern "C" int janus_page_demand(const int32_t* idx, int64_t n_rows, int k, int6
     const int64_t n_idx = n_rows * static_cast<int64_t>(k);
     if (n_idx > 0 && (!idx || !aligned16(idx))) return JANUS_ERR_INVALID_ARG;
 
-    const int n_words = static_cast<int>((n_phys_pages + 31) / 32);
-    JANUS_CUDA_CHECK(cudaMemsetAsync(bitmap, 0, sizeof(uint32_t) * n_words, stream));
-    if (n_idx > 0) {
-        int page_shift = -1;
-        if ((page_size & (page_size - 1)) == 0) {
-            page_shift = 0;
-            while ((1 << page_shift) < page_size) ++page_shift;
-        }
-        const int64_t n_vec = (n_idx + 3) / 4;
-        int64_t blocks = (n_vec + MARK_THREADS * 8 - 1) / (MARK_THREADS * 8);
-        if (blocks < 1) blocks = 1;
-        if (blocks > 148 * 8) blocks = 148 * 8;
-        if (n_words <= MARK_SMEM_WORDS)
-            page_mark_kernel<true><<<static_cast<unsigned>(blocks), MARK_THREADS, 0, stream>>>(
-                idx, n_idx, demand_limit, page_size, page_shift, page_table, n_logical_pages, n_phys_pages, bitmap, n_words, dev_status);
-        else
-            page_mark_kernel<false><<<static_cast<unsigned>(blocks), MARK_THREADS, 0, stream>>>(
-                idx, n_idx, demand_limit, page_size, page_shift, page_table, n_logical_pages, n_phys_pages, bitmap, n_words, dev_status);
-        JANUS_CUDA_CHECK(cudaGetLastError());
-    }
-    return launch_page_lists(bitmap, predicted_bitmap, n_words, n_phys_pages, pages, n_pages, runs, n_runs, miss_pages, n_miss, miss_runs,
-                             n_miss_runs, capacity, dev_status, stream);
+    PdParams p = {};
+    p.idx = idx; p.n_idx = n_idx; p.k = k;
+    p.demand_limit = demand_limit;
+    p.page_size = page_size; p.page_shift = page_shift_of(page_size);
+    p.page_table = page_table; p.n_logical_pages = n_logical_pages;
+    p.n_phys_pages = n_phys_pages; p.n_words = static_cast<int>((n_phys_pages + 31) / 32);
+    p.predicted = predicted_bitmap; p.bitmap = bitmap;
+    p.pages = pages; p.n_pages = n_pages; p.runs = runs; p.n_runs = n_runs;
+    p.miss_pages = miss_pages; p.n_miss = n_miss; p.miss_runs = miss_runs; p.n_miss_runs = n_miss_runs;
+    p.capacity = capacity; p.dev_status = dev_status;
+    return run_page_demand<PD_MARK>(p, stream);
 }
 
 extern "C" int janus_page_demand_batch(const int32_t* idx, int64_t n_rows, int k, const int64_t* demand_limits, int page_size,
@@ -338,21 +480,15 @@ extern "C" int janus_page_demand_batch(const int32_t* idx, int64_t n_rows, int k
     const int64_t n_idx = n_rows * static_cast<int64_t>(k);
     if (n_idx > 0 && (!idx || !demand_limits || !page_tables || !table_offsets)) return JANUS_ERR_INVALID_ARG;
 
-    const int n_words = static_cast<int>((n_phys_pages + 31) / 32);
-    JANUS_CUDA_CHECK(cudaMemsetAsync(bitmap, 0, sizeof(uint32_t) * n_words, stream));
-    if (n_idx > 0) {
-        int page_shift = -1;
-        if ((page_size & (page_size - 1)) == 0) {
-            page_shift = 0;
-            while ((1 << page_shift) < page_size) ++page_shift;
-        }
-        int64_t blocks = (n_idx + MARK_THREADS * 4 - 1) / (MARK_THREADS * 4);
-        if (blocks > 148 * 8) blocks = 148 * 8;
-        page_mark_rows_kernel<<<static_cast<unsigned>(blocks), MARK_THREADS, 0, stream>>>(idx, n_rows, k, demand_limits, page_size, page_shift,
-                                                                                          page_tables, table_offsets, n_phys_pages, bitmap,
-                                                                                          dev_status);
-        JANUS_CUDA_CHECK(cudaGetLastError());
-    }
-    return launch_page_lists(bitmap, predicted_bitmap, n_words, n_phys_pages, pages, n_pages, runs, n_runs, miss_pages, n_miss, miss_runs,
-                             n_miss_runs, capacity, dev_status, stream);
+    PdParams p = {};
+    p.idx = idx; p.n_idx = n_idx; p.k = k;
+    p.demand_limits = demand_limits; p.table_offsets = table_offsets;
+    p.page_size = page_size; p.page_shift = page_shift_of(page_size);
+    p.page_table = page_tables;
+    p.n_phys_pages = n_phys_pages; p.n_words = static_cast<int>((n_phys_pages + 31) / 32);
+    p.predicted = predicted_bitmap; p.bitmap = bitmap;
+    p.pages = pages; p.n_pages = n_pages; p.runs = runs; p.n_runs = n_runs;
+    p.miss_pages = miss_pages; p.n_miss = n_miss; p.miss_runs = miss_runs; p.n_miss_runs = n_miss_runs;
+    p.capacity = capacity; p.dev_status = dev_status;
+    return run_page_demand<PD_MARK_ROWS>(p, stream);
 }

@@ -333,6 +333,16 @@ __device__ __forceinline__ void st_async_cluster_f32x4(uint32_t cluster_addr, fl
 __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t cluster_addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint64_t ld_cluster_u64(uint32_t cluster_addr) {
+    uint64_t v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
 // Arrive on an mbarrier of another CTA of the cluster; orders this thread's earlier (remote) stores before it.
 // A cluster-scope release costs on the order of a thousand cycles on this part: keep it off hot paths.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {

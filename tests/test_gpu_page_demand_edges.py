@@ -1,0 +1,83 @@
+"""Page demand where its dispatch changes: bitmaps around one word, one chunk of 1024 words, the slices of 4, 8 and 16 CTAs, and past what a
+CTA keeps in shared memory; index counts on either side of the one-launch limit; runs that cross words, slices and CTAs; lists that exceed
+their capacity; rows with their own tables.  Exact against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import helpers as Hp
+from oracle import janus_oracle as O
+from paper_2609_36938_b200 import binding as B
+from paper_2609_36938_b200 import build
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    B.load()
+    yield
+    B.check_dev_status()
+
+
+def dev32(x):
+    return torch.from_numpy(np.ascontiguousarray(x, dtype=np.int32)).cuda()
+
+
+def bitmap_of(pages, n_phys):
+    bits = np.zeros((n_phys + 31) // 32 * 32, np.uint8)
+    bits[pages] = 1
+    return np.packbits(bits, bitorder="little").view(np.int32)
+
+
+@pytest.mark.parametrize("n_rows,k,n_phys,page", [
+    (1, 7, 31, 64), (3, 700, 33, 16), (2, 2048, 32768, 1), (5, 1000, 32800, 64), (40, 1639, 262144, 1), (33, 2048, 262176, 1),
+    (64, 2048, 2049, 48), (65, 2048, 2049, 64), (70, 2000, 300000, 1), (3, 2048, 600000, 1), (90, 2048, 900000, 1),
+])
+def test_page_demand_edges(n_rows, k, n_phys, page):
+    rng = np.random.default_rng(n_rows * 7 + n_phys)
+    n_log = n_phys
+    L = n_log * page - page // 2
+    lo = rng.integers(0, L, (n_rows, k))
+    run = (rng.integers(0, max(1, L - 40 * k), (n_rows, 1)) + np.arange(k) * max(1, page // 2)) % L       # neighbouring pages: long runs
+    idx = np.where(rng.random((n_rows, 1)) < 0.5, lo, run).astype(np.int32)
+    idx[rng.random(idx.shape) < 0.05] = -1
+    table = np.arange(n_log, dtype=np.int32) if n_rows % 2 else rng.permutation(n_log).astype(np.int32)
+    limit = L - L // 10
+    ref = O.page_demand(idx, limit, page, table)
+    predicted = np.array(sorted(rng.permutation(ref["pages"])[: len(ref["pages"]) // 2]), np.int64)
+    pd = B.janus_page_demand(dev32(idx), demand_limit=limit, page_size=page, page_table=dev32(table), n_phys_pages=n_phys,
+                             predicted_bitmap=torch.from_numpy(bitmap_of(predicted, n_phys)).cuda())
+    B.check_dev_status()
+    got = Hp.page_lists_from_device(pd)
+    miss = sorted(set(ref["pages"]) - set(predicted.tolist()))
+    assert Hp.bitmap_to_pages(pd["bitmap"], n_phys) == list(ref["pages"])
+    assert got["pages"] == list(ref["pages"]) and got["runs"] == [tuple(r) for r in ref["runs"]]
+    assert got["miss"] == miss and got["miss_runs"] == [tuple(r) for r in O.maximal_runs(miss)]
+    # lists shorter than the set: the first entries, true counts, and the status word
+    cap = max(1, len(ref["runs"]) // 3)
+    small = B.janus_page_demand(dev32(idx), demand_limit=limit, page_size=page, page_table=dev32(table), n_phys_pages=n_phys, capacity=cap, want_miss=False)
+    assert small["counts"][:2].tolist() == [len(ref["pages"]), len(ref["runs"])]
+    assert small["pages"].tolist() == list(ref["pages"])[:cap] and [tuple(r) for r in small["runs"].tolist()] == [tuple(r) for r in ref["runs"]][:cap]
+    if len(ref["pages"]) > cap:
+        with pytest.raises(B.JanusError, match="CAPACITY"):
+            B.check_dev_status()
+
+
+@pytest.mark.parametrize("n_rows,k", [(1, 2048), (20, 2048), (70, 2048)])
+def test_page_demand_batch_edges(n_rows, k):
+    rng = np.random.default_rng(n_rows)
+    page = 64
+    n_pages = rng.integers(1, 900, n_rows)
+    off = np.concatenate([[0], np.cumsum(n_pages)]).astype(np.int64)
+    n_phys = int(off[-1]) + 5
+    tables = rng.permutation(n_phys)[:off[-1]].astype(np.int32)
+    limits = n_pages * page - rng.integers(0, page, n_rows)
+    idx = (rng.random((n_rows, k)) * n_pages[:, None] * page).astype(np.int32)
+    pd = B.janus_page_demand_batch(dev32(idx), demand_limits=torch.from_numpy(limits.astype(np.int64)).cuda(), page_size=page, page_tables=dev32(tables),
+                                   table_offsets=torch.from_numpy(off).cuda(), n_phys_pages=n_phys)
+    B.check_dev_status()
+    want = sorted(set().union(*[O.page_demand(idx[r:r + 1], int(limits[r]), page, tables[off[r]:off[r + 1]])["pages"] for r in range(n_rows)]))
+    got = Hp.page_lists_from_device(pd)
+    assert got["pages"] == want and got["runs"] == [tuple(r) for r in O.maximal_runs(want)] and got["miss"] == want
