@@ -1,14 +1,17 @@
-"""Builds libjanus.so (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds libjanus.so (the C-ABI library) in-tree with nvcc for sm_100a, and _native.so (the native half of binding.py) with g++."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libjanus.so")
+NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")
 SOURCES = ["janus_api.cu", "indexer_generic.cu", "indexer_tc.cu", "topk.cu", "page_demand.cu", "sparse_attn_generic.cu", "sparse_attn_heads.cu",
            "sparse_attn_latent_pair.cu", "indexer_topk.cu", "diagnostics.cu"]
 
@@ -21,15 +24,24 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(NATIVE_PATH):
         return True
-    t = os.path.getmtime(LIB_PATH)
+    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(NATIVE_PATH))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(PKG_DIR, "..", "include", "janus.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _native_command() -> list:
+    """g++ command for the extension module: torch's C++ headers and libraries are the ones the process has loaded already."""
+    torch_dir = list(importlib.util.find_spec("torch").submodule_search_locations)[0]
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    inc = [os.path.join(torch_dir, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", *[f"-I{d}" for d in inc], os.path.join(CSRC, "py_binding.cpp"), "-o",
+            NATIVE_PATH, "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda", "-ldl"]
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every kernel for sm_100a into one shared library; returns its path."""
+    """Compile every kernel for sm_100a into one shared library, and the binding's extension module; returns the library's path."""
     if not force and not _stale():
         return LIB_PATH
     build_dir = os.path.join(PKG_DIR, "build")
@@ -43,14 +55,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
         objs.append(obj)
         cmd = [_nvcc(), *flags, "-c", os.path.join(CSRC, src), "-o", obj]
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    procs.append(("py_binding.cpp", subprocess.Popen(_native_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
     for src, pr in procs:
         out, _ = pr.communicate()
         if pr.returncode != 0 or verbose:
-            sys.stderr.write(f"--- nvcc {src}\n{out}\n")
+            sys.stderr.write(f"--- {src}\n{out}\n")
         failed |= pr.returncode != 0
     if failed:
-        raise RuntimeError("nvcc failed")
+        raise RuntimeError("compilation failed")
     subprocess.check_call([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB_PATH, *objs, "-lcudart_static", "-ldl", "-lrt", "-lpthread"])
     return LIB_PATH
 

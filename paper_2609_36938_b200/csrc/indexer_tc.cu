@@ -470,7 +470,9 @@ bool indexer_tc_candidates_supported(int H, int D, int dtype) {
 template <int H, bool FP8, bool CAND, bool RAGGED = false>
 static int launch_tc(const CUtensorMap& tq, const CUtensorMap& tk, const TcParams& p, const TcCandParams& cp, dim3 grid, size_t smem,
                      cudaStream_t stream) {
-    JANUS_CUDA_CHECK(cudaFuncSetAttribute(indexer_tc_kernel<H, FP8, CAND, RAGGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    static once_per_device attributes;
+    JANUS_CUDA_CHECK(attributes.run(
+        [] { return cudaFuncSetAttribute(indexer_tc_kernel<H, FP8, CAND, RAGGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET); }));
     indexer_tc_kernel<H, FP8, CAND, RAGGED><<<grid, RAGGED ? TC_THREADS_RAGGED : (CAND ? TC_THREADS : TC_THREADS16), smem, stream>>>(tq, tk, p, cp);
     JANUS_CUDA_CHECK(cudaGetLastError());
     return JANUS_OK;

@@ -321,7 +321,9 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
                                H_I, D_I, FT_NS, q_pos0, 0, dtype, sc_sample, FT_NS, dev_status, stream, nullptr, nullptr, nullptr, 0);
     if (rc != JANUS_OK) return rc;
     // 2. thresholds (also clears the candidate counters)
-    JANUS_CUDA_CHECK(cudaFuncSetAttribute(ft_threshold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(SampleShared))));
+    static once_per_device threshold_attributes, select_attributes, fallback_attributes;
+    JANUS_CUDA_CHECK(threshold_attributes.run(
+        [] { return cudaFuncSetAttribute(ft_threshold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(SampleShared))); }));
     ft_threshold_kernel<<<M, TK_THREADS, sizeof(SampleShared), stream>>>(sc_sample, M, n_keys, q_pos0, causal, k, L.cap, thr, cand_cnt, fb_count);
     JANUS_CUDA_CHECK(cudaGetLastError());
     // 3. the indexer over all keys, appending candidates
@@ -329,13 +331,16 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
                            dtype, nullptr, 0, dev_status, stream, thr, cand_cnt, cand, L.cap);
     if (rc != JANUS_OK) return rc;
     // 4. exact selection per row
+    JANUS_CUDA_CHECK(select_attributes.run([] {
+        const cudaError_t e = cudaFuncSetAttribute(ft_select_kernel<FT_CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(TopkSharedT<FT_CAP>)));
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(ft_select_kernel<FT_CAP / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           static_cast<int>(sizeof(TopkSharedT<FT_CAP / 2>)));
+    }));
     if (L.cap == FT_CAP) {
         using Sh = TopkSharedT<FT_CAP>;
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(ft_select_kernel<FT_CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(Sh))));
         ft_select_kernel<FT_CAP><<<M, TK_THREADS, sizeof(Sh), stream>>>(cand, cand_cnt, M, n_keys, q_pos0, causal, k, idx, count, kth, fb_count, fb_rows);
     } else {
         using Sh = TopkSharedT<FT_CAP / 2>;
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(ft_select_kernel<FT_CAP / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(Sh))));
         ft_select_kernel<FT_CAP / 2><<<M, TK_THREADS, sizeof(Sh), stream>>>(cand, cand_cnt, M, n_keys, q_pos0, causal, k, idx, count, kth, fb_count,
                                                                            fb_rows);
     }
@@ -344,13 +349,16 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
     const size_t fb_smem = sizeof(FallbackShared) + sizeof(float) * (static_cast<size_t>(H_I) * D_I + H_I);
     const unsigned char* qb = static_cast<const unsigned char*>(q_idx);
     const unsigned char* kb = static_cast<const unsigned char*>(k_idx);
+    constexpr int fb_smem_max = static_cast<int>(sizeof(FallbackShared) + sizeof(float) * (64 * 256 + 64));      // the largest shape of the fused route: 64 heads of 256 E4M3 bytes
+    JANUS_CUDA_CHECK(fallback_attributes.run([] {
+        const cudaError_t e = cudaFuncSetAttribute(ft_fallback_kernel<JANUS_DTYPE_FP8_E4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, fb_smem_max);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(ft_fallback_kernel<JANUS_DTYPE_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, fb_smem_max);
+    }));
     if (fp8) {
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(ft_fallback_kernel<JANUS_DTYPE_FP8_E4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(fb_smem)));
         ft_fallback_kernel<JANUS_DTYPE_FP8_E4M3><<<FT_FB_CTAS, TK_THREADS, fb_smem, stream>>>(
             qb, kb, k_stride_tok * esz, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H_I, D_I, n_keys, q_pos0, causal, k, idx, count,
             kth, fb_count, fb_rows, fb_buf, L.ld);
     } else {
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(ft_fallback_kernel<JANUS_DTYPE_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(fb_smem)));
         ft_fallback_kernel<JANUS_DTYPE_BF16><<<FT_FB_CTAS, TK_THREADS, fb_smem, stream>>>(
             qb, kb, k_stride_tok * esz, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H_I, D_I, n_keys, q_pos0, causal, k, idx, count,
             kth, fb_count, fb_rows, fb_buf, L.ld);
