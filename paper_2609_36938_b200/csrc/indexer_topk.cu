@@ -128,12 +128,13 @@ ft_threshold_kernel(const float* __restrict__ sc_sample, int M, int64_t n_keys, 
         if (tid == 0) thr[t] = neg_inf;
         return;
     }
-    const float* row = sc_sample + static_cast<int64_t>(t) * FT_NS;
-    for (int i = tid; i < FT_NS; i += TK_THREADS) sh.cand_key[i] = float_to_key(row[i]);
-    __syncthreads();
-    int dummy;
-    SmemSource s{sh.cand_key, nullptr, FT_NS};
-    const uint32_t T = select_kth(s, r, sh, &dummy);
+    const float4* row = reinterpret_cast<const float4*>(sc_sample + static_cast<int64_t>(t) * FT_NS);
+    static_assert(FT_NS == 8 * TK_THREADS, "eight sample scores per thread");
+    const float4 a = row[tid], b = row[TK_THREADS + tid];
+    const uint32_t key[8] = {float_to_key(a.x), float_to_key(a.y), float_to_key(a.z), float_to_key(a.w),
+                             float_to_key(b.x), float_to_key(b.y), float_to_key(b.z), float_to_key(b.w)};
+    uint32_t hi;
+    const uint32_t T = sample_threshold(key, r, hi, sh);
     if (tid == 0) thr[t] = key_to_float(T);
 }
 
@@ -156,25 +157,28 @@ ft_select_kernel(const int2* __restrict__ cand, const int32_t* __restrict__ cand
         if (tid == 0) fb_rows[atomicAdd(fb_count, 1)] = t;
         return;
     }
-    if (tid == 0) { sh.out_pos = 0; sh.eq_taken = 0; }
-    const int2* row = cand + static_cast<int64_t>(t) * CAP;
-    for (int i = tid; i < n_c; i += TK_THREADS) {
-        const int2 c = row[i];
-        sh.cand_key[i] = float_to_key(__int_as_float(c.x));
-        sh.cand_idx[i] = c.y;
-    }
-    __syncthreads();
-    SmemSource s{sh.cand_key, sh.cand_idx, n_c};
-    uint32_t T = 0u;
     if (n_sel > 0) {
-        int n_eq;
-        T = select_kth(s, n_sel, sh, &n_eq);
-        emit_selection(s, T, n_eq, out, sh);
+        const int2* row = cand + static_cast<int64_t>(t) * CAP;
+        uint32_t lo = 0xffffffffu, hi = 0u;
+        for (int i = tid; i < n_c; i += TK_THREADS) {
+            const int2 c = row[i];
+            const uint32_t key = float_to_key(__int_as_float(c.x));
+            sh.cand_key[i] = key;
+            sh.cand_idx[i] = c.y;
+            lo = min(lo, key);
+            hi = max(hi, key);
+        }
+        clear_hist(sh);
+        block_key_range(lo, hi, sh);
+        const BucketMap map(lo, hi);
+        for (int i = tid; i < n_c; i += TK_THREADS) atomicAdd(&sh.hist[map(sh.cand_key[i])], 1);
+        __syncthreads();
+        select_and_emit(SmemSource{sh.cand_key, sh.cand_idx, n_c}, map, n_sel, out, kth != nullptr ? kth + t : nullptr, sh);
     }
     for (int i = n_sel + tid; i < k; i += TK_THREADS) out[i] = -1;
     if (tid == 0) {
         if (count) count[t] = n_sel;
-        if (kth) kth[t] = n_sel > 0 ? key_to_float(T) : __int_as_float(0xff800000);
+        if (kth && n_sel == 0) kth[t] = __int_as_float(0xff800000);
     }
 }
 
@@ -251,7 +255,7 @@ ft_fallback_kernel(const unsigned char* __restrict__ q_idx, const unsigned char*
             buf[s] = acc;
         }
         __syncthreads();
-        topk_row(buf, n, k, t, idx + static_cast<int64_t>(t) * k, count, kth, sh);
+        topk_row(buf, n, k, idx + static_cast<int64_t>(t) * k, count != nullptr ? count + t : nullptr, kth != nullptr ? kth + t : nullptr, sh);
     }
 }
 

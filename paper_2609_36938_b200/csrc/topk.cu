@@ -1,18 +1,16 @@
 // janus_topk: per-row selection of the k largest scores over the causal prefix (Eq. 1, Sec. 2.2).
 //
-// A CTA works on one query row at a time; the CTAs resident on the device walk the rows with stride gridDim.x.  The row
-// (0.5-1 MB of fp32 at 128K-256K keys) is read from HBM once:
+// A CTA works on one query row at a time; the CTAs resident on the device walk the rows with stride gridDim.x, or, while rows
+// are few, a cluster of CTAs shares a row.  The row (0.5-1 MB of fp32 at 128K-256K keys) is read from HBM once:
 //   1. a strided sample of the row (512 x 32-byte sectors) gives a conservative threshold whose
 //      expected rank is a little above k;
 //   2. one streaming pass with 16-byte loads keeps only the elements at or above that threshold
 //      in a shared-memory candidate buffer (~1.5-3 % of the row pass the one-compare filter);
-//   3. an exact selection runs on the candidates in shared memory: 2048-bucket histograms over a
-//      shrinking key range (buckets are linear in the order-preserving integer key, so they spread
-//      over whatever range the scores occupy) until the bucket of the k-th key holds at most 256
-//      keys, which are then ranked directly.
-// If the sample misjudges the row (fewer than k candidates, or more than the buffer holds) the
-// same exact selection runs over the row in global memory instead; that path is slower, never
-// wrong.  Rows that fit the buffer skip the sampling step.
+//   3. a 2048-bucket histogram of the candidates (linear in the order-preserving integer key) gives the bucket of the k-th
+//      key; one pass emits everything above it and the keys inside are ranked directly.
+// If the sample misjudges the row (fewer than k candidates, or more than the buffer holds) an exact selection over repeated
+// histograms runs over the row in global memory instead; that path is slower, never wrong.  Rows that fit the buffer skip the
+// sampling step.
 #include <algorithm>
 
 #include "topk_select.cuh"
@@ -34,10 +32,22 @@ topk_rows_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_
         const int64_t prefix64 = causal ? min(n_keys, q_pos0 + t + 1) : n_keys;
         const int t_next = t + gridDim.x;
         const int64_t prefix_next = t_next < M ? (causal ? min(n_keys, q_pos0 + t_next + 1) : n_keys) : 0;
-        topk_row(scores + static_cast<int64_t>(t) * ld, static_cast<int>(prefix64), k, t, idx + static_cast<int64_t>(t) * k, count, kth, sh,
-                 t_next < M ? scores + static_cast<int64_t>(t_next) * ld : nullptr, static_cast<int>(prefix_next));
+        topk_row(scores + static_cast<int64_t>(t) * ld, static_cast<int>(prefix64), k, idx + static_cast<int64_t>(t) * k,
+                 count != nullptr ? count + t : nullptr, kth != nullptr ? kth + t : nullptr, sh, t_next < M ? scores + static_cast<int64_t>(t_next) * ld : nullptr, static_cast<int>(prefix_next));
         __syncthreads();   // the selection state in shared memory is reused by the next row
     }
+}
+
+// Few rows: one cluster of CTAs per row.
+__global__ void __launch_bounds__(TK_THREADS)
+topk_rows_cluster_kernel(const float* __restrict__ scores, int64_t ld, int64_t n_keys, int64_t q_pos0, int causal, int k,
+                         int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TopkSharedT<TK_CAP>& sh = *reinterpret_cast<TopkSharedT<TK_CAP>*>(smem_raw);
+    const int t = blockIdx.x / ptx::cluster_nctarank();
+    const int64_t prefix = causal ? min(n_keys, q_pos0 + t + 1) : n_keys;
+    topk_row_cluster(scores + static_cast<int64_t>(t) * ld, static_cast<int>(prefix), k, idx + static_cast<int64_t>(t) * k,
+                     count != nullptr ? count + t : nullptr, kth != nullptr ? kth + t : nullptr, sh);
 }
 
 // Entry granularity (footnote of Sec. 2.2): columns are entries of `entry_size` consecutive tokens; row t (position
@@ -52,7 +62,8 @@ topk_entries_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t
     const int t = blockIdx.x;
     int64_t prefix = (q_pos0 + t) / entry_size + 1;
     if (prefix > n_entries) prefix = n_entries;
-    topk_row(scores + static_cast<int64_t>(t) * ld, static_cast<int>(prefix), k, t, idx + static_cast<int64_t>(t) * k, count, kth, sh);
+    topk_row(scores + static_cast<int64_t>(t) * ld, static_cast<int>(prefix), k, idx + static_cast<int64_t>(t) * k,
+             count != nullptr ? count + t : nullptr, kth != nullptr ? kth + t : nullptr, sh);
 }
 
 // Token selection of an entry selection: slot e * E + j of row t = entry * E + j if that token is at or before q_pos0 + t.
@@ -94,20 +105,19 @@ entry_pool_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n
 
 // Batch form (decode over many sessions): row b starts at scores[row_offsets[b]] and has row_lengths[b] elements (or runs
 // up to the next row's start when row_lengths is NULL), every element visible.
-template <int CAP>
+template <bool CLUSTER>
 __global__ void __launch_bounds__(TK_THREADS)
 topk_ragged_kernel(const float* __restrict__ scores, const int64_t* __restrict__ row_offsets, const int64_t* __restrict__ row_lengths, int k,
                    int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth, int32_t* dev_status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    using TopkShared = TopkSharedT<CAP>;
-    TopkShared& sh = *reinterpret_cast<TopkShared*>(smem_raw);
-    const int b = blockIdx.x;
+    TopkSharedT<TK_CAP>& sh = *reinterpret_cast<TopkSharedT<TK_CAP>*>(smem_raw);
+    const int b = CLUSTER ? blockIdx.x / ptx::cluster_nctarank() : blockIdx.x;
     const int64_t off = row_offsets[b];
     const int64_t n = row_lengths != nullptr ? row_lengths[b] : row_offsets[b + 1] - off;
     // the offsets come from device memory: a row that starts before the array, off a 16-byte boundary (the row is read with
     // 16-byte loads) or has a negative or unrepresentable length is reported and left empty, never read
     if (off < 0 || (off & 3) != 0 || n < 0 || n > 2147483639) {
-        for (int i = threadIdx.x; i < k; i += blockDim.x) idx[static_cast<int64_t>(b) * k + i] = -1;
+        for (int i = threadIdx.x; i < k; i += blockDim.x) idx[static_cast<int64_t>(b) * k + i] = -1;      // (every CTA of a cluster: the same values)
         if (threadIdx.x == 0) {
             if (count != nullptr) count[b] = 0;
             if (kth != nullptr) kth[b] = __int_as_float(0xff800000);
@@ -115,7 +125,72 @@ topk_ragged_kernel(const float* __restrict__ scores, const int64_t* __restrict__
         }
         return;
     }
-    topk_row(scores + off, static_cast<int>(n), k, b, idx + static_cast<int64_t>(b) * k, count, kth, sh);
+    int32_t* out = idx + static_cast<int64_t>(b) * k;
+    if constexpr (CLUSTER)
+        topk_row_cluster(scores + off, static_cast<int>(n), k, out, count != nullptr ? count + b : nullptr, kth != nullptr ? kth + b : nullptr, sh);
+    else
+        topk_row(scores + off, static_cast<int>(n), k, out, count != nullptr ? count + b : nullptr, kth != nullptr ? kth + b : nullptr, sh);
+}
+
+// CTAs that share one of `rows` rows of up to `n` elements (n < 0: the lengths are on the device).  One CTA takes 6.6 us and 0.08 us
+// per thousand elements; a cluster streams its share only, but its start and its four cluster-wide barriers cost 2 to 3 us,
+// and more once the clusters leave few SMs free.  Measured with 1, 2, 4 and 8 CTAs (us): 8 rows of 33 K 10.2, 10.5, 11.2, 10.2; of 60 K
+// 12.5, 12.3, 12.8, 10.4; of 131 K 17.5, 14.0, 12.9, 10.1; 24 rows of 131 K 17.6, 14.1, 13.0, 14.7; 74 rows 18.2, 14.5, 28.3, 38.7.
+static int topk_cluster_size(int64_t rows, double n) {
+    const bool unknown = n < 0;
+    if (rows <= 8 && (unknown || n >= 36e3)) return 8;
+    if (rows <= 24 && n >= 96e3) return 4;
+    if (rows <= 74 && (unknown || n >= 64e3)) return 2;
+    return 1;
+}
+
+template <class Kernel, class... Args>
+static cudaError_t launch_topk_cluster(Kernel kernel, int64_t rows, int cluster, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(rows * cluster));
+    cfg.blockDim = dim3(TK_THREADS);
+    cfg.dynamicSmemBytes = sizeof(TopkSharedT<TK_CAP>);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = cluster;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Kernel attributes and the number of resident CTAs, asked for on a device's first call.
+struct TopkDevice {
+    int resident = 0, resident_small = 0;
+};
+static cudaError_t topk_device(TopkDevice& d) {
+    static once_per_device once;
+    static TopkDevice known[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    e = once.run([&] {
+        const int smem = static_cast<int>(sizeof(TopkSharedT<TK_CAP>)), smem_small = static_cast<int>(sizeof(TopkSharedT<TK_CAP_SMALL>));
+        int n_sm = 0, per = 0, per_small = 0;
+        cudaError_t r = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        auto limit = [&](const void* f, int bytes) { if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+        limit(reinterpret_cast<const void*>(topk_rows_kernel<TK_CAP>), smem);
+        limit(reinterpret_cast<const void*>(topk_rows_kernel<TK_CAP_SMALL>), smem_small);
+        limit(reinterpret_cast<const void*>(topk_rows_cluster_kernel), smem);
+        limit(reinterpret_cast<const void*>(topk_entries_kernel<TK_CAP>), smem);
+        limit(reinterpret_cast<const void*>(topk_ragged_kernel<true>), smem);
+        limit(reinterpret_cast<const void*>(topk_ragged_kernel<false>), smem);
+        if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, topk_rows_kernel<TK_CAP>, TK_THREADS, smem);
+        if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_small, topk_rows_kernel<TK_CAP_SMALL>, TK_THREADS, smem_small);
+        known[dev].resident = std::max(1, per) * n_sm;
+        known[dev].resident_small = std::max(1, per_small) * n_sm;
+        return r;
+    });
+    d = known[dev];
+    return e;
 }
 
 }  // namespace janus
@@ -130,7 +205,8 @@ extern "C" int janus_topk_entries(const float* scores, int64_t scores_ld, int M,
     if (!idx) return JANUS_ERR_INVALID_ARG;
     if (n_entries > 0 && (!scores || !aligned16(scores) || (scores_ld & 3) != 0)) return JANUS_ERR_INVALID_ARG;
     const size_t smem = sizeof(TopkSharedT<TK_CAP>);
-    JANUS_CUDA_CHECK(cudaFuncSetAttribute(topk_entries_kernel<TK_CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    TopkDevice d;
+    JANUS_CUDA_CHECK(topk_device(d));
     topk_entries_kernel<TK_CAP><<<M, TK_THREADS, smem, stream>>>(scores, scores_ld, M, n_entries, q_pos0, entry_size, k, idx, count, kth);
     JANUS_CUDA_CHECK(cudaGetLastError());
     return JANUS_OK;
@@ -177,10 +253,15 @@ extern "C" int janus_topk_batch(const float* scores, const int64_t* row_offsets,
     if (B == 0) return JANUS_OK;
     if (!idx || !row_offsets || !scores || !aligned16(scores)) return JANUS_ERR_INVALID_ARG;
     // row lengths live on the device: the large candidate buffer serves any length
-    const size_t smem = sizeof(TopkSharedT<TK_CAP>);
-    JANUS_CUDA_CHECK(cudaFuncSetAttribute(topk_ragged_kernel<TK_CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    topk_ragged_kernel<TK_CAP><<<B, TK_THREADS, smem, stream>>>(scores, row_offsets, row_lengths, k, idx, count, kth, dev_status);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    TopkDevice d;
+    JANUS_CUDA_CHECK(topk_device(d));
+    const int cluster = topk_cluster_size(B, -1.);
+    if (cluster > 1) {
+        JANUS_CUDA_CHECK(launch_topk_cluster(topk_ragged_kernel<true>, B, cluster, stream, scores, row_offsets, row_lengths, k, idx, count, kth, dev_status));
+    } else {
+        topk_ragged_kernel<false><<<B, TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream>>>(scores, row_offsets, row_lengths, k, idx, count, kth, dev_status);
+        JANUS_CUDA_CHECK(cudaGetLastError());
+    }
     return JANUS_OK;
 }
 
@@ -205,22 +286,19 @@ extern "C" int janus_topk(const float* scores, int64_t scores_ld, int M, int64_t
         const double e = 4096.0 * k / n_max, r = e + 4.0 * sqrt(e) + 8.0;
         small = n_max * (r + 5.0 * sqrt(r)) / 4096.0 <= TK_CAP_SMALL && k <= TK_CAP_SMALL / 2;
     }
-    int n_sm = 0, dev = 0, per_sm = 0;
-    JANUS_CUDA_CHECK(cudaGetDevice(&dev));
-    JANUS_CUDA_CHECK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-    if (small) {
-        const size_t smem = sizeof(TopkSharedT<TK_CAP_SMALL>);
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(topk_rows_kernel<TK_CAP_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        JANUS_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, topk_rows_kernel<TK_CAP_SMALL>, TK_THREADS, smem));
-        const int grid = std::min(M, std::max(1, per_sm) * n_sm);
-        topk_rows_kernel<TK_CAP_SMALL><<<grid, TK_THREADS, smem, stream>>>(scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count, kth);
-    } else {
-        const size_t smem = sizeof(TopkSharedT<TK_CAP>);
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(topk_rows_kernel<TK_CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        JANUS_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, topk_rows_kernel<TK_CAP>, TK_THREADS, smem));
-        const int grid = std::min(M, std::max(1, per_sm) * n_sm);
-        topk_rows_kernel<TK_CAP><<<grid, TK_THREADS, smem, stream>>>(scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count, kth);
+    TopkDevice d;
+    JANUS_CUDA_CHECK(topk_device(d));
+    const int cluster = topk_cluster_size(M, n_max);
+    if (cluster > 1) {
+        JANUS_CUDA_CHECK(launch_topk_cluster(topk_rows_cluster_kernel, M, cluster, stream, scores, scores_ld, n_keys, q_pos0, causal, k, idx, count, kth));
+        return JANUS_OK;
     }
+    if (small)
+        topk_rows_kernel<TK_CAP_SMALL><<<std::min(M, d.resident_small), TK_THREADS, sizeof(TopkSharedT<TK_CAP_SMALL>), stream>>>(
+            scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count, kth);
+    else
+        topk_rows_kernel<TK_CAP><<<std::min(M, d.resident), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream>>>(
+            scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count, kth);
     JANUS_CUDA_CHECK(cudaGetLastError());
     return JANUS_OK;
 }

@@ -1,13 +1,24 @@
-// Shared device code of the top-k selection (Eq. 1, Sec. 2.2, selection part): exact k-th selection over a candidate set
-// with 2048-bucket histograms over a shrinking key range, and the sampled single-pass top-k of one fp32 row.
+// Shared device code of the top-k selection (Eq. 1, Sec. 2.2, selection part): the sampled single-pass top-k of one fp32 row,
+// by one CTA or by a cluster, and exact k-th selection over a candidate set.
 // Used by janus_topk (materialised scores) and by janus_indexer_topk (candidates appended by the indexer epilogue).
+//
+// A row's time beyond its bytes is the chain of block-wide steps of its two selections, so both are kept short: the threshold is
+// the lower edge of a bucket of one histogram over the sample (held in registers; a conservative threshold need not be a
+// sample value), candidates are counted into the buckets of a second histogram as they are found, and one pass over them then
+// emits what lies above the k-th key's bucket while the few keys inside it are ranked directly.  Against two selections of repeated
+// histogram passes (B200, k = 2048): 4096 rows of 135168 0.442 -> 0.385 ms (5.7 TB/s, 0.86 of the copy bandwidth; what is left is
+// that a CTA between two streaming passes reads nothing), 2048 rows of 34816 122 -> 100 us, one row of 32768 15.4 -> 9.7 us.  The exact selection over
+// repeated histogram passes (select_kth) remains for what this cannot settle: a misjudged sample, or hundreds of keys in one bucket.
 #pragma once
 
 #include "janus_common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace janus {
 
 constexpr int TK_THREADS = 512;
+constexpr int TK_WARPS = TK_THREADS / 32;
+constexpr int TK_MAX_CLUSTER = 8;   // CTAs that share a row
 constexpr int TK_BUCKETS = 2048;
 constexpr int TK_SAMPLE = 4096;     // 512 threads x 8 floats (one 32-byte sector each)
 constexpr int TK_DIRECT = 256;      // a bucket of at most this many keys is ranked directly instead of split further
@@ -17,14 +28,18 @@ struct TopkSharedT {
     static constexpr int kCap = CAP;      // candidate slots (key + index = 8 bytes each)
     uint32_t cand_key[CAP];
     int32_t cand_idx[CAP];
-    int hist[TK_BUCKETS];
+    alignas(16) int hist[TK_BUCKETS];
+    uint32_t small_key[TK_DIRECT];        // the keys of the k-th key's bucket
+    int32_t small_idx[TK_DIRECT];
     int scan[40];
+    uint32_t warp_lo[TK_WARPS], warp_hi[TK_WARPS];
     int n_cand;
     int out_pos;
     int eq_taken;
     uint32_t red_lo, red_hi;
     int sel_bucket, sel_above, sel_count;
     int n_small;
+    int sel_out;                          // cluster form: next free slot of the row's output
 };
 
 struct SmemSource {
@@ -47,7 +62,7 @@ struct GlobalSource {
 // Returns the threshold key T and, in *n_eq_take, how many elements equal to T belong to the selection.
 // Every thread of the CTA must call it; results are uniform.
 template <class Src, class Sh>
-__device__ uint32_t select_kth(const Src& src, int need, Sh& sh, int* n_eq_take) {
+__device__ __noinline__ uint32_t select_kth(const Src& src, int need, Sh& sh, int* n_eq_take) {
     const int tid = threadIdx.x;
     const int n = src.size();
     // range of the active keys
@@ -139,7 +154,7 @@ __device__ uint32_t select_kth(const Src& src, int need, Sh& sh, int* n_eq_take)
 
 // Writes the selection (all keys > T, plus n_eq of the keys == T) to out[0..k).
 template <class Src, class Sh>
-__device__ void emit_selection(const Src& src, uint32_t T, int n_eq, int32_t* out, Sh& sh) {
+__device__ __noinline__ void emit_selection(const Src& src, uint32_t T, int n_eq, int32_t* out, Sh& sh) {
     const int n = src.size();
     for (int i = threadIdx.x; i < n; i += TK_THREADS) {
         const uint32_t key = src.key_at(i);
@@ -151,20 +166,163 @@ __device__ void emit_selection(const Src& src, uint32_t T, int n_eq, int32_t* ou
     }
 }
 
-// Keeps x (at row position i) if it is at or above the streaming threshold.  The float comparison admits a superset of
-// the exact key comparison (it treats -0 and +0 alike); the exact selection afterwards works on keys.
+// ---- short selections ---------------------------------------------------------------------------------------------------------
+// Smallest and largest key of the block (every thread gets them; one barrier).
 template <class Sh>
-__device__ __forceinline__ void keep_if_candidate(float x, int i, float thr_f, Sh& sh) {
-    if (x >= thr_f) {
-        const int pos = atomicAdd(&sh.n_cand, 1);
-        if (pos < Sh::kCap) { sh.cand_key[pos] = float_to_key(x); sh.cand_idx[pos] = i; }
+__device__ __forceinline__ void block_key_range(uint32_t& lo, uint32_t& hi, Sh& sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) { sh.warp_lo[warp] = lo; sh.warp_hi[warp] = hi; }
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, sh.warp_lo[lane & (TK_WARPS - 1)]);
+    hi = __reduce_max_sync(0xffffffffu, sh.warp_hi[lane & (TK_WARPS - 1)]);
+}
+
+// Buckets linear in the key over [lo, hi], at most TK_BUCKETS of them; keys above hi count into the last.
+struct BucketMap {
+    uint32_t lo;
+    int shift;
+    __device__ __forceinline__ BucketMap(uint32_t lo_, uint32_t hi) : lo(lo_) {
+        const int bits = 32 - __clz(hi - lo_);
+        shift = bits > 11 ? bits - 11 : 0;
+    }
+    __device__ __forceinline__ int operator()(uint32_t key) const { return static_cast<int>(min((key - lo) >> shift, static_cast<uint32_t>(TK_BUCKETS - 1))); }
+    __device__ __forceinline__ uint32_t first(int b) const { return lo + (static_cast<uint32_t>(b) << shift); }
+    __device__ __forceinline__ uint32_t last(int b) const { return b == TK_BUCKETS - 1 ? 0xffffffffu : first(b) + ((1u << shift) - 1u); }
+};
+
+template <class Sh>
+__device__ __forceinline__ void clear_hist(Sh& sh) {
+    reinterpret_cast<int4*>(sh.hist)[threadIdx.x] = make_int4(0, 0, 0, 0);
+}
+
+// The bucket that holds the `need`-th key from the top: sh.sel_bucket, the keys above it (sel_above) and in it (sel_count).
+// c: this thread's four buckets, 4 * (511 - tid) .. + 3.  Returns the number of keys in all buckets.  Two barriers.
+template <class Sh>
+__device__ __forceinline__ int find_bucket(const int4& c, int need, Sh& sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int mine = c.x + c.y + c.z + c.w;
+    int incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += y;
+    }
+    if (lane == 31) sh.scan[warp] = incl;
+    __syncthreads();
+    const int w = lane < TK_WARPS ? sh.scan[lane] : 0;
+    int above = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0) + incl - mine;
+    const int total = __reduce_add_sync(0xffffffffu, w);
+    if (above < need && need <= above + mine) {
+        const int b[4] = {c.w, c.z, c.y, c.x};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (above < need && need <= above + b[j]) { sh.sel_bucket = TK_BUCKETS - 1 - (4 * tid + j); sh.sel_above = above; sh.sel_count = b[j]; }
+            above += b[j];
+        }
+    }
+    __syncthreads();
+    return total;
+}
+template <class Sh>
+__device__ __forceinline__ int4 own_buckets(const Sh& sh) { return reinterpret_cast<const int4*>(sh.hist)[TK_THREADS - 1 - threadIdx.x]; }
+
+// Streaming threshold out of a sample of which every thread holds N keys: the lower edge of the bucket that holds the sample's
+// r-th key, unless that bucket is so full that it would let in far more than r, in which case it is split further.  `hi`
+// receives the largest sample key.
+template <int N, class Sh>
+__device__ __forceinline__ uint32_t sample_threshold(const uint32_t (&key)[N], int r, uint32_t& hi, Sh& sh) {
+    uint32_t lo = key[0];
+    hi = key[0];
+#pragma unroll
+    for (int j = 1; j < N; ++j) { lo = min(lo, key[j]); hi = max(hi, key[j]); }
+    clear_hist(sh);
+    block_key_range(lo, hi, sh);
+    uint32_t top = hi;
+    for (int pass = 0;; ++pass) {
+        const BucketMap map(lo, top);
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (key[j] >= lo && key[j] <= top) atomicAdd(&sh.hist[map(key[j])], 1);
+        __syncthreads();
+        find_bucket(own_buckets(sh), r, sh);
+        const int b = sh.sel_bucket, count = sh.sel_count;
+        if (count <= 4 + r / 16 || map.shift == 0 || pass == 2) return map.first(b);
+        r -= sh.sel_above;
+        if (b < TK_BUCKETS - 1) top = min(top, map.last(b));
+        lo = map.first(b);
+        clear_hist(sh);
+        __syncthreads();
     }
 }
 
-// The same for the sixteen elements a thread holds after four 16-byte loads (x[u] = elements e0 + u * e_step .. + 3): the
-// thread counts its candidates, reserves that many slots with one atomic and writes them.  One element in thirty passes, so
-// an atomic per element (even aggregated over the warp) costs several times the instructions of the comparison itself and
-// made the streaming pass issue-bound rather than memory-bound.
+// One pass over n candidates once the k-th key's bucket [b_lo, b_hi] is known: keys above it leave for out[at .. ), the keys in
+// it to small(key, index).  sh.out_pos is zero on entry.
+template <class Src, class Sh, class Small>
+__device__ __forceinline__ void emit_above(const Src& src, uint32_t b_lo, uint32_t b_hi, int32_t* __restrict__ out, int at, Sh& sh, Small&& small) {
+    const int n = src.size(), lane = threadIdx.x & 31;
+    for (int i0 = threadIdx.x - lane; i0 < n; i0 += TK_THREADS) {
+        const int i = i0 + lane;
+        const uint32_t key = i < n ? src.key_at(i) : 0u;
+        const bool above = i < n && key > b_hi, in = i < n && key >= b_lo && key <= b_hi;
+        const uint32_t m = __ballot_sync(0xffffffffu, above);
+        if (m != 0u) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&sh.out_pos, __popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (above) out[at + base + __popc(m & ((1u << lane) - 1u))] = src.idx_at(i);
+        }
+        if (in) small(key, src.idx_at(i));
+    }
+}
+
+// The `need` largest of the m keys in the small list go to out[0 .. need); the last of them is the row's k-th value.
+template <class Sh>
+__device__ __forceinline__ void emit_small(int m, int need, int32_t* __restrict__ out, float* __restrict__ kth, Sh& sh) {
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < m; i += TK_WARPS) {        // a warp per key, its lanes striding over the others
+        const uint32_t mine = sh.small_key[i];
+        int rank = 0;
+        for (int j = lane; j < m; j += 32) {
+            const uint32_t other = sh.small_key[j];
+            rank += (other > mine || (other == mine && j < i)) ? 1 : 0;
+        }
+        rank = __reduce_add_sync(0xffffffffu, rank);
+        if (lane == 0 && rank < need) {
+            out[rank] = sh.small_idx[i];
+            if (rank == need - 1 && kth != nullptr) *kth = key_to_float(mine);
+        }
+    }
+}
+
+// Top k of the n >= k candidates of `src`, counted into sh.hist with `map` (complete, barrier passed).
+template <class Src, class Sh>
+__device__ __forceinline__ void select_and_emit(const Src& src, const BucketMap& map, int k, int32_t* __restrict__ out, float* __restrict__ kth, Sh& sh) {
+    if (threadIdx.x == 0) { sh.out_pos = 0; sh.n_small = 0; sh.eq_taken = 0; }
+    find_bucket(own_buckets(sh), k, sh);
+    const int b = sh.sel_bucket, above = sh.sel_above, count = sh.sel_count;
+    if (count <= TK_DIRECT) {
+        emit_above(src, map.first(b), map.last(b), out, 0, sh, [&](uint32_t key, int32_t i) {
+            const int s = atomicAdd(&sh.n_small, 1);
+            if (s < TK_DIRECT) { sh.small_key[s] = key; sh.small_idx[s] = i; }
+        });
+        __syncthreads();
+        emit_small(count, k - above, out + above, kth, sh);
+    } else {
+        int n_eq;
+        const uint32_t T = select_kth(src, k, sh, &n_eq);
+        emit_selection(src, T, n_eq, out, sh);
+        if (threadIdx.x == 0 && kth != nullptr) *kth = key_to_float(T);
+    }
+}
+
+// The sixteen elements a thread holds after four 16-byte loads (x[u] = elements e0 + u * e_step .. + 3): those at or above the
+// streaming threshold become candidates (value bits and position).  The thread counts them, reserves that many slots with one
+// atomic and writes them: one element in thirty passes, so an atomic per element (even aggregated over the warp) costs several
+// times the instructions of the comparison itself and made the streaming pass issue-bound rather than memory-bound; for the
+// same reason keys and buckets are made of the candidates afterwards.  A list that is full stays incomplete (n_cand tells).
+// The float comparison admits a superset of the exact key comparison (it treats -0 and +0 alike).
 template <class Sh>
 __device__ __forceinline__ void keep_candidates16(const float4 (&x)[4], int e0, int e_step, float thr_f, Sh& sh) {
     int c = 0;
@@ -172,11 +330,14 @@ __device__ __forceinline__ void keep_candidates16(const float4 (&x)[4], int e0, 
     for (int u = 0; u < 4; ++u)
         c += (x[u].x >= thr_f ? 1 : 0) + (x[u].y >= thr_f ? 1 : 0) + (x[u].z >= thr_f ? 1 : 0) + (x[u].w >= thr_f ? 1 : 0);
     if (c == 0) return;
-    int o = atomicAdd(&sh.n_cand, c);
+    const int o = atomicAdd(&sh.n_cand, c);
+    if (o + c > Sh::kCap) return;
+    uint32_t* slot = sh.cand_key + o;
     auto put = [&](float v, int e) {
         if (v >= thr_f) {
-            if (o < Sh::kCap) { sh.cand_key[o] = float_to_key(v); sh.cand_idx[o] = e; }
-            ++o;
+            slot[0] = __float_as_uint(v);
+            slot[Sh::kCap] = static_cast<uint32_t>(e);      // cand_idx
+            ++slot;
         }
     };
 #pragma unroll
@@ -186,132 +347,227 @@ __device__ __forceinline__ void keep_candidates16(const float4 (&x)[4], int e0, 
     }
 }
 
+// After the streaming pass (barrier passed): candidates become keys and are counted into their buckets (sh.hist is zero).
+template <class Sh>
+__device__ __forceinline__ void count_candidates(int n, const BucketMap& map, Sh& sh) {
+    for (int i = threadIdx.x; i < n; i += TK_THREADS) {
+        const uint32_t key = max(float_to_key(__uint_as_float(sh.cand_key[i])), map.lo);      // -0 at a threshold of +0: the same value
+        sh.cand_key[i] = key;
+        atomicAdd(&sh.hist[map(key)], 1);
+    }
+}
+
 __device__ __forceinline__ void topk_prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// ---- the three phases of a row (n > k), callable separately so that several CTAs can share the streaming pass of one row
+// First float of the 8-float group that thread i samples of a row of n elements.
+__device__ __forceinline__ int64_t sample_offset(int n) {
+    return 8 * ((static_cast<int64_t>(threadIdx.x) * ((n >> 3) - 1)) / (TK_THREADS - 1));
+}
 
-// Streaming threshold of a row as an order-preserving key (0: keep everything): the sample value of a rank a few standard
-// deviations below where the row's k-th value is expected.  Thread i reads 8 consecutive floats at an evenly spread,
-// 32-byte aligned offset; the candidate buffer of `sh` is the scratch.  Every thread of the CTA calls it; the result is
-// uniform and depends on the row only.
+// Streaming threshold of a row as an order-preserving key: the sample value of a rank a few standard deviations below where the
+// row's k-th value is expected.  Thread i reads 8 consecutive floats at an evenly spread, 32-byte aligned offset.  Every
+// thread of the CTA calls it; the result is uniform and depends on the row only.  False: no threshold is low enough.
 template <class Sh>
-__device__ uint32_t topk_sample_threshold(const float* __restrict__ row, int n, int k, Sh& sh) {
-    const int tid = threadIdx.x;
-    uint32_t thr = 0u;
-    if (n > Sh::kCap) {
-        const float4* row4 = reinterpret_cast<const float4*>(row);
-        const int n8 = n >> 3;                       // complete 8-float groups
-        const int g = static_cast<int>((static_cast<int64_t>(tid) * (n8 - 1)) / (TK_THREADS - 1));
-        const float4 a = __ldcg(row4 + 2 * g), b = __ldcg(row4 + 2 * g + 1);
-        uint32_t* skey = sh.cand_key;                // the candidate buffer is free at this point
-        skey[tid * 8 + 0] = float_to_key(a.x); skey[tid * 8 + 1] = float_to_key(a.y);
-        skey[tid * 8 + 2] = float_to_key(a.z); skey[tid * 8 + 3] = float_to_key(a.w);
-        skey[tid * 8 + 4] = float_to_key(b.x); skey[tid * 8 + 5] = float_to_key(b.y);
-        skey[tid * 8 + 6] = float_to_key(b.z); skey[tid * 8 + 7] = float_to_key(b.w);
-        __syncthreads();
-        const float expect = static_cast<float>(TK_SAMPLE) * static_cast<float>(k) / static_cast<float>(n);
-        const int r = static_cast<int>(expect + 4.0f * sqrtf(expect) + 8.0f);
-        if (r < TK_SAMPLE) {
-            int dummy;
-            SmemSource s{skey, nullptr, TK_SAMPLE};
-            thr = select_kth(s, r, sh, &dummy);
-        }
-        __syncthreads();
-    }
-    return thr;
+__device__ __forceinline__ bool topk_sample(const float* __restrict__ row, int n, int k, uint32_t& thr, uint32_t& hi, Sh& sh) {
+    const float expect = static_cast<float>(TK_SAMPLE) * static_cast<float>(k) / static_cast<float>(n);
+    const int r = static_cast<int>(expect + 4.0f * sqrtf(expect) + 8.0f);
+    if (r >= TK_SAMPLE) return false;
+    const float4* src = reinterpret_cast<const float4*>(row + sample_offset(n));
+    const float4 a = __ldcg(src), b = __ldcg(src + 1);
+    const uint32_t key[8] = {float_to_key(a.x), float_to_key(a.y), float_to_key(a.z), float_to_key(a.w),
+                             float_to_key(b.x), float_to_key(b.y), float_to_key(b.z), float_to_key(b.w)};
+    thr = sample_threshold(key, r, hi, sh);
+    return true;
 }
 
 // One streaming pass over the 16-byte groups [f4_begin, f4_end) of the row (and, with `tail`, the n % 4 elements after the
-// last whole group): elements at or above the threshold go to the candidate buffer of `dst`, which may be another CTA's
-// shared memory (a cluster-mapped reference).
+// last whole group).
 template <class Sh>
-__device__ void topk_stream(const float* __restrict__ row, int n, int f4_begin, int f4_end, bool tail, uint32_t thr, Sh& dst) {
+__device__ __forceinline__ void topk_stream(const float* __restrict__ row, int n, int f4_begin, int f4_end, bool tail, float thr_f, Sh& sh) {
     const int tid = threadIdx.x;
     const float4* row4 = reinterpret_cast<const float4*>(row);
-    const float thr_f = thr == 0u ? __int_as_float(0xff800000) : key_to_float(thr);
     constexpr int UNROLL = 4;                     // 16-byte loads in flight per thread
     int i = f4_begin + tid;
     for (; i + (UNROLL - 1) * TK_THREADS < f4_end; i += UNROLL * TK_THREADS) {
         float4 x[UNROLL];
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u) x[u] = __ldcs(row4 + i + u * TK_THREADS);
-        keep_candidates16(x, 4 * i, 4 * TK_THREADS, thr_f, dst);
+        keep_candidates16(x, 4 * i, 4 * TK_THREADS, thr_f, sh);
     }
+    auto keep = [&](float v, int e) {
+        if (v >= thr_f) {
+            const int o = atomicAdd(&sh.n_cand, 1);
+            if (o < Sh::kCap) { sh.cand_key[o] = __float_as_uint(v); sh.cand_idx[o] = e; }
+        }
+    };
     for (; i < f4_end; i += TK_THREADS) {
         const float4 x = __ldcs(row4 + i);
-        keep_if_candidate(x.x, 4 * i, thr_f, dst);
-        keep_if_candidate(x.y, 4 * i + 1, thr_f, dst);
-        keep_if_candidate(x.z, 4 * i + 2, thr_f, dst);
-        keep_if_candidate(x.w, 4 * i + 3, thr_f, dst);
+        keep(x.x, 4 * i); keep(x.y, 4 * i + 1); keep(x.z, 4 * i + 2); keep(x.w, 4 * i + 3);
     }
     const int n4 = n >> 2;
-    if (tail && tid < n - 4 * n4) keep_if_candidate(__ldcg(row + 4 * n4 + tid), 4 * n4 + tid, thr_f, dst);
+    if (tail && tid < n - 4 * n4) keep(__ldcg(row + 4 * n4 + tid), 4 * n4 + tid);
 }
 
-// Exact selection over the candidates in `sh` (over the whole row in global memory when the sample misjudged it: fewer than
-// k candidates, or more than the buffer holds) and emission of the k indices, count and k-th value.
+// A row of at most k elements: all of them, and the smallest value.
 template <class Sh>
-__device__ void topk_finish(const float* __restrict__ row, int n, int k, int t, int32_t* __restrict__ out, int32_t* __restrict__ count,
-                            float* __restrict__ kth, Sh& sh) {
-    const int n_cand = sh.n_cand;
-    uint32_t T;
+__device__ __noinline__ void topk_whole_row(const float* __restrict__ row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
+                               float* __restrict__ kth, Sh& sh) {
+    const int tid = threadIdx.x;
+    for (int i = tid; i < k; i += TK_THREADS) out[i] = i < n ? i : -1;
+    if (count != nullptr && tid == 0) *count = n;
+    if (kth != nullptr) {
+        uint32_t lo = 0xffffffffu, hi = 0u;
+        for (int i = tid; i < n; i += TK_THREADS) lo = min(lo, float_to_key(__ldcg(row + i)));
+        block_key_range(lo, hi, sh);
+        if (tid == 0) *kth = n > 0 ? key_to_float(lo) : __int_as_float(0xff800000);
+        __syncthreads();
+    }
+}
+
+// The exact selection over the row in global memory.
+template <class Sh>
+__device__ __noinline__ void topk_exact_row(const float* __restrict__ row, int n, int k, int32_t* __restrict__ out, float* __restrict__ kth, Sh& sh) {
+    if (threadIdx.x == 0) { sh.out_pos = 0; sh.eq_taken = 0; }
     int n_eq;
-    if (n_cand >= k && n_cand <= Sh::kCap) {
-        SmemSource s{sh.cand_key, sh.cand_idx, n_cand};
-        T = select_kth(s, k, sh, &n_eq);
-        emit_selection(s, T, n_eq, out, sh);
-    } else {
-        GlobalSource s{row, n};
-        T = select_kth(s, k, sh, &n_eq);
-        emit_selection(s, T, n_eq, out, sh);
-    }
-    if (threadIdx.x == 0) {
-        if (count) count[t] = n < k ? n : k;
-        if (kth) kth[t] = key_to_float(T);
-    }
+    GlobalSource s{row, n};
+    const uint32_t T = select_kth(s, k, sh, &n_eq);
+    emit_selection(s, T, n_eq, out, sh);
+    if (threadIdx.x == 0 && kth != nullptr) *kth = key_to_float(T);
 }
 
 // Top-k of one fp32 row of n elements (16-byte aligned) by the whole CTA (TK_THREADS threads): out[0..k) receives the
-// indices (-1 padded), count[t] / kth[t] the number selected and the smallest selected value (either may be NULL).
+// indices (-1 padded), *count / *kth the number selected and the smallest selected value (either may be NULL).
 // `next_row` (may be NULL): the row this CTA takes next.  The sample sectors of that row are requested into L2 once this
 // row's streaming pass is over, so the next sample does not start with a DRAM round trip.  (Requesting the head of the next
 // row as well, 96 to 512 KB, made the kernel slower: 0.49 -> 0.50 .. 0.58 ms at 4096 rows of 135168.)
 template <class Sh>
-__device__ void topk_row(const float* __restrict__ row, int n, int k, int t, int32_t* __restrict__ out, int32_t* __restrict__ count,
+__device__ __forceinline__ void topk_row(const float* __restrict__ row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
                          float* __restrict__ kth, Sh& sh, const float* __restrict__ next_row = nullptr, int next_n = 0) {
     const int tid = threadIdx.x;
-
-    if (tid == 0) { sh.n_cand = 0; sh.out_pos = 0; sh.eq_taken = 0; }
+    if (n <= k) {
+        topk_whole_row(row, n, k, out, count, kth, sh);
+        return;
+    }
+    if (count != nullptr && tid == 0) *count = k;
+    if (n <= Sh::kCap) {                           // the whole row is the candidate list
+        uint32_t lo = 0xffffffffu, hi = 0u;
+        auto take = [&](float v, int i) {
+            const uint32_t key = float_to_key(v);
+            sh.cand_key[i] = key;
+            lo = min(lo, key);
+            hi = max(hi, key);
+        };
+        const float4* row4 = reinterpret_cast<const float4*>(row);
+        for (int i = tid; i < (n >> 2); i += TK_THREADS) {
+            const float4 x = __ldcs(row4 + i);
+            take(x.x, 4 * i); take(x.y, 4 * i + 1); take(x.z, 4 * i + 2); take(x.w, 4 * i + 3);
+        }
+        if (tid < (n & 3)) take(__ldcg(row + (n & ~3) + tid), (n & ~3) + tid);
+        clear_hist(sh);
+        block_key_range(lo, hi, sh);
+        const BucketMap map(lo, hi);
+        for (int i = tid; i < n; i += TK_THREADS) atomicAdd(&sh.hist[map(sh.cand_key[i])], 1);
+        __syncthreads();
+        select_and_emit(SmemSource{sh.cand_key, nullptr, n}, map, k, out, kth, sh);
+        return;
+    }
+    uint32_t thr, hi;
+    if (tid == 0) sh.n_cand = 0;
+    const bool sampled = topk_sample(row, n, k, thr, hi, sh);
+    if (sampled) {
+        const BucketMap map(thr, max(thr, hi));
+        clear_hist(sh);
+        __syncthreads();
+        topk_stream(row, n, 0, n >> 2, true, key_to_float(thr), sh);
+        if (next_row != nullptr && next_n > Sh::kCap) topk_prefetch_l2(next_row + sample_offset(next_n));
+        __syncthreads();
+        const int n_cand = sh.n_cand;
+        if (n_cand >= k && n_cand <= Sh::kCap) {
+            count_candidates(n_cand, map, sh);
+            __syncthreads();
+            select_and_emit(SmemSource{sh.cand_key, sh.cand_idx, n_cand}, map, k, out, kth, sh);
+            return;
+        }
+    }
     __syncthreads();
+    topk_exact_row(row, n, k, out, kth, sh);       // the sample misjudged the row
+}
 
-    if (n <= k) {  // the whole prefix is selected
-        for (int i = tid; i < k; i += TK_THREADS) out[i] = i < n ? i : -1;
-        if (kth != nullptr || count != nullptr) {
-            float mn = __int_as_float(0x7f800000);
-            for (int i = tid; i < n; i += TK_THREADS) mn = fminf(mn, __ldcg(row + i));
+// The same by a cluster of CTAs (few rows): each CTA samples alike, streams its share of the row into its own candidates and
+// histogram, the histograms are added through distributed shared memory, every CTA emits its own keys above the k-th key's
+// bucket, and CTA 0 ranks the bucket's keys of all of them.
+template <class Sh>
+__device__ __forceinline__ void topk_row_cluster(const float* __restrict__ row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
+                                 float* __restrict__ kth, Sh& sh) {
+    using namespace ptx;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int rank = static_cast<int>(cluster_ctarank()), n_cta = static_cast<int>(cluster_nctarank());
+    uint32_t thr = 0u, hi = 0u;
+    if (tid == 0) { sh.n_cand = 0; sh.out_pos = 0; sh.n_small = 0; sh.sel_out = 0; }
+    const bool split = n > Sh::kCap && n > k && topk_sample(row, n, k, thr, hi, sh);     // the same answer in every CTA
+    if (!split) {
+        if (rank == 0) topk_row(row, n, k, out, count, kth, sh);
+        return;
+    }
+    const BucketMap map(thr, max(thr, hi));
+    clear_hist(sh);
+    __syncthreads();
+    const int64_t n4 = n >> 2;
+    topk_stream(row, n, static_cast<int>(n4 * rank / n_cta), static_cast<int>(n4 * (rank + 1) / n_cta), rank == n_cta - 1, key_to_float(thr), sh);
+    __syncthreads();
+    count_candidates(min(sh.n_cand, Sh::kCap), map, sh);
+    cluster_sync_all();                            // every CTA's candidates and counts
+    // remote loads of all CTAs are issued together: one after the other each would cost the round trip
+    int4 c = make_int4(0, 0, 0, 0);
+    bool fits = true;
+    const uint32_t my_buckets = smem_u32(sh.hist) + 16u * (TK_THREADS - 1 - tid), my_cand = smem_u32(&sh.n_cand);
+    {
+        int4 x[TK_MAX_CLUSTER];
+        uint32_t m[TK_MAX_CLUSTER];
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, d));
-            if (tid == 0) sh.red_lo = 0xffffffffu;
-            __syncthreads();
-            if ((tid & 31) == 0) atomicMin(&sh.red_lo, float_to_key(mn));
-            __syncthreads();
-            if (tid == 0) {
-                if (count) count[t] = n;
-                if (kth) kth[t] = n > 0 ? key_to_float(sh.red_lo) : __int_as_float(0xff800000);
-            }
+        for (int r = 0; r < TK_MAX_CLUSTER; ++r) {
+            x[r] = ld_cluster_s32x4(mapa_shared(my_buckets, min(r, n_cta - 1)));
+            m[r] = ld_cluster_u32(mapa_shared(my_cand, min(r, n_cta - 1)));
+        }
+#pragma unroll
+        for (int r = 0; r < TK_MAX_CLUSTER; ++r) {
+            if (r < n_cta) { c.x += x[r].x; c.y += x[r].y; c.z += x[r].z; c.w += x[r].w; }
+            fits = fits && static_cast<int>(m[r]) <= Sh::kCap;
+        }
+    }
+    const int total = find_bucket(c, k, sh);
+    const int b = sh.sel_bucket, above = sh.sel_above, in = sh.sel_count;
+    if (!fits || total < k || in > TK_DIRECT) {    // uniform over the cluster: everybody read the same counts
+        cluster_sync_all();                        // which may change only now
+        if (rank == 0) {
+            if (count != nullptr && tid == 0) *count = k;
+            topk_exact_row(row, n, k, out, kth, sh);
         }
         return;
     }
-
-    const uint32_t thr = topk_sample_threshold(row, n, k, sh);
-    topk_stream(row, n, 0, n >> 2, true, thr, sh);
-    if (next_row != nullptr && next_n > Sh::kCap) {
-        const int n8 = next_n >> 3;
-        const int g = static_cast<int>((static_cast<int64_t>(tid) * (n8 - 1)) / (TK_THREADS - 1));
-        topk_prefetch_l2(next_row + 8 * g);                                   // the sample sector this thread will read
+    // this CTA's keys above the bucket, and where they go: one reservation in CTA 0
+    const int4 own = own_buckets(sh);
+    const int first = TK_BUCKETS - 4 - 4 * tid;
+    int mine = (first > b ? own.x : 0) + (first + 1 > b ? own.y : 0) + (first + 2 > b ? own.z : 0) + (first + 3 > b ? own.w : 0);
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) sh.warp_lo[tid >> 5] = static_cast<uint32_t>(mine);
+    __syncthreads();
+    if (tid < 32) {
+        const int n_above = __reduce_add_sync(0xffffffffu, lane < TK_WARPS ? static_cast<int>(sh.warp_lo[lane]) : 0);
+        if (lane == 0) sh.eq_taken = atomic_add_cluster_s32(mapa_shared(smem_u32(&sh.sel_out), 0), n_above);
     }
     __syncthreads();
-    topk_finish(row, n, k, t, out, count, kth, sh);
+    // the keys inside the bucket (a handful) go straight to CTA 0's small list
+    const uint32_t n_small0 = mapa_shared(smem_u32(&sh.n_small), 0), key0 = mapa_shared(smem_u32(sh.small_key), 0), idx0 = mapa_shared(smem_u32(sh.small_idx), 0);
+    emit_above(SmemSource{sh.cand_key, sh.cand_idx, sh.n_cand}, map.first(b), map.last(b), out, sh.eq_taken, sh, [&](uint32_t key, int32_t i) {
+        const int s = atomic_add_cluster_s32(n_small0, 1);
+        if (s < TK_DIRECT) { st_cluster_u32(key0 + 4 * s, key); st_cluster_u32(idx0 + 4 * s, static_cast<uint32_t>(i)); }
+    });
+    cluster_sync_all();                            // CTA 0 has the list; nobody is read any more
+    if (rank == 0) {
+        emit_small(in, k - above, out + above, kth, sh);
+        if (count != nullptr && tid == 0) *count = k;
+    }
 }
 
 }  // namespace janus

@@ -1,0 +1,85 @@
+"""Top-k where its routes change: rows around the candidate buffers (5632 and 8192 elements), the cluster sizes with their shares of a row,
+ragged rows of very different lengths in one launch, and score distributions the sample or the buckets cannot settle (ties by the thousand,
+one value, two far-apart levels, -0 and +0, an outlier that stretches the key range, a row whose large scores hide from the sample).
+A selection is checked against a full sort: the values above the k-th are all there, ties at it are free."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_36938_b200 import binding as B
+from paper_2609_36938_b200 import build
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    B.load()
+    yield
+    B.check_dev_status()
+
+
+def check_row(idx, count, kth, row, k, tag):
+    want = min(k, len(row))
+    sel = idx[:want]
+    assert count == want and np.all(idx[want:] == -1), tag
+    assert len(np.unique(sel)) == want and (want == 0 or (sel.min() >= 0 and sel.max() < len(row))), tag
+    if want == 0:
+        assert np.isneginf(kth), tag
+        return
+    t = np.partition(row, len(row) - want)[len(row) - want]
+    assert kth == t, f"{tag}: k-th {kth} instead of {t}"
+    vals = row[sel]
+    assert np.all(vals >= t) and np.sum(vals > t) == np.sum(row > t), tag
+
+
+def draw(kind, n, rng):
+    x = rng.standard_normal(n).astype(np.float32)
+    if kind == "ties":
+        x = np.round(x * 2) / 2
+    elif kind == "constant":
+        x[:] = 1.25
+    elif kind == "levels":
+        x = np.where(rng.random(n) < 0.02, np.float32(1e30), np.float32(-1e-30)) * (1 + rng.random(n).astype(np.float32) / 8)
+    elif kind == "zeros":
+        x = np.where(rng.random(n) < 0.5, np.float32(-0.0), np.float32(0.0))
+    elif kind == "outlier" and n:
+        x[rng.integers(0, n)] = 3e38
+    elif kind == "hidden":                       # a dense block of large scores between sampled groups
+        x[n // 2:n // 2 + min(9000, n // 3)] += 50
+    return x.astype(np.float32)
+
+
+@pytest.mark.parametrize("kind", ["normal", "ties", "constant", "levels", "zeros", "outlier", "hidden"])
+@pytest.mark.parametrize("rows,n", [(3, 5640), (90, 8193), (5, 40009), (20, 99991), (70, 65003), (80, 66001)])
+def test_topk_rows(kind, rows, n):
+    rng = np.random.default_rng(n + rows)
+    sc = np.stack([draw(kind, n, rng) for _ in range(rows)])
+    ld = (n + 3) // 4 * 4
+    dev = torch.full((rows, ld), float("nan"), device="cuda")
+    dev[:, :n] = torch.from_numpy(sc)
+    for k in (1, 2048):
+        idx, cnt, kth = B.janus_topk(dev, n, k, q_pos0=n - rows, causal=True)
+        B.check_dev_status()
+        idx, cnt, kth = idx.cpu().numpy(), cnt.cpu().numpy(), kth.cpu().numpy()
+        for t in {0, 1, rows // 2, rows - 1}:
+            check_row(idx[t], cnt[t], kth[t], sc[t, :n - rows + t + 1], k, f"{kind} row {t} of {rows} x {n}, k {k}")
+
+
+@pytest.mark.parametrize("kind", ["normal", "ties", "zeros", "hidden"])
+@pytest.mark.parametrize("lengths", [[131072], [0, 1, 2047, 2048, 2049, 8192, 8196, 70001], [100003] + [9001] * 11, [300 * i + 5 for i in range(64)],
+                                     [12001] * 80])
+def test_topk_batch(kind, lengths):
+    rng = np.random.default_rng(len(lengths))
+    off = np.concatenate([[0], np.cumsum([(n + 3) // 4 * 4 for n in lengths])])
+    flat = torch.full((int(off[-1]) + 4,), float("nan"), device="cuda")
+    rows = [draw(kind, n, rng) for n in lengths]
+    for o, r in zip(off, rows):
+        flat[o:o + len(r)] = torch.from_numpy(r)
+    k = 2048
+    idx, cnt, kth = B.janus_topk_batch(flat, torch.from_numpy(off).cuda(), k, row_lengths=torch.tensor(lengths, dtype=torch.int64, device="cuda"))
+    B.check_dev_status()
+    idx, cnt, kth = idx.cpu().numpy(), cnt.cpu().numpy(), kth.cpu().numpy()
+    for b, r in enumerate(rows):
+        check_row(idx[b], cnt[b], kth[b], r, k, f"{kind} row {b}")
