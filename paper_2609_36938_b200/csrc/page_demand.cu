@@ -58,7 +58,7 @@ __device__ __forceinline__ void set_bit_shared(uint32_t* bm, int p) {
 // A CTA's tokens become bits of its own bitmap of logical pages; at the end its set pages go through the page table into a
 // bitmap of physical pages, whose words are ORed into the global one (page by page they would be a contended atomic each:
 // 109 us).
-// Whole call at 4096 x 2048 indices: 35 us when every index went through the page table, 25.9 now; 8192 x 2048: 65.8 and 36.9.
+// Whole call at 4096 x 2048 indices: 35 us when every index went through the page table, 24.7 now; 8192 x 2048: 65.8 and 35.7.
 __global__ void __launch_bounds__(MARK_THREADS)
 page_mark_kernel(const PdParams p, int n_log_words) {
     extern __shared__ uint32_t lbm[];
@@ -242,9 +242,12 @@ page_demand_kernel(const PdParams p) {
         } else {
             const uint32_t addr = smem_u32(bm + i);
             uint32_t v = 0u;
+            for (int r0 = 0; r0 < n_cta; r0 += 4) {      // clusters of 4, 8 or 16; four round trips overlap
+                uint32_t x[4];
 #pragma unroll
-            for (int r = 0; r < PD_MAX_CLUSTER; ++r)
-                if (r < n_cta) v |= ld_cluster_u32(mapa_shared(addr, r));
+                for (int r = 0; r < 4; ++r) x[r] = ld_cluster_u32(mapa_shared(addr, r0 + r));
+                v |= (x[0] | x[1]) | (x[2] | x[3]);
+            }
             return v;
         }
     };
@@ -289,18 +292,18 @@ page_demand_kernel(const PdParams p) {
     }
     if (tid == 0) { sh.totals[0] = sum[0]; sh.totals[1] = sum[1]; }
     cluster_sync_all();                   // counts are there; nobody reads the private bitmaps any more
-    uint64_t base[2] = {0, 0}, all[2] = {0, 0};
+    uint64_t base[2], all[2];             // lane r fetches CTA r's counts
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        const uint32_t addr = smem_u32(&sh.totals[q]);
+        uint64_t x = lane < n_cta ? ld_cluster_u64(mapa_shared(smem_u32(&sh.totals[q]), lane)) : 0;
+        uint64_t y = lane < rank ? x : 0;
 #pragma unroll
-        for (int r = 0; r < PD_MAX_CLUSTER; ++r) {
-            if (r < n_cta) {
-                const uint64_t x = ld_cluster_u64(mapa_shared(addr, r));
-                all[q] += x;
-                if (r < rank) base[q] += x;
-            }
+        for (int d = PD_MAX_CLUSTER / 2; d > 0; d >>= 1) {
+            x += __shfl_xor_sync(0xffffffffu, x, d);
+            y += __shfl_xor_sync(0xffffffffu, y, d);
         }
+        all[q] = __shfl_sync(0xffffffffu, x, 0);
+        base[q] = __shfl_sync(0xffffffffu, y, 0);
     }
     for (int c0 = w0; c0 < w1; c0 += PD_THREADS) {
         if (!one_chunk) {
@@ -381,11 +384,11 @@ static int launch_page_demand(const PdParams& p, int cluster, cudaStream_t strea
     return JANUS_OK;
 }
 
-// One launch of one cluster while it reads the indices as fast as memset, chip-wide marking and lists would (14.4 us up to 512 K
-// indices): 128 K indices in 13 us, 256 K in 15.  Four CTAs up to 4 K indices (9.1 us, 9.6 with eight, 11.8 with sixteen), eight
-// up to 64 K (10.9 against 12.6 and 11.8 with four and sixteen at 256 x 256), sixteen beyond (64 rows of a 131136-page pool: 25.3
-// against 35.5 with eight and 27.5 for the three launches).  Memset, marking and one-CTA lists took 14.6, 18.5 and 36.6 us
-// for these three.
+// One launch of one cluster while it reads the indices as fast as memset, chip-wide marking and lists would (14 us up to 512 K
+// indices): 128 K indices in 12 us, 256 K in 15.  Four CTAs up to 4 K indices (7.6 us; eight and sixteen cost 0.5 and 2.5 us more),
+// eight up to 64 K (9.3 us at 256 x 256, four and sixteen 1 to 2 us more), sixteen beyond (64 rows of a 131136-page pool: 24.9
+// against 35 with eight and 27 for the three launches).  Memset, marking and one-CTA lists took 14.6, 18.5 and 36.6 us for these
+// three.
 constexpr int64_t PD_ONE_LAUNCH_INDICES = 1 << 17;
 
 template <int MODE>

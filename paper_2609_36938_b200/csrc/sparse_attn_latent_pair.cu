@@ -134,37 +134,42 @@ __device__ __forceinline__ float4 lp_ld_cluster4(uint32_t addr) {
     return v;
 }
 
-// Output of token t from the `n_split` pairs' unnormalised outputs: CTA (s, c) takes every n_split-th block of 16 columns of value
-// half c, a thread one block of one head at a time.
-__device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s, int n_split, uint32_t c, uint32_t o_addr, uint32_t stats_addr) {
+// Output of token t from the N pairs' unnormalised outputs: CTA (s, c) takes every N-th block of 16 columns of value half c, a
+// thread one block of one head at a time.  N is a compile-time number so that all remote loads are issued together.
+template <int N>
+__device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s, uint32_t c, uint32_t o_addr, uint32_t stats_addr) {
     const int h = threadIdx.x & (LP_HEADS - 1);
-    float f[LP_MAX_SPLIT];
-    float m_all = __int_as_float(0xff800000), l_all = 0.f;
+    const float neg_inf = __int_as_float(0xff800000);
+    float f[N], l[N];
+    float m_all = neg_inf, l_all = 0.f;
 #pragma unroll
-    for (int r = 0; r < LP_MAX_SPLIT; ++r) {
-        f[r] = r < n_split ? lp_ld_cluster(mapa_shared(stats_addr + 4 * h, 2 * r + c)) : __int_as_float(0xff800000);
-        m_all = fmaxf(m_all, f[r]);
+    for (int r = 0; r < N; ++r) {
+        f[r] = lp_ld_cluster(mapa_shared(stats_addr + 4 * h, 2 * r + c));
+        l[r] = lp_ld_cluster(mapa_shared(stats_addr + 4 * (LP_HEADS + h), 2 * r + c));
     }
 #pragma unroll
-    for (int r = 0; r < LP_MAX_SPLIT; ++r) {
-        f[r] = m_all == __int_as_float(0xff800000) ? 0.f : lp_exp2(f[r] - m_all);
-        if (r < n_split) l_all += f[r] * lp_ld_cluster(mapa_shared(stats_addr + 4 * (LP_HEADS + h), 2 * r + c));
+    for (int r = 0; r < N; ++r) m_all = fmaxf(m_all, f[r]);
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+        f[r] = m_all == neg_inf ? 0.f : lp_exp2(f[r] - m_all);
+        l_all = fmaf(f[r], l[r], l_all);
     }
     const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
-    for (int blk = s + n_split * (threadIdx.x / LP_HEADS); blk < LP_DVH / 16; blk += n_split * (LP_THREADS / LP_HEADS)) {
-        float4 acc[4] = {};
+    for (int blk = s + N * (threadIdx.x / LP_HEADS); blk < LP_DVH / 16; blk += N * (LP_THREADS / LP_HEADS)) {
+        float4 x[N][4], acc[4] = {};
 #pragma unroll
-        for (int r = 0; r < LP_MAX_SPLIT; ++r) {
-            if (r < n_split && f[r] != 0.f) {
-                const uint32_t src = mapa_shared(o_addr + static_cast<uint32_t>((blk * 4 * LP_HEADS + h) * 16), 2 * r + c);
+        for (int r = 0; r < N; ++r) {
+            const uint32_t src = mapa_shared(o_addr + static_cast<uint32_t>((blk * 4 * LP_HEADS + h) * 16), 2 * r + c);
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const float4 x = lp_ld_cluster4(src + v * LP_HEADS * 16);
-                    acc[v].x = fmaf(f[r], x.x, acc[v].x); acc[v].y = fmaf(f[r], x.y, acc[v].y);
-                    acc[v].z = fmaf(f[r], x.z, acc[v].z); acc[v].w = fmaf(f[r], x.w, acc[v].w);
-                }
-            }
+            for (int v = 0; v < 4; ++v) x[r][v] = lp_ld_cluster4(src + v * LP_HEADS * 16);
         }
+#pragma unroll
+        for (int r = 0; r < N; ++r)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                acc[v].x = fmaf(f[r], x[r][v].x, acc[v].x); acc[v].y = fmaf(f[r], x[r][v].y, acc[v].y);
+                acc[v].z = fmaf(f[r], x[r][v].z, acc[v].z); acc[v].w = fmaf(f[r], x[r][v].w, acc[v].w);
+            }
         uint4* dst = reinterpret_cast<uint4*>(p.out + (static_cast<int64_t>(t) * LP_HEADS + h) * LP_DV + c * LP_DVH + blk * 16);
         uint32_t w[8];
 #pragma unroll
@@ -176,7 +181,7 @@ __device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s,
         dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
     }
     if (p.lse != nullptr && c == 0u && s == 0 && threadIdx.x < LP_HEADS)
-        p.lse[static_cast<int64_t>(t) * LP_HEADS + h] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : __int_as_float(0xff800000);
+        p.lse[static_cast<int64_t>(t) * LP_HEADS + h] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : neg_inf;
 }
 
 // SPLIT = false: clusters of two CTAs, persistent over tokens.  SPLIT = true: a cluster of 2 n CTAs takes one token, pair s of it
@@ -690,7 +695,20 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     }
     if constexpr (SPLIT) {
         cluster_sync_all();         // every pair's output lies in its shared memory
-        if (!start_abort && n_my > 0) lp_merge_splits(p, cid, static_cast<int>(rank >> 1), n_split, c, smem_u32(k_smem), smem_u32(xbuf));
+        if (!start_abort && n_my > 0) {
+            const uint32_t o_addr = smem_u32(k_smem), stats_addr = smem_u32(xbuf);
+            const int sp = static_cast<int>(rank >> 1);
+            static_assert(LP_MAX_SPLIT == 8, "cases below");
+            switch (n_split) {
+                case 2: lp_merge_splits<2>(p, cid, sp, c, o_addr, stats_addr); break;
+                case 3: lp_merge_splits<3>(p, cid, sp, c, o_addr, stats_addr); break;
+                case 4: lp_merge_splits<4>(p, cid, sp, c, o_addr, stats_addr); break;
+                case 5: lp_merge_splits<5>(p, cid, sp, c, o_addr, stats_addr); break;
+                case 6: lp_merge_splits<6>(p, cid, sp, c, o_addr, stats_addr); break;
+                case 7: lp_merge_splits<7>(p, cid, sp, c, o_addr, stats_addr); break;
+                case 8: lp_merge_splits<8>(p, cid, sp, c, o_addr, stats_addr); break;
+            }
+        }
     }
     cluster_sync_all();   // neither CTA leaves while the other may still write into its shared memory or arrive on its barriers
 }
@@ -785,16 +803,16 @@ int launch_sparse_attn_latent_tc(const void* q, int M, const void* pool, int64_t
     const int rc = lp_resident_clusters(dev, smem, n_resident);
     if (rc != JANUS_OK) return rc;
     // A pair takes 1.16 us per tile of 64 keys and 8.7 us around them.  While the tokens are few, clusters of 2 n CTAs share a
-    // token's tiles; the merge, whose 112 KB per CTA cross the SM-to-SM network, makes that 12 + 0.6 n us.  The n with the least
-    // waves x time is taken.  Measured at 2048 keys: 1 token 45.8 us with one pair, 31.4 / 26.1 / 24.2 / 21.5 with 2 / 3 / 4 / 8;
-    // 19 tokens 47.6, 32.9 and 28.4 with 1, 2 and 3 (22 clusters of six CTAs are resident at once), 49.0 with 4 (two waves);
-    // 512 keys: 18.0 with one pair, 17.5 and 16.7 with 2 and 3.
+    // token's tiles; start and merge, whose 112 KB per CTA cross the SM-to-SM network, make that 12 + 0.4 n us.  The n with the least
+    // waves x time is taken.  Measured at 2048 keys: 1 token 45.8 us with one pair, 20.0 with eight; 19 tokens 47.6 and 27.6 with one
+    // and three (22 clusters of six CTAs are resident at once; four take two waves, 49); 512 keys: 18.0 with one pair, 16.0 with
+    // eight.  (Remote loads one pair after the other instead of all at once: 21.6, 28.3 and 17.5.)
     const int all_tiles = (k + LP_TILE - 1) / LP_TILE;
     int split = 1;
     double best = 0.;
     for (int n = 1; n <= LP_MAX_SPLIT && n <= all_tiles; ++n) {
         if (n_resident[n] <= 0) break;
-        const double t = ((M + n_resident[n] - 1) / n_resident[n]) * (((all_tiles + n - 1) / n) * 1.16 + (n > 1 ? 12. + 0.6 * n : 8.7));
+        const double t = ((M + n_resident[n] - 1) / n_resident[n]) * (((all_tiles + n - 1) / n) * 1.16 + (n > 1 ? 12. + 0.4 * n : 8.7));
         if (n == 1 || t < best) { best = t; split = n; }
     }
     const int n_clusters = split > 1 ? M : (M < n_resident[1] ? M : n_resident[1]);     // one pair per cluster: persistent over tokens
