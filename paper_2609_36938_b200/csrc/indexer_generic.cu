@@ -21,6 +21,8 @@ indexer_generic_kernel(const void* __restrict__ q_idx, int64_t q_stride_tok, con
                        const float* __restrict__ w, const float* __restrict__ q_scale, int64_t q_scale_stride_tok,
                        const float* __restrict__ k_scale, const float* __restrict__ row_bias, const float* __restrict__ col_bias,
                        int M, int H, int D, int64_t n_keys, int64_t q_pos0, int causal, float* __restrict__ scores, int64_t ld) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ float smem[];
     float* ks = smem;                       // [D][IG_KEYS] transposed key tile
     float* qs = smem + D * IG_KEYS;         // [H][D] one query token
@@ -80,14 +82,15 @@ int launch_indexer_generic(const void* q_idx, int64_t q_stride_tok, const void* 
     if (grid.y > 65535) return JANUS_ERR_UNSUPPORTED;
     if (dtype == JANUS_DTYPE_BF16) {
         JANUS_CUDA_CHECK(cudaFuncSetAttribute(indexer_generic_kernel<JANUS_DTYPE_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        indexer_generic_kernel<JANUS_DTYPE_BF16><<<grid, IG_KEYS, smem, stream>>>(q_idx, q_stride_tok, k_idx, k_stride_tok, w, q_scale, q_scale_stride_tok,
-                                                                                k_scale, row_bias, col_bias, M, H, D, n_keys, q_pos0, causal, scores, ld);
+        JANUS_CUDA_CHECK(launch_kernel(indexer_generic_kernel<JANUS_DTYPE_BF16>, grid, IG_KEYS, smem, stream, 1, q_idx, q_stride_tok, k_idx,
+                                       k_stride_tok, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H, D, n_keys, q_pos0, causal,
+                                       scores, ld));
     } else {
         JANUS_CUDA_CHECK(cudaFuncSetAttribute(indexer_generic_kernel<JANUS_DTYPE_FP8_E4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        indexer_generic_kernel<JANUS_DTYPE_FP8_E4M3><<<grid, IG_KEYS, smem, stream>>>(q_idx, q_stride_tok, k_idx, k_stride_tok, w, q_scale, q_scale_stride_tok,
-                                                                                    k_scale, row_bias, col_bias, M, H, D, n_keys, q_pos0, causal, scores, ld);
+        JANUS_CUDA_CHECK(launch_kernel(indexer_generic_kernel<JANUS_DTYPE_FP8_E4M3>, grid, IG_KEYS, smem, stream, 1, q_idx, q_stride_tok, k_idx,
+                                       k_stride_tok, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H, D, n_keys, q_pos0, causal,
+                                       scores, ld));
     }
-    JANUS_CUDA_CHECK(cudaGetLastError());
     return JANUS_OK;
 }
 

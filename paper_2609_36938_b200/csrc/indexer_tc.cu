@@ -259,6 +259,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     const int tpc = RAGGED ? 1 : nq * TPS;                      // tokens per group (ragged: a session's one query row)
 
     if ((smem_u32(smem) & 1023u) != 0u) {   // swizzled tiles need 1024-byte alignment
+        grid_wait();
         if (threadIdx.x == 0) report(p.dev_status, JANUS_DEV_WAIT_TIMEOUT);
         return;
     }
@@ -266,13 +267,15 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&bars->tmem_full[s]), 1); mbar_init(smem_u32(&bars->tmem_empty[s]), RAGGED ? 4 : 8); }
         mbar_init(smem_u32(&bars->mma_drain), 1);
-        // an earlier CTA of this launch gave up on a wait: this one starts no work on a broken pipeline.  One thread reads the
-        // status word and the whole CTA follows that one reading (a second reading could differ and split the roles).
-        bars->aborted = (p.dev_status != nullptr && *reinterpret_cast<volatile int32_t*>(p.dev_status) == JANUS_DEV_WAIT_TIMEOUT) ? 1 : 0;
         fence_mbar_init();
         prefetch_tensormap(&tmap_q);
         prefetch_tensormap(&tmap_k);
+        grid_wait();
+        // an earlier CTA of this launch gave up on a wait: this one starts no work on a broken pipeline.  One thread reads the
+        // status word and the whole CTA follows that one reading (a second reading could differ and split the roles).
+        bars->aborted = (p.dev_status != nullptr && *reinterpret_cast<volatile int32_t*>(p.dev_status) == JANUS_DEV_WAIT_TIMEOUT) ? 1 : 0;
     }
+    grid_wait();
     // per-column weights (w * q_scale) and per-token bias factors and thresholds of group g, by threads first, first + step, ..
     auto load_weights = [&](int g, int first, int step) {
         const int t0 = g * tpc;
@@ -659,10 +662,10 @@ static int launch_tc(const CUtensorMap& tq, const CUtensorMap& tk, const TcParam
         [] { return cudaFuncSetAttribute(indexer_tc_kernel<H, FP8, CAND, RAGGED, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET); }));
     constexpr int threads = RAGGED ? TC_THREADS_RAGGED : TC_THREADS;
     if constexpr (MULTI && !RAGGED)
-        indexer_tc_kernel<H, FP8, CAND, RAGGED, MULTI><<<grid, threads, smem, stream>>>(tq, tk, p, cp, sched);
+        JANUS_CUDA_CHECK(launch_kernel(indexer_tc_kernel<H, FP8, CAND, RAGGED, MULTI>, grid, threads, smem, stream, 1, tq, tk, p, cp, sched));
     else
-        indexer_tc_kernel<H, FP8, CAND, RAGGED, MULTI><<<grid, threads, smem, stream>>>(tq, tk, p, cp, TcNoSchedule{});
-    JANUS_CUDA_CHECK(cudaGetLastError());
+        JANUS_CUDA_CHECK(launch_kernel(indexer_tc_kernel<H, FP8, CAND, RAGGED, MULTI>, grid, threads, smem, stream, 1, tq, tk, p, cp,
+                                       TcNoSchedule{}));
     return JANUS_OK;
 }
 

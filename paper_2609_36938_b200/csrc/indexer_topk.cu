@@ -93,6 +93,8 @@ __device__ __forceinline__ int64_t sample_position(int j, int64_t p0) {
 __global__ void ft_gather_sample_kernel(const unsigned char* __restrict__ k_idx, int64_t k_row_bytes, int row_vecs, const float* __restrict__ k_scale,
                                         const float* __restrict__ col_bias, int64_t p0, uint4* __restrict__ k_sample, float* __restrict__ ks_sample,
                                         float* __restrict__ cb_sample) {
+    grid_launch_next();
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;      // one 16-byte vector of one sampled key row
     if (i >= FT_NS * row_vecs) return;
     const int j = i / row_vecs, v = i - j * row_vecs;
@@ -108,6 +110,8 @@ __global__ void ft_gather_sample_kernel(const unsigned char* __restrict__ k_idx,
 __global__ void __launch_bounds__(TK_THREADS)
 ft_threshold_kernel(const float* __restrict__ sc_sample, int M, int64_t n_keys, int64_t q_pos0, int causal, int k, int cap, float* __restrict__ thr,
                     int32_t* __restrict__ cand_cnt, int32_t* __restrict__ fb_count) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SampleShared& sh = *reinterpret_cast<SampleShared*>(smem_raw);
     const int t = blockIdx.x, tid = threadIdx.x;
@@ -144,6 +148,8 @@ __global__ void __launch_bounds__(TK_THREADS)
 ft_select_kernel(const int2* __restrict__ cand, const int32_t* __restrict__ cand_cnt, int M, int64_t n_keys, int64_t q_pos0, int causal, int k,
                  int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth, int32_t* __restrict__ fb_count,
                  int32_t* __restrict__ fb_rows) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using Shared = TopkSharedT<CAP>;
     Shared& sh = *reinterpret_cast<Shared*>(smem_raw);
@@ -206,6 +212,8 @@ ft_fallback_kernel(const unsigned char* __restrict__ q_idx, const unsigned char*
                    const float* __restrict__ row_bias, const float* __restrict__ col_bias, int M, int H, int D, int64_t n_keys, int64_t q_pos0,
                    int causal, int k, int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth,
                    const int32_t* __restrict__ fb_count, const int32_t* __restrict__ fb_rows, float* __restrict__ fb_buf, int64_t ld) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FallbackShared& sh = *reinterpret_cast<FallbackShared*>(smem_raw);
     float* qs = reinterpret_cast<float*>(smem_raw + sizeof(FallbackShared));   // [H][D] query of the row, pre-multiplied by q_scale
@@ -317,10 +325,9 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
     float* fb_buf = reinterpret_cast<float*>(base + L.fb_buf);
 
     // 1. sample
-    ft_gather_sample_kernel<<<(FT_NS * row_vecs + 255) / 256, 256, 0, stream>>>(static_cast<const unsigned char*>(k_idx), k_stride_tok * esz, row_vecs,
-                                                                                k_scale, col_bias, L.p0,
-                                                                                reinterpret_cast<uint4*>(base + L.k_sample), ks_sample, cb_sample);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    JANUS_CUDA_CHECK(launch_kernel(ft_gather_sample_kernel, dim3((FT_NS * row_vecs + 255) / 256), 256, 0, stream, 1,
+                                   static_cast<const unsigned char*>(k_idx), k_stride_tok * esz, row_vecs, k_scale, col_bias, L.p0,
+                                   reinterpret_cast<uint4*>(base + L.k_sample), ks_sample, cb_sample));
     int rc = launch_indexer_tc(q_idx, base + L.k_sample, D_I, w, q_scale, q_scale_stride_tok, ks_sample, cb_sample ? row_bias : nullptr, cb_sample, M,
                                H_I, D_I, FT_NS, q_pos0, 0, dtype, sc_sample, FT_NS, dev_status, stream, nullptr, nullptr, nullptr, 0);
     if (rc != JANUS_OK) return rc;
@@ -328,8 +335,8 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
     static once_per_device threshold_attributes, select_attributes, fallback_attributes;
     JANUS_CUDA_CHECK(threshold_attributes.run(
         [] { return cudaFuncSetAttribute(ft_threshold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(SampleShared))); }));
-    ft_threshold_kernel<<<M, TK_THREADS, sizeof(SampleShared), stream>>>(sc_sample, M, n_keys, q_pos0, causal, k, L.cap, thr, cand_cnt, fb_count);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    JANUS_CUDA_CHECK(launch_kernel(ft_threshold_kernel, dim3(M), TK_THREADS, sizeof(SampleShared), stream, 1, sc_sample, M, n_keys, q_pos0, causal, k,
+                                   L.cap, thr, cand_cnt, fb_count));
     // 3. the indexer over all keys, appending candidates
     rc = launch_indexer_tc(q_idx, k_idx, k_stride_tok, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H_I, D_I, n_keys, q_pos0, causal,
                            dtype, nullptr, 0, dev_status, stream, thr, cand_cnt, cand, L.cap);
@@ -342,13 +349,13 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
     }));
     if (L.cap == FT_CAP) {
         using Sh = TopkSharedT<FT_CAP>;
-        ft_select_kernel<FT_CAP><<<M, TK_THREADS, sizeof(Sh), stream>>>(cand, cand_cnt, M, n_keys, q_pos0, causal, k, idx, count, kth, fb_count, fb_rows);
+        JANUS_CUDA_CHECK(launch_kernel(ft_select_kernel<FT_CAP>, dim3(M), TK_THREADS, sizeof(Sh), stream, 1, cand, cand_cnt, M, n_keys, q_pos0, causal,
+                                       k, idx, count, kth, fb_count, fb_rows));
     } else {
         using Sh = TopkSharedT<FT_CAP / 2>;
-        ft_select_kernel<FT_CAP / 2><<<M, TK_THREADS, sizeof(Sh), stream>>>(cand, cand_cnt, M, n_keys, q_pos0, causal, k, idx, count, kth, fb_count,
-                                                                           fb_rows);
+        JANUS_CUDA_CHECK(launch_kernel(ft_select_kernel<FT_CAP / 2>, dim3(M), TK_THREADS, sizeof(Sh), stream, 1, cand, cand_cnt, M, n_keys, q_pos0,
+                                       causal, k, idx, count, kth, fb_count, fb_rows));
     }
-    JANUS_CUDA_CHECK(cudaGetLastError());
     // 5. rows the sample misjudged (normally none: the kernel then returns at once)
     const size_t fb_smem = sizeof(FallbackShared) + sizeof(float) * (static_cast<size_t>(H_I) * D_I + H_I);
     const unsigned char* qb = static_cast<const unsigned char*>(q_idx);
@@ -359,15 +366,14 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
         return e != cudaSuccess ? e : cudaFuncSetAttribute(ft_fallback_kernel<JANUS_DTYPE_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, fb_smem_max);
     }));
     if (fp8) {
-        ft_fallback_kernel<JANUS_DTYPE_FP8_E4M3><<<FT_FB_CTAS, TK_THREADS, fb_smem, stream>>>(
-            qb, kb, k_stride_tok * esz, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H_I, D_I, n_keys, q_pos0, causal, k, idx, count,
-            kth, fb_count, fb_rows, fb_buf, L.ld);
+        JANUS_CUDA_CHECK(launch_kernel(ft_fallback_kernel<JANUS_DTYPE_FP8_E4M3>, dim3(FT_FB_CTAS), TK_THREADS, fb_smem, stream, 1, qb, kb,
+                                       k_stride_tok * esz, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H_I, D_I, n_keys, q_pos0,
+                                       causal, k, idx, count, kth, fb_count, fb_rows, fb_buf, L.ld));
     } else {
-        ft_fallback_kernel<JANUS_DTYPE_BF16><<<FT_FB_CTAS, TK_THREADS, fb_smem, stream>>>(
-            qb, kb, k_stride_tok * esz, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H_I, D_I, n_keys, q_pos0, causal, k, idx, count,
-            kth, fb_count, fb_rows, fb_buf, L.ld);
+        JANUS_CUDA_CHECK(launch_kernel(ft_fallback_kernel<JANUS_DTYPE_BF16>, dim3(FT_FB_CTAS), TK_THREADS, fb_smem, stream, 1, qb, kb,
+                                       k_stride_tok * esz, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H_I, D_I, n_keys, q_pos0,
+                                       causal, k, idx, count, kth, fb_count, fb_rows, fb_buf, L.ld));
     }
-    JANUS_CUDA_CHECK(cudaGetLastError());
     return JANUS_OK;
 }
 

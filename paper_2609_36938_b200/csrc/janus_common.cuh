@@ -46,6 +46,36 @@ class once_per_device {
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// ---- launches that overlap the end of the kernel before them -----------------------------------------------------------------
+// Every kernel here is launched as a programmatic dependent of its predecessor in the stream: its CTAs may become resident, and
+// run up to grid_wait(), while the predecessor still runs.  The order of memory accesses stays that of the stream, because every
+// kernel waits, on every path, before its first access to global memory; grid_wait() returns when the predecessor has completed
+// and its writes are visible, and the predecessor has itself waited for what came before.  Tensor memory is allocated after
+// grid_wait(), so that no CTA holds it while it waits.  A short kernel lets its successor in at once with grid_launch_next(); the
+// indexer and the attention of many tokens do not, because CTAs that wait beside them made them 1 % slower.  One-session decode step
+// 51.2 -> 44.2 us, short message 59.9 -> 52.8, sharded prediction 1.70 -> 1.66 ms; the large passes are unchanged.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class Kernel, class... Args>
+inline cudaError_t launch_kernel(Kernel kernel, dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster, const Args&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // ---- device-side status word: first error wins ------------------------------------------------
 __device__ __forceinline__ void report(int32_t* dev_status, int code) {
     if (dev_status != nullptr) atomicCAS(dev_status, 0, code);

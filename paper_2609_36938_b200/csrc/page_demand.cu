@@ -63,7 +63,9 @@ __global__ void __launch_bounds__(MARK_THREADS)
 page_mark_kernel(const PdParams p, int n_log_words) {
     extern __shared__ uint32_t lbm[];
     uint32_t* pbm = lbm + n_log_words;
+    grid_launch_next();
     for (int i = threadIdx.x; i < n_log_words + p.n_words; i += MARK_THREADS) lbm[i] = 0u;
+    grid_wait();
     __syncthreads();
     const PageDiv page{p.page_size, p.page_shift};
     bool bad = false;
@@ -127,6 +129,8 @@ __device__ __forceinline__ int32_t page_of_token(int s, int64_t limit, const Pag
 template <int MODE>
 __global__ void __launch_bounds__(256)
 page_mark_global_kernel(const PdParams p) {
+    grid_launch_next();
+    grid_wait();
     const PageDiv page{p.page_size, p.page_shift};
     bool bad = false;
     for (int64_t e = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; e < p.n_idx; e += static_cast<int64_t>(gridDim.x) * 256) {
@@ -199,8 +203,10 @@ page_demand_kernel(const PdParams p) {
     const int wps = (p.n_words + n_cta - 1) / n_cta;        // words of a slice; at most one chunk of PD_THREADS in the marking modes
     const int w0 = min(p.n_words, rank * wps), w1 = min(p.n_words, w0 + wps);
 
+    grid_launch_next();
     if constexpr (MODE != PD_LISTS) {
         for (int i = tid; i < p.n_words; i += PD_THREADS) bm[i] = 0u;
+        grid_wait();
         __syncthreads();
         const PageDiv page{p.page_size, p.page_shift};
         bool bad = false;
@@ -232,6 +238,7 @@ page_demand_kernel(const PdParams p) {
         cluster_sync_all();               // every private bitmap is complete
     }
 
+    if constexpr (MODE == PD_LISTS) grid_wait();
     // ---- lists of this CTA's slice, a chunk of words at a time
     const bool want_miss = p.miss_pages != nullptr;
     // word i of the set: ORed over the CTAs' bitmaps, or as page_mark_kernel left it
@@ -355,6 +362,8 @@ page_demand_kernel(const PdParams p) {
 }
 
 __global__ void page_union_kernel(uint32_t* __restrict__ dst, const uint32_t* __restrict__ src, int n_words) {
+    grid_launch_next();
+    grid_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_words; i += gridDim.x * blockDim.x) dst[i] |= src[i];
 }
 
@@ -368,19 +377,7 @@ static int launch_page_demand(const PdParams& p, int cluster, cudaStream_t strea
             e = cudaFuncSetAttribute(page_demand_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PD_SMEM_WORDS * static_cast<int>(sizeof(uint32_t)));
         return e;
     }));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cluster);
-    cfg.blockDim = dim3(PD_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = cluster;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, page_demand_kernel<MODE>, p));
+    JANUS_CUDA_CHECK(launch_kernel(page_demand_kernel<MODE>, dim3(cluster), PD_THREADS, smem, stream, cluster, p));
     return JANUS_OK;
 }
 
@@ -407,12 +404,13 @@ static int run_page_demand(const PdParams& p, cudaStream_t stream) {
         }));
         const int64_t want = ((p.n_idx >> 2) + MARK_THREADS - 1) / MARK_THREADS;
         const unsigned grid = static_cast<unsigned>(want < 1 ? 1 : want < 148 * 2 ? want : 148 * 2);
-        page_mark_kernel<<<grid, MARK_THREADS, sizeof(uint32_t) * (n_log_words + p.n_words), stream>>>(p, static_cast<int>(n_log_words));
+        JANUS_CUDA_CHECK(launch_kernel(page_mark_kernel, dim3(grid), MARK_THREADS, sizeof(uint32_t) * (n_log_words + p.n_words), stream, 1, p,
+                                       static_cast<int>(n_log_words)));
     } else if (p.n_idx > 0) {
         const int64_t want = (p.n_idx + 1023) / 1024;
-        page_mark_global_kernel<MODE><<<static_cast<unsigned>(want < 148 * 8 ? want : 148 * 8), 256, 0, stream>>>(p);
+        JANUS_CUDA_CHECK(launch_kernel(page_mark_global_kernel<MODE>, dim3(static_cast<unsigned>(want < 148 * 8 ? want : 148 * 8)), 256, 0, stream, 1,
+                                       p));
     }
-    JANUS_CUDA_CHECK(cudaGetLastError());
     return launch_page_demand<PD_LISTS>(p, p.n_words <= 8 * PD_THREADS ? 8 : 16, stream);     // 131136 pages: 27.5 us with 16, 32.7 with 8; 2112 pages: 14.4 with 8, 16.5 with 16
 }
 
@@ -431,8 +429,7 @@ extern "C" int janus_page_union(uint32_t* dst, const uint32_t* src, int64_t n_ph
     if (n_phys_pages > (int64_t(1) << 31) - 64) return JANUS_ERR_UNSUPPORTED;
     const int n_words = static_cast<int>((n_phys_pages + 31) / 32);
     const int blocks = n_words < 256 * 148 ? (n_words + 255) / 256 : 148;
-    page_union_kernel<<<blocks, 256, 0, static_cast<cudaStream_t>(stream_)>>>(dst, src, n_words);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    JANUS_CUDA_CHECK(launch_kernel(page_union_kernel, dim3(blocks), 256, 0, static_cast<cudaStream_t>(stream_), 1, dst, src, n_words));
     return JANUS_OK;
 }
 

@@ -18,6 +18,8 @@ sparse_attn_generic_kernel(const uint16_t* __restrict__ q, int M, int H_q, int d
                            int n_kv_heads, int d_v, const int32_t* __restrict__ idx, int k, int page_size,
                            const int32_t* __restrict__ page_table, int64_t n_logical_pages, const int64_t* __restrict__ table_offsets,
                            float softmax_scale, uint16_t* __restrict__ out, float* __restrict__ lse, int32_t* dev_status) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int kpad = d_qk + 8, vpad = d_v + 8;             // row pitch in bf16: odd multiple of 16 bytes -> conflict-free 16 B reads
     const bool v_alias = (v_pool == k_pool);
@@ -173,11 +175,10 @@ static int launch_g(const void* q, int M, int H_q, int d_qk, const void* k_pool,
     JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_generic_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
     const int heads_per_kv = H_q / n_kv_heads;
     dim3 grid(M, n_kv_heads * ((heads_per_kv + G - 1) / G));
-    sparse_attn_generic_kernel<G><<<grid, AG_THREADS, smem, stream>>>(
-        static_cast<const uint16_t*>(q), M, H_q, d_qk, static_cast<const uint16_t*>(k_pool), static_cast<const uint16_t*>(v_pool),
-        page_stride, tok_stride, head_stride, n_kv_heads, d_v, idx, k, page_size, page_table, n_logical_pages, table_offsets,
-        softmax_scale, static_cast<uint16_t*>(out), lse, dev_status);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    JANUS_CUDA_CHECK(launch_kernel(sparse_attn_generic_kernel<G>, grid, AG_THREADS, smem, stream, 1, static_cast<const uint16_t*>(q), M, H_q, d_qk,
+                                   static_cast<const uint16_t*>(k_pool), static_cast<const uint16_t*>(v_pool), page_stride, tok_stride, head_stride,
+                                   n_kv_heads, d_v, idx, k, page_size, page_table, n_logical_pages, table_offsets, softmax_scale,
+                                   static_cast<uint16_t*>(out), lse, dev_status));
     return JANUS_OK;
 }
 

@@ -91,6 +91,8 @@ constexpr int ah_ctas_per_sm(int warps) { return 12 / warps; }
 template <int DQK, int DV, bool WIDE, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, ah_ctas_per_sm(WARPS))
 sparse_attn_heads_kernel(const AhParams p) {
+    grid_launch_next();
+    grid_wait();
     __shared__ AhShared<DV, WARPS> sh;
     constexpr int KE = WIDE ? 16 : 8;     // elements of a key row per load: four lanes read 128 or 64 contiguous bytes of it
     constexpr int KB = DQK / (4 * KE);
@@ -341,24 +343,14 @@ static int launch_heads(const AhParams& p, int M, int n_kv_heads, cudaStream_t s
     } else {
         warps = steps >= 16 ? 4 : 2;
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(M) * split, groups);
-    cfg.blockDim = dim3(32 * warps);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = split;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = split > 1 ? 1 : 0;
+    const dim3 grid(static_cast<unsigned>(M) * split, groups);
     // 32-byte loads where every row starts on 32 bytes
     const bool wide = ((reinterpret_cast<uintptr_t>(p.k_pool) | reinterpret_cast<uintptr_t>(p.v_pool)) & 31u) == 0 &&
                       ((p.page_stride | p.tok_stride | p.head_stride) & 15) == 0;
 #define JANUS_AH_CASE(WIDE)                                                                                       \
-    if (warps == 2) JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sparse_attn_heads_kernel<DQK, DV, WIDE, 2>, p));    \
-    else if (warps == 4) JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sparse_attn_heads_kernel<DQK, DV, WIDE, 4>, p)); \
-    else JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sparse_attn_heads_kernel<DQK, DV, WIDE, 8>, p));
+    if (warps == 2) JANUS_CUDA_CHECK(launch_kernel(sparse_attn_heads_kernel<DQK, DV, WIDE, 2>, grid, 32 * warps, 0, stream, split, p));    \
+    else if (warps == 4) JANUS_CUDA_CHECK(launch_kernel(sparse_attn_heads_kernel<DQK, DV, WIDE, 4>, grid, 32 * warps, 0, stream, split, p)); \
+    else JANUS_CUDA_CHECK(launch_kernel(sparse_attn_heads_kernel<DQK, DV, WIDE, 8>, grid, 32 * warps, 0, stream, split, p));
     if (wide) {
         JANUS_AH_CASE(true)
     } else {

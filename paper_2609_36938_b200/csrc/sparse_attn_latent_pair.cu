@@ -224,6 +224,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
         mbar_init(smem_u32(&sh->p_full), 4);
         fence_mbar_init();
         prefetch_tensormap(&tmap_q);
+        grid_wait();
         // start-up agreement: if this CTA should not start (misaligned shared memory, or an earlier CTA of the launch gave
         // up on a wait), both CTAs of the cluster must skip the work, so the flag is written to both of them
         uint32_t flag = ((smem_u32(smem) & 1023u) != 0u) ? 1u : 0u;
@@ -231,6 +232,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
         sh->start_abort[c] = flag;
         st_cluster_u32(mapa_shared(smem_u32(&sh->start_abort[c]), peer), flag);
     }
+    grid_wait();
     if (warp == 0) {
         tmem_alloc(smem_u32(&sh->tmem_base), 512);
         tmem_relinquish();
@@ -238,6 +240,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();                            // barriers of both CTAs are initialised, start flags exchanged
+    if constexpr (SPLIT) grid_launch_next();       // (tensor memory is allocated)
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
     const bool start_abort = (sh->start_abort[0] | sh->start_abort[1]) != 0u;
@@ -733,7 +736,7 @@ bool sparse_attn_latent_tc_supported(int M, int H_q, int d_qk, const void* k_poo
     return true;
 }
 
-static cudaLaunchConfig_t lp_launch_config(int cluster_size, int n_clusters, size_t smem, cudaLaunchAttribute* attr) {
+static cudaLaunchConfig_t lp_occupancy_config(int cluster_size, int n_clusters, size_t smem, cudaLaunchAttribute* attr) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(cluster_size) * n_clusters);
     cfg.blockDim = dim3(LP_THREADS);
@@ -762,7 +765,7 @@ static int lp_resident_clusters(int dev, size_t smem, int (&n)[LP_MAX_SPLIT + 1]
         JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         for (int s = LP_MAX_SPLIT; s >= 1; --s) {
             cudaLaunchAttribute attr;
-            const cudaLaunchConfig_t cfg = lp_launch_config(2 * s, 148, smem, &attr);
+            const cudaLaunchConfig_t cfg = lp_occupancy_config(2 * s, 148, smem, &attr);
             const cudaError_t e = s > 1 ? cudaOccupancyMaxActiveClusters(&k[s], sparse_attn_latent_pair_kernel<true>, &cfg)
                                         : cudaOccupancyMaxActiveClusters(&k[s], sparse_attn_latent_pair_kernel<false>, &cfg);
             if (e != cudaSuccess) {
@@ -828,11 +831,9 @@ int launch_sparse_attn_latent_tc(const void* q, int M, const void* pool, int64_t
         if (n == 1 || t < best) { best = t; split = n; }
     }
     const int n_clusters = split > 1 ? M : (M < n_resident[1] ? M : n_resident[1]);     // one pair per cluster: persistent over tokens
-    cudaLaunchAttribute attr;
-    cudaLaunchConfig_t cfg = lp_launch_config(2 * split, n_clusters, smem, &attr);
-    cfg.stream = stream;
-    if (split > 1) JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sparse_attn_latent_pair_kernel<true>, tq, p));
-    else JANUS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sparse_attn_latent_pair_kernel<false>, tq, p));
+    const dim3 grid(static_cast<unsigned>(2 * split) * n_clusters);
+    if (split > 1) JANUS_CUDA_CHECK(launch_kernel(sparse_attn_latent_pair_kernel<true>, grid, LP_THREADS, smem, stream, 2 * split, tq, p));
+    else JANUS_CUDA_CHECK(launch_kernel(sparse_attn_latent_pair_kernel<false>, grid, LP_THREADS, smem, stream, 2, tq, p));
     return JANUS_OK;
 }
 

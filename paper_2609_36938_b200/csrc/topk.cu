@@ -24,6 +24,8 @@ template <int CAP>
 __global__ void __launch_bounds__(TK_THREADS)
 topk_rows_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int k,
                  int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using TopkShared = TopkSharedT<CAP>;
     TopkShared& sh = *reinterpret_cast<TopkShared*>(smem_raw);
@@ -42,6 +44,8 @@ topk_rows_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_
 __global__ void __launch_bounds__(TK_THREADS)
 topk_rows_cluster_kernel(const float* __restrict__ scores, int64_t ld, int64_t n_keys, int64_t q_pos0, int causal, int k,
                          int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TopkSharedT<TK_CAP>& sh = *reinterpret_cast<TopkSharedT<TK_CAP>*>(smem_raw);
     const int t = blockIdx.x / ptx::cluster_nctarank();
@@ -56,6 +60,8 @@ template <int CAP>
 __global__ void __launch_bounds__(TK_THREADS)
 topk_entries_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_entries, int64_t q_pos0, int entry_size, int k,
                     int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using TopkShared = TopkSharedT<CAP>;
     TopkShared& sh = *reinterpret_cast<TopkShared*>(smem_raw);
@@ -69,6 +75,8 @@ topk_entries_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t
 // Token selection of an entry selection: slot e * E + j of row t = entry * E + j if that token is at or before q_pos0 + t.
 __global__ void entry_expand_kernel(const int32_t* __restrict__ idx_e, int M, int k_e, int entry_size, int64_t q_pos0,
                                     int32_t* __restrict__ idx_tok) {
+    grid_launch_next();
+    grid_wait();
     const int64_t n = static_cast<int64_t>(M) * k_e * entry_size;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int64_t slot = i / entry_size;            // (t, e)
@@ -85,6 +93,8 @@ __global__ void entry_expand_kernel(const int32_t* __restrict__ idx_e, int M, in
 __global__ void __launch_bounds__(256)
 entry_pool_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int entry_size,
                   int64_t n_entries, float* __restrict__ out, int64_t out_ld) {
+    grid_launch_next();
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t warp_id = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t n_warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -109,6 +119,8 @@ template <bool CLUSTER>
 __global__ void __launch_bounds__(TK_THREADS)
 topk_ragged_kernel(const float* __restrict__ scores, const int64_t* __restrict__ row_offsets, const int64_t* __restrict__ row_lengths, int k,
                    int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth, int32_t* dev_status) {
+    grid_launch_next();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TopkSharedT<TK_CAP>& sh = *reinterpret_cast<TopkSharedT<TK_CAP>*>(smem_raw);
     const int b = CLUSTER ? blockIdx.x / ptx::cluster_nctarank() : blockIdx.x;
@@ -142,23 +154,6 @@ static int topk_cluster_size(int64_t rows, double n) {
     if (rows <= 24 && n >= 96e3) return 4;
     if (rows <= 74 && (unknown || n >= 64e3)) return 2;
     return 1;
-}
-
-template <class Kernel, class... Args>
-static cudaError_t launch_topk_cluster(Kernel kernel, int64_t rows, int cluster, cudaStream_t stream, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(rows * cluster));
-    cfg.blockDim = dim3(TK_THREADS);
-    cfg.dynamicSmemBytes = sizeof(TopkSharedT<TK_CAP>);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = cluster;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Kernel attributes and the number of resident CTAs, asked for on a device's first call.
@@ -207,8 +202,8 @@ extern "C" int janus_topk_entries(const float* scores, int64_t scores_ld, int M,
     const size_t smem = sizeof(TopkSharedT<TK_CAP>);
     TopkDevice d;
     JANUS_CUDA_CHECK(topk_device(d));
-    topk_entries_kernel<TK_CAP><<<M, TK_THREADS, smem, stream>>>(scores, scores_ld, M, n_entries, q_pos0, entry_size, k, idx, count, kth);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    JANUS_CUDA_CHECK(launch_kernel(topk_entries_kernel<TK_CAP>, dim3(M), TK_THREADS, smem, stream, 1, scores, scores_ld, M, n_entries, q_pos0,
+                                   entry_size, k, idx, count, kth));
     return JANUS_OK;
 }
 
@@ -223,9 +218,8 @@ extern "C" int janus_entry_pool_scores(const float* scores, int64_t scores_ld, i
     const int64_t items = static_cast<int64_t>(M) * n_entries;
     int64_t blocks = (items + 7) / 8;                        // eight warps per block, one strip each
     if (blocks > 148 * 16) blocks = 148 * 16;
-    entry_pool_kernel<<<static_cast<unsigned>(blocks), 256, 0, static_cast<cudaStream_t>(stream_)>>>(scores, scores_ld, M, n_keys, q_pos0, causal,
-                                                                                                    entry_size, n_entries, entry_scores, entry_ld);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    JANUS_CUDA_CHECK(launch_kernel(entry_pool_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, static_cast<cudaStream_t>(stream_), 1, scores,
+                                   scores_ld, M, n_keys, q_pos0, causal, entry_size, n_entries, entry_scores, entry_ld));
     return JANUS_OK;
 }
 
@@ -239,9 +233,8 @@ extern "C" int janus_entry_expand(const int32_t* idx_entries, int M, int k_e, in
     if (static_cast<int64_t>(k_e) * entry_size > 2147483647) return JANUS_ERR_UNSUPPORTED;
     int64_t blocks = (n + 255) / 256;
     if (blocks > 148 * 16) blocks = 148 * 16;
-    entry_expand_kernel<<<static_cast<unsigned>(blocks), 256, 0, static_cast<cudaStream_t>(stream_)>>>(idx_entries, M, k_e, entry_size, q_pos0,
-                                                                                                       idx_tokens);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+    JANUS_CUDA_CHECK(launch_kernel(entry_expand_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, static_cast<cudaStream_t>(stream_), 1,
+                                   idx_entries, M, k_e, entry_size, q_pos0, idx_tokens));
     return JANUS_OK;
 }
 
@@ -257,10 +250,11 @@ extern "C" int janus_topk_batch(const float* scores, const int64_t* row_offsets,
     JANUS_CUDA_CHECK(topk_device(d));
     const int cluster = topk_cluster_size(B, -1.);
     if (cluster > 1) {
-        JANUS_CUDA_CHECK(launch_topk_cluster(topk_ragged_kernel<true>, B, cluster, stream, scores, row_offsets, row_lengths, k, idx, count, kth, dev_status));
+        JANUS_CUDA_CHECK(launch_kernel(topk_ragged_kernel<true>, dim3(B * cluster), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream, cluster, scores,
+                                       row_offsets, row_lengths, k, idx, count, kth, dev_status));
     } else {
-        topk_ragged_kernel<false><<<B, TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream>>>(scores, row_offsets, row_lengths, k, idx, count, kth, dev_status);
-        JANUS_CUDA_CHECK(cudaGetLastError());
+        JANUS_CUDA_CHECK(launch_kernel(topk_ragged_kernel<false>, dim3(B), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream, 1, scores, row_offsets,
+                                       row_lengths, k, idx, count, kth, dev_status));
     }
     return JANUS_OK;
 }
@@ -290,15 +284,16 @@ extern "C" int janus_topk(const float* scores, int64_t scores_ld, int M, int64_t
     JANUS_CUDA_CHECK(topk_device(d));
     const int cluster = topk_cluster_size(M, n_max);
     if (cluster > 1) {
-        JANUS_CUDA_CHECK(launch_topk_cluster(topk_rows_cluster_kernel, M, cluster, stream, scores, scores_ld, n_keys, q_pos0, causal, k, idx, count, kth));
+        JANUS_CUDA_CHECK(launch_kernel(topk_rows_cluster_kernel, dim3(M * cluster), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream, cluster, scores,
+                                       scores_ld, n_keys, q_pos0, causal, k, idx, count, kth));
         return JANUS_OK;
     }
     if (small)
-        topk_rows_kernel<TK_CAP_SMALL><<<std::min(M, d.resident_small), TK_THREADS, sizeof(TopkSharedT<TK_CAP_SMALL>), stream>>>(
-            scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count, kth);
+        JANUS_CUDA_CHECK(launch_kernel(topk_rows_kernel<TK_CAP_SMALL>, dim3(std::min(M, d.resident_small)), TK_THREADS,
+                                       sizeof(TopkSharedT<TK_CAP_SMALL>), stream, 1, scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count,
+                                       kth));
     else
-        topk_rows_kernel<TK_CAP><<<std::min(M, d.resident), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream>>>(
-            scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count, kth);
-    JANUS_CUDA_CHECK(cudaGetLastError());
+        JANUS_CUDA_CHECK(launch_kernel(topk_rows_kernel<TK_CAP>, dim3(std::min(M, d.resident)), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream, 1,
+                                       scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count, kth));
     return JANUS_OK;
 }
