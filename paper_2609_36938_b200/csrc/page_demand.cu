@@ -2,7 +2,7 @@
 // maximal runs of adjacent physical pages, and the miss set "exact minus predicted"
 // (union of selections: Sec. 2.2; corrective reads: Sec. 4.2; read packing: Sec. 4.3).
 //
-// Latency bounds all of it: a few hundred kilobytes in, a few kilobytes out, but several dependent steps.  Up to a million
+// Latency bounds all of it: a few hundred kilobytes in, a few kilobytes out, but several dependent steps.  Up to 128 K
 // indices one launch of one cluster does everything (page_demand_kernel): every CTA marks its share of the indices in a private
 // bitmap in shared memory, the cluster ORs the bitmaps slice by slice through distributed shared memory, and each CTA
 // turns its slice of the set into its part of the lists, offsets coming from one exchange of the CTAs' counts.  Larger blocks of
