@@ -12,8 +12,8 @@ PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libjanus.so")
 NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")
-SOURCES = ["janus_api.cu", "indexer_generic.cu", "indexer_tc.cu", "topk.cu", "page_demand.cu", "sparse_attn_generic.cu", "sparse_attn_heads.cu",
-           "sparse_attn_latent_pair.cu", "indexer_topk.cu", "diagnostics.cu"]
+SOURCES = ["janus_api.cu", "indexer_generic.cu", "indexer_tc.cu", "indexer_tc_batch.cu", "topk.cu", "page_demand.cu", "sparse_attn_generic.cu",
+           "sparse_attn_heads.cu", "sparse_attn_latent_pair.cu", "indexer_topk.cu", "diagnostics.cu"]
 
 
 def _nvcc() -> str:

@@ -13,7 +13,7 @@
 // overlaps the MMA of the next.  Warp roles: warp 0 issues TMA, warp 1 issues MMA (one thread each) and owns
 // the TMEM allocation, the other warps are two epilogue groups (one per TMEM half) of eight warps (two per TMEM lane
 // quadrant, each reducing half of the slot's columns): with four epilogue warps per scheduler one warp's wait for its
-// tensor-memory load or its weights is covered by the others.  The ragged decode mode has one group of four warps.
+// tensor-memory load or its weights is covered by the others.
 //
 // The launch is persistent: the visible (token group, key tile) pairs, group by group, are cut into as many equal contiguous
 // ranges as CTAs are resident, and a CTA walks its range in segments of one group each.  The key ring, the TMEM slots and
@@ -22,18 +22,12 @@
 // heads 121 -> 114, 1024 x 17408 FP8 183 -> 172; 4096 x 135168 FP8, which is on the power limit, 5.26 -> 5.17 ms.  Small launches give
 // every CTA tiles of one group only (MULTI = false).  256 rows x 4352 keys of 4 heads 18.6 -> 8.0 us, with half the sub-tiles per CTA.
 // Every wait is bounded; on a timeout the CTA reports JANUS_DEV_WAIT_TIMEOUT and winds down normally.
-#include "janus_common.cuh"
-#include "sm100_ptx.cuh"
+#include "indexer_tc.cuh"
 
 namespace janus {
 
-using namespace ptx;
-
-constexpr int TC_KEYS = 128;        // keys per tile = MMA M
 constexpr int TC_N = 256;           // (token, head) rows per MMA = MMA N
 constexpr int TC_THREADS = 576;     // 1 TMA warp + 1 MMA warp + 16 epilogue warps, two per TMEM lane quadrant and slot, each takes half the columns
-constexpr int TC_THREADS_RAGGED = 192;   // ragged mode: one epilogue group (4 warps), so that four CTAs fit an SM
-constexpr int TC_SMEM_BUDGET = 227 * 1024;
 constexpr int TC_MAX_STAGES = 6;
 
 struct TcParams {
@@ -49,7 +43,7 @@ struct TcParams {
     int64_t q_pos0;
     int M, H, causal;
     int n_tiles;          // ceil(n_keys / 128)
-    int n_groups;         // token groups (ragged: sessions)
+    int n_groups;         // token groups
     int tiles_per_cta;    // without MULTI: CTA (x, y) has the tiles x * tiles_per_cta .. of group y
     int nq;               // query sub-tiles per CTA
     int atoms;            // 128-byte swizzle atoms per row (row bytes / 128)
@@ -64,15 +58,10 @@ struct TcCandParams {
     int32_t* cand_cnt;    // [M] candidates appended so far (may exceed cand_cap: only the first cand_cap are stored)
     int2* cand;           // [M, cand_cap] (score bits, key index)
     int cand_cap;
-    // ragged batch mode (decode over many sessions): query row b scores the keys key_offsets[b] .. key_offsets[b+1] of one
-    // concatenated key array, no causal mask, and its scores go to scores[key_offsets[b] + s]
-    const int64_t* key_offsets;
-    // ragged batch mode only: keys are FP4 E2M1, two per byte; the TMA expands 16 of them into the first 8 bytes of every
-    // 16-byte shared-memory chunk, which is the layout the f8f6f4 MMA expects for 4-bit operands
+    // keys are FP4 E2M1, two per byte; the TMA expands 16 of them into the first 8 bytes of every 16-byte shared-memory chunk, which
+    // is the layout the f8f6f4 MMA expects for 4-bit operands
     int k_fp4;
 };
-
-constexpr int TC_MAX_CTAS = 148;      // SMs: CTAs of a persistent launch that are resident at once
 
 // Even shares (MULTI): where each CTA's range begins, (token group, key tile).  Made on the host and read from constant memory:
 // found by the device it was not known to be uniform, which made the issuing threads' loops up to 8 % slower.  Its 1.2 KB make
@@ -99,48 +88,7 @@ struct TcBarriers {
     uint64_t mma_drain;       // abort path only: every MMA issued so far has completed
     uint32_t tmem_base;
     int aborted;
-    int first_group, first_tile;        // where this CTA's range begins (even shares)
 };
-
-// Barrier of the epilogue warps alone.
-template <int THREADS>
-__device__ __forceinline__ void epilogue_barrier() {
-    asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
-}
-
-// One 32-column chunk of accumulators: 2 * ReLU, half weight, reduce over heads; a token's sum is complete every H columns.
-// Pairs of columns go through packed fp32 FMAs into up to four independent accumulator pairs, so the reduction is
-// neither one long dependent chain nor one instruction per element.
-template <int H, class Store>
-__device__ __forceinline__ void reduce_chunk(const uint32_t (&r)[32], const float* __restrict__ wchunk, int col0, float2 (&acc)[4], Store&& store) {
-    constexpr int NACC = (H / 2 < 4) ? H / 2 : 4;
-#pragma unroll
-    for (int i4 = 0; i4 < 8; ++i4) {
-        const float4 wv = *reinterpret_cast<const float4*>(wchunk + 4 * i4);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int i = 4 * i4 + 2 * j;                      // first column of the pair inside the chunk
-            const int col = col0 + i;
-            const float2 w2 = j == 0 ? make_float2(wv.x, wv.y) : make_float2(wv.z, wv.w);
-            // 2 * max(x, 0) = x + |x|, exactly: an add (full-rate FMA pipe, |x| is an operand modifier) instead of a max (the
-            // half-rate pipe, which 256 of them per thread and tile would saturate before the tensor pipe); the weights
-            // carry the factor 1/2
-            const float xa = __uint_as_float(r[i]), xb = __uint_as_float(r[i + 1]);
-            const float2 x2 = make_float2(xa + fabsf(xa), xb + fabsf(xb));
-            float2& a = acc[(col / 2) % NACC];
-            a = ffma2(w2, x2, a);
-            if (((col + 2) % H) == 0) {
-                float v = 0.f;
-#pragma unroll
-                for (int q = 0; q < NACC; ++q) {
-                    v += acc[q].x + acc[q].y;
-                    acc[q] = make_float2(0.f, 0.f);
-                }
-                store(col / H, v);
-            }
-        }
-    }
-}
 
 // Key tiles visible to some token of group g (tpc tokens per group) under the causal mask.
 __host__ __device__ __forceinline__ int tc_causal_tiles(int M, int64_t q_pos0, int n_tiles, int tpc, int g) {
@@ -168,41 +116,17 @@ __device__ __noinline__ void fill_masked_tails(float* scores, int64_t ld, int M,
     }
 }
 
-// Ragged mode: keys of session b, cut back to the part inside the key array (p.n_keys rows).
-struct TcSession {
-    int64_t base, count;
-    int tiles;
-    bool bad;
-};
-__device__ __forceinline__ TcSession tc_session(int64_t begin, int64_t end, int64_t n_keys, int max_tiles) {
-    TcSession s;
-    s.base = begin;
-    s.count = end - begin;
-    // the offsets come from device memory: neither the per-key scale / bias reads nor the score writes may leave their arrays
-    s.bad = s.base < 0 || s.count < 0 || s.base > n_keys || s.count > n_keys - s.base;
-    if (s.bad) {
-        if (s.base < 0 || s.base > n_keys) { s.base = 0; s.count = 0; }
-        if (s.count < 0) s.count = 0;
-        if (s.count > n_keys - s.base) s.count = n_keys - s.base;
-    }
-    s.tiles = static_cast<int>(min((s.count + TC_KEYS - 1) / TC_KEYS, static_cast<int64_t>(max_tiles)));      // max_keys bounds every session
-    return s;
-}
-
-// A CTA's range, one token group (or session) at a time: key tiles [tb, te) of group `g`.  Without MULTI there is one.
-template <bool RAGGED, bool MULTI>
+// A CTA's range, one token group at a time: key tiles [tb, te) of group `g`.  Without MULTI there is one.
+template <bool MULTI>
 struct TcSegments {
     const TcParams& p;
-    const int64_t* offsets;
     int tpc, g, tb, te, left;
     bool first;
-    int64_t key_base, key_count;              // rows key_base .. key_base + key_count of k_idx
-    __device__ __forceinline__ TcSegments(const TcParams& p_, const int64_t* offsets_, int tpc_, int g0, int t0, int work)
-        : p(p_), offsets(offsets_), tpc(tpc_), g(g0), tb(t0), te(t0), left(work), first(true), key_base(0), key_count(p_.n_keys) {}
+    __device__ __forceinline__ TcSegments(const TcParams& p_, int tpc_, int g0, int t0, int work)
+        : p(p_), tpc(tpc_), g(g0), tb(t0), te(t0), left(work), first(true) {}
     __device__ __forceinline__ bool next() {
         if (left <= 0) return false;
         if constexpr (!MULTI) {
-            if constexpr (RAGGED) load(g);
             te = tb + left;
             left = 0;
             return true;
@@ -211,39 +135,23 @@ struct TcSegments {
             do {
                 if (!first) { ++g; tb = 0; }
                 first = false;
-                if constexpr (RAGGED) {
-                    if (g >= p.n_groups) { left = 0; return false; }
-                    tiles = load(g);
-                } else {
-                    tiles = tc_visible_tiles(p, tpc, g);
-                }
-            } while (tiles <= tb);            // (sessions without keys)
+                tiles = tc_visible_tiles(p, tpc, g);
+            } while (tiles <= tb);
             te = min(tiles, tb + left);
             left -= te - tb;
             return true;
         }
     }
-    __device__ __forceinline__ int load(int b) {
-        const TcSession s = tc_session(__ldg(offsets + b), __ldg(offsets + b + 1), p.n_keys, p.n_tiles);
-        key_base = s.base;
-        key_count = s.count;
-        return s.tiles;
-    }
 };
 
-template <int H, bool FP8, bool CAND, bool RAGGED, bool MULTI>
-__global__ void __launch_bounds__(RAGGED ? TC_THREADS_RAGGED : TC_THREADS, RAGGED ? 4 : 1)
+template <int H, bool FP8, bool CAND, bool MULTI>
+__global__ void __launch_bounds__(TC_THREADS, 1)
 indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, const TcParams p, const TcCandParams cp,
-                  const __grid_constant__ typename TcScheduleOf<MULTI && !RAGGED>::type sched) {
+                  const __grid_constant__ typename TcScheduleOf<MULTI>::type sched) {
     extern __shared__ __align__(1024) unsigned char smem[];
     constexpr int TPS = TC_N / H;                      // tokens per query sub-tile
     const int atoms = p.atoms, nq = p.nq, stages = p.stages;
-    // ragged mode keeps only what one query row needs (H rows of Q, H accumulator columns per slot), so that several CTAs fit an SM
-    constexpr int QROWS = RAGGED ? H : TC_N;           // rows of a query sub-tile in shared memory
-    constexpr int SLOT_COLS = RAGGED ? H : TC_N;       // TMEM columns of one accumulator slot
-    constexpr int TMEM_COLS = RAGGED ? 2 * H : 512;
-    static_assert(TMEM_COLS >= 32 && (TMEM_COLS & (TMEM_COLS - 1)) == 0, "TMEM allocations are powers of two of at least 32 columns");
-    const int q_sub_bytes = atoms * QROWS * 128;       // one query sub-tile
+    const int q_sub_bytes = atoms * TC_N * 128;        // one query sub-tile
     const int k_stage_bytes = atoms * TC_KEYS * 128;   // one key tile
     unsigned char* q_smem = smem;
     unsigned char* k_smem = smem + nq * q_sub_bytes;
@@ -254,9 +162,8 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     TcBarriers* bars = reinterpret_cast<TcBarriers*>(reinterpret_cast<unsigned char*>(cstage) + (CAND ? TC_CAND_STAGE_BYTES : 0));
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int NTHREADS = RAGGED ? TC_THREADS_RAGGED : TC_THREADS;
-    constexpr int NEPI = NTHREADS - 64;                         // epilogue threads
-    const int tpc = RAGGED ? 1 : nq * TPS;                      // tokens per group (ragged: a session's one query row)
+    constexpr int NEPI = TC_THREADS - 64;                         // epilogue threads
+    const int tpc = nq * TPS;                                   // tokens per group
 
     if ((smem_u32(smem) & 1023u) != 0u) {   // swizzled tiles need 1024-byte alignment
         grid_wait();
@@ -265,7 +172,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     }
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&bars->k_full[s]), 1); mbar_init(smem_u32(&bars->k_empty[s]), 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&bars->tmem_full[s]), 1); mbar_init(smem_u32(&bars->tmem_empty[s]), RAGGED ? 4 : 8); }
+        for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&bars->tmem_full[s]), 1); mbar_init(smem_u32(&bars->tmem_empty[s]), 8); }
         mbar_init(smem_u32(&bars->mma_drain), 1);
         fence_mbar_init();
         prefetch_tensormap(&tmap_q);
@@ -298,65 +205,17 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     if constexpr (!MULTI) {
         g0 = blockIdx.y;
         tile0 = blockIdx.x * p.tiles_per_cta;
-        int64_t key_begin = 0, key_end = 0;
-        if constexpr (RAGGED) { key_begin = __ldg(cp.key_offsets + g0); key_end = __ldg(cp.key_offsets + g0 + 1); }
-        load_weights(g0, threadIdx.x, NTHREADS);                // (while the offsets are on their way)
-        int tiles;
-        if constexpr (RAGGED) {
-            const TcSession ses = tc_session(key_begin, key_end, p.n_keys, p.n_tiles);
-            if (ses.bad && tile0 == 0 && threadIdx.x == 0) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
-            tiles = ses.tiles;
-        } else {
-            tiles = tc_visible_tiles(p, tpc, g0);
-        }
-        n_work = min(tiles - tile0, p.tiles_per_cta);
+        load_weights(g0, threadIdx.x, TC_THREADS);
+        n_work = min(tc_visible_tiles(p, tpc, g0) - tile0, p.tiles_per_cta);
         if (n_work <= 0) return;
-    } else if constexpr (!RAGGED) {
+    } else {
         g0 = sched.first[blockIdx.x].x;
         tile0 = sched.first[blockIdx.x].y;
         n_work = sched.count + (static_cast<int>(blockIdx.x) < sched.longer ? 1 : 0);
-        load_weights(g0, threadIdx.x, NTHREADS);
-    } else {
-        // the sessions' tile counts are scanned by the block: where this CTA's share of their sum begins
-        int* sums = reinterpret_cast<int*>(ws);                 // (the weights come later)
-        const bool one_round = p.n_groups <= NTHREADS;
-        int64_t total = 0, begin = 0, end = 0;
-        for (int pass = one_round ? 1 : 0; pass < 2; ++pass) {
-            int64_t before = 0;                                 // tiles of the groups of earlier rounds
-            if (pass == 1 && threadIdx.x == 0) bars->first_group = p.n_groups;
-            for (int b0 = 0; b0 < p.n_groups; b0 += NTHREADS) {
-                const int b = b0 + threadIdx.x;
-                int tiles = 0;
-                if (b < p.n_groups) {
-                    const TcSession ses = tc_session(__ldg(cp.key_offsets + b), __ldg(cp.key_offsets + b + 1), p.n_keys, p.n_tiles);
-                    if (ses.bad && pass == 1 && blockIdx.x == 0) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
-                    tiles = ses.tiles;
-                }
-                int block_total;
-                const int mine = block_exclusive_scan<NTHREADS>(tiles, sums, &block_total);
-                if (one_round) total = block_total;
-                if (pass == 1) {
-                    if (b0 == 0) {
-                        const uint32_t each = static_cast<uint32_t>(total) / gridDim.x, more = static_cast<uint32_t>(total) - each * gridDim.x;
-                        begin = static_cast<int64_t>(each) * blockIdx.x + min(blockIdx.x, more);
-                        end = begin + each + (blockIdx.x < more ? 1 : 0);
-                    }
-                    const int64_t at = before + mine;
-                    if (at <= begin && begin < at + tiles) { bars->first_group = b; bars->first_tile = static_cast<int>(begin - at); }
-                }
-                before += block_total;
-            }
-            total = before;
-        }
-        __syncthreads();
-        n_work = static_cast<int>(end - begin);
-        g0 = bars->first_group;
-        tile0 = bars->first_tile;
-        if (n_work <= 0 || g0 >= p.n_groups) return;
-        load_weights(g0, threadIdx.x, NTHREADS);                // (overwrites the scan's scratch: the barrier above is behind its last reader)
+        load_weights(g0, threadIdx.x, TC_THREADS);
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32(&bars->tmem_base), TMEM_COLS);
+        tmem_alloc(smem_u32(&bars->tmem_base), 512);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -379,7 +238,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             // The queries of a segment are counted on the barrier of its first key tile, so the MMA warp needs to know nothing of
             // segments.  They may be replaced when the previous segment's last key tile has been released: every MMA up to it has
             // completed then.
-            TcSegments<RAGGED, MULTI> seg(p, cp.key_offsets, tpc, g0, tile0, n_work);
+            TcSegments<MULTI> seg(p, tpc, g0, tile0, n_work);
             int left = 0;                               // tiles of this segment still to load
             int q_at = -1;                              // the queries are loaded when `left` has come down to this
             int key_row = 0;
@@ -387,7 +246,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             auto load_q = [&]() {
                 for (int j = 0; j < nq; ++j)
                     for (int a = 0; a < atoms; ++a)
-                        tma_load_2d(smem_u32(q_smem + j * q_sub_bytes + a * QROWS * 128), &tmap_q, a * atom_elems, (seg.g * tpc + j * TPS) * H, q_bar);
+                        tma_load_2d(smem_u32(q_smem + j * q_sub_bytes + a * TC_N * 128), &tmap_q, a * atom_elems, (seg.g * tpc + j * TPS) * H, q_bar);
             };
             const uint32_t tile_bytes = static_cast<uint32_t>((FP8 && cp.k_fp4) ? k_stage_bytes / 2 : k_stage_bytes);   // packed 4-bit keys are counted in the bytes read
             for (int it = 0; it < n_work; ++it, s = (s + 1 == stages ? 0 : s + 1), ph ^= (s == 0 ? 1u : 0u)) {
@@ -396,7 +255,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                 if (left == 0) {
                     if (!seg.next()) break;
                     left = seg.te - seg.tb;
-                    key_row = static_cast<int>(seg.key_base) + seg.tb * TC_KEYS;
+                    key_row = seg.tb * TC_KEYS;
                     bytes += static_cast<uint32_t>(nq * q_sub_bytes);
                     q_bar = kf;
                     q_at = MULTI && it > 0 ? max(0, left - (stages - 1)) : -1;    // later segments: the other stages are filled first
@@ -429,8 +288,8 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            // ragged: only the first query row's heads (N = H); the keys (the A operand) may be E2M1 (format 5) against E4M3 queries
-            const uint32_t idesc = umma_idesc(FP8 ? 0u : 1u, TC_KEYS, RAGGED ? H : TC_N) | ((FP8 && cp.k_fp4) ? (5u << 7) : 0u);
+            // the keys (the A operand) may be E2M1 (format 5) against E4M3 queries
+            const uint32_t idesc = umma_idesc(FP8 ? 0u : 1u, TC_KEYS, TC_N) | ((FP8 && cp.k_fp4) ? (5u << 7) : 0u);
             bool ok = true;
             uint32_t cnt = 0;
             // descriptors of the first key stage / first query sub-tile; every other operand is a constant number of 16-byte
@@ -442,19 +301,18 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                 ok = mbar_wait(smem_u32(&bars->k_full[s]), ph) && !*aborted;
                 if (!ok) break;
                 const uint64_t kdesc_s = kdesc0 + static_cast<uint64_t>((s * k_stage_bytes) >> 4);
-                // ragged mode has one query sub-tile, so consecutive key tiles alternate between the two TMEM halves
                 for (int j = 0; j < nq; ++j, ++cnt) {
                     const uint32_t slot = cnt & 1u, use = cnt >> 1;
                     ok = mbar_wait(smem_u32(&bars->tmem_empty[slot]), (use & 1u) ^ 1u) && !*aborted;
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + slot * SLOT_COLS;
+                    const uint32_t d_tmem = tmem_base + slot * TC_N;
                     const uint64_t qdesc_j = qdesc0 + static_cast<uint64_t>((j * q_sub_bytes) >> 4);
                     {
                         uint32_t acc = 0;
                         for (int a = 0; a < atoms; ++a) {
                             const uint64_t ka = kdesc_s + static_cast<uint64_t>((a * TC_KEYS * 128) >> 4);
-                            const uint64_t qa = qdesc_j + static_cast<uint64_t>((a * QROWS * 128) >> 4);
+                            const uint64_t qa = qdesc_j + static_cast<uint64_t>((a * TC_N * 128) >> 4);
 #pragma unroll
                             for (int ks = 0; ks < 4; ++ks) {   // 32 bytes of K per instruction (16 bf16 or 32 e4m3)
                                 umma<FP8>(d_tmem, ka + 2 * ks, qa + 2 * ks, idesc, acc);
@@ -478,13 +336,11 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         }
     } else {
         // ------------------------------------------------------------------ epilogue: warps 2 and up
-        constexpr bool W16 = !RAGGED;
-        constexpr int NCHUNK = RAGGED ? H / 32 : TC_N / 32;   // 32-column chunks of a slot (ragged: the first query row only)
-        constexpr int CPW = W16 ? NCHUNK / 2 : NCHUNK;        // chunks a warp reduces
-        constexpr int TPH = W16 ? TPS / 2 : TPS;              // tokens of a slot a warp reduces
+        constexpr int CPW = TC_N / 32 / 2;      // 32-column chunks a warp reduces: half a slot
+        constexpr int TPH = TPS / 2;            // tokens of a slot a warp reduces
         static_assert(CPW % 2 == 0, "chunks are processed in pairs");
         const int e = ((warp - 2) >> 2) & 1;    // epilogue group = TMEM half it drains
-        const int chalf = W16 ? (warp - 2) >> 3 : 0;   // which half of the slot's columns
+        const int chalf = (warp - 2) >> 3;   // which half of the slot's columns
         const int quad = warp & 3;              // TMEM lanes 32*quad .. 32*quad+31
         const float neg_inf = __int_as_float(0xff800000);
         bool ok = true;
@@ -499,7 +355,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             if (lane < c && base + lane < cp.cand_cap) cp.cand[static_cast<int64_t>(t) * cp.cand_cap + base + lane] = my_stage[slot * TC_CAND_SLOTS + lane];
             __syncwarp();                                        // slots are free again
         };
-        if constexpr (!CAND && !RAGGED) {
+        if constexpr (!CAND) {
             if (p.causal) {
                 // the CTAs that work on a group share its rows; with even shares all CTAs share all rows
                 constexpr bool own = !MULTI;
@@ -512,7 +368,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         uint32_t it = 0;                        // tiles done so far, over all segments
         bool later = false;
         // every wait is bounded and a warp that gives up keeps to the barriers of the segments that follow
-        for (TcSegments<RAGGED, MULTI> seg(p, cp.key_offsets, tpc, g0, tile0, n_work); seg.next(); later = true) {
+        for (TcSegments<MULTI> seg(p, tpc, g0, tile0, n_work); seg.next(); later = true) {
             if (MULTI && later) {
                 epilogue_barrier<NEPI>();       // nobody reads the previous weights any more
                 load_weights(seg.g, threadIdx.x - 64, NEPI);
@@ -520,33 +376,25 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             }
             const int t0 = seg.g * tpc;
             for (int tile = seg.tb; tile < seg.te && ok; ++tile, ++it) {
-                const int64_t s_local = static_cast<int64_t>(tile) * TC_KEYS + quad * 32 + lane;
-                const bool key_ok = s_local < seg.key_count;
-                const int64_t s = seg.key_base + s_local;           // row of k_idx (and of k_scale / col_bias; ragged: of scores)
+                const int64_t s = static_cast<int64_t>(tile) * TC_KEYS + quad * 32 + lane;
+                const bool key_ok = s < p.n_keys;
                 const float kscale = (FP8 && key_ok) ? p.k_scale[s] : 1.f;
                 const float cb = (p.col_bias != nullptr && key_ok) ? p.col_bias[s] : 0.f;
-                // group e drains the sub-tiles j = e, e+2, .. of every key tile (nq is even);
-                // ragged mode (nq = 1, one group): consecutive key tiles sit in slots 0, 1, 0, ..
-                for (int j = RAGGED ? 0 : e; j < nq; j += 2) {
-                    const int slot = RAGGED ? static_cast<int>(it & 1u) : e;     // ragged: the one group takes both slots in turn
+                // group e drains the sub-tiles j = e, e+2, .. of every key tile (nq is even)
+                for (int j = e; j < nq; j += 2) {
+                    const int slot = e;
                     const uint32_t use = (it * static_cast<uint32_t>(nq) + static_cast<uint32_t>(j)) >> 1;
                     ok = mbar_wait(smem_u32(&bars->tmem_full[slot]), use & 1u) && !*aborted;
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + slot * SLOT_COLS + chalf * CPW * 32;
+                    const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + slot * TC_N + chalf * CPW * 32;
                     const int tsub0 = t0 + j * TPS + chalf * TPH;
                     const float* wrow = ws + j * TC_N + chalf * CPW * 32;
                     const float* rb = rbs + j * TPS + chalf * TPH;
                     float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
                     auto store = [&](int tt, float v) {
                         const int t = tsub0 + tt;
-                        if constexpr (RAGGED) {
-                            if (tt == 0 && key_ok) {
-                                float out = v * kscale;
-                                out = fmaf(rb[0], cb, out);
-                                p.scores[s] = out;
-                            }
-                        } else if constexpr (!CAND) {
+                        if constexpr (!CAND) {
                             if (t < p.M && key_ok) {
                                 float out = v * kscale;
                                 out = fmaf(rb[tt], cb, out);
@@ -605,7 +453,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, TMEM_COLS);
+        tmem_dealloc(tmem_base, 512);
     }
 }
 
@@ -654,17 +502,16 @@ bool indexer_tc_candidates_supported(int H, int D, int dtype) {
     return (H == 32 || H == 64) && (nq_max / 2) * (TC_N / H / 2) <= TC_CAND_TPW;
 }
 
-template <int H, bool FP8, bool CAND, bool RAGGED, bool MULTI>
+template <int H, bool FP8, bool CAND, bool MULTI>
 static int launch_tc(const CUtensorMap& tq, const CUtensorMap& tk, const TcParams& p, const TcCandParams& cp, const TcSchedule& sched, dim3 grid,
                      size_t smem, cudaStream_t stream) {
     static once_per_device attributes;
     JANUS_CUDA_CHECK(attributes.run(
-        [] { return cudaFuncSetAttribute(indexer_tc_kernel<H, FP8, CAND, RAGGED, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET); }));
-    constexpr int threads = RAGGED ? TC_THREADS_RAGGED : TC_THREADS;
-    if constexpr (MULTI && !RAGGED)
-        JANUS_CUDA_CHECK(launch_kernel(indexer_tc_kernel<H, FP8, CAND, RAGGED, MULTI>, grid, threads, smem, stream, 1, tq, tk, p, cp, sched));
+        [] { return cudaFuncSetAttribute(indexer_tc_kernel<H, FP8, CAND, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET); }));
+    if constexpr (MULTI)
+        JANUS_CUDA_CHECK(launch_kernel(indexer_tc_kernel<H, FP8, CAND, MULTI>, grid, TC_THREADS, smem, stream, 1, tq, tk, p, cp, sched));
     else
-        JANUS_CUDA_CHECK(launch_kernel(indexer_tc_kernel<H, FP8, CAND, RAGGED, MULTI>, grid, threads, smem, stream, 1, tq, tk, p, cp,
+        JANUS_CUDA_CHECK(launch_kernel(indexer_tc_kernel<H, FP8, CAND, MULTI>, grid, TC_THREADS, smem, stream, 1, tq, tk, p, cp,
                                        TcNoSchedule{}));
     return JANUS_OK;
 }
@@ -680,7 +527,7 @@ int launch_indexer_tc(const void* q_idx, const void* k_idx, int64_t k_stride_tok
     p.w = w; p.q_scale = q_scale; p.q_scale_stride_tok = q_scale_stride_tok; p.k_scale = k_scale;
     p.row_bias = row_bias; p.col_bias = col_bias; p.scores = scores; p.ld = ld; p.n_keys = n_keys; p.q_pos0 = q_pos0;
     p.M = M; p.H = H; p.causal = causal; p.dev_status = dev_status;
-    const TcCandParams cp{thr, cand_cnt, static_cast<int2*>(cand), cand_cap, nullptr, k_fp4 ? 1 : 0};
+    const TcCandParams cp{thr, cand_cnt, static_cast<int2*>(cand), cand_cap, k_fp4 ? 1 : 0};
     p.atoms = D * esz / 128;
     p.n_tiles = static_cast<int>((n_keys + TC_KEYS - 1) / TC_KEYS);
     const int tps = TC_N / H;
@@ -754,10 +601,10 @@ int launch_indexer_tc(const void* q_idx, const void* k_idx, int64_t k_stride_tok
 
 #define JANUS_TC_CASE(HH, CC)                                                         \
     case HH:                                                                          \
-        if (multi) return fp8 ? launch_tc<HH, true, CC, false, true>(tq, tk, p, cp, sched, grid, smem, stream)          \
-                              : launch_tc<HH, false, CC, false, true>(tq, tk, p, cp, sched, grid, smem, stream);        \
-        return fp8 ? launch_tc<HH, true, CC, false, false>(tq, tk, p, cp, sched, grid, smem, stream)                    \
-                   : launch_tc<HH, false, CC, false, false>(tq, tk, p, cp, sched, grid, smem, stream);
+        if (multi) return fp8 ? launch_tc<HH, true, CC, true>(tq, tk, p, cp, sched, grid, smem, stream)          \
+                              : launch_tc<HH, false, CC, true>(tq, tk, p, cp, sched, grid, smem, stream);        \
+        return fp8 ? launch_tc<HH, true, CC, false>(tq, tk, p, cp, sched, grid, smem, stream)                    \
+                   : launch_tc<HH, false, CC, false>(tq, tk, p, cp, sched, grid, smem, stream);
     if (cand_mode) {
         switch (H) {   // head counts whose tokens per epilogue warp fit the staging slots
             JANUS_TC_CASE(32, true)
@@ -774,73 +621,6 @@ int launch_indexer_tc(const void* q_idx, const void* k_idx, int64_t k_stride_tok
     }
 #undef JANUS_TC_CASE
     return JANUS_ERR_UNSUPPORTED;
-}
-
-// Ragged batch (decode): B query rows, row b against keys key_offsets[b] .. key_offsets[b+1] of one concatenated array.
-bool indexer_tc_batch_supported(int B, int H, int D, int64_t total_keys, int dtype) {
-    const int row_bytes = D * (dtype == JANUS_DTYPE_BF16 ? 2 : 1);
-    if (dtype == JANUS_DTYPE_FP8_Q_FP4_K && D != 128) return false;      // the packed 4-bit TMA box is 128 elements
-    return H == 64 && (row_bytes == 128 || row_bytes == 256) && static_cast<int64_t>(B) * H < (int64_t(1) << 31) &&
-           total_keys < (int64_t(1) << 31) - 256 && B <= 65535;
-}
-
-int launch_indexer_tc_batch(const void* q_idx, const void* k_idx, int64_t k_stride_tok, const float* w, const float* q_scale,
-                            int64_t q_scale_stride_tok, const float* k_scale, const float* row_bias, const float* col_bias, int B, int H, int D,
-                            int64_t total_keys, int64_t max_keys, const int64_t* key_offsets, int dtype, float* scores, int32_t* dev_status,
-                            cudaStream_t stream) {
-    const bool k_fp4 = dtype == JANUS_DTYPE_FP8_Q_FP4_K;
-    const bool fp8 = dtype == JANUS_DTYPE_FP8_E4M3 || k_fp4;
-    const int esz = fp8 ? 1 : 2;
-    TcParams p;
-    p.w = w; p.q_scale = q_scale; p.q_scale_stride_tok = q_scale_stride_tok; p.k_scale = k_scale;
-    p.row_bias = row_bias; p.col_bias = col_bias; p.scores = scores; p.ld = 0; p.n_keys = total_keys; p.q_pos0 = 0;
-    p.M = B; p.H = H; p.causal = 0; p.dev_status = dev_status;
-    const TcCandParams cp{nullptr, nullptr, nullptr, 0, key_offsets, k_fp4 ? 1 : 0};
-    p.atoms = D * esz / 128;
-    p.nq = 1;
-    const int tps = TC_N / H;
-    const int q_bytes = p.nq * p.atoms * H * 128;           // one query row: H (head) rows of the B operand
-    const int k_stage = p.atoms * TC_KEYS * 128;
-    const int tail = static_cast<int>(sizeof(float)) * (p.nq * TC_N + 2 * p.nq * tps) + static_cast<int>(sizeof(TcBarriers)) + 16;
-    // One query row per CTA leaves the single MMA-issuing thread as the limit of a CTA, so several CTAs share an SM: four with
-    // one-byte operands (each a quarter of the SM's shared memory less the 1 KB the system keeps per CTA, 2 x H of the 512
-    // TMEM columns, 6 warps of at most 80 registers), two with bf16 (a key stage is 32 KB).
-    const int budget = (227 * 1024) / (fp8 ? 4 : 2) - 1024;
-    p.stages = (budget - q_bytes - tail) / k_stage;
-    if (p.stages > TC_MAX_STAGES) p.stages = TC_MAX_STAGES;
-    if (p.stages < 2) return JANUS_ERR_UNSUPPORTED;
-    const size_t smem = static_cast<size_t>(q_bytes) + static_cast<size_t>(p.stages) * k_stage + tail;
-    const int64_t max_tiles = (max_keys + TC_KEYS - 1) / TC_KEYS;
-    if (max_tiles == 0) return JANUS_OK;
-    p.n_tiles = static_cast<int>(max_tiles);
-    // Either every CTA gets the same number of one session's tiles (a 2-D grid that is resident at once), or the tiles of all
-    // sessions, whose number only the device knows, are shared out evenly.  The second needs a scan of the offsets and changes of
-    // session, together about three tiles' time, so it is taken when the first would leave some CTA that much more than the
-    // average, as far as the host can tell from total_keys.  64 sessions of 30000 FP8 keys 58.5 -> 46 us against chunks of fixed
-    // length in part-filled waves, 64 of 81920 FP4 keys 112 -> 84, ragged ones (a quarter to all of 131072) 120 -> 91.
-    const int64_t resident = static_cast<int64_t>(TC_MAX_CTAS) * (fp8 ? 4 : 2);
-    const int64_t chunks = resident / B > max_tiles ? max_tiles : resident / B;
-    int64_t per = chunks > 0 ? (max_tiles + chunks - 1) / chunks : 0;
-    if (per == 1 && max_tiles > 1) per = 2;
-    const bool direct = chunks > 0 && per <= total_keys / TC_KEYS / resident + 4;
-    p.tiles_per_cta = direct ? static_cast<int>(per) : 0;
-    p.n_groups = B;
-    const dim3 grid(static_cast<unsigned>(direct ? (max_tiles + per - 1) / per : resident), direct ? B : 1);
-    CUtensorMap tq, tk;
-    const uint32_t box_cols = fp8 ? 128 : 64;
-    if (!make_tmap_2d_sw128(&tq, q_idx, esz, static_cast<uint64_t>(B) * H, D, static_cast<uint64_t>(D) * esz, H, box_cols)) return JANUS_ERR_CUDA;
-    if (k_fp4) {
-        if (!make_tmap_2d_sw128(&tk, k_idx, 0, static_cast<uint64_t>(total_keys), D, static_cast<uint64_t>(k_stride_tok) / 2, TC_KEYS, 128))
-            return JANUS_ERR_CUDA;
-    } else if (!make_tmap_2d_sw128(&tk, k_idx, esz, static_cast<uint64_t>(total_keys), D, static_cast<uint64_t>(k_stride_tok) * esz, TC_KEYS, box_cols)) {
-        return JANUS_ERR_CUDA;
-    }
-    const TcSchedule sched{};
-    if (direct)
-        return fp8 ? launch_tc<64, true, false, true, false>(tq, tk, p, cp, sched, grid, smem, stream)
-                   : launch_tc<64, false, false, true, false>(tq, tk, p, cp, sched, grid, smem, stream);
-    return fp8 ? launch_tc<64, true, false, true, true>(tq, tk, p, cp, sched, grid, smem, stream)
-               : launch_tc<64, false, false, true, true>(tq, tk, p, cp, sched, grid, smem, stream);
 }
 
 }  // namespace janus
