@@ -156,6 +156,7 @@ page_mark_global_kernel(const PdParams p) {
 struct PdShared {
     uint64_t warp_sums[2][33];
     uint64_t totals[2];                       // this CTA's slice: the set, the miss set
+    uint64_t before[2], all[2];               // the slices before it, all slices
     uint64_t at[2][PD_THREADS];               // counts before each word of a chunk
     uint32_t word[2][PD_THREADS + 2];         // the words of a chunk and one neighbour on either side
 };
@@ -211,7 +212,7 @@ page_demand_kernel(const PdParams p) {
         const PageDiv page{p.page_size, p.page_shift};
         bool bad = false;
         // Eight indices per thread at a time, in rounds of loads that are all in flight together: indices and their rows' table and
-        // limit, then page table entries (one index after the other: 24.2 instead of 21.9 us for 64 decode rows of 2048)
+        // limit, then page table entries (one index after the other: 24.2 us instead of 21.9 for 64 decode rows of 2048, when the rest took 5 us longer)
         constexpr int U = 8;
         const int stride = n_cta * PD_THREADS, n_idx = static_cast<int>(p.n_idx);
         for (int base = rank * PD_THREADS + tid; base < n_idx; base += U * stride) {
@@ -325,19 +326,24 @@ page_demand_kernel(const PdParams p) {
     }
     if (tid == 0) { sh.totals[0] = sum[0]; sh.totals[1] = sum[1]; }
     cluster_sync_all();                   // counts are there; nobody reads the private bitmaps any more
-    uint64_t base[2], all[2];             // lane r fetches CTA r's counts
+    // Warp 0 fetches everybody's counts, lane r those of CTA r: from all 32 warps they were a thousand small remote loads per CTA, which
+    // took 4 us with sixteen CTAs.
+    if (warp == 0) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        uint64_t x = lane < n_cta ? ld_cluster_u64(mapa_shared(smem_u32(&sh.totals[q]), lane)) : 0;
-        uint64_t y = lane < rank ? x : 0;
+        for (int q = 0; q < 2; ++q) {
+            uint64_t x = lane < n_cta ? ld_cluster_u64(mapa_shared(smem_u32(&sh.totals[q]), lane)) : 0;
+            uint64_t y = lane < rank ? x : 0;
 #pragma unroll
-        for (int d = PD_MAX_CLUSTER / 2; d > 0; d >>= 1) {
-            x += __shfl_xor_sync(0xffffffffu, x, d);
-            y += __shfl_xor_sync(0xffffffffu, y, d);
+            for (int d = PD_MAX_CLUSTER / 2; d > 0; d >>= 1) {
+                x += __shfl_xor_sync(0xffffffffu, x, d);
+                y += __shfl_xor_sync(0xffffffffu, y, d);
+            }
+            if (lane == 0) { sh.all[q] = x; sh.before[q] = y; }
         }
-        all[q] = __shfl_sync(0xffffffffu, x, 0);
-        base[q] = __shfl_sync(0xffffffffu, y, 0);
     }
+    __syncthreads();
+    uint64_t base[2] = {sh.before[0], sh.before[1]};
+    const int cap = static_cast<int>(min(p.capacity, static_cast<int64_t>(0x7fffffff)));
     for (int c0 = w0; c0 < w1; c0 += PD_THREADS) {
         if (!one_chunk) {
             uint64_t mine[2];
@@ -348,24 +354,28 @@ page_demand_kernel(const PdParams p) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) sh.at[q][tid] = base[q] + excl[q];
         __syncthreads();
-        // a warp writes one word's entries at a time, a lane per page: neighbouring entries leave in one store
+        // A warp writes one word's entries at a time, a lane per page: neighbouring entries leave in one store.  Bound by its instructions.
         const int n_in = min(PD_THREADS, w1 - c0);
-        for (int jq = warp; jq < (want_miss ? 2 * n_in : n_in); jq += PD_THREADS / 32) {
-            const int q = jq >= n_in ? 1 : 0, j = jq - q * n_in;
-            const uint32_t w = sh.word[q][j + 1];
-            if (w == 0u) continue;
+        const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q == 1 && !want_miss) break;
             int32_t* ids = q ? p.miss_pages : p.pages;
             int32_t* runs = q ? p.miss_runs : p.runs;
-            const uint32_t b = sh.word[q][j] >> 31, a = sh.word[q][j + 2] & 1u;
-            const uint64_t o = sh.at[q][j];
-            const uint32_t starts = w & ~((w << 1) | b), ends = w & ~((w >> 1) | (a << 31)), below = (1u << lane) - 1u;
-            const int64_t o_id = static_cast<int64_t>(o >> 32) + __popc(w & below);
-            const int64_t o_st = static_cast<int64_t>(o & 0xffffffffu) + __popc(starts & below);
-            const int64_t o_en = static_cast<int64_t>(o & 0xffffffffu) - (b & w & 1u) + __popc(ends & below);
-            const int32_t page = (c0 + j) * 32 + lane;
-            if (((w >> lane) & 1u) && o_id < p.capacity) ids[o_id] = page;
-            if (((starts >> lane) & 1u) && o_st < p.capacity) runs[2 * o_st] = page;
-            if (((ends >> lane) & 1u) && o_en < p.capacity) runs[2 * o_en + 1] = page + 1;     // becomes a length below
+            for (int j = warp; j < n_in; j += PD_THREADS / 32) {
+                const uint32_t w = sh.word[q][j + 1];
+                if (((w >> lane) & 1u) == 0u) continue;
+                const uint32_t starts = w & ~((w << 1) | (sh.word[q][j] >> 31)), ends = w & ~((w >> 1) | (sh.word[q][j + 2] << 31));
+                const uint64_t o = sh.at[q][j];
+                const int o_id = static_cast<int>(o >> 32) + __popc(w & below);
+                const int run = static_cast<int>(o & 0xffffffffu) + __popc(starts & (below | (1u << lane))) - 1;      // the page's run
+                const int32_t page = (c0 + j) * 32 + lane;
+                if (o_id < cap) ids[o_id] = page;
+                if (run < cap) {
+                    if ((starts >> lane) & 1u) runs[2 * static_cast<int64_t>(run)] = page;
+                    if ((ends >> lane) & 1u) runs[2 * static_cast<int64_t>(run) + 1] = page + 1;        // becomes a length below
+                }
+            }
         }
         base[0] += sum[0];
         base[1] += sum[1];
@@ -375,7 +385,7 @@ page_demand_kernel(const PdParams p) {
     for (int q = 0; q < 2; ++q) {
         if (q == 1 && !want_miss) break;
         int32_t* runs = q ? p.miss_runs : p.runs;
-        const int64_t n_runs = static_cast<int64_t>(all[q] & 0xffffffffu), n_ids = static_cast<int64_t>(all[q] >> 32);
+        const int64_t n_runs = static_cast<int64_t>(sh.all[q] & 0xffffffffu), n_ids = static_cast<int64_t>(sh.all[q] >> 32);
         const int64_t n = n_runs < p.capacity ? n_runs : p.capacity;
         for (int64_t j = static_cast<int64_t>(rank) * PD_THREADS + tid; j < n; j += static_cast<int64_t>(n_cta) * PD_THREADS)
             runs[2 * j + 1] = __ldcg(runs + 2 * j + 1) - __ldcg(runs + 2 * j);
@@ -407,17 +417,16 @@ static int launch_page_demand(const PdParams& p, int cluster, cudaStream_t strea
     return JANUS_OK;
 }
 
-// One launch of one cluster while it reads the indices as fast as memset, chip-wide marking and lists would (14 us up to 512 K
-// indices): 128 K indices in 12 us, 256 K in 15.  Four CTAs up to 4 K indices (7.6 us; eight and sixteen cost 0.5 and 2.5 us more),
-// eight up to 64 K (9.3 us at 256 x 256, four and sixteen 1 to 2 us more), sixteen beyond (64 rows of a 131136-page pool: 21.9
-// against 35 with eight and 27 for the three launches).  Memset, marking and one-CTA lists took 14.6, 18.5 and 36.6 us for these
-// three.
+// One launch of one cluster while it reads the indices as fast as memset, chip-wide marking and lists would (12.4 us up to 512 K
+// indices): 128 K indices in 9.6 us, 256 K in 12.3, 512 K in 17.4.  Four CTAs up to 8 K indices (7.1 us; eight and sixteen cost 0.1 and 0.3 us more),
+// sixteen beyond (256 x 256 8.0 us against 10.7 with four and 8.6 with eight, 12 decode rows 8.4, 10.5 and 9.1, 64 rows of a 131136-page
+// pool 17.1, 26.4 and 26.4).
 constexpr int64_t PD_ONE_LAUNCH_INDICES = 1 << 17;
 
 template <int MODE>
 static int run_page_demand(const PdParams& p, cudaStream_t stream) {
     if (p.n_idx <= PD_ONE_LAUNCH_INDICES && p.n_words <= PD_SMEM_WORDS) {
-        int cluster = p.n_idx <= 4096 ? 4 : p.n_idx <= 65536 ? 8 : 16;
+        int cluster = p.n_idx <= 8192 ? 4 : 16;
         while (p.n_words > cluster * PD_THREADS) cluster *= 2;      // a slice is one chunk
         return launch_page_demand<MODE>(p, cluster, stream);
     }
