@@ -17,8 +17,11 @@
 
 namespace janus {
 
-constexpr int TK_CAP = 8192;        // 73 KB of shared memory per CTA keeps three CTAs on an SM
-constexpr int TK_CAP_SMALL = 5632;  // 54 KB: four CTAs on an SM (all 2048 threads), for rows whose candidate list is sure to fit
+// Three CTAs share an SM (registers).  With 73 KB of shared memory each they leave next to nothing of it to L1, through which the
+// streaming loads pass, with 54 KB a third: 4096 rows of 135168 390 us against 498, 1024 of 16384 28 against 35.  (Four CTAs of 54 KB and
+// 32 registers: 497.)
+constexpr int TK_CAP = 8192;
+constexpr int TK_CAP_SMALL = 5632;  // for rows whose candidate list is sure to fit
 
 template <int CAP>
 __global__ void __launch_bounds__(TK_THREADS)
@@ -339,7 +342,7 @@ extern "C" int janus_topk(const float* scores, int64_t scores_ld, int M, int64_t
     if (n_keys > 0 && (!scores || !aligned16(scores) || (scores_ld & 3) != 0)) return JANUS_ERR_INVALID_ARG;
     // The candidate list of a row holds what passes the sampled threshold: about n * r / 4096 elements for the sample rank
     // r = e + 4 sqrt(e) + 8, e = 4096 k / n, give or take n sqrt(r) / 4096.  When that plus five deviations fits the small
-    // buffer for the longest row, four CTAs share an SM instead of three.
+    // buffer for the longest row, that is taken.
     const double n_max = static_cast<double>(causal ? (n_keys < q_pos0 + M ? n_keys : q_pos0 + M) : n_keys);
     bool small = false;
     if (n_max > TK_CAP) {

@@ -7,7 +7,8 @@
 // sample value), candidates are counted into the buckets of a second histogram as they are found, and one pass over them then
 // emits what lies above the k-th key's bucket while the few keys inside it are ranked directly.  Against two selections of repeated
 // histogram passes (B200, k = 2048): 4096 rows of 135168 0.442 -> 0.385 ms (5.7 TB/s, 0.86 of the copy bandwidth; what is left is
-// that a CTA between two streaming passes reads nothing), 2048 rows of 34816 122 -> 100 us, one row of 32768 15.4 -> 9.7 us.  The exact selection over
+// that a CTA between two streaming passes reads nothing), 2048 rows of 34816 122 -> 100 us, one row of 32768 (a cluster) 15.4 -> 9.6, and 8.2 us
+// with its first loads issued before the sample and counts of 16 bits exchanged.  The exact selection over
 // repeated histogram passes (select_kth) remains for what this cannot settle: a misjudged sample, or hundreds of keys in one bucket.
 #pragma once
 
@@ -21,6 +22,7 @@ constexpr int TK_WARPS = TK_THREADS / 32;
 constexpr int TK_MAX_CLUSTER = 8;   // CTAs that share a row
 constexpr int TK_BUCKETS = 2048;
 constexpr int TK_SAMPLE = 4096;     // 512 threads x 8 floats (one 32-byte sector each)
+constexpr int TK_FULL = 1 << 26;    // more than the counts of all buckets of a cluster
 constexpr int TK_DIRECT = 256;      // a bucket of at most this many keys is ranked directly instead of split further
 
 template <int CAP>
@@ -380,32 +382,47 @@ __device__ __forceinline__ bool topk_sample(const float* __restrict__ row, int n
     return true;
 }
 
+// Four 16-byte groups of a thread: i, i + TK_THREADS, ..; past the end NaN, which no threshold lets in.
+__device__ __forceinline__ void load_groups(const float4* __restrict__ row4, int i, int f4_end, float4 (&x)[4]) {
+    if (i + 3 * TK_THREADS < f4_end) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = __ldcs(row4 + i + u * TK_THREADS);
+    } else {
+        const float nan = __int_as_float(0x7fffffff);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            x[u] = make_float4(nan, nan, nan, nan);
+            if (i + u * TK_THREADS < f4_end) x[u] = __ldcs(row4 + i + u * TK_THREADS);
+        }
+    }
+}
+
 // One streaming pass over the 16-byte groups [f4_begin, f4_end) of the row (and, with `tail`, the n % 4 elements after the
 // last whole group).
 template <class Sh>
 __device__ __forceinline__ void topk_stream(const float* __restrict__ row, int n, int f4_begin, int f4_end, bool tail, float thr_f, Sh& sh) {
     const int tid = threadIdx.x;
     const float4* row4 = reinterpret_cast<const float4*>(row);
-    constexpr int UNROLL = 4;                     // 16-byte loads in flight per thread
     int i = f4_begin + tid;
-    for (; i + (UNROLL - 1) * TK_THREADS < f4_end; i += UNROLL * TK_THREADS) {
-        float4 x[UNROLL];
+    for (; i + 3 * TK_THREADS < f4_end; i += 4 * TK_THREADS) {
+        float4 x[4];                              // 16-byte loads in flight per thread
 #pragma unroll
-        for (int u = 0; u < UNROLL; ++u) x[u] = __ldcs(row4 + i + u * TK_THREADS);
+        for (int u = 0; u < 4; ++u) x[u] = __ldcs(row4 + i + u * TK_THREADS);
         keep_candidates16(x, 4 * i, 4 * TK_THREADS, thr_f, sh);
     }
-    auto keep = [&](float v, int e) {
-        if (v >= thr_f) {
-            const int o = atomicAdd(&sh.n_cand, 1);
-            if (o < Sh::kCap) { sh.cand_key[o] = __float_as_uint(v); sh.cand_idx[o] = e; }
-        }
-    };
-    for (; i < f4_end; i += TK_THREADS) {
-        const float4 x = __ldcs(row4 + i);
-        keep(x.x, 4 * i); keep(x.y, 4 * i + 1); keep(x.z, 4 * i + 2); keep(x.w, 4 * i + 3);
+    if (i < f4_end) {
+        float4 x[4];
+        load_groups(row4, i, f4_end, x);
+        keep_candidates16(x, 4 * i, 4 * TK_THREADS, thr_f, sh);
     }
     const int n4 = n >> 2;
-    if (tail && tid < n - 4 * n4) keep(__ldcg(row + 4 * n4 + tid), 4 * n4 + tid);
+    if (tail && tid < n - 4 * n4) {
+        const float v = __ldcg(row + 4 * n4 + tid);
+        if (v >= thr_f) {
+            const int o = atomicAdd(&sh.n_cand, 1);
+            if (o < Sh::kCap) { sh.cand_key[o] = __float_as_uint(v); sh.cand_idx[o] = 4 * n4 + tid; }
+        }
+    }
 }
 
 // A row of at most k elements: all of them, and the smallest value.
@@ -504,7 +521,15 @@ __device__ __forceinline__ void topk_row_cluster(const float* __restrict__ row, 
     const int rank = static_cast<int>(cluster_ctarank()), n_cta = static_cast<int>(cluster_nctarank());
     uint32_t thr = 0u, hi = 0u;
     if (tid == 0) { sh.n_cand = 0; sh.out_pos = 0; sh.n_small = 0; sh.sel_out = 0; }
-    const bool split = n > Sh::kCap && n > k && topk_sample(row, n, k, thr, hi, sh);     // the same answer in every CTA
+    // the first of this CTA's share is on its way while the sample is worked on
+    const int64_t n4 = n >> 2;
+    const int f4_begin = static_cast<int>(n4 * rank / n_cta), f4_end = static_cast<int>(n4 * (rank + 1) / n_cta);
+    float4 x[4];
+    bool split = n > Sh::kCap && n > k;            // the same answer in every CTA
+    if (split) {
+        load_groups(reinterpret_cast<const float4*>(row), f4_begin + tid, f4_end, x);
+        split = topk_sample(row, n, k, thr, hi, sh);
+    }
     if (!split) {
         if (rank == 0) topk_row(row, n, k, out, count, kth, sh);
         return;
@@ -512,32 +537,39 @@ __device__ __forceinline__ void topk_row_cluster(const float* __restrict__ row, 
     const BucketMap map(thr, max(thr, hi));
     clear_hist(sh);
     __syncthreads();
-    const int64_t n4 = n >> 2;
-    topk_stream(row, n, static_cast<int>(n4 * rank / n_cta), static_cast<int>(n4 * (rank + 1) / n_cta), rank == n_cta - 1, key_to_float(thr), sh);
+    keep_candidates16(x, 4 * (f4_begin + tid), 4 * TK_THREADS, key_to_float(thr), sh);
+    topk_stream(row, n, f4_begin + 4 * TK_THREADS, f4_end, rank == n_cta - 1, key_to_float(thr), sh);
     __syncthreads();
     count_candidates(min(sh.n_cand, Sh::kCap), map, sh);
+    __syncthreads();
+    // The counts travel as 16 bits each, four buckets in 8 bytes where the histogram was (its bytes are what the exchange takes); bit 15 of
+    // the lowest bucket says that the list was full.
+    const int4 own = own_buckets(sh);
+    __syncthreads();
+    const uint32_t full = tid == TK_THREADS - 1 && sh.n_cand > Sh::kCap ? 0x8000u : 0u;
+    reinterpret_cast<uint2*>(sh.hist)[TK_THREADS - 1 - tid] = make_uint2(static_cast<uint32_t>(own.x) | full | static_cast<uint32_t>(own.y) << 16,
+                                                                         static_cast<uint32_t>(own.z) | static_cast<uint32_t>(own.w) << 16);
     cluster_sync_all();                            // every CTA's candidates and counts
     // remote loads of all CTAs are issued together: one after the other each would cost the round trip
     int4 c = make_int4(0, 0, 0, 0);
-    bool fits = true;
-    const uint32_t my_buckets = smem_u32(sh.hist) + 16u * (TK_THREADS - 1 - tid), my_cand = smem_u32(&sh.n_cand);
     {
-        int4 x[TK_MAX_CLUSTER];
-        uint32_t m[TK_MAX_CLUSTER];
+        const uint32_t my_buckets = smem_u32(sh.hist) + 8u * (TK_THREADS - 1 - tid);
+        uint64_t v[TK_MAX_CLUSTER];
+#pragma unroll
+        for (int r = 0; r < TK_MAX_CLUSTER; ++r) v[r] = ld_cluster_u64(mapa_shared(my_buckets, min(r, n_cta - 1)));
 #pragma unroll
         for (int r = 0; r < TK_MAX_CLUSTER; ++r) {
-            x[r] = ld_cluster_s32x4(mapa_shared(my_buckets, min(r, n_cta - 1)));
-            m[r] = ld_cluster_u32(mapa_shared(my_cand, min(r, n_cta - 1)));
-        }
-#pragma unroll
-        for (int r = 0; r < TK_MAX_CLUSTER; ++r) {
-            if (r < n_cta) { c.x += x[r].x; c.y += x[r].y; c.z += x[r].z; c.w += x[r].w; }
-            fits = fits && static_cast<int>(m[r]) <= Sh::kCap;
+            if (r >= n_cta) continue;
+            const uint32_t lo = static_cast<uint32_t>(v[r]), up = static_cast<uint32_t>(v[r] >> 32);
+            c.x += static_cast<int>(lo & 0x7fffu) + ((lo & 0x8000u) != 0u ? TK_FULL : 0);
+            c.y += static_cast<int>(lo >> 16);
+            c.z += static_cast<int>(up & 0xffffu);
+            c.w += static_cast<int>(up >> 16);
         }
     }
     const int total = find_bucket(c, k, sh);
     const int b = sh.sel_bucket, above = sh.sel_above, in = sh.sel_count;
-    if (!fits || total < k || in > TK_DIRECT) {    // uniform over the cluster: everybody read the same counts
+    if (total >= TK_FULL || total < k || in > TK_DIRECT) {    // uniform over the cluster: everybody read the same counts
         cluster_sync_all();                        // which may change only now
         if (rank == 0) {
             if (count != nullptr && tid == 0) *count = k;
@@ -546,7 +578,6 @@ __device__ __forceinline__ void topk_row_cluster(const float* __restrict__ row, 
         return;
     }
     // this CTA's keys above the bucket, and where they go: one reservation in CTA 0
-    const int4 own = own_buckets(sh);
     const int first = TK_BUCKETS - 4 - 4 * tid;
     int mine = (first > b ? own.x : 0) + (first + 1 > b ? own.y : 0) + (first + 2 > b ? own.z : 0) + (first + 3 > b ? own.w : 0);
     mine = __reduce_add_sync(0xffffffffu, mine);
