@@ -12,13 +12,18 @@
 //                   accumulators with a pack and a movmatrix transpose.
 // No shared memory and no block barrier in the key loop: every warp walks its own steps of 32 keys with its own online
 // softmax, the next 16 keys' loads are issued before this 16's arithmetic, and the warps merge once at the end.  P is
-// carried as three bf16 terms (24 significant bits), so that the tensor cores see what fp32 arithmetic would.
+// carried as three bf16 terms (24 significant bits), so that the tensor cores see what fp32 arithmetic would.  The rounded terms, and the
+// rows that stand in for padding, make NaN of an infinite value; a warp whose outputs hold a NaN walks its keys once more with
+// terms that are all positive and with zeros in place of padding, which leaves infinities as they are.  (Those terms for every
+// warp: 220 -> 242 us at 300 tokens x 8 kv heads x 2048 keys.)
 // With few (token, kv head) pairs a cluster of CTAs splits the keys of one pair and merges through distributed shared memory.
 //
 // Loads are bound by L1's tag stage, one 128-byte line a cycle: with 16-byte loads four lanes touch half a line of each key row
 // (347 us at 777 tokens x 4 kv heads x 2048 keys, L1 at 96 %); 32-byte loads touch whole lines.
 // Measured (B200, 128 / 128 dims): 777 tokens x 32 heads in 4 groups x 2048 keys 5785 -> 271 us = 12.0 TB/s out of L2 (kernel on
 // the fp32 ALUs before); 256 tokens x 8 heads x 256 keys 180 -> 34 us.
+#include <type_traits>
+
 #include "janus_common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -135,7 +140,7 @@ sparse_attn_heads_kernel(const AhParams p) {
         return i < p.k ? __ldg(my_idx + i) : -1;
     };
     // Element offset of the lane's key row.  A padding slot (or a token without a page) takes the row of the first valid lane, so
-    // that no load needs a predicate; its logit is masked, and a row that is attended anyway cannot add a NaN of its own.
+    // that no load needs a predicate; its logit is masked, and a row that is attended anyway adds no NaN but those of infinities.
     auto resolve = [&](int tok, uint32_t& mask) -> int64_t {
         int64_t off = 0;
         bool valid = false;
@@ -168,99 +173,129 @@ sparse_attn_heads_kernel(const AhParams p) {
     };
 
     float o[VB][VE / 2][4];               // [block][dims VE g + 2j, VE g + 2j + 1][heads 2t, 2t+1 of either dim]
+    float m_ref[2], l_sum[2];             // heads 2t, 2t + 1 (l: this lane's keys only)
+    auto walk = [&](auto keep_infinities) {
+        constexpr bool KEEP_INF = decltype(keep_infinities)::value;
+#pragma unroll
+        for (int b = 0; b < VB; ++b)
+#pragma unroll
+            for (int j = 0; j < VE / 2; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) o[b][j][e] = 0.f;
+        m_ref[0] = m_ref[1] = neg_inf;
+        l_sum[0] = l_sum[1] = 0.f;
+
+        int s = static_cast<int>(split) * WARPS + warp;
+        uint32_t mask = 0u;
+        int64_t off = resolve(s < n_steps ? load_raw(s) : -1, mask);
+        int raw_next = s + stride < n_steps ? load_raw(s + stride) : -1;
+        if (mask != 0u) load_k(off, 0);
+        for (; s < n_steps; s += stride) {
+            uint32_t mask_next;
+            const int64_t off_next = resolve(raw_next, mask_next);
+            raw_next = s + 2 * stride < n_steps ? load_raw(s + 2 * stride) : -1;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (mask != 0u) {
+                    uint32_t vf[4][VB][VE / 2];      // rows 2t, 2t+1, 2t+8, 2t+9 of these 16 keys
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const uint16_t* src = p.v_pool + __shfl_sync(0xffffffffu, off, 16 * u + 2 * t4 + (r & 1) + 8 * (r >> 1)) + g * VE;
+#pragma unroll
+                        for (int b = 0; b < VB; ++b) ah_load(vf[r][b], src + b * 8 * VE);
+                    }
+                    float sc[4] = {0.f, 0.f, 0.f, 0.f};      // keys g, g + 8 x heads 2t, 2t+1
+#pragma unroll
+                    for (int c = 0; c < KB; ++c)
+#pragma unroll
+                        for (int e = 0; e < KE / 2; e += 2)
+                            ah_mma(sc, kf[0][c][e], kf[1][c][e], kf[0][c][e + 1], kf[1][c][e + 1], qf[c][e], qf[c][e + 1]);
+                    if (u == 0) load_k(off, 1);
+                    else if (mask_next != 0u) load_k(off_next, 0);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) sc[e] *= p.scale_log2e;
+                    const uint32_t mk = mask >> (16 * u);
+                    if ((mk & 0xffffu) != 0xffffu) {
+                        if (((mk >> g) & 1u) == 0u) sc[0] = sc[1] = neg_inf;
+                        if (((mk >> (g + 8)) & 1u) == 0u) sc[2] = sc[3] = neg_inf;
+                        if constexpr (KEEP_INF) {
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) {
+                                if (((mk >> (2 * t4 + (r & 1) + 8 * (r >> 1))) & 1u) != 0u) continue;
+#pragma unroll
+                                for (int b = 0; b < VB; ++b)
+#pragma unroll
+                                    for (int j = 0; j < VE / 2; ++j) vf[r][b][j] = 0u;
+                            }
+                        }
+                    }
+                    // the reference maximum moves only when a key exceeds it by more than 2^8 (the sums are fp32)
+                    const float mx0 = fmaxf(sc[0], sc[2]), mx1 = fmaxf(sc[1], sc[3]);
+                    if (__any_sync(0xffffffffu, mx0 > m_ref[0] + 8.f || mx1 > m_ref[1] + 8.f)) {
+                        float mx[2] = {mx0, mx1};
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                            for (int d = 4; d < 32; d <<= 1) mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], d));
+                            const float m_new = fmaxf(m_ref[h], mx[h]);
+                            const float corr = m_ref[h] == neg_inf ? 1.f : ah_exp2(m_ref[h] - m_new);   // nothing accumulated yet: nothing to scale
+                            m_ref[h] = m_new;
+                            l_sum[h] *= corr;
+#pragma unroll
+                            for (int b = 0; b < VB; ++b)
+#pragma unroll
+                                for (int j = 0; j < VE / 2; ++j) { o[b][j][h] *= corr; o[b][j][2 + h] *= corr; }
+                        }
+                    }
+                    const float nm0 = m_ref[0] == neg_inf ? 0.f : m_ref[0], nm1 = m_ref[1] == neg_inf ? 0.f : m_ref[1];
+                    float pr[4] = {ah_exp2(sc[0] - nm0), ah_exp2(sc[1] - nm1), ah_exp2(sc[2] - nm0), ah_exp2(sc[3] - nm1)};
+                    l_sum[0] += pr[0] + pr[2];
+                    l_sum[1] += pr[1] + pr[3];
+                    // P = three bf16 terms; each becomes the B fragment (head g, keys 2t, 2t+1 | 2t+8, 2t+9)
+                    uint32_t pb[3][2];
+#pragma unroll
+                    for (int term = 0; term < 3; ++term) {
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            uint32_t bits;
+                            if constexpr (KEEP_INF) {      // the largest bf16 below P, the largest below the rest, and what is left: eight bits
+                                const int below = term < 2 ? 1 : 0;
+                                bits = __byte_perm(max(__float_as_int(pr[2 * r]) - below, 0), max(__float_as_int(pr[2 * r + 1]) - below, 0), 0x7632);
+                            } else {
+                                const __nv_bfloat162 v = __floats2bfloat162_rn(pr[2 * r], pr[2 * r + 1]);
+                                bits = *reinterpret_cast<const uint32_t*>(&v);
+                            }
+                            pb[term][r] = ah_transpose(bits);
+                            pr[2 * r] -= __uint_as_float(bits << 16);
+                            pr[2 * r + 1] -= __uint_as_float(bits & 0xffff0000u);
+                        }
+                    }
+#pragma unroll
+                    for (int b = 0; b < VB; ++b)
+#pragma unroll
+                        for (int j = 0; j < VE / 2; ++j) {
+                            const uint32_t a0 = __byte_perm(vf[0][b][j], vf[1][b][j], 0x5410), a1 = __byte_perm(vf[0][b][j], vf[1][b][j], 0x7632);
+                            const uint32_t a2 = __byte_perm(vf[2][b][j], vf[3][b][j], 0x5410), a3 = __byte_perm(vf[2][b][j], vf[3][b][j], 0x7632);
+#pragma unroll
+                            for (int term = 2; term >= 0; --term) ah_mma(o[b][j], a0, a1, a2, a3, pb[term][0], pb[term][1]);
+                        }
+                } else if (u == 1 && mask_next != 0u) {
+                    load_k(off_next, 0);
+                }
+            }
+            mask = mask_next;
+            off = off_next;
+        }
+    };
+    walk(std::false_type{});
+    bool has_nan = false;
 #pragma unroll
     for (int b = 0; b < VB; ++b)
 #pragma unroll
         for (int j = 0; j < VE / 2; ++j)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) o[b][j][e] = 0.f;
-    float m_ref[2] = {neg_inf, neg_inf}, l_sum[2] = {0.f, 0.f};      // heads 2t, 2t + 1 (l: this lane's keys only)
-
-    int s = static_cast<int>(split) * WARPS + warp;
-    uint32_t mask = 0u;
-    int64_t off = resolve(s < n_steps ? load_raw(s) : -1, mask);
-    int raw_next = s + stride < n_steps ? load_raw(s + stride) : -1;
-    if (mask != 0u) load_k(off, 0);
-    for (; s < n_steps; s += stride) {
-        uint32_t mask_next;
-        const int64_t off_next = resolve(raw_next, mask_next);
-        raw_next = s + 2 * stride < n_steps ? load_raw(s + 2 * stride) : -1;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (mask != 0u) {
-                uint32_t vf[4][VB][VE / 2];      // rows 2t, 2t+1, 2t+8, 2t+9 of these 16 keys
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const uint16_t* src = p.v_pool + __shfl_sync(0xffffffffu, off, 16 * u + 2 * t4 + (r & 1) + 8 * (r >> 1)) + g * VE;
-#pragma unroll
-                    for (int b = 0; b < VB; ++b) ah_load(vf[r][b], src + b * 8 * VE);
-                }
-                float sc[4] = {0.f, 0.f, 0.f, 0.f};      // keys g, g + 8 x heads 2t, 2t+1
-#pragma unroll
-                for (int c = 0; c < KB; ++c)
-#pragma unroll
-                    for (int e = 0; e < KE / 2; e += 2)
-                        ah_mma(sc, kf[0][c][e], kf[1][c][e], kf[0][c][e + 1], kf[1][c][e + 1], qf[c][e], qf[c][e + 1]);
-                if (u == 0) load_k(off, 1);
-                else if (mask_next != 0u) load_k(off_next, 0);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) sc[e] *= p.scale_log2e;
-                const uint32_t mk = mask >> (16 * u);
-                if ((mk & 0xffffu) != 0xffffu) {
-                    if (((mk >> g) & 1u) == 0u) sc[0] = sc[1] = neg_inf;
-                    if (((mk >> (g + 8)) & 1u) == 0u) sc[2] = sc[3] = neg_inf;
-                }
-                // the reference maximum moves only when a key exceeds it by more than 2^8 (the sums are fp32)
-                const float mx0 = fmaxf(sc[0], sc[2]), mx1 = fmaxf(sc[1], sc[3]);
-                if (__any_sync(0xffffffffu, mx0 > m_ref[0] + 8.f || mx1 > m_ref[1] + 8.f)) {
-                    float mx[2] = {mx0, mx1};
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                        for (int d = 4; d < 32; d <<= 1) mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], d));
-                        const float m_new = fmaxf(m_ref[h], mx[h]);
-                        const float corr = m_ref[h] == neg_inf ? 1.f : ah_exp2(m_ref[h] - m_new);   // nothing accumulated yet: nothing to scale
-                        m_ref[h] = m_new;
-                        l_sum[h] *= corr;
-#pragma unroll
-                        for (int b = 0; b < VB; ++b)
-#pragma unroll
-                            for (int j = 0; j < VE / 2; ++j) { o[b][j][h] *= corr; o[b][j][2 + h] *= corr; }
-                    }
-                }
-                const float nm0 = m_ref[0] == neg_inf ? 0.f : m_ref[0], nm1 = m_ref[1] == neg_inf ? 0.f : m_ref[1];
-                float pr[4] = {ah_exp2(sc[0] - nm0), ah_exp2(sc[1] - nm1), ah_exp2(sc[2] - nm0), ah_exp2(sc[3] - nm1)};
-                l_sum[0] += pr[0] + pr[2];
-                l_sum[1] += pr[1] + pr[3];
-                // P = three bf16 terms; each becomes the B fragment (head g, keys 2t, 2t+1 | 2t+8, 2t+9)
-                uint32_t pb[3][2];
-#pragma unroll
-                for (int term = 0; term < 3; ++term) {
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const __nv_bfloat162 v = __floats2bfloat162_rn(pr[2 * r], pr[2 * r + 1]);
-                        const uint32_t bits = *reinterpret_cast<const uint32_t*>(&v);
-                        pb[term][r] = ah_transpose(bits);
-                        pr[2 * r] -= __uint_as_float(bits << 16);
-                        pr[2 * r + 1] -= __uint_as_float(bits & 0xffff0000u);
-                    }
-                }
-#pragma unroll
-                for (int b = 0; b < VB; ++b)
-#pragma unroll
-                    for (int j = 0; j < VE / 2; ++j) {
-                        const uint32_t a0 = __byte_perm(vf[0][b][j], vf[1][b][j], 0x5410), a1 = __byte_perm(vf[0][b][j], vf[1][b][j], 0x7632);
-                        const uint32_t a2 = __byte_perm(vf[2][b][j], vf[3][b][j], 0x5410), a3 = __byte_perm(vf[2][b][j], vf[3][b][j], 0x7632);
-#pragma unroll
-                        for (int term = 2; term >= 0; --term) ah_mma(o[b][j], a0, a1, a2, a3, pb[term][0], pb[term][1]);
-                    }
-            } else if (u == 1 && mask_next != 0u) {
-                load_k(off_next, 0);
-            }
-        }
-        mask = mask_next;
-        off = off_next;
-    }
+            for (int e = 0; e < 4; ++e) has_nan = has_nan || isnan(o[b][j][e]);
+    if (__any_sync(0xffffffffu, has_nan)) walk(std::true_type{});
 
     // ---- merge: the warps of the CTA, then the CTAs of the cluster
 #pragma unroll

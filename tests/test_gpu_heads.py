@@ -60,3 +60,24 @@ def test_heads_kernel_matches_oracle(M, n_kv, group, d_qk, d_v, k, shift):
     assert np.array_equal(np.isfinite(got), fin)
     # logits are fp32 sums of d_qk exact products (relative error d_qk 2^-24 of their absolute sum, below 1e-4 here)
     assert np.all(np.abs(got[fin] - ref_l[fin]) <= 1e-4 * (1 + np.abs(ref_l[fin])))
+
+
+@pytest.mark.parametrize("M,n_kv,group,d_qk,d_v,k", [(3, 2, 4, 128, 128, 1), (5, 4, 8, 64, 64, 37), (2, 1, 8, 192, 128, 2048), (300, 1, 1, 128, 64, 45)])
+def test_infinite_values_come_out_as_they_are(M, n_kv, group, d_qk, d_v, k):
+    """Every token's value is +Inf in one dim, -Inf in another and finite elsewhere: so are the outputs, whatever padding is near."""
+    rng = np.random.default_rng(M + k)
+    H_q, page, S = n_kv * group, 16, 2500
+    n_log = (S + page - 1) // page
+    table = np.arange(n_log, dtype=np.int32)
+    kp, v = rng.standard_normal((n_log, page, n_kv, max(d_qk, d_v))).astype(np.float32) / 4, rng.standard_normal((n_log, page, n_kv, max(d_qk, d_v))).astype(np.float32)
+    v[..., 5], v[..., d_v - 2] = np.inf, -np.inf
+    Q = W.to_bf16_bits(rng.standard_normal((M, H_q, d_qk)).astype(np.float32))
+    idx = np.stack([rng.permutation(S)[:k] for _ in range(M)]).astype(np.int32)
+    idx[(rng.random(idx.shape) < 0.3) & (np.arange(k) > 0)] = -1
+    out, _ = B.janus_sparse_attn_prefill(B.to_device(Q, "bf16"), B.to_device(W.to_bf16_bits(kp), "bf16"), B.to_device(W.to_bf16_bits(v), "bf16"), B.to_device(idx, "i32"),
+                                         page_table=B.to_device(table, "i32"), page_size=page, softmax_scale=d_qk ** -0.5, d_v=d_v)
+    B.check_dev_status()
+    got = Hp.bf16_tensor_to_f64(out)
+    want = np.zeros(d_v)
+    want[5], want[d_v - 2] = np.inf, -np.inf
+    assert np.array_equal(np.where(np.isfinite(got), 0, got), np.broadcast_to(want, got.shape))
