@@ -17,9 +17,9 @@ __device__ __forceinline__ float load_elem(const void* base, int64_t i) {
 
 template <int DTYPE>
 __global__ void __launch_bounds__(IG_KEYS)
-indexer_generic_kernel(const void* __restrict__ q_idx, int64_t q_stride_tok, const void* __restrict__ k_idx, int64_t k_stride_tok,
-                       const float* __restrict__ w, const float* __restrict__ q_scale, int64_t q_scale_stride_tok,
-                       const float* __restrict__ k_scale, const float* __restrict__ row_bias, const float* __restrict__ col_bias,
+indexer_generic_kernel(const void* q_idx, int64_t q_stride_tok, const void* k_idx, int64_t k_stride_tok,
+                       const float* w, const float* q_scale, int64_t q_scale_stride_tok,
+                       const float* k_scale, const float* row_bias, const float* col_bias,
                        int M, int H, int D, int64_t n_keys, int64_t q_pos0, int causal, float* __restrict__ scores, int64_t ld) {
     grid_launch_next();
     grid_wait();

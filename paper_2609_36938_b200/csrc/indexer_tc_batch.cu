@@ -99,7 +99,7 @@ struct TbSegments {
             if (!first) { ++b; tb = 0; }
             first = false;
             if (MULTI && b >= p.n_sessions) { left = 0; return false; }
-            const TbSession s = tb_session<KEYS>(__ldg(p.key_offsets + b), __ldg(p.key_offsets + b + 1), p.n_keys, p.max_tiles);
+            const TbSession s = tb_session<KEYS>(ld_input(p.key_offsets + b), ld_input(p.key_offsets + b + 1), p.n_keys, p.max_tiles);
             key_base = s.base;
             key_count = s.count;
             tiles = s.tiles;
@@ -154,7 +154,7 @@ indexer_tc_batch_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
     if constexpr (!MULTI) {
         b0 = blockIdx.y;
         tile0 = blockIdx.x * p.tiles_per_cta;
-        const int64_t key_begin = __ldg(p.key_offsets + b0), key_end = __ldg(p.key_offsets + b0 + 1);
+        const int64_t key_begin = ld_input(p.key_offsets + b0), key_end = ld_input(p.key_offsets + b0 + 1);
         load_weights(b0, threadIdx.x);                     // (while the offsets are on their way)
         const TbSession ses = tb_session<KEYS>(key_begin, key_end, p.n_keys, p.max_tiles);
         if (ses.bad && tile0 == 0 && threadIdx.x == 0) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
@@ -171,7 +171,7 @@ indexer_tc_batch_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
                 const int b = r0 + threadIdx.x;
                 int tiles = 0;
                 if (b < p.n_sessions) {
-                    const TbSession ses = tb_session<KEYS>(__ldg(p.key_offsets + b), __ldg(p.key_offsets + b + 1), p.n_keys, p.max_tiles);
+                    const TbSession ses = tb_session<KEYS>(ld_input(p.key_offsets + b), ld_input(p.key_offsets + b + 1), p.n_keys, p.max_tiles);
                     if (ses.bad && pass == 1 && blockIdx.x == 0) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
                     tiles = ses.tiles;
                 }

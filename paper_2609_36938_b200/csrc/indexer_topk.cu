@@ -90,8 +90,8 @@ __device__ __forceinline__ int64_t sample_position(int j, int64_t p0) {
     return 8 * ((static_cast<int64_t>(j >> 3) * (n8 - 1)) / 511) + (j & 7);
 }
 
-__global__ void ft_gather_sample_kernel(const unsigned char* __restrict__ k_idx, int64_t k_row_bytes, int row_vecs, const float* __restrict__ k_scale,
-                                        const float* __restrict__ col_bias, int64_t p0, uint4* __restrict__ k_sample, float* __restrict__ ks_sample,
+__global__ void ft_gather_sample_kernel(const unsigned char* k_idx, int64_t k_row_bytes, int row_vecs, const float* k_scale,
+                                        const float* col_bias, int64_t p0, uint4* __restrict__ k_sample, float* __restrict__ ks_sample,
                                         float* __restrict__ cb_sample) {
     grid_launch_next();
     grid_wait();
@@ -99,7 +99,7 @@ __global__ void ft_gather_sample_kernel(const unsigned char* __restrict__ k_idx,
     if (i >= FT_NS * row_vecs) return;
     const int j = i / row_vecs, v = i - j * row_vecs;
     const int64_t pos = sample_position(j, p0);
-    k_sample[i] = __ldg(reinterpret_cast<const uint4*>(k_idx + pos * k_row_bytes) + v);
+    k_sample[i] = ld_input(reinterpret_cast<const uint4*>(k_idx + pos * k_row_bytes) + v);
     if (v == 0) {
         if (k_scale != nullptr) ks_sample[j] = k_scale[pos];
         if (col_bias != nullptr) cb_sample[j] = col_bias[pos];
@@ -108,7 +108,7 @@ __global__ void ft_gather_sample_kernel(const unsigned char* __restrict__ k_idx,
 
 // ---- 2. per-row threshold from the sample ----------------------------------------------------------------------------------
 __global__ void __launch_bounds__(TK_THREADS)
-ft_threshold_kernel(const float* __restrict__ sc_sample, int M, int64_t n_keys, int64_t q_pos0, int causal, int k, int cap, float* __restrict__ thr,
+ft_threshold_kernel(const float* sc_sample, int M, int64_t n_keys, int64_t q_pos0, int causal, int k, int cap, float* __restrict__ thr,
                     int32_t* __restrict__ cand_cnt, int32_t* __restrict__ fb_count) {
     grid_launch_next();
     grid_wait();
@@ -145,7 +145,7 @@ ft_threshold_kernel(const float* __restrict__ sc_sample, int M, int64_t n_keys, 
 // ---- 4. exact selection among a row's candidates ------------------------------------------------------------------------------
 template <int CAP>
 __global__ void __launch_bounds__(TK_THREADS)
-ft_select_kernel(const int2* __restrict__ cand, const int32_t* __restrict__ cand_cnt, int M, int64_t n_keys, int64_t q_pos0, int causal, int k,
+ft_select_kernel(const int2* cand, const int32_t* cand_cnt, int M, int64_t n_keys, int64_t q_pos0, int causal, int k,
                  int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth, int32_t* __restrict__ fb_count,
                  int32_t* __restrict__ fb_rows) {
     grid_launch_next();
@@ -207,11 +207,11 @@ __device__ __forceinline__ void decode16(const uint4& u, float (&v)[16], int& n)
 
 template <int DTYPE>
 __global__ void __launch_bounds__(TK_THREADS)
-ft_fallback_kernel(const unsigned char* __restrict__ q_idx, const unsigned char* __restrict__ k_idx, int64_t k_row_bytes, const float* __restrict__ w,
-                   const float* __restrict__ q_scale, int64_t q_scale_stride_tok, const float* __restrict__ k_scale,
-                   const float* __restrict__ row_bias, const float* __restrict__ col_bias, int M, int H, int D, int64_t n_keys, int64_t q_pos0,
+ft_fallback_kernel(const unsigned char* q_idx, const unsigned char* k_idx, int64_t k_row_bytes, const float* w,
+                   const float* q_scale, int64_t q_scale_stride_tok, const float* k_scale,
+                   const float* row_bias, const float* col_bias, int M, int H, int D, int64_t n_keys, int64_t q_pos0,
                    int causal, int k, int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth,
-                   const int32_t* __restrict__ fb_count, const int32_t* __restrict__ fb_rows, float* __restrict__ fb_buf, int64_t ld) {
+                   const int32_t* fb_count, const int32_t* fb_rows, float* __restrict__ fb_buf, int64_t ld) {
     grid_launch_next();
     grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -245,7 +245,7 @@ ft_fallback_kernel(const unsigned char* __restrict__ q_idx, const unsigned char*
                 for (int v = 0; d < D; ++v) {
                     float kv[16];
                     int nv;
-                    decode16<DTYPE>(__ldg(krow + v), kv, nv);
+                    decode16<DTYPE>(ld_input(krow + v), kv, nv);
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
                         if (e < nv) {

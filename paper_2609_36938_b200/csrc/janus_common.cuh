@@ -51,11 +51,16 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // run up to grid_wait(), while the predecessor still runs.  The order of memory accesses stays that of the stream, because every
 // kernel waits, on every path, before its first access to global memory; grid_wait() returns when the predecessor has completed
 // and its writes are visible, and the predecessor has itself waited for what came before.  Tensor memory is allocated after
-// grid_wait(), so that no CTA holds it while it waits.  A short kernel lets its successor in at once with grid_launch_next(); the
+// grid_wait(), so that no CTA holds it while it waits.  Inputs are read with ordinary loads (ld_input, __ldcg, __ldcs, asynchronous
+// copies), never with read-only ones (__ldg, ld.global.nc, or const __restrict__ parameters, which the compiler may turn into them): those
+// require memory that nobody writes while the kernel exists, and it exists while its predecessor still writes.  A short kernel lets its successor in at once with grid_launch_next(); the
 // indexer and the attention of many tokens do not, because CTAs that wait beside them made them 1 % slower.  One-session decode step
 // 51.2 -> 44.2 us, short message 59.9 -> 52.8, sharded prediction 1.70 -> 1.66 ms; the large passes are unchanged.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class T>
+__device__ __forceinline__ T ld_input(const T* p) { return __ldca(p); }
 
 template <class Kernel, class... Args>
 inline cudaError_t launch_kernel(Kernel kernel, dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster, const Args&... args) {

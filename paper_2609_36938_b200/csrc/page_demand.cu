@@ -94,16 +94,16 @@ page_mark_kernel(const PdParams p, int n_log_words) {
     for (; i + 3 * stride < n_vec; i += 4 * stride) {
         int4 v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldg(idx4 + i + u * stride);
+        for (int u = 0; u < 4; ++u) v[u] = ld_input(idx4 + i + u * stride);
 #pragma unroll
         for (int u = 0; u < 4; ++u) mark4(v[u]);
     }
-    for (; i < n_vec; i += stride) mark4(__ldg(idx4 + i));
+    for (; i < n_vec; i += stride) mark4(ld_input(idx4 + i));
     if (blockIdx.x == 0 && threadIdx.x < (p.n_idx & 3)) mark4(make_int4(p.idx[(n_vec << 2) + threadIdx.x], -1, -1, -1));
     __syncthreads();
     for (int lp = threadIdx.x; lp < n_log_words * 32; lp += MARK_THREADS) {
         if (((lbm[lp >> 5] >> (lp & 31)) & 1u) == 0u) continue;
-        const int32_t q = __ldg(p.page_table + lp);
+        const int32_t q = ld_input(p.page_table + lp);
         if (q < 0 || q >= p.n_phys_pages) bad = true;
         else atomicOr(pbm + (q >> 5), 1u << (q & 31));
     }
@@ -116,11 +116,11 @@ page_mark_kernel(const PdParams p, int n_log_words) {
 }
 
 // Physical page of a token, -1 for none (padding, past the limit) and after reporting what is out of range.
-__device__ __forceinline__ int32_t page_of_token(int s, int64_t limit, const PageDiv& page, const int32_t* __restrict__ table, int64_t n_logical,
+__device__ __forceinline__ int32_t page_of_token(int s, int64_t limit, const PageDiv& page, const int32_t* table, int64_t n_logical,
                                                  int64_t n_phys, bool& bad) {
     if (s < 0 || s >= limit) return -1;
     const int64_t lp = page(s);
-    const int32_t q = lp < n_logical ? __ldg(table + lp) : -1;
+    const int32_t q = lp < n_logical ? ld_input(table + lp) : -1;
     if (q < 0 || q >= n_phys) { bad = true; return -1; }
     return q;
 }
@@ -137,12 +137,12 @@ page_mark_global_kernel(const PdParams p) {
         const int32_t* table = p.page_table;
         int64_t n_log = p.n_logical_pages, limit = p.demand_limit;
         if (MODE == PD_MARK_ROWS) {
-            const int64_t r = e / p.k, off = __ldg(p.table_offsets + r);
-            n_log = off < 0 ? 0 : __ldg(p.table_offsets + r + 1) - off;       // a table that starts before the array has no pages
+            const int64_t r = e / p.k, off = ld_input(p.table_offsets + r);
+            n_log = off < 0 ? 0 : ld_input(p.table_offsets + r + 1) - off;       // a table that starts before the array has no pages
             table += off < 0 ? 0 : off;
-            limit = __ldg(p.demand_limits + r);
+            limit = ld_input(p.demand_limits + r);
         }
-        const int32_t q = page_of_token(__ldg(p.idx + e), limit, page, table, n_log, p.n_phys_pages, bad);
+        const int32_t q = page_of_token(ld_input(p.idx + e), limit, page, table, n_log, p.n_phys_pages, bad);
         if (q < 0) continue;
         const uint32_t bit = 1u << (q & 31);
         if ((__ldcg(p.bitmap + (q >> 5)) & bit) == 0u) atomicOr(p.bitmap + (q >> 5), bit);
@@ -220,7 +220,7 @@ page_demand_kernel(const PdParams p) {
             int32_t q[U];
             const int32_t* entry[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) s[u] = base + u * stride < n_idx ? __ldg(p.idx + base + u * stride) : -1;
+            for (int u = 0; u < U; ++u) s[u] = base + u * stride < n_idx ? ld_input(p.idx + base + u * stride) : -1;
             if constexpr (MODE == PD_MARK_ROWS) {
                 int64_t off[U], end[U], limit[U];
 #pragma unroll
@@ -228,9 +228,9 @@ page_demand_kernel(const PdParams p) {
                     off[u] = end[u] = limit[u] = 0;
                     if (base + u * stride >= n_idx) continue;
                     const int r = (base + u * stride) / p.k;
-                    off[u] = __ldg(p.table_offsets + r);
-                    end[u] = __ldg(p.table_offsets + r + 1);
-                    limit[u] = __ldg(p.demand_limits + r);
+                    off[u] = ld_input(p.table_offsets + r);
+                    end[u] = ld_input(p.table_offsets + r + 1);
+                    limit[u] = ld_input(p.demand_limits + r);
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
@@ -253,7 +253,7 @@ page_demand_kernel(const PdParams p) {
                 }
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) q[u] = entry[u] != nullptr ? __ldg(entry[u]) : -1;
+            for (int u = 0; u < U; ++u) q[u] = entry[u] != nullptr ? ld_input(entry[u]) : -1;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 if (entry[u] == nullptr) continue;
@@ -397,7 +397,7 @@ page_demand_kernel(const PdParams p) {
     }
 }
 
-__global__ void page_union_kernel(uint32_t* __restrict__ dst, const uint32_t* __restrict__ src, int n_words) {
+__global__ void page_union_kernel(uint32_t* __restrict__ dst, const uint32_t* src, int n_words) {
     grid_launch_next();
     grid_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_words; i += gridDim.x * blockDim.x) dst[i] |= src[i];

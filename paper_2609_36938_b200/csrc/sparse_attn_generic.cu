@@ -13,10 +13,10 @@ constexpr int AG_KT = 32;  // keys per tile
 
 template <int G>
 __global__ void __launch_bounds__(AG_THREADS)
-sparse_attn_generic_kernel(const uint16_t* __restrict__ q, int M, int H_q, int d_qk, const uint16_t* __restrict__ k_pool,
-                           const uint16_t* __restrict__ v_pool, int64_t page_stride, int64_t tok_stride, int64_t head_stride,
-                           int n_kv_heads, int d_v, const int32_t* __restrict__ idx, int k, int page_size,
-                           const int32_t* __restrict__ page_table, int64_t n_logical_pages, const int64_t* __restrict__ table_offsets,
+sparse_attn_generic_kernel(const uint16_t* q, int M, int H_q, int d_qk, const uint16_t* k_pool,
+                           const uint16_t* v_pool, int64_t page_stride, int64_t tok_stride, int64_t head_stride,
+                           int n_kv_heads, int d_v, const int32_t* idx, int k, int page_size,
+                           const int32_t* page_table, int64_t n_logical_pages, const int64_t* table_offsets,
                            float softmax_scale, uint16_t* __restrict__ out, float* __restrict__ lse, int32_t* dev_status) {
     grid_launch_next();
     grid_wait();
@@ -66,7 +66,7 @@ sparse_attn_generic_kernel(const uint16_t* __restrict__ q, int M, int H_q, int d
         if (tid < AG_KT) {
             int s = base + tid < k ? my_idx[base + tid] : -1;
             // a token beyond the page table, or a negative physical page id in it, is reported and skipped
-            if (s >= 0 && (s / page_size >= n_logical_pages || __ldg(page_table + s / page_size) < 0)) { report(dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE); s = -1; }
+            if (s >= 0 && (s / page_size >= n_logical_pages || ld_input(page_table + s / page_size) < 0)) { report(dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE); s = -1; }
             srow[tid] = s;
         }
         __syncthreads();
@@ -74,15 +74,15 @@ sparse_attn_generic_kernel(const uint16_t* __restrict__ q, int M, int H_q, int d
         for (int r = warp; r < AG_KT; r += AG_THREADS / 32) {
             const int s = srow[r];
             if (s < 0) continue;
-            const int64_t off = static_cast<int64_t>(__ldg(page_table + s / page_size)) * page_stride +
+            const int64_t off = static_cast<int64_t>(ld_input(page_table + s / page_size)) * page_stride +
                                 static_cast<int64_t>(s % page_size) * tok_stride + static_cast<int64_t>(hk) * head_stride;
             const uint4* src = reinterpret_cast<const uint4*>(k_pool + off);
             uint4* dst = reinterpret_cast<uint4*>(ks + r * kpad);
-            for (int c = lane; c < d_qk / 8; c += 32) dst[c] = __ldg(src + c);
+            for (int c = lane; c < d_qk / 8; c += 32) dst[c] = ld_input(src + c);
             if (!v_alias) {
                 const uint4* vsrc = reinterpret_cast<const uint4*>(v_pool + off);
                 uint4* vdst = reinterpret_cast<uint4*>(vs + r * vpad);
-                for (int c = lane; c < d_v / 8; c += 32) vdst[c] = __ldg(vsrc + c);
+                for (int c = lane; c < d_v / 8; c += 32) vdst[c] = ld_input(vsrc + c);
             }
         }
         __syncthreads();

@@ -68,10 +68,10 @@ __device__ __forceinline__ float ah_exp2(float x) {
 }
 // One load of 16 or 32 bytes; rows are used once and not kept in L1.
 __device__ __forceinline__ void ah_load(uint32_t (&v)[4], const uint16_t* p) {
-    asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(p));
 }
 __device__ __forceinline__ void ah_load(uint32_t (&v)[8], const uint16_t* p) {
-    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
                  : "l"(p));
 }
@@ -113,8 +113,8 @@ sparse_attn_heads_kernel(const AhParams p) {
     const int32_t* table = p.page_table;
     int64_t n_pages = p.n_logical_pages;
     if (p.table_offsets != nullptr) {
-        const int64_t tbl = __ldg(p.table_offsets + row);
-        n_pages = __ldg(p.table_offsets + row + 1) - tbl;
+        const int64_t tbl = ld_input(p.table_offsets + row);
+        n_pages = ld_input(p.table_offsets + row + 1) - tbl;
         if (tbl < 0) n_pages = 0;         // a table that starts before the array: every selected token is reported and skipped
         else table += tbl;
     }
@@ -126,7 +126,7 @@ sparse_attn_heads_kernel(const AhParams p) {
         for (int c = 0; c < KB; ++c)
 #pragma unroll
             for (int v = 0; v < KE / 8; ++v) {
-                uint4 u = __ldg(reinterpret_cast<const uint4*>(qrow + c * 4 * KE + v * 8));
+                uint4 u = ld_input(reinterpret_cast<const uint4*>(qrow + c * 4 * KE + v * 8));
                 if (g >= n_heads) u = make_uint4(0u, 0u, 0u, 0u);
                 qf[c][4 * v] = u.x; qf[c][4 * v + 1] = u.y; qf[c][4 * v + 2] = u.z; qf[c][4 * v + 3] = u.w;
             }
@@ -137,7 +137,7 @@ sparse_attn_heads_kernel(const AhParams p) {
     const int stride = WARPS * static_cast<int>(n_split);
     auto load_raw = [&](int s) -> int {
         const int i = s * AH_STEP + lane;
-        return i < p.k ? __ldg(my_idx + i) : -1;
+        return i < p.k ? ld_input(my_idx + i) : -1;
     };
     // Element offset of the lane's key row.  A padding slot (or a token without a page) takes the row of the first valid lane, so
     // that no load needs a predicate; its logit is masked, and a row that is attended anyway adds no NaN but those of infinities.
@@ -147,7 +147,7 @@ sparse_attn_heads_kernel(const AhParams p) {
         if (tok >= 0) {
             const int64_t lp = p.page_shift >= 0 ? (tok >> p.page_shift) : (tok / p.page_size);
             const int within = p.page_shift >= 0 ? (tok & (p.page_size - 1)) : (tok % p.page_size);
-            const int32_t phys = lp < n_pages ? __ldg(table + lp) : -1;
+            const int32_t phys = lp < n_pages ? ld_input(table + lp) : -1;
             if (phys < 0) {
                 report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
             } else {

@@ -360,11 +360,11 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
             const int slot = (2 * tile0 + gh - it * n_half) * LP_HALF + lane;
             const int64_t t_row = cid + it * n_clusters;
             if (p.table_offsets != nullptr) {                  // every query row has a page table of its own (a batch of sessions)
-                tbl_nxt = __ldg(p.table_offsets + t_row);
-                tbl_n_nxt = __ldg(p.table_offsets + t_row + 1) - tbl_nxt;
+                tbl_nxt = ld_input(p.table_offsets + t_row);
+                tbl_n_nxt = ld_input(p.table_offsets + t_row + 1) - tbl_nxt;
                 if (tbl_nxt < 0) tbl_n_nxt = 0;                // a table that starts before the array: its tokens are reported and skipped
             }
-            return slot < p.k ? __ldg(p.idx + t_row * p.k + slot) : -1;
+            return slot < p.k ? ld_input(p.idx + t_row * p.k + slot) : -1;
         };
         auto resolve = [&](int s_tok, int64_t tbl, int64_t tbl_n, bool& valid) -> const unsigned char* {   // first owned byte of the row of token s_tok
             const unsigned char* ptr = reinterpret_cast<const unsigned char*>(p.pool) + seg_off;
@@ -372,7 +372,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
             if (s_tok >= 0) {
                 const int64_t lp = p.page_shift >= 0 ? (s_tok >> p.page_shift) : (s_tok / p.page_size);
                 const int within = p.page_shift >= 0 ? (s_tok & (p.page_size - 1)) : (s_tok % p.page_size);
-                const int32_t phys = lp < tbl_n ? __ldg(p.page_table + tbl + lp) : -1;
+                const int32_t phys = lp < tbl_n ? ld_input(p.page_table + tbl + lp) : -1;
                 if (phys < 0) {     // beyond the page table, or a negative physical page id in it
                     report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
                 } else {
@@ -446,7 +446,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
                 uint32_t r[32];
 #pragma unroll
                 for (int v = 0; v < 8; ++v) {
-                    const uint4 u = __ldg(src + a * 8 + v);
+                    const uint4 u = ld_input(src + a * 8 + v);
                     r[4 * v + 0] = u.x; r[4 * v + 1] = u.y; r[4 * v + 2] = u.z; r[4 * v + 3] = u.w;
                 }
                 tmem_st32_wait(lane_addr + LP_COL_Q + a * 32, r);

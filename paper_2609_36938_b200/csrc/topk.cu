@@ -25,7 +25,7 @@ constexpr int TK_CAP_SMALL = 5632;  // for rows whose candidate list is sure to 
 
 template <int CAP>
 __global__ void __launch_bounds__(TK_THREADS)
-topk_rows_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int k,
+topk_rows_kernel(const float* scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int k,
                  int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth) {
     grid_launch_next();
     grid_wait();
@@ -45,7 +45,7 @@ topk_rows_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_
 
 // Few rows: one cluster of CTAs per row.
 __global__ void __launch_bounds__(TK_THREADS)
-topk_rows_cluster_kernel(const float* __restrict__ scores, int64_t ld, int64_t n_keys, int64_t q_pos0, int causal, int k,
+topk_rows_cluster_kernel(const float* scores, int64_t ld, int64_t n_keys, int64_t q_pos0, int causal, int k,
                          int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth) {
     grid_launch_next();
     grid_wait();
@@ -61,7 +61,7 @@ topk_rows_cluster_kernel(const float* __restrict__ scores, int64_t ld, int64_t n
 // q_pos0 + t) may select the entries that hold a token at or before its position: entries 0 .. (q_pos0 + t) / entry_size.
 template <int CAP>
 __global__ void __launch_bounds__(TK_THREADS)
-topk_entries_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_entries, int64_t q_pos0, int entry_size, int k,
+topk_entries_kernel(const float* scores, int64_t ld, int M, int64_t n_entries, int64_t q_pos0, int entry_size, int k,
                     int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth) {
     grid_launch_next();
     grid_wait();
@@ -76,7 +76,7 @@ topk_entries_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t
 }
 
 // Token selection of an entry selection: slot e * E + j of row t = entry * E + j if that token is at or before q_pos0 + t.
-__global__ void entry_expand_kernel(const int32_t* __restrict__ idx_e, int M, int k_e, int entry_size, int64_t q_pos0,
+__global__ void entry_expand_kernel(const int32_t* idx_e, int M, int k_e, int entry_size, int64_t q_pos0,
                                     int32_t* __restrict__ idx_tok) {
     grid_launch_next();
     grid_wait();
@@ -85,7 +85,7 @@ __global__ void entry_expand_kernel(const int32_t* __restrict__ idx_e, int M, in
         const int64_t slot = i / entry_size;            // (t, e)
         const int j = static_cast<int>(i - slot * entry_size);
         const int64_t t = slot / k_e;
-        const int32_t ent = __ldg(idx_e + slot);
+        const int32_t ent = ld_input(idx_e + slot);
         const int64_t tok = static_cast<int64_t>(ent) * entry_size + j;
         idx_tok[i] = (ent >= 0 && tok <= q_pos0 + t) ? static_cast<int32_t>(tok) : -1;
     }
@@ -99,7 +99,7 @@ __global__ void entry_expand_kernel(const int32_t* __restrict__ idx_e, int M, in
 // a warp per entry (four 4-byte loads and a 64-bit division each), 19 us so; entries of 16 tokens 200 and 18.
 template <int ENTRY>
 __global__ void __launch_bounds__(256)
-entry_pool_vec_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int n_entries,
+entry_pool_vec_kernel(const float* scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int n_entries,
                       float* __restrict__ out, int64_t out_ld) {
     grid_launch_next();
     grid_wait();
@@ -141,7 +141,7 @@ entry_pool_vec_kernel(const float* __restrict__ scores, int64_t ld, int M, int64
 
 // Any entry size: one warp per (row, entry) strip, lanes read consecutive floats, a warp shuffle takes the maximum.
 __global__ void __launch_bounds__(256)
-entry_pool_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int entry_size,
+entry_pool_kernel(const float* scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int entry_size,
                   int64_t n_entries, float* __restrict__ out, int64_t out_ld) {
     grid_launch_next();
     grid_wait();
@@ -156,7 +156,7 @@ entry_pool_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n
         const int64_t b = a + entry_size < prefix ? a + entry_size : prefix;
         const float* row = scores + t * ld;
         float m = neg_inf;
-        for (int64_t s = a + lane; s < b; s += 32) m = fmaxf(m, __ldg(row + s));
+        for (int64_t s = a + lane; s < b; s += 32) m = fmaxf(m, ld_input(row + s));
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
         if (lane == 0) out[t * out_ld + e] = m;
@@ -167,7 +167,7 @@ entry_pool_kernel(const float* __restrict__ scores, int64_t ld, int M, int64_t n
 // up to the next row's start when row_lengths is NULL), every element visible.
 template <bool CLUSTER>
 __global__ void __launch_bounds__(TK_THREADS)
-topk_ragged_kernel(const float* __restrict__ scores, const int64_t* __restrict__ row_offsets, const int64_t* __restrict__ row_lengths, int k,
+topk_ragged_kernel(const float* scores, const int64_t* row_offsets, const int64_t* row_lengths, int k,
                    int32_t* __restrict__ idx, int32_t* __restrict__ count, float* __restrict__ kth, int32_t* dev_status) {
     grid_launch_next();
     grid_wait();

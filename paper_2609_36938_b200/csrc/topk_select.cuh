@@ -370,7 +370,7 @@ __device__ __forceinline__ int64_t sample_offset(int n) {
 // row's k-th value is expected.  Thread i reads 8 consecutive floats at an evenly spread, 32-byte aligned offset.  Every
 // thread of the CTA calls it; the result is uniform and depends on the row only.  False: no threshold is low enough.
 template <class Sh>
-__device__ __forceinline__ bool topk_sample(const float* __restrict__ row, int n, int k, uint32_t& thr, uint32_t& hi, Sh& sh) {
+__device__ __forceinline__ bool topk_sample(const float* row, int n, int k, uint32_t& thr, uint32_t& hi, Sh& sh) {
     const float expect = static_cast<float>(TK_SAMPLE) * static_cast<float>(k) / static_cast<float>(n);
     const int r = static_cast<int>(expect + 4.0f * sqrtf(expect) + 8.0f);
     if (r >= TK_SAMPLE) return false;
@@ -383,7 +383,7 @@ __device__ __forceinline__ bool topk_sample(const float* __restrict__ row, int n
 }
 
 // Four 16-byte groups of a thread: i, i + TK_THREADS, ..; past the end NaN, which no threshold lets in.
-__device__ __forceinline__ void load_groups(const float4* __restrict__ row4, int i, int f4_end, float4 (&x)[4]) {
+__device__ __forceinline__ void load_groups(const float4* row4, int i, int f4_end, float4 (&x)[4]) {
     if (i + 3 * TK_THREADS < f4_end) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) x[u] = __ldcs(row4 + i + u * TK_THREADS);
@@ -400,7 +400,7 @@ __device__ __forceinline__ void load_groups(const float4* __restrict__ row4, int
 // One streaming pass over the 16-byte groups [f4_begin, f4_end) of the row (and, with `tail`, the n % 4 elements after the
 // last whole group).
 template <class Sh>
-__device__ __forceinline__ void topk_stream(const float* __restrict__ row, int n, int f4_begin, int f4_end, bool tail, float thr_f, Sh& sh) {
+__device__ __forceinline__ void topk_stream(const float* row, int n, int f4_begin, int f4_end, bool tail, float thr_f, Sh& sh) {
     const int tid = threadIdx.x;
     const float4* row4 = reinterpret_cast<const float4*>(row);
     int i = f4_begin + tid;
@@ -427,7 +427,7 @@ __device__ __forceinline__ void topk_stream(const float* __restrict__ row, int n
 
 // A row of at most k elements: all of them, and the smallest value.
 template <class Sh>
-__device__ __noinline__ void topk_whole_row(const float* __restrict__ row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
+__device__ __noinline__ void topk_whole_row(const float* row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
                                float* __restrict__ kth, Sh& sh) {
     const int tid = threadIdx.x;
     for (int i = tid; i < k; i += TK_THREADS) out[i] = i < n ? i : -1;
@@ -443,7 +443,7 @@ __device__ __noinline__ void topk_whole_row(const float* __restrict__ row, int n
 
 // The exact selection over the row in global memory.
 template <class Sh>
-__device__ __noinline__ void topk_exact_row(const float* __restrict__ row, int n, int k, int32_t* __restrict__ out, float* __restrict__ kth, Sh& sh) {
+__device__ __noinline__ void topk_exact_row(const float* row, int n, int k, int32_t* __restrict__ out, float* __restrict__ kth, Sh& sh) {
     if (threadIdx.x == 0) { sh.out_pos = 0; sh.eq_taken = 0; }
     int n_eq;
     GlobalSource s{row, n};
@@ -458,8 +458,8 @@ __device__ __noinline__ void topk_exact_row(const float* __restrict__ row, int n
 // row's streaming pass is over, so the next sample does not start with a DRAM round trip.  (Requesting the head of the next
 // row as well, 96 to 512 KB, made the kernel slower: 0.49 -> 0.50 .. 0.58 ms at 4096 rows of 135168.)
 template <class Sh>
-__device__ __forceinline__ void topk_row(const float* __restrict__ row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
-                         float* __restrict__ kth, Sh& sh, const float* __restrict__ next_row = nullptr, int next_n = 0) {
+__device__ __forceinline__ void topk_row(const float* row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
+                         float* __restrict__ kth, Sh& sh, const float* next_row = nullptr, int next_n = 0) {
     const int tid = threadIdx.x;
     if (n <= k) {
         topk_whole_row(row, n, k, out, count, kth, sh);
@@ -514,7 +514,7 @@ __device__ __forceinline__ void topk_row(const float* __restrict__ row, int n, i
 // histogram, the histograms are added through distributed shared memory, every CTA emits its own keys above the k-th key's
 // bucket, and CTA 0 ranks the bucket's keys of all of them.
 template <class Sh>
-__device__ __forceinline__ void topk_row_cluster(const float* __restrict__ row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
+__device__ __forceinline__ void topk_row_cluster(const float* row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
                                  float* __restrict__ kth, Sh& sh) {
     using namespace ptx;
     const int tid = threadIdx.x, lane = tid & 31;
