@@ -7,7 +7,7 @@
 // a commit costs its issuing thread more than the tensor pipe needs for them.  Hence
 //   - the TMA and the MMA warp stay converged and one elected lane issues (in a branch on the lane number the addresses are not
 //     known to be uniform: 1300 cycles per 128 keys in the MMA warp, 660 in the TMA warp, whatever the number of MMAs);
-//   - a step is 256 keys with one-byte operands: one copy, two accumulators, one commit, whose barrier tells the epilogue that the
+//   - a step is 256 keys of 128 one-byte elements: one copy, two accumulators, one commit, whose barrier tells the epilogue that the
 //     accumulators are complete and the TMA warp that the stage is free;
 //   - eight epilogue warps, one group of four per 128 keys, load the next keys' scales a step ahead;
 //   - two CTAs share an SM, three stages of 32 KB each.
@@ -25,7 +25,9 @@ constexpr int TB_THREADS = 320;      // 1 TMA warp + 1 MMA warp + 8 epilogue war
 constexpr int TB_NEPI = TB_THREADS - 64;
 constexpr int TB_CTAS = 2;           // per SM
 constexpr int TB_MAX_STAGES = 6;
-constexpr int tb_subs(bool fp8) { return fp8 ? 2 : 1; }      // accumulators of 128 keys x 64 heads per step; bf16 stages hold 128 keys
+// Accumulators of 128 keys x 64 heads per step: a stage holds 32 KB, 256 keys of 128 bytes or 128 keys of 256 (bf16, and E4M3 of 256 dims, of
+// which half an SM would hold one stage of 256).
+constexpr int tb_subs(int atoms, bool fp8) { return fp8 && atoms == 1 ? 2 : 1; }
 
 struct TbParams {
     const float* w;
@@ -110,11 +112,10 @@ struct TbSegments {
     }
 };
 
-template <bool FP8, bool MULTI>
+template <bool FP8, int SUBS, bool MULTI>
 __global__ void __launch_bounds__(TB_THREADS, TB_CTAS)
 indexer_tc_batch_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, const TbParams p) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    constexpr int SUBS = tb_subs(FP8);
     constexpr int KEYS = SUBS * TC_KEYS;                   // keys per step
     constexpr int SLOT_COLS = SUBS * TB_HEADS;             // TMEM columns of a step's accumulators, two sets in turn
     const int atoms = p.atoms, stages = p.stages;
@@ -244,7 +245,7 @@ indexer_tc_batch_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
                     const uint32_t full = k_full + 8 * s, dst = ring + s * stage_bytes;
                     mbar_expect_tx(full, tile_bytes + (i == 0 ? static_cast<uint32_t>(q_bytes) : 0u));
                     tma_load_2d(dst, &tmap_k, 0, key_row, full);
-                    if (atoms == 2) tma_load_2d(dst + KEYS * 128, &tmap_k, ATOM, key_row, full);
+                    if (SUBS == 1 && atoms == 2) tma_load_2d(dst + KEYS * 128, &tmap_k, ATOM, key_row, full);
                 }
                 __syncwarp();
                 if (issued == 0) load_q();
@@ -291,7 +292,7 @@ indexer_tc_batch_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
                     const uint64_t ka = kdesc + sub * (TC_KEYS * 128 >> 4);
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks) umma<FP8>(d, ka + 2 * ks, qdesc + 2 * ks, idesc, ks > 0 ? 1u : 0u);     // 32 bytes of K per instruction
-                    if (atoms == 2) {
+                    if (SUBS == 1 && atoms == 2) {
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
                             umma<FP8>(d, ka + (KEYS * 128 >> 4) + 2 * ks, qdesc + (TB_HEADS * 128 >> 4) + 2 * ks, idesc, 1u);
@@ -383,12 +384,12 @@ indexer_tc_batch_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
     }
 }
 
-template <bool FP8, bool MULTI>
+template <bool FP8, int SUBS, bool MULTI>
 static int launch_tb(const CUtensorMap& tq, const CUtensorMap& tk, const TbParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
     static once_per_device attributes;
     JANUS_CUDA_CHECK(attributes.run(
-        [] { return cudaFuncSetAttribute(indexer_tc_batch_kernel<FP8, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET / TB_CTAS); }));
-    JANUS_CUDA_CHECK(launch_kernel(indexer_tc_batch_kernel<FP8, MULTI>, grid, TB_THREADS, smem, stream, 1, tq, tk, p));
+        [] { return cudaFuncSetAttribute(indexer_tc_batch_kernel<FP8, SUBS, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET / TB_CTAS); }));
+    JANUS_CUDA_CHECK(launch_kernel(indexer_tc_batch_kernel<FP8, SUBS, MULTI>, grid, TB_THREADS, smem, stream, 1, tq, tk, p));
     return JANUS_OK;
 }
 
@@ -406,12 +407,12 @@ int launch_indexer_tc_batch(const void* q_idx, const void* k_idx, int64_t k_stri
     const bool k_fp4 = dtype == JANUS_DTYPE_FP8_Q_FP4_K;
     const bool fp8 = dtype == JANUS_DTYPE_FP8_E4M3 || k_fp4;
     const int esz = fp8 ? 1 : 2;
-    const int keys = tb_subs(fp8) * TC_KEYS;
     TbParams p;
     p.w = w; p.q_scale = q_scale; p.q_scale_stride_tok = q_scale_stride_tok; p.k_scale = k_scale;
     p.row_bias = row_bias; p.col_bias = col_bias; p.scores = scores; p.n_keys = total_keys;
     p.key_offsets = key_offsets; p.n_sessions = B; p.k_fp4 = k_fp4 ? 1 : 0; p.dev_status = dev_status;
     p.atoms = D * esz / 128;
+    const int subs = tb_subs(p.atoms, fp8), keys = subs * TC_KEYS;
     const int q_bytes = p.atoms * TB_HEADS * 128, stage_bytes = p.atoms * keys * 128, tail = static_cast<int>(sizeof(TbShared));
     const int budget = TC_SMEM_BUDGET / TB_CTAS - 1024;      // (the system keeps 1 KB per CTA)
     p.stages = (budget - q_bytes - tail) / stage_bytes;
@@ -441,9 +442,9 @@ int launch_indexer_tc_batch(const void* q_idx, const void* k_idx, int64_t k_stri
     } else if (!make_tmap_2d_sw128(&tk, k_idx, esz, static_cast<uint64_t>(total_keys), D, static_cast<uint64_t>(k_stride_tok) * esz, keys, box_cols)) {
         return JANUS_ERR_CUDA;
     }
-    if (direct)
-        return fp8 ? launch_tb<true, false>(tq, tk, p, grid, smem, stream) : launch_tb<false, false>(tq, tk, p, grid, smem, stream);
-    return fp8 ? launch_tb<true, true>(tq, tk, p, grid, smem, stream) : launch_tb<false, true>(tq, tk, p, grid, smem, stream);
+    if (!fp8) return direct ? launch_tb<false, 1, false>(tq, tk, p, grid, smem, stream) : launch_tb<false, 1, true>(tq, tk, p, grid, smem, stream);
+    if (subs == 1) return direct ? launch_tb<true, 1, false>(tq, tk, p, grid, smem, stream) : launch_tb<true, 1, true>(tq, tk, p, grid, smem, stream);
+    return direct ? launch_tb<true, 2, false>(tq, tk, p, grid, smem, stream) : launch_tb<true, 2, true>(tq, tk, p, grid, smem, stream);
 }
 
 }  // namespace janus

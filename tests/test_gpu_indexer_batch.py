@@ -25,7 +25,7 @@ def _lib():
 
 
 @pytest.mark.parametrize("lengths", [EDGES, EDGES * 30, [40000] + EDGES, [20000, 1, 20001, 129, 19999, 257] * 8])
-@pytest.mark.parametrize("dtype,D", [("bf16", 128), ("bf16", 64), ("fp8", 128), ("fp4", 128)])
+@pytest.mark.parametrize("dtype,D", [("bf16", 128), ("bf16", 64), ("fp8", 128), ("fp8", 256), ("fp4", 128)])
 def test_steps_of_every_session(lengths, dtype, D):
     rng = np.random.default_rng(len(lengths) + D)
     n, total = len(lengths), sum(lengths)
