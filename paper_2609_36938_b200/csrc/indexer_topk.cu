@@ -12,6 +12,7 @@
 // Shapes the tensor-core indexer does not take, and problems too small to sample, run the two-call path
 // (scores in the workspace, then the row-wise top-k).
 #include <mutex>
+#include <type_traits>
 
 #include "sm100_ptx.cuh"
 #include "topk_select.cuh"
@@ -19,7 +20,8 @@
 namespace janus {
 
 constexpr int FT_NS = 4096;          // sampled keys (512 chunks of 8 consecutive keys)
-constexpr int FT_CAP = 16384;        // candidate slots per row; FT_CAP / 2 when the expected lists are short enough
+constexpr int FT_CAP = 16384;        // candidate slots per row; three quarters or half of them when the lists are sure to be short enough
+constexpr int FT_SLACK = 2;          // sample keys in the bucket of the threshold, at most (but for equal keys)
 constexpr int FT_FB_CTAS = 32;       // CTAs (and scratch rows) of the fallback kernel
 constexpr int FT_FB_CAP = 8192;      // candidate slots of the fallback's row-wise top-k
 
@@ -47,7 +49,9 @@ struct FusedLayout {
 
 static size_t align_up(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
-FusedLayout fused_layout(int M, int H, int D, int64_t n_keys, int64_t q_pos0, int causal, int dtype, int k) {
+// `tight`: the shortest list that the expected number of candidates fits, without the margin for a sample that is off.  Only for a
+// workspace that holds no more: some rows then take the fallback.
+FusedLayout fused_layout(int M, int H, int D, int64_t n_keys, int64_t q_pos0, int causal, int dtype, int k, bool tight = false) {
     FusedLayout L{};
     const int esz = dtype == JANUS_DTYPE_BF16 ? 2 : 1;
     L.p0 = causal ? (n_keys < q_pos0 + 1 ? n_keys : q_pos0 + 1) : n_keys;
@@ -57,11 +61,17 @@ FusedLayout fused_layout(int M, int H, int D, int64_t n_keys, int64_t q_pos0, in
               k <= FT_CAP / 4 && n_keys - L.p0 <= FT_CAP / 2;
     L.cap = FT_CAP;
     if (L.fused) {
-        // half-size lists (three selection CTAs per SM instead of one) when the list expected at the sampled threshold, plus
-        // every key beyond the sampled range, still fits them
+        // Shorter lists let three (half) or two (three quarters) selection CTAs share an SM instead of one.  A list receives what
+        // passes the sampled threshold among the p0 keys every row sees, and in the worst case (a recency bias) every key beyond
+        // them.  The threshold is the lower edge of the histogram bucket that holds the sample's r-th key (ft_threshold_kernel), so up to
+        // FT_SLACK more sample keys may lie above it, give or take the sample's own deviation of sqrt(r), of which four are allowed
+        // for.  A list that overflows costs its row a pass over all keys on the fp32 ALUs.
         const double expect = static_cast<double>(FT_NS) * k / static_cast<double>(L.p0);
-        const double frac = (expect + 6.0 * sqrt(expect) + 8.0) / FT_NS;
-        if (k <= FT_CAP / 8 && frac * static_cast<double>(n_keys) + static_cast<double>(n_keys - L.p0) <= FT_CAP / 2) L.cap = FT_CAP / 2;
+        const double r = expect + 6.0 * sqrt(expect) + 8.0, beyond = static_cast<double>(n_keys - L.p0);
+        const double rank = r + FT_SLACK + 4.0 * sqrt(r);
+        const double need = tight ? r / FT_NS * static_cast<double>(n_keys) + beyond : rank / FT_NS * static_cast<double>(L.p0) + beyond;
+        if (k <= FT_CAP / 8 && need <= FT_CAP / 2) L.cap = FT_CAP / 2;
+        else if (!tight && k <= FT_CAP / 8 && need <= FT_CAP / 4 * 3) L.cap = FT_CAP / 4 * 3;
     }
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += align_up(bytes); return o; };
@@ -138,7 +148,7 @@ ft_threshold_kernel(const float* sc_sample, int M, int64_t n_keys, int64_t q_pos
     const uint32_t key[8] = {float_to_key(a.x), float_to_key(a.y), float_to_key(a.z), float_to_key(a.w),
                              float_to_key(b.x), float_to_key(b.y), float_to_key(b.z), float_to_key(b.w)};
     uint32_t hi;
-    const uint32_t T = sample_threshold(key, r, hi, sh);
+    const uint32_t T = sample_threshold(key, r, FT_SLACK, hi, sh);
     if (tid == 0) thr[t] = key_to_float(T);
 }
 
@@ -300,6 +310,7 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
         L.ld = (n_keys + 3) / 4 * 4;
         L.total = align_up(sizeof(float) * static_cast<size_t>(L.ld) * M);
     }
+    if (L.fused && ws_bytes < L.total) L = fused_layout(M, H_I, D_I, n_keys, q_pos0, causal, dtype, k, true);
     if (n_keys > 0 && (ws == nullptr || ws_bytes < L.total || !aligned16(ws))) return JANUS_ERR_WORKSPACE_TOO_SMALL;
     unsigned char* base = static_cast<unsigned char*>(ws);
 
@@ -332,7 +343,7 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
                                H_I, D_I, FT_NS, q_pos0, 0, dtype, sc_sample, FT_NS, dev_status, stream, nullptr, nullptr, nullptr, 0);
     if (rc != JANUS_OK) return rc;
     // 2. thresholds (also clears the candidate counters)
-    static once_per_device threshold_attributes, select_attributes, fallback_attributes;
+    static once_per_device threshold_attributes, fallback_attributes;
     JANUS_CUDA_CHECK(threshold_attributes.run(
         [] { return cudaFuncSetAttribute(ft_threshold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(SampleShared))); }));
     JANUS_CUDA_CHECK(launch_kernel(ft_threshold_kernel, dim3(M), TK_THREADS, sizeof(SampleShared), stream, 1, sc_sample, M, n_keys, q_pos0, causal, k,
@@ -342,20 +353,19 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
                            dtype, nullptr, 0, dev_status, stream, thr, cand_cnt, cand, L.cap);
     if (rc != JANUS_OK) return rc;
     // 4. exact selection per row
-    JANUS_CUDA_CHECK(select_attributes.run([] {
-        const cudaError_t e = cudaFuncSetAttribute(ft_select_kernel<FT_CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(TopkSharedT<FT_CAP>)));
-        return e != cudaSuccess ? e : cudaFuncSetAttribute(ft_select_kernel<FT_CAP / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           static_cast<int>(sizeof(TopkSharedT<FT_CAP / 2>)));
-    }));
-    if (L.cap == FT_CAP) {
-        using Sh = TopkSharedT<FT_CAP>;
-        JANUS_CUDA_CHECK(launch_kernel(ft_select_kernel<FT_CAP>, dim3(M), TK_THREADS, sizeof(Sh), stream, 1, cand, cand_cnt, M, n_keys, q_pos0, causal,
-                                       k, idx, count, kth, fb_count, fb_rows));
-    } else {
-        using Sh = TopkSharedT<FT_CAP / 2>;
-        JANUS_CUDA_CHECK(launch_kernel(ft_select_kernel<FT_CAP / 2>, dim3(M), TK_THREADS, sizeof(Sh), stream, 1, cand, cand_cnt, M, n_keys, q_pos0,
+    auto select = [&](auto cap) -> int {
+        constexpr int CAP = decltype(cap)::value;
+        static once_per_device attributes;
+        JANUS_CUDA_CHECK(attributes.run([] {
+            return cudaFuncSetAttribute(ft_select_kernel<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(TopkSharedT<CAP>)));
+        }));
+        JANUS_CUDA_CHECK(launch_kernel(ft_select_kernel<CAP>, dim3(M), TK_THREADS, sizeof(TopkSharedT<CAP>), stream, 1, cand, cand_cnt, M, n_keys, q_pos0,
                                        causal, k, idx, count, kth, fb_count, fb_rows));
-    }
+        return JANUS_OK;
+    };
+    rc = L.cap == FT_CAP ? select(std::integral_constant<int, FT_CAP>{})
+                         : L.cap == FT_CAP / 2 ? select(std::integral_constant<int, FT_CAP / 2>{}) : select(std::integral_constant<int, FT_CAP / 4 * 3>{});
+    if (rc != JANUS_OK) return rc;
     // 5. rows the sample misjudged (normally none: the kernel then returns at once)
     const size_t fb_smem = sizeof(FallbackShared) + sizeof(float) * (static_cast<size_t>(H_I) * D_I + H_I);
     const unsigned char* qb = static_cast<const unsigned char*>(q_idx);
@@ -416,7 +426,7 @@ extern "C" int janus_indexer_topk_static(const void* q_idx, int64_t q_stride_tok
     // the size check comes first: a problem that does not fit is refused before anything touches the device
     if (M < 0 || H_I <= 0 || D_I <= 0 || n_keys < 0 || k <= 0) return JANUS_ERR_INVALID_ARG;
     if (M > 0 && n_keys > 0) {
-        const FusedLayout L = fused_layout(M, H_I, D_I, n_keys, q_pos0, causal, dtype, k);
+        const FusedLayout L = fused_layout(M, H_I, D_I, n_keys, q_pos0, causal, dtype, k, true);
         size_t need = L.total;
         if (L.fused && q_stride_tok != static_cast<int64_t>(H_I) * D_I)   // strided queries take the two-call route
             need = align_up(sizeof(float) * static_cast<size_t>(L.ld) * M);

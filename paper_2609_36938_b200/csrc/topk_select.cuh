@@ -231,10 +231,10 @@ template <class Sh>
 __device__ __forceinline__ int4 own_buckets(const Sh& sh) { return reinterpret_cast<const int4*>(sh.hist)[TK_THREADS - 1 - threadIdx.x]; }
 
 // Streaming threshold out of a sample of which every thread holds N keys: the lower edge of the bucket that holds the sample's
-// r-th key, unless that bucket is so full that it would let in far more than r, in which case it is split further.  `hi`
-// receives the largest sample key.
+// r-th key, once that bucket holds no more than `slack` keys; a fuller one is split further, up to a width of one key.  `hi` receives
+// the largest sample key.
 template <int N, class Sh>
-__device__ __forceinline__ uint32_t sample_threshold(const uint32_t (&key)[N], int r, uint32_t& hi, Sh& sh) {
+__device__ __forceinline__ uint32_t sample_threshold(const uint32_t (&key)[N], int r, int slack, uint32_t& hi, Sh& sh) {
     uint32_t lo = key[0];
     hi = key[0];
 #pragma unroll
@@ -250,7 +250,7 @@ __device__ __forceinline__ uint32_t sample_threshold(const uint32_t (&key)[N], i
         __syncthreads();
         find_bucket(own_buckets(sh), r, sh);
         const int b = sh.sel_bucket, count = sh.sel_count;
-        if (count <= 4 + r / 16 || map.shift == 0 || pass == 2) return map.first(b);
+        if (count <= slack || map.shift == 0 || pass == 2) return map.first(b);
         r -= sh.sel_above;
         if (b < TK_BUCKETS - 1) top = min(top, map.last(b));
         lo = map.first(b);
@@ -378,7 +378,7 @@ __device__ __forceinline__ bool topk_sample(const float* row, int n, int k, uint
     const float4 a = __ldcg(src), b = __ldcg(src + 1);
     const uint32_t key[8] = {float_to_key(a.x), float_to_key(a.y), float_to_key(a.z), float_to_key(a.w),
                              float_to_key(b.x), float_to_key(b.y), float_to_key(b.z), float_to_key(b.w)};
-    thr = sample_threshold(key, r, hi, sh);
+    thr = sample_threshold(key, r, 4 + r / 16, hi, sh);
     return true;
 }
 

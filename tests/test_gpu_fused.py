@@ -157,3 +157,32 @@ def test_workspace_contract():
     rc = lib.janus_indexer_topk(q.data_ptr(), 64 * 128, kk.data_ptr(), 128, w.data_ptr(), None, 0, None, None, None, 8, 64, 128, 20008, 20000, 1, 0,
                                 0, idx.data_ptr(), None, None, small.data_ptr(), small.numel(), None, None)
     assert rc == 1                                            # k = 0
+
+
+def test_recency_bias_stays_within_the_candidate_lists():
+    """Every key beyond the sampled range scores above it, so a late row's list takes all of them beside what passes the sampled
+    threshold: no row may overflow its list (it would be recomputed on the fp32 ALUs).  A workspace of half-size lists, which hold no
+    more than the expected number, is still taken and gives the same selections, by the fallback where it must."""
+    M, L, k = 4096, 131072, 2048
+    g = torch.Generator(device="cuda").manual_seed(3)
+    S = L + M
+    q = torch.randn((M, 64, 128), device="cuda", generator=g).to(torch.float8_e4m3fn)
+    kk = torch.randn((S, 128), device="cuda", generator=g).to(torch.float8_e4m3fn)
+    w, qs, ks = torch.rand((M, 64), device="cuda", generator=g) / 8, torch.full((64,), 0.5, device="cuda"), torch.ones(S, device="cuda")
+    row_bias, col_bias = torch.full((M,), 1e3, device="cuda"), (torch.arange(S, device="cuda") >= L).float()
+    lib = B.load()
+    args = (M, 64, 128, S, L, 1, B.DTYPE_FP8_E4M3, k)
+    need, at = int(lib.janus_indexer_topk_workspace_size(*args)), int(lib.janus_indexer_topk_fallback_counter_offset(*args))
+    idx, kth = torch.empty((2, M, k), dtype=torch.int32, device="cuda"), torch.empty((2, M), device="cuda")
+    new = torch.minimum(torch.arange(1, M + 1, device="cuda"), torch.tensor(k, device="cuda"))
+    for i, nbytes in enumerate((need, need - 8 * M * (12288 - 8192))):
+        ws = torch.empty((nbytes,), dtype=torch.uint8, device="cuda")
+        rc = lib.janus_indexer_topk(q.data_ptr(), 64 * 128, kk.data_ptr(), 128, w.data_ptr(), qs.data_ptr(), 0, ks.data_ptr(), row_bias.data_ptr(),
+                                    col_bias.data_ptr(), M, 64, 128, S, L, 1, B.DTYPE_FP8_E4M3, k, idx[i].data_ptr(), None, kth[i].data_ptr(), ws.data_ptr(),
+                                    nbytes, B.dev_status_tensor().data_ptr(), torch.cuda.current_stream().cuda_stream)
+        assert rc == B.JANUS_OK
+        B.check_dev_status()
+        if i == 0:
+            assert int(ws[at:at + 4].view(torch.int32).item()) == 0
+        assert torch.equal((idx[i] >= L).sum(1), new)
+    torch.testing.assert_close(kth[0], kth[1], rtol=1e-5, atol=0.0)
