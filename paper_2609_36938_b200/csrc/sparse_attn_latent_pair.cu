@@ -69,6 +69,7 @@ constexpr int LP_SMAX_WARP0 = LP_XCHG_WARP0 + 4;                 // first softma
 constexpr int LP_THREADS = 32 * (LP_SMAX_WARP0 + 4);             // 12 warps
 constexpr int LP_Q_TMEM_ATOMS = 3;                               // query atoms kept in tensor memory; the others sit in shared memory
 constexpr int LP_QS_BYTES = 2 * LP_Q_ATOM_BYTES;                 // 32 KB: owned query atom 3 (and 4 on CTA 1)
+constexpr int LP_MAX_SPLIT = 8;             // pairs of a cluster that share the keys of one token
 constexpr uint32_t LP_COL_O = 0, LP_COL_S = 256, LP_COL_P = 384, LP_COL_Q = 416;   // O 256 | 2 x 64 logits | P 32 | 3 x 32 query
 
 struct LpShared {
@@ -81,12 +82,11 @@ struct LpShared {
     uint64_t x_empty[2];                          // the PEER has read this CTA's previous partial logits out of its exchange buffer b
     uint32_t vmask[LP_SLOTS];
     uint32_t tmem_base;
-    uint32_t start_abort[2];
+    uint32_t start_abort[2 * LP_MAX_SPLIT];       // by CTA of the cluster
 };
 
 // Keys of one token split over several pairs of a cluster (few query rows): what a pair leaves for the merge.  Its fp32 output
 // goes where its key ring was, [column / 4][head][4]; reference maximum (log2 domain) and row sum of every head beside it.
-constexpr int LP_MAX_SPLIT = 8;
 struct LpSplitStats {
     float m[LP_HEADS], l[LP_HEADS];
 };
@@ -195,6 +195,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     unsigned char* q_smem = smem + LP_BUFS * LP_TILE_BYTES + 2 * LP_XBUF_BYTES;    // owned query atom 3 (and 4 on CTA 1), each [128 heads x 128 B]
     LpShared* sh = reinterpret_cast<LpShared*>(q_smem + LP_QS_BYTES);
 
+    cluster_arrive();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t c = rank & 1u;                  // 0 or 1: which bytes of the rows this CTA owns
@@ -224,15 +225,18 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
         mbar_init(smem_u32(&sh->p_full), 4);
         fence_mbar_init();
         prefetch_tensormap(&tmap_q);
-        grid_wait();
+    }
+    __syncwarp();
+    grid_wait();
+    cluster_wait();                                // every CTA of the cluster runs: its shared memory may be written
+    if (threadIdx.x == 0) {
         // start-up agreement: if this CTA should not start (misaligned shared memory, or an earlier CTA of the launch gave
-        // up on a wait), both CTAs of the cluster must skip the work, so the flag is written to both of them
+        // up on a wait), every CTA of the cluster must skip the work, so the flag is written to all of them
         uint32_t flag = ((smem_u32(smem) & 1023u) != 0u) ? 1u : 0u;
         if (p.dev_status != nullptr && *reinterpret_cast<volatile int32_t*>(p.dev_status) == JANUS_DEV_WAIT_TIMEOUT) flag = 1u;
-        sh->start_abort[c] = flag;
-        st_cluster_u32(mapa_shared(smem_u32(&sh->start_abort[c]), peer), flag);
+        for (uint32_t r = 0; r < cluster_nctarank(); ++r) st_cluster_u32(mapa_shared(smem_u32(&sh->start_abort[rank]), r), flag);
     }
-    grid_wait();
+    __syncwarp();
     if (warp == 0) {
         tmem_alloc(smem_u32(&sh->tmem_base), 512);
         tmem_relinquish();
@@ -243,7 +247,9 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     if constexpr (SPLIT) grid_launch_next();       // (tensor memory is allocated)
     tc_fence_after();
     const uint32_t tmem_base = sh->tmem_base;
-    const bool start_abort = (sh->start_abort[0] | sh->start_abort[1]) != 0u;
+    uint32_t abort_flags = 0u;
+    for (int r = 0; r < 2 * n_split; ++r) abort_flags |= sh->start_abort[r];
+    const bool start_abort = abort_flags != 0u;
     if (start_abort && threadIdx.x == 0 && (smem_u32(smem) & 1023u) != 0u) report(p.dev_status, JANUS_DEV_WAIT_TIMEOUT);
 
     if (start_abort) {

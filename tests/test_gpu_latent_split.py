@@ -2,6 +2,7 @@
 tiles, pairs without a single valid key, rows without any, logits whose maximum sits in one pair only.  Reference: the oracle."""
 import numpy as np
 import pytest
+import torch
 
 import helpers as Hp
 from oracle import janus_oracle as O
@@ -46,3 +47,17 @@ def test_split_latent_attention_matches_oracle(M, k, gain):
     assert np.array_equal(np.isfinite(got), fin)
     # partial logits cross between the two SMs as fp16: 2^-11 of a partial logit (up to 40 here), and P is bf16
     assert np.all(np.abs(got[fin] - ref_l[fin]) <= 2e-2 + 1e-3 * np.abs(ref_l[fin]))
+
+
+@pytest.mark.parametrize("M", [1, 5, 200])
+def test_a_call_on_a_broken_pipeline_does_nothing(M):
+    """The status word says that a wait has given up: no CTA starts, all of a cluster agree on it, and the outputs stay as they were."""
+    q, pool = torch.zeros((M, 128, 576), dtype=torch.bfloat16, device="cuda"), torch.zeros((8, 64, 1, 576), dtype=torch.bfloat16, device="cuda")
+    idx, table = torch.arange(512, dtype=torch.int32, device="cuda").repeat(M, 1), torch.arange(8, dtype=torch.int32, device="cuda")
+    out, lse = torch.full((M, 128, 512), 7.0, dtype=torch.bfloat16, device="cuda"), torch.full((M, 128), 7.0, device="cuda")
+    status = torch.full((1,), 103, dtype=torch.int32, device="cuda")
+    rc = B.load().janus_sparse_attn_prefill(q.data_ptr(), M, 128, 576, pool.data_ptr(), pool.data_ptr(), pool.stride(0), pool.stride(1), pool.stride(2), 1, 512,
+                                            idx.data_ptr(), 512, 64, table.data_ptr(), 8, 1.0, out.data_ptr(), lse.data_ptr(), None, 0, status.data_ptr(),
+                                            torch.cuda.current_stream().cuda_stream)
+    assert rc == B.JANUS_OK
+    assert bool((out == 7).all()) and bool((lse == 7).all()) and int(status.item()) == 103
