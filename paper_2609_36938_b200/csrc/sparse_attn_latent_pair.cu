@@ -83,14 +83,14 @@ struct LpShared {
     uint32_t vmask[LP_SLOTS];
     uint32_t tmem_base;
     uint32_t start_abort[2 * LP_MAX_SPLIT];       // by CTA of the cluster
+    // reference maximum (log2 domain) and row sum of every head, for the merge: -inf and 0 until the pair has left its output
+    float split_m[LP_HEADS], split_l[LP_HEADS];
+    alignas(16) float split_zero[4];
 };
 
-// Keys of one token split over several pairs of a cluster (few query rows): what a pair leaves for the merge.  Its fp32 output
-// goes where its key ring was, [column / 4][head][4]; reference maximum (log2 domain) and row sum of every head beside it.
-struct LpSplitStats {
-    float m[LP_HEADS], l[LP_HEADS];
-};
-static_assert(LP_DVH * LP_HEADS * 4 <= LP_BUFS * LP_TILE_BYTES && sizeof(LpSplitStats) <= 2 * LP_XBUF_BYTES, "merge buffers reuse the ring and the exchange buffers");
+// Keys of one token split over several pairs of a cluster (few query rows): a pair leaves its fp32 output for the merge where its
+// key ring was, [column / 4][head][4], and LpShared::split_m / split_l.
+static_assert(LP_DVH * LP_HEADS * 4 <= LP_BUFS * LP_TILE_BYTES, "the merge buffer reuses the ring");
 
 struct LpParams {
     const uint16_t* q;
@@ -137,15 +137,15 @@ __device__ __forceinline__ float4 lp_ld_cluster4(uint32_t addr) {
 // Output of token t from the N pairs' unnormalised outputs: CTA (s, c) takes every N-th block of 16 columns of value half c, a
 // thread one block of one head at a time.  N is a compile-time number so that all remote loads are issued together.
 template <int N>
-__device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s, uint32_t c, uint32_t o_addr, uint32_t stats_addr) {
+__device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s, uint32_t c, uint32_t o_addr, uint32_t m_addr, uint32_t l_addr, uint32_t zero_addr) {
     const int h = threadIdx.x & (LP_HEADS - 1);
     const float neg_inf = __int_as_float(0xff800000);
     float f[N], l[N];
     float m_all = neg_inf, l_all = 0.f;
 #pragma unroll
     for (int r = 0; r < N; ++r) {
-        f[r] = lp_ld_cluster(mapa_shared(stats_addr + 4 * h, 2 * r + c));
-        l[r] = lp_ld_cluster(mapa_shared(stats_addr + 4 * (LP_HEADS + h), 2 * r + c));
+        f[r] = lp_ld_cluster(mapa_shared(m_addr + 4 * h, 2 * r + c));
+        l[r] = lp_ld_cluster(mapa_shared(l_addr + 4 * h, 2 * r + c));
     }
 #pragma unroll
     for (int r = 0; r < N; ++r) m_all = fmaxf(m_all, f[r]);
@@ -159,9 +159,12 @@ __device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s,
         float4 x[N][4], acc[4] = {};
 #pragma unroll
         for (int r = 0; r < N; ++r) {
-            const uint32_t src = mapa_shared(o_addr + static_cast<uint32_t>((blk * 4 * LP_HEADS + h) * 16), 2 * r + c);
+            // a pair without a key, or one that gave up, counts as zeros: what lies in its buffer may be anything, a NaN even
+            const bool empty = f[r] == 0.f;
+            const uint32_t src = empty ? mapa_shared(zero_addr, 2 * s + c) : mapa_shared(o_addr + static_cast<uint32_t>((blk * 4 * LP_HEADS + h) * 16), 2 * r + c);
+            const uint32_t step = empty ? 0u : LP_HEADS * 16u;
 #pragma unroll
-            for (int v = 0; v < 4; ++v) x[r][v] = lp_ld_cluster4(src + v * LP_HEADS * 16);
+            for (int v = 0; v < 4; ++v) x[r][v] = lp_ld_cluster4(src + v * step);
         }
 #pragma unroll
         for (int r = 0; r < N; ++r)
@@ -212,6 +215,11 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     const int n_tiles = SPLIT ? (static_cast<int>(rank >> 1) + 1) * all_tiles / n_split - tile0 : all_tiles;
     const int n_half = 2 * n_tiles;
 
+    if (SPLIT && threadIdx.x < LP_HEADS) {
+        sh->split_m[threadIdx.x] = __int_as_float(0xff800000);
+        sh->split_l[threadIdx.x] = 0.f;
+        if (threadIdx.x < 4) sh->split_zero[threadIdx.x] = 0.f;
+    }
     if (threadIdx.x == 0) {
         mbar_init(smem_u32(&sh->q_full), 1);
         mbar_init(smem_u32(&sh->qt_full), 4);
@@ -525,7 +533,6 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
         const float neg_inf = __int_as_float(0xff800000);
         const bool out_al32 = (reinterpret_cast<uint64_t>(p.out) & 31u) == 0u;
         bool ok = true;
-        bool merged = false;        // SPLIT: the output was left for the merge
         const uint32_t peer_xempty = mapa_shared(smem_u32(&sh->x_empty[0]), peer);
         int gi = 0;                 // tiles done so far, over all tokens
         for (int it = 0; it < n_my && ok; ++it) {
@@ -654,11 +661,10 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
         tc_fence_after();
         const bool have_o = __any_sync(0xffffffffu, l_sum > 0.f);   // some P.V of this token has written O
         if constexpr (SPLIT) {
-            // this pair's last P.V is complete, so nothing reads the ring or the exchange buffer any more: leave O for the merge
+            // this pair's last P.V is complete, so nothing reads the ring any more: leave O for the merge
             float* mo = reinterpret_cast<float*>(k_smem);
-            LpSplitStats* stats = reinterpret_cast<LpSplitStats*>(xbuf);
-            stats->m[h] = m_ref;
-            stats->l[h] = l_sum;
+            sh->split_m[h] = m_ref;
+            sh->split_l[h] = l_sum;
 #pragma unroll 1
             for (int cc = 0; cc < LP_DVH / 32; ++cc) {
                 uint32_t o[32];
@@ -672,7 +678,6 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
                 for (int v = 0; v < 8; ++v)
                     *reinterpret_cast<uint4*>(mo + ((cc * 8 + v) * LP_HEADS + h) * 4) = make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
             }
-            merged = true;
             break;
         }
         const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
@@ -702,11 +707,6 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
             p.lse[static_cast<int64_t>(t) * LP_HEADS + h] = l_sum > 0.f ? (m_ref + log2f(l_sum)) * 0.6931471805599453f : neg_inf;
         }
         if (!ok && lane == 0) report(p.dev_status, JANUS_DEV_WAIT_TIMEOUT);
-        if (SPLIT && !merged) {     // gave up: the merge below reads zeros instead of leftovers
-            LpSplitStats* stats = reinterpret_cast<LpSplitStats*>(xbuf);
-            stats->m[h] = neg_inf;
-            stats->l[h] = 0.f;
-        }
     }
     tc_fence_before();
     __syncthreads();
@@ -717,17 +717,17 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     if constexpr (SPLIT) {
         cluster_sync_all();         // every pair's output lies in its shared memory
         if (!start_abort && n_my > 0) {
-            const uint32_t o_addr = smem_u32(k_smem), stats_addr = smem_u32(xbuf);
+            const uint32_t o_addr = smem_u32(k_smem), m_addr = smem_u32(sh->split_m), l_addr = smem_u32(sh->split_l), zero_addr = smem_u32(sh->split_zero);
             const int sp = static_cast<int>(rank >> 1);
             static_assert(LP_MAX_SPLIT == 8, "cases below");
             switch (n_split) {
-                case 2: lp_merge_splits<2>(p, cid, sp, c, o_addr, stats_addr); break;
-                case 3: lp_merge_splits<3>(p, cid, sp, c, o_addr, stats_addr); break;
-                case 4: lp_merge_splits<4>(p, cid, sp, c, o_addr, stats_addr); break;
-                case 5: lp_merge_splits<5>(p, cid, sp, c, o_addr, stats_addr); break;
-                case 6: lp_merge_splits<6>(p, cid, sp, c, o_addr, stats_addr); break;
-                case 7: lp_merge_splits<7>(p, cid, sp, c, o_addr, stats_addr); break;
-                case 8: lp_merge_splits<8>(p, cid, sp, c, o_addr, stats_addr); break;
+                case 2: lp_merge_splits<2>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
+                case 3: lp_merge_splits<3>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
+                case 4: lp_merge_splits<4>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
+                case 5: lp_merge_splits<5>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
+                case 6: lp_merge_splits<6>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
+                case 7: lp_merge_splits<7>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
+                case 8: lp_merge_splits<8>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
             }
         }
     }
