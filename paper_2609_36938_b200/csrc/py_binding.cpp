@@ -11,9 +11,10 @@
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
-#include <stdexcept>
+#include <exception>
 #include <string>
 #include <vector>
 
@@ -67,6 +68,15 @@ int64_t integer(PyObject* o) {
         return v;
     }
     PyObject* n = PyNumber_Long(o);
+    if (n == nullptr) throw PyError{};
+    const long long v = PyLong_AsLongLong(n);
+    Py_DECREF(n);
+    if (v == -1 && PyErr_Occurred()) throw PyError{};
+    return v;
+}
+// A size of something this call allocates: whole numbers only, as for any tensor's shape.
+int64_t size(PyObject* o) {
+    PyObject* n = PyNumber_Index(o);
     if (n == nullptr) throw PyError{};
     const long long v = PyLong_AsLongLong(n);
     Py_DECREF(n);
@@ -185,7 +195,7 @@ PyObject* indexer_scores(Args a) {
 
 PyObject* topk(Args a) {
     const at::Tensor& scores = tensor(a[0]);
-    const int64_t M = scores.size(0), k = integer(a[2]);
+    const int64_t M = scores.size(0), k = a[7] == Py_None ? size(a[2]) : integer(a[2]);
     at::Tensor idx = a[7] == Py_None ? make({M, k}, at::kInt, scores) : tensor(a[7]), count, kth;
     if (truth(a[5])) count = make({M}, at::kInt, scores);
     if (truth(a[6])) kth = make({M}, at::kFloat, scores);
@@ -198,7 +208,7 @@ PyObject* topk(Args a) {
 PyObject* indexer_topk(Args a) {
     const at::Tensor &q = tensor(a[0]), &k_idx = tensor(a[1]);
     want_dims(q, 3, "q_idx");
-    const int64_t M = q.size(0), H = q.size(1), D = q.size(2), n_keys = k_idx.size(0), k = integer(a[3]), q_pos0 = integer(a[8]);
+    const int64_t M = q.size(0), H = q.size(1), D = q.size(2), n_keys = k_idx.size(0), k = a[13] == Py_None ? size(a[3]) : integer(a[3]), q_pos0 = integer(a[8]);
     const IdxDtypes dt = idx_dtypes(q, k_idx, truth(a[14]));
     const int causal = i32(truth(a[9]));
     const size_t need = api.indexer_topk_workspace_size(i32(M), i32(H), i32(D), n_keys, q_pos0, causal, dt.code, i32(k));
@@ -210,7 +220,7 @@ PyObject* indexer_topk(Args a) {
         idx = make({M, k}, at::kInt, q);
     } else {
         idx = tensor(a[13]);
-        if (idx.dim() != 2 || idx.size(0) != M || idx.size(1) != k || idx.scalar_type() != at::kInt || !idx.is_contiguous())
+        if (idx.dim() != 2 || idx.size(0) != M || idx.size(1) != k || number(a[3]) != static_cast<double>(k) || idx.scalar_type() != at::kInt || !idx.is_contiguous())
             fail(janus_error, "idx must be a contiguous [M, k] int32 tensor");
     }
     if (truth(a[10])) count = make({M}, at::kInt, q);
@@ -279,7 +289,7 @@ PyObject* sparse_attn(Args a) {
     const at::Tensor &q = tensor(a[0]), &kp = tensor(a[1]), &vp = tensor(a[2]), &idx = tensor(a[3]), &table = tensor(a[4]);
     want_dims(q, 3, "q");
     const bool batch = a[5] != Py_None;
-    const int64_t M = q.size(0), H = q.size(1), d_qk = q.size(2), n_kv = kp.size(2), d_v = integer(a[8]);
+    const int64_t M = q.size(0), H = q.size(1), d_qk = q.size(2), n_kv = kp.size(2), d_v = a[10] == Py_None ? size(a[8]) : integer(a[8]);
     at::Tensor out = a[10] == Py_None ? make({M, H, d_v}, at::kBFloat16, q) : tensor(a[10]), lse;
     if (truth(a[9])) lse = make({M, H}, at::kFloat, q);
     if (!batch && vp.data_ptr() != kp.data_ptr() && vp.strides() != kp.strides()) fail(janus_error, "k_pool and v_pool must share strides");
@@ -300,7 +310,7 @@ PyObject* sparse_attn(Args a) {
 
 PyObject* topk_entries(Args a) {      // scores, n_entries, k, q_pos0, entry_size, want_count, want_kth
     const at::Tensor& scores = tensor(a[0]);
-    const int64_t M = scores.size(0), k = integer(a[2]);
+    const int64_t M = scores.size(0), k = size(a[2]);
     at::Tensor idx = make({M, k}, at::kInt, scores), count, kth;
     if (truth(a[5])) count = make({M}, at::kInt, scores);
     if (truth(a[6])) kth = make({M}, at::kFloat, scores);
@@ -312,7 +322,7 @@ PyObject* topk_entries(Args a) {      // scores, n_entries, k, q_pos0, entry_siz
 
 PyObject* entry_pool_scores(Args a) { // scores, n_keys, entry_size, q_pos0, causal
     const at::Tensor& scores = tensor(a[0]);
-    const int64_t M = scores.size(0), n_keys = integer(a[1]), entry = integer(a[2]);
+    const int64_t M = scores.size(0), n_keys = integer(a[1]), entry = size(a[2]);
     if (entry == 0) fail(PyExc_ZeroDivisionError, "entry_size is zero");
     const int64_t n_entries = (n_keys + entry - 1) / entry, ld = n_entries > 4 ? (n_entries + 3) / 4 * 4 : 4;
     at::Tensor out = make({M, ld}, at::kFloat, scores);
@@ -324,9 +334,9 @@ PyObject* entry_pool_scores(Args a) { // scores, n_keys, entry_size, q_pos0, cau
 PyObject* entry_expand(Args a) {      // idx_entries, q_pos0, entry_size
     const at::Tensor& e = tensor(a[0]);
     want_dims(e, 2, "idx_entries");
-    const int64_t M = e.size(0), k_e = e.size(1), size = integer(a[2]);
-    at::Tensor out = make({M, k_e * size}, at::kInt, e);
-    call("janus_entry_expand", api.entry_expand, as<const int32_t>(ptr(e)), i32(M), i32(k_e), i32(size), integer(a[1]), as<int32_t>(ptr(out)), stream());
+    const int64_t M = e.size(0), k_e = e.size(1), entry = size(a[2]);
+    at::Tensor out = make({M, k_e * entry}, at::kInt, e);
+    call("janus_entry_expand", api.entry_expand, as<const int32_t>(ptr(e)), i32(M), i32(k_e), i32(entry), integer(a[1]), as<int32_t>(ptr(out)), stream());
     return wrap(out);
 }
 
@@ -346,7 +356,7 @@ PyObject* indexer_scores_batch(Args a) {      // q, k, w, key_offsets, max_keys,
 
 PyObject* topk_batch(Args a) {        // scores, row_offsets, k, row_lengths, want_count, want_kth
     const at::Tensor &scores = tensor(a[0]), &off = tensor(a[1]);
-    const int64_t n = off.numel() - 1, k = integer(a[2]);
+    const int64_t n = off.numel() - 1, k = size(a[2]);
     at::Tensor idx = make({n, k}, at::kInt, scores), count, kth;
     if (truth(a[4])) count = make({n}, at::kInt, scores);
     if (truth(a[5])) kth = make({n}, at::kFloat, scores);
@@ -366,10 +376,8 @@ PyObject* entry(PyObject*, Args args, Py_ssize_t n) {
     try {
         return F(args);
     } catch (const PyError&) {
-    } catch (const c10::Error& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {      // torch's own exceptions by their own names: out of memory, a dimension that is not there
+        torch::translate_exception_to_python(std::current_exception());
     }
     return nullptr;
 }

@@ -19,6 +19,31 @@ def test_loads_and_counts_its_arguments():
             getattr(native, name)()
 
 
+def test_sizes_are_whole_numbers_and_errors_keep_their_types():
+    """Where a size shapes an output, only a whole number is taken; a missing dimension and a failed allocation raise what torch raises."""
+    sc, e = torch.zeros(4, 8), torch.zeros(4, 2, dtype=torch.int32)
+    with pytest.raises(TypeError):
+        B.janus_topk(sc, 8, 2.5)
+    with pytest.raises(TypeError):
+        B.janus_topk_entries(sc, 8, 2.0, q_pos0=0, entry_size=4)
+    with pytest.raises(TypeError):
+        B.janus_topk_batch(sc, torch.zeros(3, dtype=torch.int64), 2.0)
+    with pytest.raises(TypeError):
+        B.janus_entry_expand(e, q_pos0=0, entry_size=4.0)
+    with pytest.raises(TypeError):
+        B.janus_entry_pool_scores(sc, 8, entry_size=4.0)
+    with pytest.raises(IndexError):
+        B.janus_topk(torch.zeros(()), 8, 2)
+
+
+@pytest.mark.gpu
+def test_out_of_memory_is_torch_s_own_error():
+    off = torch.arange(65, device="cuda") * 4
+    with pytest.raises(torch.OutOfMemoryError):
+        B.janus_topk_batch(torch.zeros(256, device="cuda"), off, 1 << 30)      # 256 GB of indices
+    torch.cuda.empty_cache()
+
+
 @pytest.mark.gpu
 def test_bad_tensors_raise():
     q, k, w = torch.zeros(4, 64, 128).bfloat16(), torch.zeros(32, 128).bfloat16(), torch.zeros(4, 64)
