@@ -505,7 +505,7 @@ bool indexer_tc_candidates_supported(int H, int D, int dtype) {
 template <int H, bool FP8, bool CAND, bool MULTI>
 static int launch_tc(const CUtensorMap& tq, const CUtensorMap& tk, const TcParams& p, const TcCandParams& cp, const TcSchedule& sched, dim3 grid,
                      size_t smem, cudaStream_t stream) {
-    static once_per_device attributes;
+    static once_per_context attributes;
     JANUS_CUDA_CHECK(attributes.run(
         [] { return cudaFuncSetAttribute(indexer_tc_kernel<H, FP8, CAND, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET); }));
     if constexpr (MULTI)

@@ -386,7 +386,7 @@ indexer_tc_batch_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid
 
 template <bool FP8, int SUBS, bool MULTI>
 static int launch_tb(const CUtensorMap& tq, const CUtensorMap& tk, const TbParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
-    static once_per_device attributes;
+    static once_per_context attributes;
     JANUS_CUDA_CHECK(attributes.run(
         [] { return cudaFuncSetAttribute(indexer_tc_batch_kernel<FP8, SUBS, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BUDGET / TB_CTAS); }));
     JANUS_CUDA_CHECK(launch_kernel(indexer_tc_batch_kernel<FP8, SUBS, MULTI>, grid, TB_THREADS, smem, stream, 1, tq, tk, p));

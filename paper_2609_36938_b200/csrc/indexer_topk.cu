@@ -343,7 +343,7 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
                                H_I, D_I, FT_NS, q_pos0, 0, dtype, sc_sample, FT_NS, dev_status, stream, nullptr, nullptr, nullptr, 0);
     if (rc != JANUS_OK) return rc;
     // 2. thresholds (also clears the candidate counters)
-    static once_per_device threshold_attributes, fallback_attributes;
+    static once_per_context threshold_attributes, fallback_attributes;
     JANUS_CUDA_CHECK(threshold_attributes.run(
         [] { return cudaFuncSetAttribute(ft_threshold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(SampleShared))); }));
     JANUS_CUDA_CHECK(launch_kernel(ft_threshold_kernel, dim3(M), TK_THREADS, sizeof(SampleShared), stream, 1, sc_sample, M, n_keys, q_pos0, causal, k,
@@ -355,7 +355,7 @@ extern "C" int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok, const
     // 4. exact selection per row
     auto select = [&](auto cap) -> int {
         constexpr int CAP = decltype(cap)::value;
-        static once_per_device attributes;
+        static once_per_context attributes;
         JANUS_CUDA_CHECK(attributes.run([] {
             return cudaFuncSetAttribute(ft_select_kernel<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(TopkSharedT<CAP>)));
         }));

@@ -1,11 +1,26 @@
 // Entry points that validate arguments and pick a kernel: janus_indexer_scores, janus_sparse_attn_prefill,
 // plus the version / error queries.  janus_topk and janus_page_demand live beside their kernels.
+#include <cuda.h>
+
 #include "janus_common.cuh"
 
 namespace janus {
 
 static thread_local int g_last_cuda_error = 0;
 void set_last_cuda_error(cudaError_t e) { g_last_cuda_error = static_cast<int>(e); }
+
+uint64_t current_context_id() {
+    using GetId = CUresult (*)(CUcontext, unsigned long long*);
+    static const GetId get = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        return cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess
+                   ? reinterpret_cast<GetId>(p)
+                   : nullptr;
+    }();
+    unsigned long long id = 0;
+    return get != nullptr && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
 
 int launch_indexer_generic(const void* q_idx, int64_t q_stride_tok, const void* k_idx, int64_t k_stride_tok, const float* w,
                            const float* q_scale, int64_t q_scale_stride_tok, const float* k_scale, const float* row_bias,

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 
 #include "../../include/janus.h"
 
@@ -24,24 +25,41 @@ void set_last_cuda_error(cudaError_t e);
         }                                              \
     } while (0)
 
-// Runs a function once on every device (kernel attributes: they stay set, and setting them on each call costs a microsecond).
-class once_per_device {
+// Id of the CUDA context that is current on this thread; 0 while there is none (the runtime makes one on its first call that needs it).
+uint64_t current_context_id();
+
+// Runs a function once in every context: kernel attributes belong to a context (a device may have several, one after the other or
+// side by side) and setting them on each call costs a microsecond.  Callers on other threads wait until it has run.
+class once_per_context {
   public:
     template <class F>
-    cudaError_t run(F&& f) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return f();
-        const uint64_t bit = uint64_t(1) << dev;
-        if ((done_.load(std::memory_order_acquire) & bit) != 0) return cudaSuccess;
-        e = f();
-        if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_release);
-        return e;
+    cudaError_t run(F&& f) { return run_in(current_context_id(), f); }
+    template <class F>
+    cudaError_t run_in(uint64_t id, F&& f) {
+        if (seen(id)) return cudaSuccess;
+        std::lock_guard<std::mutex> lock(mu_);
+        if (seen(id)) return cudaSuccess;
+        const cudaError_t e = f();
+        if (e != cudaSuccess || id == 0) return e;
+        for (auto& d : done_) {
+            if (d.load(std::memory_order_relaxed) != 0) continue;
+            d.store(id, std::memory_order_release);
+            break;
+        }
+        return e;      // (with more contexts than places the function runs on each call)
     }
 
   private:
-    std::atomic<uint64_t> done_{0};
+    bool seen(uint64_t id) const {
+        for (const auto& d : done_) {
+            const uint64_t v = d.load(std::memory_order_acquire);
+            if (v == 0) return false;
+            if (v == id) return true;
+        }
+        return false;
+    }
+    std::atomic<uint64_t> done_[32] = {};
+    std::mutex mu_;
 };
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

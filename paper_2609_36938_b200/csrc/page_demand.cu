@@ -406,7 +406,7 @@ __global__ void page_union_kernel(uint32_t* __restrict__ dst, const uint32_t* sr
 template <int MODE>
 static int launch_page_demand(const PdParams& p, int cluster, cudaStream_t stream) {
     const size_t smem = MODE == PD_LISTS ? 0 : sizeof(uint32_t) * static_cast<size_t>(p.n_words);
-    static once_per_device attributes;
+    static once_per_context attributes;
     JANUS_CUDA_CHECK(attributes.run([] {
         cudaError_t e = cudaFuncSetAttribute(page_demand_kernel<MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e == cudaSuccess && MODE != PD_LISTS)
@@ -433,7 +433,7 @@ static int run_page_demand(const PdParams& p, cudaStream_t stream) {
     JANUS_CUDA_CHECK(cudaMemsetAsync(p.bitmap, 0, sizeof(uint32_t) * p.n_words, stream));
     const int64_t n_log_words = (p.n_logical_pages + 31) / 32;
     if (MODE == PD_MARK && n_log_words + p.n_words <= MARK_SMEM_WORDS) {
-        static once_per_device attributes;
+        static once_per_context attributes;
         JANUS_CUDA_CHECK(attributes.run([] {
             return cudaFuncSetAttribute(page_mark_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MARK_SMEM_WORDS * static_cast<int>(sizeof(uint32_t)));
         }));

@@ -757,18 +757,22 @@ static cudaLaunchConfig_t lp_occupancy_config(int cluster_size, int n_clusters, 
 }
 
 // n[s] = clusters of 2 s CTAs the device keeps resident at once (one CTA per SM), 0 where it takes none.  A property of the
-// device, asked for on its first call; so are the kernels' attributes.
+// device, asked for on its first call; the kernels' attributes are set once in every context.
 static int lp_resident_clusters(int dev, size_t smem, int (&n)[LP_MAX_SPLIT + 1]) {
     constexpr int MAX_DEVICES = 64;
     static std::mutex mu;
     static int known[MAX_DEVICES][LP_MAX_SPLIT + 1] = {};
     if (dev < 0 || dev >= MAX_DEVICES) return JANUS_ERR_UNSUPPORTED;
+    static once_per_context attributes;
+    JANUS_CUDA_CHECK(attributes.run([&] {
+        const int bytes = static_cast<int>(smem);
+        cudaError_t e = cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }));
     std::lock_guard<std::mutex> lock(mu);
     int (&k)[LP_MAX_SPLIT + 1] = known[dev];
     if (k[1] == 0) {
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_latent_pair_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         for (int s = LP_MAX_SPLIT; s >= 1; --s) {
             cudaLaunchAttribute attr;
             const cudaLaunchConfig_t cfg = lp_occupancy_config(2 * s, 148, smem, &attr);

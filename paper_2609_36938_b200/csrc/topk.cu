@@ -206,13 +206,13 @@ static int topk_cluster_size(int64_t rows, double n) {
     return 1;
 }
 
-// Kernel attributes and the number of resident CTAs, asked for on a device's first call.
+// Kernel attributes, set once in every context, and the number of resident CTAs, a property of the device.
 struct TopkDevice {
     int resident = 0, resident_small = 0;
 };
 static cudaError_t topk_device(TopkDevice& d) {
-    static once_per_device once;
-    static TopkDevice known[64];
+    static once_per_context once;
+    static std::atomic<int> resident[64], resident_small[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -230,11 +230,12 @@ static cudaError_t topk_device(TopkDevice& d) {
         limit(reinterpret_cast<const void*>(topk_ragged_kernel<false>), smem);
         if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, topk_rows_kernel<TK_CAP>, TK_THREADS, smem);
         if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_small, topk_rows_kernel<TK_CAP_SMALL>, TK_THREADS, smem_small);
-        known[dev].resident = std::max(1, per) * n_sm;
-        known[dev].resident_small = std::max(1, per_small) * n_sm;
+        resident[dev] = std::max(1, per) * n_sm;
+        resident_small[dev] = std::max(1, per_small) * n_sm;
         return r;
     });
-    d = known[dev];
+    d.resident = resident[dev];
+    d.resident_small = resident_small[dev];
     return e;
 }
 

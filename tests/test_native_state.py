@@ -1,0 +1,76 @@
+"""What the library keeps between calls: kernel attributes, set once in every CUDA context, however many threads make the first call."""
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+from paper_2609_36938_b200 import build
+
+
+def test_a_first_call_from_many_threads_runs_once_and_is_waited_for(tmp_path):
+    src = tmp_path / "once.cu"
+    src.write_text(textwrap.dedent("""
+        #include <chrono>
+        #include <thread>
+        #include <vector>
+        #include "janus_common.cuh"
+        uint64_t janus::current_context_id() { return 0; }
+        int main() {
+            janus::once_per_context once;
+            std::atomic<int> runs{0}, early{0};
+            int value[3] = {0, 0, 0};                       // plain memory: visible to whoever has returned from run_in
+            std::vector<std::thread> threads;
+            for (int i = 0; i < 24; ++i)
+                threads.emplace_back([&, i] {
+                    const int c = i % 3;
+                    once.run_in(100 + c, [&] {
+                        std::this_thread::sleep_for(std::chrono::milliseconds(20));
+                        ++runs;
+                        value[c] = 1;
+                        return cudaSuccess;
+                    });
+                    if (value[c] != 1) ++early;
+                });
+            for (auto& t : threads) t.join();
+            for (int i = 0; i < 2; ++i) once.run_in(0, [&] { ++runs; return cudaSuccess; });        // no context yet: nothing to remember
+            for (int i = 0; i < 2; ++i) once.run_in(7, [&] { ++runs; return i == 0 ? cudaErrorUnknown : cudaSuccess; });      // a failure is not remembered
+            once.run_in(7, [&] { ++runs; return cudaSuccess; });
+            return runs == 7 && early == 0 ? 0 : 1;
+        }
+    """))
+    exe = tmp_path / "once"
+    subprocess.check_call([build._nvcc(), "-std=c++17", "-I", build.CSRC, str(src), "-o", str(exe)])
+    assert subprocess.run([str(exe)]).returncode == 0
+
+
+@pytest.mark.gpu
+def test_calls_work_in_every_context_of_a_device():
+    """The C library in a process with two contexts on one device, without torch: each needs the kernels' attributes."""
+    build.build()
+    script = textwrap.dedent("""
+        import ctypes, struct, sys
+        cu, lib = ctypes.CDLL("libcuda.so.1"), ctypes.CDLL(sys.argv[1])
+        def ck(r):
+            assert r == 0, r
+        ck(cu.cuInit(0))
+        dev, primary, second = ctypes.c_int(), ctypes.c_void_p(), ctypes.c_void_p()
+        ck(cu.cuDeviceGet(ctypes.byref(dev), 0))
+        ck(cu.cuDevicePrimaryCtxRetain(ctypes.byref(primary), dev))
+        ck(cu.cuCtxCreate_v2(ctypes.byref(second), 0, dev))
+        lib.janus_topk.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_int64, ctypes.c_int64, ctypes.c_int, ctypes.c_int] + [ctypes.c_void_p] * 4 + [ctypes.c_size_t] + [ctypes.c_void_p] * 2
+        n, k = 10000, 5
+        scores = struct.pack(f"{n}f", *[float((i * 7919) % n) for i in range(n)])
+        for ctx in (primary, second, primary):
+            ck(cu.cuCtxSetCurrent(ctx))
+            src, idx = ctypes.c_void_p(), ctypes.c_void_p()
+            ck(cu.cuMemAlloc_v2(ctypes.byref(src), ctypes.c_size_t(4 * n)))
+            ck(cu.cuMemAlloc_v2(ctypes.byref(idx), ctypes.c_size_t(4 * k)))
+            ck(cu.cuMemcpyHtoD_v2(src, scores, ctypes.c_size_t(4 * n)))
+            ck(lib.janus_topk(src, n, 1, n, 0, 0, k, idx, None, None, None, 0, None, None))
+            ck(cu.cuCtxSynchronize())
+            got = (ctypes.c_int * k)()
+            ck(cu.cuMemcpyDtoH_v2(got, idx, ctypes.c_size_t(4 * k)))
+            assert sorted((i * 7919) % n for i in got) == list(range(n - k, n)), list(got)
+    """)
+    subprocess.run([sys.executable, "-c", script, build.LIB_PATH], check=True, timeout=120)
