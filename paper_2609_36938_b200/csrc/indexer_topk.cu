@@ -397,22 +397,29 @@ namespace janus {
 
 static __device__ __align__(256) unsigned char ft_static_scratch[JANUS_STATIC_SCRATCH_BYTES];
 
-// Device address of the array on the device that is current now, looked up the first time that device is seen.
+// Address of the array in the context that is current now, looked up the first time that context is seen (every context has an array of
+// its own).
 static int static_scratch_address(void** out) {
-    constexpr int MAX_DEVICES = 64;
+    constexpr int MAX_CONTEXTS = 64;
     static std::mutex mu;
-    static void* address[MAX_DEVICES] = {};
-    int dev = -1;
-    JANUS_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= MAX_DEVICES) return JANUS_ERR_UNSUPPORTED;
+    static uint64_t id[MAX_CONTEXTS] = {};
+    static void* address[MAX_CONTEXTS] = {};
+    const uint64_t now = current_context_id();
     std::lock_guard<std::mutex> lock(mu);
-    if (address[dev] == nullptr) {
-        void* ptr = nullptr;
-        JANUS_CUDA_CHECK(cudaGetSymbolAddress((void**)&ptr, ft_static_scratch));
-        if (ptr == nullptr || !aligned16(ptr)) return JANUS_ERR_CUDA;
-        address[dev] = ptr;
+    int i = 0;
+    while (i < MAX_CONTEXTS && id[i] != 0 && id[i] != now) ++i;
+    if (now != 0 && i < MAX_CONTEXTS && id[i] == now) {
+        *out = address[i];
+        return JANUS_OK;
     }
-    *out = address[dev];
+    void* ptr = nullptr;
+    JANUS_CUDA_CHECK(cudaGetSymbolAddress((void**)&ptr, ft_static_scratch));
+    if (ptr == nullptr || !aligned16(ptr)) return JANUS_ERR_CUDA;
+    if (now != 0 && i < MAX_CONTEXTS) {
+        id[i] = now;
+        address[i] = ptr;
+    }
+    *out = ptr;
     return JANUS_OK;
 }
 

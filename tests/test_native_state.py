@@ -59,6 +59,8 @@ def test_calls_work_in_every_context_of_a_device():
         ck(cu.cuDevicePrimaryCtxRetain(ctypes.byref(primary), dev))
         ck(cu.cuCtxCreate_v2(ctypes.byref(second), 0, dev))
         lib.janus_topk.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_int64, ctypes.c_int64, ctypes.c_int, ctypes.c_int] + [ctypes.c_void_p] * 4 + [ctypes.c_size_t] + [ctypes.c_void_p] * 2
+        lib.janus_indexer_topk_static.argtypes = [ctypes.c_void_p, ctypes.c_int64] * 2 + [ctypes.c_void_p] * 2 + [ctypes.c_int64] + [ctypes.c_void_p] * 3 + [
+            ctypes.c_int] * 3 + [ctypes.c_int64] * 2 + [ctypes.c_int] * 3 + [ctypes.c_void_p] * 5
         n, k = 10000, 5
         scores = struct.pack(f"{n}f", *[float((i * 7919) % n) for i in range(n)])
         for ctx in (primary, second, primary):
@@ -72,5 +74,17 @@ def test_calls_work_in_every_context_of_a_device():
             got = (ctypes.c_int * k)()
             ck(cu.cuMemcpyDtoH_v2(got, idx, ctypes.c_size_t(4 * k)))
             assert sorted((i * 7919) % n for i in got) == list(range(n - k, n)), list(got)
+            # one key of 64 that looks at the query, on the library's own scratch: every context has an array of its own
+            ops, row = ctypes.c_void_p(), [0x3f80] * 64
+            ck(cu.cuMemAlloc_v2(ctypes.byref(ops), ctypes.c_size_t(1 << 16)))
+            ck(cu.cuMemsetD8_v2(ops, 0, ctypes.c_size_t(1 << 16)))
+            q, w, keys = ops.value, ops.value + 4096, ops.value + 8192
+            ck(cu.cuMemcpyHtoD_v2(ctypes.c_uint64(q), struct.pack("256H", *(row * 4)), ctypes.c_size_t(512)))
+            ck(cu.cuMemcpyHtoD_v2(ctypes.c_uint64(w), struct.pack("4f", 1, 1, 1, 1), ctypes.c_size_t(16)))
+            ck(cu.cuMemcpyHtoD_v2(ctypes.c_uint64(keys + 128 * 37), struct.pack("64H", *row), ctypes.c_size_t(128)))
+            ck(lib.janus_indexer_topk_static(q, 256, keys, 64, w, None, 0, None, None, None, 1, 4, 64, 64, 0, 0, 0, 1, idx, None, None, None, None))
+            ck(cu.cuCtxSynchronize())
+            ck(cu.cuMemcpyDtoH_v2(got, idx, ctypes.c_size_t(4)))
+            assert got[0] == 37, got[0]
     """)
     subprocess.run([sys.executable, "-c", script, build.LIB_PATH], check=True, timeout=120)
