@@ -9,15 +9,13 @@
 // indices are marked by the whole chip first (page_mark_kernel, one bitmap of *logical* pages per CTA, so that an index costs
 // one shared-memory test and the page table is read once per page and CTA), and the same kernel then only makes the lists.
 #include "janus_common.cuh"
+#include "page_demand_plan.h"
 #include "sm100_ptx.cuh"
 
 namespace janus {
 
 using namespace ptx;
 
-constexpr int PD_THREADS = 1024;
-constexpr int PD_MAX_CLUSTER = 16;
-constexpr int PD_SMEM_WORDS = PD_MAX_CLUSTER * PD_THREADS;      // private bitmap of a CTA: up to 64 KB, half a million pages
 constexpr int MARK_THREADS = 1024;
 constexpr int MARK_SMEM_WORDS = 24576;             // bitmaps of logical and physical pages of a marking CTA together: 96 KB, two CTAs per SM
 
@@ -404,7 +402,7 @@ __global__ void page_union_kernel(uint32_t* __restrict__ dst, const uint32_t* sr
 }
 
 template <int MODE>
-static int launch_page_demand(const PdParams& p, int cluster, cudaStream_t stream) {
+static int launch_page_demand(const PdParams& p, const PdPlan& plan, cudaStream_t stream) {
     const size_t smem = MODE == PD_LISTS ? 0 : sizeof(uint32_t) * static_cast<size_t>(p.n_words);
     static once_per_context attributes;
     JANUS_CUDA_CHECK(attributes.run([] {
@@ -413,23 +411,55 @@ static int launch_page_demand(const PdParams& p, int cluster, cudaStream_t strea
             e = cudaFuncSetAttribute(page_demand_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PD_SMEM_WORDS * static_cast<int>(sizeof(uint32_t)));
         return e;
     }));
-    JANUS_CUDA_CHECK(launch_kernel(page_demand_kernel<MODE>, dim3(cluster), PD_THREADS, smem, stream, cluster, p));
+    JANUS_CUDA_CHECK(launch_kernel(page_demand_kernel<MODE>, dim3(plan.cluster), PD_THREADS, smem, stream, plan.cluster, p));
     return JANUS_OK;
 }
 
-// One launch of one cluster while it reads the indices as fast as memset, chip-wide marking and lists would (12.4 us up to 512 K
-// indices): 128 K indices in 9.6 us, 256 K in 12.3, 512 K in 17.4.  Four CTAs up to 8 K indices (7.1 us; eight and sixteen cost 0.1 and 0.3 us more),
-// sixteen beyond (256 x 256 8.0 us against 10.7 with four and 8.6 with eight, 12 decode rows 8.4, 10.5 and 9.1, 64 rows of a 131136-page
-// pool 17.1, 26.4 and 26.4).
-constexpr int64_t PD_ONE_LAUNCH_INDICES = 1 << 17;
+// CTAs of the largest cluster that the device takes: clusters above eight are not granted everywhere (a part of a GPU may have fewer
+// SMs side by side).  A property of the device, asked for on its first call.
+static cudaError_t largest_cluster(int& largest) {
+    static once_per_context once;
+    static std::atomic<int> known[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) {
+        largest = PD_PORTABLE_CLUSTER;
+        return cudaSuccess;
+    }
+    e = once.run([&] {
+        cudaError_t r = cudaFuncSetAttribute(page_demand_kernel<PD_MARK>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (r == cudaSuccess)
+            r = cudaFuncSetAttribute(page_demand_kernel<PD_MARK>, cudaFuncAttributeMaxDynamicSharedMemorySize, PD_SMEM_WORDS * static_cast<int>(sizeof(uint32_t)));
+        if (r != cudaSuccess) return r;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = PD_MAX_CLUSTER;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(PD_MAX_CLUSTER);
+        cfg.blockDim = dim3(PD_THREADS);
+        cfg.dynamicSmemBytes = sizeof(uint32_t) * PD_SMEM_WORDS;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, page_demand_kernel<PD_MARK>, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        known[dev] = n > 0 ? PD_MAX_CLUSTER : PD_PORTABLE_CLUSTER;
+        return cudaSuccess;
+    });
+    largest = known[dev];
+    return e;
+}
 
 template <int MODE>
 static int run_page_demand(const PdParams& p, cudaStream_t stream) {
-    if (p.n_idx <= PD_ONE_LAUNCH_INDICES && p.n_words <= PD_SMEM_WORDS) {
-        int cluster = p.n_idx <= 8192 ? 4 : 16;
-        while (p.n_words > cluster * PD_THREADS) cluster *= 2;      // a slice is one chunk
-        return launch_page_demand<MODE>(p, cluster, stream);
-    }
+    int largest = 0;
+    JANUS_CUDA_CHECK(largest_cluster(largest));
+    const PdPlan plan = page_demand_plan(p.n_idx, p.n_words, largest);
+    if (plan.one_launch) return launch_page_demand<MODE>(p, plan, stream);
     JANUS_CUDA_CHECK(cudaMemsetAsync(p.bitmap, 0, sizeof(uint32_t) * p.n_words, stream));
     const int64_t n_log_words = (p.n_logical_pages + 31) / 32;
     if (MODE == PD_MARK && n_log_words + p.n_words <= MARK_SMEM_WORDS) {
@@ -446,7 +476,7 @@ static int run_page_demand(const PdParams& p, cudaStream_t stream) {
         JANUS_CUDA_CHECK(launch_kernel(page_mark_global_kernel<MODE>, dim3(static_cast<unsigned>(want < 148 * 8 ? want : 148 * 8)), 256, 0, stream, 1,
                                        p));
     }
-    return launch_page_demand<PD_LISTS>(p, p.n_words <= 8 * PD_THREADS ? 8 : 16, stream);     // 131136 pages: 27.5 us with 16, 32.7 with 8; 2112 pages: 14.4 with 8, 16.5 with 16
+    return launch_page_demand<PD_LISTS>(p, plan, stream);
 }
 
 static int page_shift_of(int page_size) {

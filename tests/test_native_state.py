@@ -88,3 +88,26 @@ def test_calls_work_in_every_context_of_a_device():
             assert got[0] == 37, got[0]
     """)
     subprocess.run([sys.executable, "-c", script, build.LIB_PATH], check=True, timeout=120)
+
+
+def test_page_demand_plan_keeps_to_the_clusters_of_the_device(tmp_path):
+    """The rule that sizes page demand launches: no cluster above what the device takes, a slice of one chunk where marking needs it."""
+    src = tmp_path / "plan.cpp"
+    src.write_text(textwrap.dedent("""
+        #include "page_demand_plan.h"
+        using namespace janus;
+        int main() {
+            const int64_t idx[] = {0, 1, 8192, 8193, 131072, 131073, 1 << 26};
+            for (int largest = 8; largest <= 16; largest += 8)
+                for (int64_t n_idx : idx)
+                    for (int64_t w = 1; w < (int64_t(1) << 26); w += 1 + w / 7) {
+                        const PdPlan p = page_demand_plan(n_idx, static_cast<int>(w), largest);
+                        if (p.cluster > largest || p.cluster < 4) return 1;
+                        if (p.one_launch && (w > p.cluster * PD_THREADS || n_idx > PD_ONE_LAUNCH_INDICES)) return 2;
+                    }
+            return 0;
+        }
+    """))
+    exe = tmp_path / "plan"
+    subprocess.check_call(["g++", "-std=c++17", "-I", build.CSRC, str(src), "-o", str(exe)])
+    assert subprocess.run([str(exe)]).returncode == 0
