@@ -7,7 +7,8 @@
 // bitmap in shared memory, the cluster ORs the bitmaps slice by slice through distributed shared memory, and each CTA
 // turns its slice of the set into its part of the lists, offsets coming from one exchange of the CTAs' counts.  Larger blocks of
 // indices are marked by the whole chip first (page_mark_kernel, one bitmap of *logical* pages per CTA, so that an index costs
-// one shared-memory test and the page table is read once per page and CTA), and the same kernel then only makes the lists.
+// one shared-memory test and the page table is read once per page and CTA), and the same kernel then only makes the lists, for large pools
+// in several clusters.  Which of them, and how many CTAs: page_demand_plan.h.
 #include "janus_common.cuh"
 #include "page_demand_plan.h"
 #include "sm100_ptx.cuh"
@@ -154,7 +155,10 @@ page_mark_global_kernel(const PdParams p) {
 struct PdShared {
     uint64_t warp_sums[2][33];
     uint64_t totals[2];                       // this CTA's slice: the set, the miss set
-    uint64_t before[2], all[2];               // the slices before it, all slices
+    uint64_t before[2], all[2];               // the slices before it, all slices up to the cluster's end
+    // with several clusters: this CTA's share of the counts before the cluster and of the last run start there, and those of all CTAs
+    uint64_t earlier[2], upto[2];
+    int last_start[2], open_start[2], last_of_warp[2][32];
     uint64_t at[2][PD_THREADS];               // counts before each word of a chunk
     uint32_t word[2][PD_THREADS + 2];         // the words of a chunk and one neighbour on either side
 };
@@ -199,8 +203,13 @@ page_demand_kernel(const PdParams p) {
     __shared__ PdShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = static_cast<int>(cluster_ctarank()), n_cta = static_cast<int>(cluster_nctarank());
-    const int wps = (p.n_words + n_cta - 1) / n_cta;        // words of a slice; at most one chunk of PD_THREADS in the marking modes
-    const int w0 = min(p.n_words, rank * wps), w1 = min(p.n_words, w0 + wps);
+    // words of a CTA's slice; at most one chunk of PD_THREADS in the marking modes, which are one cluster
+    const int wps = (p.n_words + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
+    const int w0 = static_cast<int>(min(static_cast<int64_t>(p.n_words), static_cast<int64_t>(blockIdx.x) * wps)), w1 = min(p.n_words, w0 + wps);
+    // the cluster's words [c_begin, c_end)
+    const int64_t first_cta = static_cast<int64_t>(blockIdx.x) - rank;
+    const int c_begin = MODE == PD_LISTS ? static_cast<int>(min(static_cast<int64_t>(p.n_words), first_cta * wps)) : 0;
+    const int c_end = MODE == PD_LISTS ? static_cast<int>(min(static_cast<int64_t>(p.n_words), (first_cta + n_cta) * wps)) : p.n_words;
 
     grid_launch_next();
     if constexpr (MODE != PD_LISTS) {
@@ -323,6 +332,36 @@ page_demand_kernel(const PdParams p) {
         block_scan2_u64(mine, sh.warp_sums, excl, sum);
     }
     if (tid == 0) { sh.totals[0] = sum[0]; sh.totals[1] = sum[1]; }
+    // Later clusters count what lies before them by themselves, a share of the words per CTA (clusters do not wait for one another), and
+    // note the last run start, of which a run that reaches into the cluster's words needs its length.
+    const bool later = MODE == PD_LISTS && c_begin > 0;
+    auto miss_word = [&](int i, uint32_t v) -> uint32_t { return v == 0u || p.predicted == nullptr ? v : v & ~__ldcg(p.predicted + i); };
+    if (later) {
+        uint64_t part[2] = {0, 0}, dummy[2], before[2];
+        int last[2] = {-1, -1};
+        for (int i = rank * PD_THREADS + tid; i < c_begin; i += n_cta * PD_THREADS) {
+            const uint32_t v0 = union_word(i), u0 = union_word(i - 1);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (q == 1 && !want_miss) break;
+                const uint32_t v = q ? miss_word(i, v0) : v0, u = q ? miss_word(i - 1, u0) : u0;
+                const uint32_t starts = v & ~((v << 1) | (u >> 31));
+                part[q] += static_cast<uint64_t>(__popc(v)) << 32 | static_cast<uint64_t>(__popc(starts));
+                if (starts != 0u) last[q] = i * 32 + 31 - __clz(starts);
+            }
+        }
+        block_scan2_u64(part, sh.warp_sums, dummy, before);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            last[q] = __reduce_max_sync(0xffffffffu, last[q]);
+            if (lane == 0) sh.last_of_warp[q][warp] = last[q];
+        }
+        __syncthreads();
+        if (warp < 2) {
+            const int m = __reduce_max_sync(0xffffffffu, sh.last_of_warp[warp][lane]);
+            if (lane == 0) { sh.earlier[warp] = before[warp]; sh.last_start[warp] = m; }
+        }
+    }
     cluster_sync_all();                   // counts are there; nobody reads the private bitmaps any more
     // Warp 0 fetches everybody's counts, lane r those of CTA r: from all 32 warps they were a thousand small remote loads per CTA, which
     // took 4 us with sixteen CTAs.
@@ -330,13 +369,20 @@ page_demand_kernel(const PdParams p) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             uint64_t x = lane < n_cta ? ld_cluster_u64(mapa_shared(smem_u32(&sh.totals[q]), lane)) : 0;
-            uint64_t y = lane < rank ? x : 0;
+            uint64_t y = lane < rank ? x : 0, z = 0;
+            int last = -1;
+            if (later && lane < n_cta) {
+                z = ld_cluster_u64(mapa_shared(smem_u32(&sh.earlier[q]), lane));
+                last = static_cast<int>(ld_cluster_u32(mapa_shared(smem_u32(&sh.last_start[q]), lane)));
+            }
 #pragma unroll
             for (int d = PD_MAX_CLUSTER / 2; d > 0; d >>= 1) {
                 x += __shfl_xor_sync(0xffffffffu, x, d);
                 y += __shfl_xor_sync(0xffffffffu, y, d);
+                if (later) z += __shfl_xor_sync(0xffffffffu, z, d);
             }
-            if (lane == 0) { sh.all[q] = x; sh.before[q] = y; }
+            if (later) last = __reduce_max_sync(0xffffffffu, last);
+            if (lane == 0) { sh.upto[q] = z; sh.all[q] = x + z; sh.before[q] = y + z; sh.open_start[q] = last; }
         }
     }
     __syncthreads();
@@ -383,11 +429,19 @@ page_demand_kernel(const PdParams p) {
     for (int q = 0; q < 2; ++q) {
         if (q == 1 && !want_miss) break;
         int32_t* runs = q ? p.miss_runs : p.runs;
+        // The runs that end in the cluster's words: one may have begun before them, and one may go on after them.
+        auto open_at = [&](int i) {       // page 32 i belongs to the run of the page before it
+            if (MODE != PD_LISTS || i <= 0 || i >= p.n_words) return false;
+            const uint32_t u = union_word(i - 1), v = union_word(i);
+            return ((q ? miss_word(i - 1, u) : u) >> 31) != 0u && ((q ? miss_word(i, v) : v) & 1u) != 0u;
+        };
+        const bool begun = later && open_at(c_begin);
         const int64_t n_runs = static_cast<int64_t>(sh.all[q] & 0xffffffffu), n_ids = static_cast<int64_t>(sh.all[q] >> 32);
-        const int64_t n = n_runs < p.capacity ? n_runs : p.capacity;
-        for (int64_t j = static_cast<int64_t>(rank) * PD_THREADS + tid; j < n; j += static_cast<int64_t>(n_cta) * PD_THREADS)
-            runs[2 * j + 1] = __ldcg(runs + 2 * j + 1) - __ldcg(runs + 2 * j);
-        if (rank == 0 && tid == 0) {
+        const int64_t j_begin = later ? static_cast<int64_t>(sh.upto[q] & 0xffffffffu) - (begun ? 1 : 0) : 0;
+        const int64_t j_end = min(n_runs - (open_at(c_end) ? 1 : 0), p.capacity);
+        for (int64_t j = j_begin + static_cast<int64_t>(rank) * PD_THREADS + tid; j < j_end; j += static_cast<int64_t>(n_cta) * PD_THREADS)
+            runs[2 * j + 1] = __ldcg(runs + 2 * j + 1) - (begun && j == j_begin ? sh.open_start[q] : __ldcg(runs + 2 * j));
+        if (c_end == p.n_words && c_begin < c_end && rank == 0 && tid == 0) {
             *(q ? p.n_miss : p.n_pages) = static_cast<int32_t>(n_ids);
             *(q ? p.n_miss_runs : p.n_runs) = static_cast<int32_t>(n_runs);
             if (n_ids > p.capacity || n_runs > p.capacity) report(p.dev_status, JANUS_DEV_CAPACITY_EXCEEDED);
@@ -411,7 +465,7 @@ static int launch_page_demand(const PdParams& p, const PdPlan& plan, cudaStream_
             e = cudaFuncSetAttribute(page_demand_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PD_SMEM_WORDS * static_cast<int>(sizeof(uint32_t)));
         return e;
     }));
-    JANUS_CUDA_CHECK(launch_kernel(page_demand_kernel<MODE>, dim3(plan.cluster), PD_THREADS, smem, stream, plan.cluster, p));
+    JANUS_CUDA_CHECK(launch_kernel(page_demand_kernel<MODE>, dim3(plan.cluster * plan.clusters), PD_THREADS, smem, stream, plan.cluster, p));
     return JANUS_OK;
 }
 

@@ -8,27 +8,37 @@ namespace janus {
 constexpr int PD_THREADS = 1024;
 constexpr int PD_MAX_CLUSTER = 16;
 constexpr int PD_PORTABLE_CLUSTER = 8;
-constexpr int PD_SMEM_WORDS = PD_MAX_CLUSTER * PD_THREADS;      // private bitmap of a CTA: up to 64 KB, half a million pages
+constexpr int PD_SMEM_WORDS = PD_PORTABLE_CLUSTER * PD_THREADS;      // private bitmap of a marking CTA: up to 32 KB, 262144 pages
+constexpr int PD_MAX_CLUSTERS = 64;
+constexpr int PD_FEW_WORDS = 256;
 
 // One launch of one cluster while it reads the indices as fast as memset, chip-wide marking and lists would (12.4 us up to 512 K
-// indices): 128 K indices in 9.6 us, 256 K in 12.3, 512 K in 17.4.
+// indices): 128 K indices in 9.6 us, 256 K in 12.3, 512 K in 17.4; and while its lists are as fast as those of several clusters: 131072
+// indices of 524288 pages 38.0 us in one launch, 20.4 without.
 constexpr int64_t PD_ONE_LAUNCH_INDICES = 1 << 17;
 
 struct PdPlan {
     bool one_launch;      // marking and lists by one cluster; otherwise the whole chip marks first
-    int cluster;          // CTAs of the cluster of page_demand_kernel
+    int cluster;          // CTAs of a cluster of page_demand_kernel
+    int clusters;         // of the lists
 };
 
 // `largest`: CTAs of the largest cluster that the device takes (8 always, 16 on a whole B200).
 inline PdPlan page_demand_plan(int64_t n_idx, int n_words, int largest) {
-    // Four CTAs up to 8 K indices (7.1 us; eight and sixteen cost 0.1 and 0.3 us more), sixteen beyond (256 x 256 8.0 us against 10.7 with
-    // four and 8.6 with eight, 12 decode rows 8.4, 10.5 and 9.1, 64 rows of a 131136-page pool 17.1, 26.4 and 26.4).
-    if (n_idx <= PD_ONE_LAUNCH_INDICES && n_words <= largest * PD_THREADS) {
-        int cluster = n_idx <= 8192 ? 4 : largest;
-        while (n_words > cluster * PD_THREADS) cluster *= 2;      // a slice is one chunk
-        return {true, cluster};
-    }
-    return {false, n_words <= PD_PORTABLE_CLUSTER * PD_THREADS ? PD_PORTABLE_CLUSTER : largest};      // 2112 pages: 14.4 us with 8, 16.5 with 16
+    // A CTA's slice of the set is one chunk, PD_THREADS words.  Four CTAs for few indices in a small pool (2048 indices of 512 pages 7.4 us, of
+    // 4096 pages 7.7; eight and sixteen cost 0.1 and 0.3 us more), all the device takes beyond: 256 x 256 indices 8.0 us against 10.7 with four
+    // and 8.6 with eight; 2048 indices of 16384 pages 8.2 against 9.6 with four, of 131072 pages 11.8 against 19.1.
+    if (n_idx <= PD_ONE_LAUNCH_INDICES && n_words <= PD_SMEM_WORDS)
+        return {true, n_idx <= 8192 && n_words <= PD_FEW_WORDS ? 4 : largest, 1};
+    // Lists alone: 2112 pages 14.4 us with a cluster of 8, 16.5 with 16; larger pools are shared by clusters, which count what lies before
+    // them: up to four while each CTA has 256 words, then as many as give each one chunk.  524288 indices of 500000 pages 43.2 us with one
+    // cluster, 30.0 with four; 131072 of 1048576 pages 55.6, 31.8, 23.5 and 29.3 with one, two, four and eight; of 2097152 pages 88 with one,
+    // 29.3 with four and 35.7 with eight.
+    if (n_words <= PD_FEW_WORDS) return {false, PD_PORTABLE_CLUSTER, 1};
+    const auto shares = [&](int64_t words) { return (n_words + words * largest - 1) / (words * largest); };
+    int64_t n = shares(256) < 4 ? shares(256) : 4;
+    if (n < shares(PD_THREADS)) n = shares(PD_THREADS);
+    return {false, largest, n < PD_MAX_CLUSTERS ? static_cast<int>(n) : PD_MAX_CLUSTERS};
 }
 
 }  // namespace janus

@@ -81,3 +81,28 @@ def test_page_demand_batch_edges(n_rows, k):
     want = sorted(set().union(*[O.page_demand(idx[r:r + 1], int(limits[r]), page, tables[off[r]:off[r + 1]])["pages"] for r in range(n_rows)]))
     got = Hp.page_lists_from_device(pd)
     assert got["pages"] == want and got["runs"] == [tuple(r) for r in O.maximal_runs(want)] and got["miss"] == want
+
+
+def test_runs_across_the_clusters_of_a_large_pool():
+    """Lists of a pool that several clusters share (four, of 16 x 831 words each): runs that cross from one cluster into the next, that end
+    or begin on the boundary, and a miss set with other runs."""
+    n_phys, step = 1_700_000, 16 * 831 * 32
+    here = np.ones(n_phys, bool)
+    here[[5, 2 * step, 3 * step - 1, n_phys - 40]] = False
+    here[n_phys - 1000:n_phys - 900] = False
+    known = np.zeros(n_phys, bool)
+    known[[step - 70, 2 * step - 1, n_phys - 1]] = True
+    known[3 * step:3 * step + 500] = True
+    idx = np.flatnonzero(here).astype(np.int32)
+    idx = np.concatenate([idx, np.full(-len(idx) % 2048, -1, np.int32)]).reshape(-1, 2048)
+    pd = B.janus_page_demand(dev32(idx), demand_limit=n_phys, page_size=1, page_table=dev32(np.arange(n_phys)), n_phys_pages=n_phys,
+                             predicted_bitmap=torch.from_numpy(bitmap_of(np.flatnonzero(known), n_phys)).cuda())
+    B.check_dev_status()
+    for want, n, n_runs, ids, runs in ((here, 0, 1, "pages", "runs"), (here & ~known, 2, 3, "miss_pages", "miss_runs")):
+        pages = np.flatnonzero(want)
+        cut = np.flatnonzero(np.diff(pages) > 1)
+        first, last = np.concatenate([[0], cut + 1]), np.concatenate([cut, [len(pages) - 1]])
+        counts = pd["counts"].cpu().numpy()
+        assert counts[n] == len(pages) and counts[n_runs] == len(first)
+        assert np.array_equal(pd[ids][:len(pages)].cpu().numpy(), pages)
+        assert np.array_equal(pd[runs][:len(first)].cpu().numpy(), np.stack([pages[first], pages[last] - pages[first] + 1], 1))

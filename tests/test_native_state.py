@@ -102,8 +102,9 @@ def test_page_demand_plan_keeps_to_the_clusters_of_the_device(tmp_path):
                 for (int64_t n_idx : idx)
                     for (int64_t w = 1; w < (int64_t(1) << 26); w += 1 + w / 7) {
                         const PdPlan p = page_demand_plan(n_idx, static_cast<int>(w), largest);
-                        if (p.cluster > largest || p.cluster < 4) return 1;
-                        if (p.one_launch && (w > p.cluster * PD_THREADS || n_idx > PD_ONE_LAUNCH_INDICES)) return 2;
+                        if (p.cluster > largest || p.cluster < 4 || p.clusters < 1 || p.clusters > PD_MAX_CLUSTERS) return 1;
+                        if (p.one_launch && (p.clusters != 1 || w > p.cluster * PD_THREADS || n_idx > PD_ONE_LAUNCH_INDICES)) return 2;
+                        if (!p.one_launch && p.clusters < PD_MAX_CLUSTERS && w > int64_t(p.cluster) * p.clusters * PD_THREADS) return 3;
                     }
             return 0;
         }
