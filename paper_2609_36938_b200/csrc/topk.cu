@@ -94,16 +94,16 @@ __global__ void entry_expand_kernel(const int32_t* idx_e, int M, int k_e, int en
 // Pooled entry scores (the second reading of the entry footnote of Sec. 2.2): an entry scores as the best of its tokens the
 // row may see.  Bound by the bytes of the score matrix.
 //
-// Entries of 4, 8, .. 128 tokens in 16-byte aligned rows: a warp takes 1024 consecutive scores with eight 16-byte loads per lane,
+// Entries of 4, 8, .. 128 tokens in 16-byte aligned rows: a warp takes 128 U consecutive scores with U 16-byte loads per lane,
 // all in flight together; ENTRY / 4 neighbouring lanes hold an entry of each load.  512 rows x 40512 in entries of 128: 32.8 us with
 // a warp per entry (four 4-byte loads and a 64-bit division each), 19 us so; entries of 16 tokens 200 and 18.
-template <int ENTRY>
+template <int ENTRY, int U>
 __global__ void __launch_bounds__(256)
 entry_pool_vec_kernel(const float* scores, int64_t ld, int M, int64_t n_keys, int64_t q_pos0, int causal, int n_entries,
                       float* __restrict__ out, int64_t out_ld) {
     grid_launch_next();
     grid_wait();
-    constexpr int U = 8, LANES = ENTRY / 4, STRIP = 128 * U;
+    constexpr int LANES = ENTRY / 4, STRIP = 128 * U;
     const int lane = threadIdx.x & 31;
     const int strip = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int64_t s0 = static_cast<int64_t>(strip) * STRIP + 4 * lane;
@@ -268,13 +268,19 @@ extern "C" int janus_entry_pool_scores(const float* scores, int64_t scores_ld, i
     if (!scores || !entry_scores) return JANUS_ERR_INVALID_ARG;
     const cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     if (aligned16(scores) && (scores_ld & 3) == 0 && n_keys < (int64_t(1) << 31) - 8192) {
-        const dim3 grid(static_cast<unsigned>((n_keys + 8 * 1024 - 1) / (8 * 1024)), static_cast<unsigned>(M < 65535 ? M : 65535));
+        // Eight loads per lane keep the most bytes in flight; two while eight would leave the chip short of warps (512 rows of 1000 in
+        // entries of 64 2.3 us against 4.6, 2000 rows of 200 3.8 against 12.9).
+        const bool few = M * ((n_keys + 1023) / 1024) < 148 * 16;
+        const int per_block = 8 * 128 * (few ? 2 : 8);
+        const dim3 grid(static_cast<unsigned>((n_keys + per_block - 1) / per_block), static_cast<unsigned>(M < 65535 ? M : 65535));
         const int n = static_cast<int>(n_entries);
         switch (entry_size) {
 #define JANUS_POOL_CASE(E)                                                                                                                    \
     case E:                                                                                                                                   \
-        JANUS_CUDA_CHECK(launch_kernel(entry_pool_vec_kernel<E>, grid, 256, 0, stream, 1, scores, scores_ld, M, n_keys, q_pos0, causal, n,    \
-                                       entry_scores, entry_ld));                                                                              \
+        if (few) JANUS_CUDA_CHECK(launch_kernel(entry_pool_vec_kernel<E, 2>, grid, 256, 0, stream, 1, scores, scores_ld, M, n_keys, q_pos0,   \
+                                                causal, n, entry_scores, entry_ld));                                                          \
+        else JANUS_CUDA_CHECK(launch_kernel(entry_pool_vec_kernel<E, 8>, grid, 256, 0, stream, 1, scores, scores_ld, M, n_keys, q_pos0,       \
+                                            causal, n, entry_scores, entry_ld));                                                              \
         return JANUS_OK;
             JANUS_POOL_CASE(4)
             JANUS_POOL_CASE(8)
