@@ -15,10 +15,10 @@
 // quadrant, each reducing half of the slot's columns): with four epilogue warps per scheduler one warp's wait for its
 // tensor-memory load or its weights is covered by the others.
 //
-// The launch is persistent: the visible (token group, key tile) pairs, group by group, are cut into as many equal contiguous
-// ranges as CTAs are resident, and a CTA walks its range in segments of one group each.  The key ring, the TMEM slots and
-// their barriers run on across segments; the queries and weights are replaced, which costs about half a tile's time once or
-// twice per CTA.  A grid of fixed chunks left waves unfilled: 2048 rows x 34816 keys 64 x 128 bf16 901 -> 857 us, 777 x 20788 of 32
+// The launch is persistent: the visible (token group, key tile) pairs, group by group, are cut into as many contiguous ranges of equal
+// cost as CTAs are resident, and a CTA walks its range in segments of one group each.  The key ring, the TMEM slots and
+// their barriers run on across segments; the queries and weights are replaced, which costs about three quarters of a tile's time,
+// once or twice per CTA in a long call.  A grid of fixed chunks left waves unfilled: 2048 rows x 34816 keys 64 x 128 bf16 901 -> 857 us, 777 x 20788 of 32
 // heads 121 -> 114, 1024 x 17408 FP8 183 -> 172; 4096 x 135168 FP8, which is on the power limit, 5.26 -> 5.17 ms.  Small launches give
 // every CTA tiles of one group only (MULTI = false).  256 rows x 4352 keys of 4 heads 18.6 -> 8.0 us, with half the sub-tiles per CTA.
 // Every wait is bounded; on a timeout the CTA reports JANUS_DEV_WAIT_TIMEOUT and winds down normally.
@@ -68,7 +68,8 @@ struct TcCandParams {
 // a launch about 0.5 us longer, so small launches do without.
 struct TcSchedule {
     int2 first[TC_MAX_CTAS];
-    int count, longer;                // a range is `count` tiles long, that of the first `longer` CTAs one more
+    uint16_t less[TC_MAX_CTAS];       // tiles that CTA c's range is shorter than the longest
+    int longest;
 };
 struct TcNoSchedule {};
 template <bool TABLE> struct TcScheduleOf { using type = TcSchedule; };
@@ -211,7 +212,7 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     } else {
         g0 = sched.first[blockIdx.x].x;
         tile0 = sched.first[blockIdx.x].y;
-        n_work = sched.count + (static_cast<int>(blockIdx.x) < sched.longer ? 1 : 0);
+        n_work = sched.longest - sched.less[blockIdx.x];
         load_weights(g0, threadIdx.x, TC_THREADS);
     }
     if (warp == 1) {
@@ -560,7 +561,7 @@ int launch_indexer_tc(const void* q_idx, const void* k_idx, int64_t k_stride_tok
     if (p.stages < 2) return JANUS_ERR_UNSUPPORTED;
     const size_t smem = static_cast<size_t>(q_bytes) + static_cast<size_t>(p.stages) * k_stage + tail;
     const int tpc = p.nq * tps;
-    // Few tiles: ranges that end with their group, when the longest is no longer for it (a change of group costs about half a
+    // Few tiles: ranges that end with their group, when the longest is no longer for it (a change of group costs most of a
     // tile's time and the table 0.5 us: 19 rows x 9020 keys 9.5 us with even shares, 8.3 without).
     p.n_groups = (M + tpc - 1) / tpc;
     TcSchedule sched;
@@ -574,16 +575,44 @@ int launch_indexer_tc(const void* q_idx, const void* k_idx, int64_t k_stride_tok
         multi = ctas > TC_MAX_CTAS;
     }
     if (multi) {
+        // Ranges whose tiles, and the changes of group inside them at three quarters of a tile each, cost at most `budget`: the smallest with
+        // which the CTAs get through.  Equal numbers of tiles left the CTAs of a causal call's first groups, which have a tile or two
+        // each, far behind: 4096 rows x 4096 keys without history, 64 heads of bf16 167 -> 125 us, FP8 127 -> 96.5; 300 keys of history 150
+        // -> 139; from 4 K on unchanged.  (A change at a whole tile: the same there, and calls of three to eight tiles per CTA 9 % slower.)
         const int n_ctas = static_cast<int>(grid.x);
-        sched.count = static_cast<int>(work / n_ctas);
-        sched.longer = static_cast<int>(work % n_ctas);
-        int g = 0;
-        int64_t at = 0, before = 0, tiles = tc_visible_tiles(p, tpc, 0);     // tiles before this CTA's range, before group g, and of g
-        for (int c = 0; c < n_ctas; ++c) {
-            while (at >= before + tiles) { before += tiles; tiles = tc_visible_tiles(p, tpc, ++g); }
-            sched.first[c] = make_int2(g, static_cast<int>(at - before));
-            at += sched.count + (c < sched.longer ? 1 : 0);
-        }
+        const int tile_cost = longest < 65536 ? 4 : 1, change_cost = longest < 65536 ? 3 : 0;
+        int used = 0;
+        int64_t counts[TC_MAX_CTAS];
+        auto pack = [&](int64_t budget) {
+            int g = 0;
+            int64_t done = 0, tile = 0, tiles = tc_visible_tiles(p, tpc, 0);
+            for (used = 0; used < n_ctas && done < work; ++used) {
+                sched.first[used] = make_int2(g, static_cast<int>(tile));
+                int64_t left = budget, count = 0;
+                for (;;) {
+                    const int64_t fit = left / tile_cost, take = fit < tiles - tile ? fit : tiles - tile;
+                    tile += take;
+                    count += take;
+                    left -= take * tile_cost;
+                    if (tile < tiles) break;
+                    tile = 0;
+                    tiles = ++g < p.n_groups ? tc_visible_tiles(p, tpc, g) : 0;
+                    left -= change_cost;
+                    if (done + count >= work || left < tile_cost) break;
+                }
+                done += count;
+                counts[used] = count;
+            }
+            return done >= work;
+        };
+        const int64_t inside = p.n_groups > n_ctas ? p.n_groups - n_ctas : 0;      // changes that no cut can avoid
+        int64_t budget = (work * tile_cost + inside * change_cost + n_ctas - 1) / n_ctas, most = 0;
+        if (budget < tile_cost) budget = tile_cost;
+        for (int64_t more = 1 + budget / 512; !pack(budget); ++more) budget += more;
+        for (int c = 0; c < used; ++c) most = counts[c] > most ? counts[c] : most;
+        for (int c = 0; c < used; ++c) sched.less[c] = static_cast<uint16_t>(most - counts[c]);
+        sched.longest = static_cast<int>(most);
+        grid.x = used;
     } else {
         p.tiles_per_cta = static_cast<int>(longest);
         grid = dim3(static_cast<unsigned>((tc_visible_tiles(p, tpc, p.n_groups - 1) + longest - 1) / longest), p.n_groups);

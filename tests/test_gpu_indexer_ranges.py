@@ -1,4 +1,4 @@
-"""How the tensor-core indexer shares its tiles out: ranges inside one token group and across several, one and many tiles per CTA, both sub-tile
+"""How the tensor-core indexer shares its tiles out: ranges inside one token group and across several or many of one tile, one and many tiles per CTA, both sub-tile
 counts, masked tails of rows (ragged ends included), and batches of sessions on either side of the even-share rule, more sessions than
 the block that scans them, empty ones and one-tile ones among them.  Against the oracle; tolerance as in test_gpu_parity.py (fp32 sums of
 exact products)."""
@@ -36,6 +36,7 @@ def operands(rng, n_q, n_k, H, D, dtype):
     (9, 4000, 4009, 64, 128, "bf16", True), (700, 0, 700, 64, 128, "fp8", True), (1300, 129, 1429, 32, 128, "bf16", True),
     (33, 5000, 4777, 64, 128, "fp8", False), (513, 3, 515, 4, 64, "bf16", True), (100, 5000, 5100, 8, 128, "fp8", True),
     (2500, 130, 2630, 64, 64, "bf16", True), (300, 1000, 1203, 16, 128, "bf16", True),
+    (3001, 0, 3001, 64, 128, "bf16", True), (1192, 0, 100, 64, 128, "bf16", True), (2400, 0, 2400, 64, 128, "fp8", True),
 ])
 def test_scores_of_every_range(M, L, n_keys, H, D, dtype, causal):
     rng = np.random.default_rng(M + n_keys)
