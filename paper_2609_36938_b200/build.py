@@ -1,6 +1,7 @@
 """Builds libjanus.so (the C-ABI library) in-tree with nvcc for sm_100a, and _native.so (the native half of binding.py) with g++."""
 from __future__ import annotations
 
+import importlib.metadata
 import importlib.util
 import os
 import shutil
@@ -28,7 +29,15 @@ def _stale() -> bool:
         return True
     t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(NATIVE_PATH))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(PKG_DIR, "..", "include", "janus.h")]
-    return any(os.path.getmtime(d) > t for d in deps)
+    if any(os.path.getmtime(d) > t for d in deps):
+        return True
+    with open(NATIVE_PATH, "rb") as f:
+        return _native_mark().encode() not in f.read()
+
+
+def _native_mark() -> str:
+    """What _native.so is bound to, and carries as a string: torch's C++ interface and the interpreter's."""
+    return f"janus native for torch {importlib.metadata.version('torch')}, {sys.implementation.cache_tag};"
 
 
 def _native_command() -> list:
@@ -36,7 +45,8 @@ def _native_command() -> list:
     torch_dir = list(importlib.util.find_spec("torch").submodule_search_locations)[0]
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
     inc = [os.path.join(torch_dir, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
-    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", *[f"-I{d}" for d in inc], os.path.join(CSRC, "py_binding.cpp"), "-o",
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", *[f"-I{d}" for d in inc],
+            f'-DJANUS_NATIVE_MARK="{_native_mark()}"', os.path.join(CSRC, "py_binding.cpp"), "-o",
             NATIVE_PATH, "-L" + os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda", "-ldl"]
 
 

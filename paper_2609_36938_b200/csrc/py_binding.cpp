@@ -20,6 +20,9 @@
 
 #include "../../include/janus.h"
 
+// read by build.py: the library is built again when torch or the interpreter is another
+extern "C" __attribute__((used, visibility("default"))) const char janus_native_mark[] = JANUS_NATIVE_MARK;
+
 namespace {
 
 // ---- state set once by init(): the C entry points and the Python objects the calls need

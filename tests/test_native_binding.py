@@ -19,6 +19,12 @@ def test_loads_and_counts_its_arguments():
             getattr(native, name)()
 
 
+def test_another_torch_makes_the_build_stale(monkeypatch):
+    assert not build._stale()
+    monkeypatch.setattr(build.importlib.metadata, "version", lambda name: "2.0.0")
+    assert build._stale()
+
+
 def test_sizes_are_whole_numbers_and_errors_keep_their_types():
     """Where a size shapes an output, only a whole number is taken; a missing dimension and a failed allocation raise what torch raises."""
     sc, e = torch.zeros(4, 8), torch.zeros(4, 2, dtype=torch.int32)
