@@ -309,29 +309,25 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + slot * TC_N;
                     const uint64_t qdesc_j = qdesc0 + static_cast<uint64_t>((j * q_sub_bytes) >> 4);
-                    {
-                        uint32_t acc = 0;
-                        for (int a = 0; a < atoms; ++a) {
-                            const uint64_t ka = kdesc_s + static_cast<uint64_t>((a * TC_KEYS * 128) >> 4);
-                            const uint64_t qa = qdesc_j + static_cast<uint64_t>((a * TC_N * 128) >> 4);
+                    uint32_t acc = 0;
+                    for (int a = 0; a < atoms; ++a) {
+                        const uint64_t ka = kdesc_s + static_cast<uint64_t>((a * TC_KEYS * 128) >> 4);
+                        const uint64_t qa = qdesc_j + static_cast<uint64_t>((a * TC_N * 128) >> 4);
 #pragma unroll
-                            for (int ks = 0; ks < 4; ++ks) {   // 32 bytes of K per instruction (16 bf16 or 32 e4m3)
-                                umma<FP8>(d_tmem, ka + 2 * ks, qa + 2 * ks, idesc, acc);
-                                acc = 1;
-                            }
+                        for (int ks = 0; ks < 4; ++ks) {   // 32 bytes of K per instruction (16 bf16 or 32 e4m3)
+                            umma<FP8>(d_tmem, ka + 2 * ks, qa + 2 * ks, idesc, acc);
+                            acc = 1;
                         }
-                        umma_commit(smem_u32(&bars->tmem_full[slot]));
-                        if (j == nq - 1) umma_commit(smem_u32(&bars->k_empty[s]));
                     }
-                    }
+                    umma_commit(smem_u32(&bars->tmem_full[slot]));
+                    if (j == nq - 1) umma_commit(smem_u32(&bars->k_empty[s]));
+                }
             }
             if (!ok) {
                 *aborted = 1;
                 // tensor memory is freed after the barrier below: the instructions already issued finish first
-                {
-                    report(p.dev_status, JANUS_DEV_WAIT_TIMEOUT);
-                    umma_commit(smem_u32(&bars->mma_drain));
-                }
+                report(p.dev_status, JANUS_DEV_WAIT_TIMEOUT);
+                umma_commit(smem_u32(&bars->mma_drain));
                 mbar_wait(smem_u32(&bars->mma_drain), 0);
             }
         }

@@ -353,11 +353,6 @@ __device__ __forceinline__ uint64_t ld_cluster_u64(uint32_t cluster_addr) {
     asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(cluster_addr) : "memory");
     return v;
 }
-__device__ __forceinline__ int4 ld_cluster_s32x4(uint32_t cluster_addr) {
-    int4 v;
-    asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(cluster_addr) : "memory");
-    return v;
-}
 __device__ __forceinline__ int atomic_add_cluster_s32(uint32_t cluster_addr, int v) {
     int old;
     asm volatile("atom.relaxed.cluster.shared::cluster.add.s32 %0, [%1], %2;" : "=r"(old) : "r"(cluster_addr), "r"(v) : "memory");

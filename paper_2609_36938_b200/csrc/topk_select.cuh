@@ -542,6 +542,7 @@ __device__ __forceinline__ void topk_row_cluster(const float* row, int n, int k,
     __syncthreads();
     count_candidates(min(sh.n_cand, Sh::kCap), map, sh);
     __syncthreads();
+    static_assert(Sh::kCap < 0x8000, "a bucket's count and the flag share 16 bits");
     // The counts travel as 16 bits each, four buckets in 8 bytes where the histogram was (its bytes are what the exchange takes); bit 15 of
     // the lowest bucket says that the list was full.
     const int4 own = own_buckets(sh);
