@@ -81,3 +81,36 @@ def test_infinite_values_come_out_as_they_are(M, n_kv, group, d_qk, d_v, k):
     want = np.zeros(d_v)
     want[5], want[d_v - 2] = np.inf, -np.inf
     assert np.array_equal(np.where(np.isfinite(got), 0, got), np.broadcast_to(want, got.shape))
+
+
+@pytest.mark.parametrize("n,n_kv,group,d_qk,d_v,k", [(1, 4, 8, 128, 128, 700), (6, 2, 4, 64, 64, 129), (200, 1, 1, 192, 128, 33)])
+def test_decode_rows_have_tables_of_their_own(n, n_kv, group, d_qk, d_v, k):
+    """One query row per session, each with its own page table and history; a table that starts before the array has no pages (reported)."""
+    rng = np.random.default_rng(n + k)
+    H_q, page = n_kv * group, 32
+    lengths = rng.integers(k, 3 * k, n)
+    pages = (lengths + page - 1) // page
+    off = np.concatenate([[0], np.cumsum(pages)]).astype(np.int64)
+    n_phys = int(off[-1])
+    tables = rng.permutation(n_phys).astype(np.int32)
+    pools = [W.to_bf16_bits((rng.standard_normal((n_phys, page, n_kv, max(d_qk, d_v))) / 4).astype(np.float32)) for _ in range(2)]
+    Q = W.to_bf16_bits(rng.standard_normal((n, H_q, d_qk)).astype(np.float32))
+    idx = np.stack([rng.permutation(int(m))[:k] for m in lengths]).astype(np.int32)
+    idx[rng.random(idx.shape) < 0.1] = -1
+    scale = float(d_qk ** -0.5)
+    args = (B.to_device(Q, "bf16"), B.to_device(pools[0], "bf16"), B.to_device(pools[1], "bf16"), B.to_device(idx, "i32"))
+    out, lse = B.janus_sparse_attn_decode(*args, page_tables=B.to_device(tables, "i32"), table_offsets=torch.from_numpy(off).cuda(), page_size=page,
+                                          softmax_scale=scale, d_v=d_v)
+    B.check_dev_status()
+    for b in sorted({0, n // 2, n - 1}):
+        ref_o, ref_l = O.sparse_attention(Q[b:b + 1], pools[0], pools[1], tables[off[b]:off[b + 1]], idx[b:b + 1], page_size=page, softmax_scale=scale,
+                                          d_qk=d_qk, d_v=d_v)
+        Hp.assert_attention_close(Hp.bf16_tensor_to_f64(out)[b:b + 1], ref_o, f"session {b}")
+        assert np.all(np.abs(lse.cpu().numpy().astype(np.float64)[b] - ref_l[0]) <= 1e-4 * (1 + np.abs(ref_l[0])))
+    bad = off.copy()
+    bad[0] = -1
+    out2, lse2 = B.janus_sparse_attn_decode(*args, page_tables=B.to_device(tables, "i32"), table_offsets=torch.from_numpy(bad).cuda(), page_size=page,
+                                            softmax_scale=scale, d_v=d_v)
+    assert bool((out2[0] == 0).all()) and bool(torch.isneginf(lse2[0]).all()) and torch.equal(out2[1:], out[1:])
+    with pytest.raises(B.JanusError, match="OUT_OF_RANGE"):
+        B.check_dev_status()
