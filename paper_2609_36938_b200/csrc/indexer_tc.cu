@@ -456,8 +456,8 @@ indexer_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
 
 // ---- host side ---------------------------------------------------------------------------------------------
 PFN_encodeTiled get_encode_tiled() {
-    static PFN_encodeTiled fn = nullptr;
-    if (fn == nullptr) {
+    static std::atomic<PFN_encodeTiled> fn{nullptr};
+    if (fn.load() == nullptr) {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult qres;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess)
@@ -477,6 +477,12 @@ bool make_tmap_2d_sw128(CUtensorMap* map, const void* base, int elem_bytes, uint
     // elem_bytes 0: 4-bit elements, 16 of them expanded to a 16-byte aligned shared-memory chunk (box_cols must be 128)
     const CUtensorMapDataType dt = elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                    : elem_bytes == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_16U4_ALIGN16B;
+    // The encoder is a driver call and wants a context on this thread; a thread whose first CUDA call this is has none yet (the runtime's
+    // own calls bring one along).
+    if (current_context_id() == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return false;
+    }
     return enc(map, dt, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
