@@ -2,12 +2,15 @@
 //     scores[t,s] = sum_h w[t,h] * relu(<q[t,h,:], k[s,:]>) + row_bias[t]*col_bias[s],  -inf where masked.
 // Serves the shapes the tensor-core kernel does not (odd head counts, strided queries).  One thread per
 // key; a tile of 128 keys is kept transposed in shared memory and reused by a chunk of query tokens.
+#include <type_traits>
+
 #include "janus_common.cuh"
 
 namespace janus {
 
 constexpr int IG_KEYS = 128;     // keys per CTA (one per thread)
 constexpr int IG_TOKENS = 16;    // query tokens per CTA
+constexpr int IG_MAX_SMEM = 200 * 1024;
 
 template <int DTYPE>
 __device__ __forceinline__ float load_elem(const void* base, int64_t i) {
@@ -77,21 +80,18 @@ int launch_indexer_generic(const void* q_idx, int64_t q_stride_tok, const void* 
                            const float* col_bias, int M, int H, int D, int64_t n_keys, int64_t q_pos0, int causal, int dtype,
                            float* scores, int64_t ld, cudaStream_t stream) {
     const size_t smem = sizeof(float) * (static_cast<size_t>(D) * IG_KEYS + static_cast<size_t>(H) * D);
-    if (smem > 200 * 1024) return JANUS_ERR_UNSUPPORTED;
+    if (smem > IG_MAX_SMEM) return JANUS_ERR_UNSUPPORTED;
     dim3 grid(static_cast<unsigned>((n_keys + IG_KEYS - 1) / IG_KEYS), static_cast<unsigned>((M + IG_TOKENS - 1) / IG_TOKENS));
     if (grid.y > 65535) return JANUS_ERR_UNSUPPORTED;
-    if (dtype == JANUS_DTYPE_BF16) {
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(indexer_generic_kernel<JANUS_DTYPE_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        JANUS_CUDA_CHECK(launch_kernel(indexer_generic_kernel<JANUS_DTYPE_BF16>, grid, IG_KEYS, smem, stream, 1, q_idx, q_stride_tok, k_idx,
-                                       k_stride_tok, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H, D, n_keys, q_pos0, causal,
-                                       scores, ld));
-    } else {
-        JANUS_CUDA_CHECK(cudaFuncSetAttribute(indexer_generic_kernel<JANUS_DTYPE_FP8_E4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        JANUS_CUDA_CHECK(launch_kernel(indexer_generic_kernel<JANUS_DTYPE_FP8_E4M3>, grid, IG_KEYS, smem, stream, 1, q_idx, q_stride_tok, k_idx,
-                                       k_stride_tok, w, q_scale, q_scale_stride_tok, k_scale, row_bias, col_bias, M, H, D, n_keys, q_pos0, causal,
-                                       scores, ld));
-    }
-    return JANUS_OK;
+    auto launch = [&](auto format) -> int {
+        constexpr int DTYPE = decltype(format)::value;
+        static once_per_context attributes;      // the largest size, not this call's: another thread's call may need more
+        JANUS_CUDA_CHECK(attributes.run([] { return cudaFuncSetAttribute(indexer_generic_kernel<DTYPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, IG_MAX_SMEM); }));
+        JANUS_CUDA_CHECK(launch_kernel(indexer_generic_kernel<DTYPE>, grid, IG_KEYS, smem, stream, 1, q_idx, q_stride_tok, k_idx, k_stride_tok, w, q_scale,
+                                       q_scale_stride_tok, k_scale, row_bias, col_bias, M, H, D, n_keys, q_pos0, causal, scores, ld));
+        return JANUS_OK;
+    };
+    return dtype == JANUS_DTYPE_BF16 ? launch(std::integral_constant<int, JANUS_DTYPE_BF16>{}) : launch(std::integral_constant<int, JANUS_DTYPE_FP8_E4M3>{});
 }
 
 }  // namespace janus

@@ -172,7 +172,9 @@ static int launch_g(const void* q, int M, int H_q, int d_qk, const void* k_pool,
     const bool v_alias = (v_pool == k_pool);
     size_t smem = sizeof(uint16_t) * AG_KT * (d_qk + 8) + (v_alias ? 0 : sizeof(uint16_t) * AG_KT * (d_v + 8)) +
                   sizeof(float) * (G * d_qk + G * AG_KT + G) + sizeof(int) * AG_KT;
-    JANUS_CUDA_CHECK(cudaFuncSetAttribute(sparse_attn_generic_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    constexpr int max_smem = static_cast<int>(sizeof(uint16_t) * AG_KT * (576 + 8 + 512 + 8) + sizeof(float) * (G * 576 + G * AG_KT + G) + sizeof(int) * AG_KT);
+    static once_per_context attributes;      // the largest size, not this call's: another thread's call may need more
+    JANUS_CUDA_CHECK(attributes.run([] { return cudaFuncSetAttribute(sparse_attn_generic_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem); }));
     const int heads_per_kv = H_q / n_kv_heads;
     dim3 grid(M, n_kv_heads * ((heads_per_kv + G - 1) / G));
     JANUS_CUDA_CHECK(launch_kernel(sparse_attn_generic_kernel<G>, grid, AG_THREADS, smem, stream, 1, static_cast<const uint16_t*>(q), M, H_q, d_qk,
