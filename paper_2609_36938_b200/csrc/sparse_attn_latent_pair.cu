@@ -83,9 +83,8 @@ struct LpShared {
     uint32_t vmask[LP_SLOTS];
     uint32_t tmem_base;
     uint32_t start_abort[2 * LP_MAX_SPLIT];       // by CTA of the cluster
-    // reference maximum (log2 domain) and row sum of every head, for the merge: -inf and 0 until the pair has left its output
+    // reference maximum (log2 domain) and row sum of every head, for the merge; the sum is negative until the pair has left its output
     float split_m[LP_HEADS], split_l[LP_HEADS];
-    alignas(16) float split_zero[4];
 };
 
 // Keys of one token split over several pairs of a cluster (few query rows): a pair leaves its fp32 output for the merge where its
@@ -137,7 +136,7 @@ __device__ __forceinline__ float4 lp_ld_cluster4(uint32_t addr) {
 // Output of token t from the N pairs' unnormalised outputs: CTA (s, c) takes every N-th block of 16 columns of value half c, a
 // thread one block of one head at a time.  N is a compile-time number so that all remote loads are issued together.
 template <int N>
-__device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s, uint32_t c, uint32_t o_addr, uint32_t m_addr, uint32_t l_addr, uint32_t zero_addr) {
+__device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s, uint32_t c, uint32_t o_addr, uint32_t m_addr, uint32_t l_addr) {
     const int h = threadIdx.x & (LP_HEADS - 1);
     const float neg_inf = __int_as_float(0xff800000);
     float f[N], l[N];
@@ -147,6 +146,9 @@ __device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s,
         f[r] = lp_ld_cluster(mapa_shared(m_addr + 4 * h, 2 * r + c));
         l[r] = lp_ld_cluster(mapa_shared(l_addr + 4 * h, 2 * r + c));
     }
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+        if (l[r] < 0.f) return;      // a pair gave up (reported): what lies in its buffer may be anything, and the row stays unwritten
 #pragma unroll
     for (int r = 0; r < N; ++r) m_all = fmaxf(m_all, f[r]);
 #pragma unroll
@@ -159,12 +161,9 @@ __device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s,
         float4 x[N][4], acc[4] = {};
 #pragma unroll
         for (int r = 0; r < N; ++r) {
-            // a pair without a key, or one that gave up, counts as zeros: what lies in its buffer may be anything, a NaN even
-            const bool empty = f[r] == 0.f;
-            const uint32_t src = empty ? mapa_shared(zero_addr, 2 * s + c) : mapa_shared(o_addr + static_cast<uint32_t>((blk * 4 * LP_HEADS + h) * 16), 2 * r + c);
-            const uint32_t step = empty ? 0u : LP_HEADS * 16u;
+            const uint32_t src = mapa_shared(o_addr + static_cast<uint32_t>((blk * 4 * LP_HEADS + h) * 16), 2 * r + c);
 #pragma unroll
-            for (int v = 0; v < 4; ++v) x[r][v] = lp_ld_cluster4(src + v * step);
+            for (int v = 0; v < 4; ++v) x[r][v] = lp_ld_cluster4(src + v * LP_HEADS * 16);
         }
 #pragma unroll
         for (int r = 0; r < N; ++r)
@@ -215,11 +214,7 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     const int n_tiles = SPLIT ? (static_cast<int>(rank >> 1) + 1) * all_tiles / n_split - tile0 : all_tiles;
     const int n_half = 2 * n_tiles;
 
-    if (SPLIT && threadIdx.x < LP_HEADS) {
-        sh->split_m[threadIdx.x] = __int_as_float(0xff800000);
-        sh->split_l[threadIdx.x] = 0.f;
-        if (threadIdx.x < 4) sh->split_zero[threadIdx.x] = 0.f;
-    }
+    if (SPLIT && threadIdx.x < LP_HEADS) sh->split_l[threadIdx.x] = -1.f;
     if (threadIdx.x == 0) {
         mbar_init(smem_u32(&sh->q_full), 1);
         mbar_init(smem_u32(&sh->qt_full), 4);
@@ -717,17 +712,17 @@ sparse_attn_latent_pair_kernel(const __grid_constant__ CUtensorMap tmap_q, const
     if constexpr (SPLIT) {
         cluster_sync_all();         // every pair's output lies in its shared memory
         if (!start_abort && n_my > 0) {
-            const uint32_t o_addr = smem_u32(k_smem), m_addr = smem_u32(sh->split_m), l_addr = smem_u32(sh->split_l), zero_addr = smem_u32(sh->split_zero);
+            const uint32_t o_addr = smem_u32(k_smem), m_addr = smem_u32(sh->split_m), l_addr = smem_u32(sh->split_l);
             const int sp = static_cast<int>(rank >> 1);
             static_assert(LP_MAX_SPLIT == 8, "cases below");
             switch (n_split) {
-                case 2: lp_merge_splits<2>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
-                case 3: lp_merge_splits<3>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
-                case 4: lp_merge_splits<4>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
-                case 5: lp_merge_splits<5>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
-                case 6: lp_merge_splits<6>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
-                case 7: lp_merge_splits<7>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
-                case 8: lp_merge_splits<8>(p, cid, sp, c, o_addr, m_addr, l_addr, zero_addr); break;
+                case 2: lp_merge_splits<2>(p, cid, sp, c, o_addr, m_addr, l_addr); break;
+                case 3: lp_merge_splits<3>(p, cid, sp, c, o_addr, m_addr, l_addr); break;
+                case 4: lp_merge_splits<4>(p, cid, sp, c, o_addr, m_addr, l_addr); break;
+                case 5: lp_merge_splits<5>(p, cid, sp, c, o_addr, m_addr, l_addr); break;
+                case 6: lp_merge_splits<6>(p, cid, sp, c, o_addr, m_addr, l_addr); break;
+                case 7: lp_merge_splits<7>(p, cid, sp, c, o_addr, m_addr, l_addr); break;
+                case 8: lp_merge_splits<8>(p, cid, sp, c, o_addr, m_addr, l_addr); break;
             }
         }
     }
