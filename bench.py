@@ -796,7 +796,7 @@ def main():
         B.check_dev_status()
         fused = {"ms": f0.elapsed_time(f1) / 5, "two_call_ms": float(per_call[:, 0].mean() + per_call[:, 1].mean()), "workspace_bytes": ws_bytes,
                  "score_matrix_bytes": int(shp.M) * int((shp.S + 31) // 32 * 32) * 4,
-                 "note": "one call that never stores the score matrix: a memory-saving path (workspace vs score matrix), not the faster one at this size"}
+                 "note": "one call that never stores the score matrix: workspace instead of score matrix; two_call_ms is the time of the two calls on the same operands"}
 
     if rank != 0:
         if world > 1:
