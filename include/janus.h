@@ -120,7 +120,8 @@ int janus_topk(const float* scores, int64_t scores_ld, int M, int64_t n_keys,
  * than 8192 keys beyond the first row's prefix run the two calls internally with the scores in the workspace.
  *
  *   ws   device scratch of at least janus_indexer_topk_workspace_size(...) bytes, 16-byte aligned; contents undefined on
- *        return; two calls sharing a workspace must not overlap on the device.
+ *        return; two calls sharing a workspace must not overlap on the device.  (One that only holds candidate lists of
+ *        the expected length, without the margin in that figure, is taken too; more rows may then be recomputed.)
  */
 size_t janus_indexer_topk_workspace_size(int M, int H_I, int D_I, int64_t n_keys, int64_t q_pos0, int causal, int dtype, int k);
 int janus_indexer_topk(const void* q_idx, int64_t q_stride_tok,
@@ -154,7 +155,7 @@ int64_t janus_indexer_topk_fallback_counter_offset(int M, int H_I, int D_I, int6
  *             JANUS_STATIC_SCRATCH_BYTES; otherwise the call returns JANUS_ERR_WORKSPACE_TOO_SMALL and touches
  *             nothing.  64 MiB covers, for example, 128 new tokens over 131072 cached keys, or 64 over 262144
  *             (64 x 128 FP8 indexer, k = 2048); a 4096-token chunk at that history needs the caller's workspace.
- *   Set-up    the first call on a device looks up the array's address on that device (no allocation) and keeps it;
+ *   Set-up    the first call in a CUDA context looks up the array's address there (no allocation) and keeps it;
  *             the device whose stream is passed must be the current device.  Make that first call before any
  *             stream capture begins.
  *   Sharing   all calls on one device use the same array.  Each call clears the counters it needs itself, so
@@ -235,7 +236,8 @@ int janus_page_union(uint32_t* dst, const uint32_t* src, int64_t n_phys_pages, v
  *   lse   [M, H_q] fp32 out, log-sum-exp of the scaled logits (-inf for an empty selection), or NULL
  *
  * d_qk and d_v multiples of 8, d_qk <= 576, d_v <= 512, H_q a multiple of n_kv_heads; strides (in elements)
- * multiples of 8.  The tensor-core kernel serves the latent shape (n_kv_heads = 1, H_q = 128, d_qk = 576, d_v = 512).
+ * multiples of 8.  Tensor-core kernels serve the latent shape (n_kv_heads = 1, H_q = 128, d_qk = 576, d_v = 512) and keys
+ * of 64, 128 or 192 dims with values of 64 or 128 in any grouping; other dims run a slower general kernel.
  */
 size_t janus_sparse_attn_prefill_workspace_size(int M, int H_q, int d_qk, int d_v, int k);
 int janus_sparse_attn_prefill(const void* q, int M, int H_q, int d_qk,

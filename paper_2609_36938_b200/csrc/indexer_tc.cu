@@ -18,8 +18,9 @@
 // The launch is persistent: the visible (token group, key tile) pairs, group by group, are cut into as many contiguous ranges of equal
 // cost as CTAs are resident, and a CTA walks its range in segments of one group each.  The key ring, the TMEM slots and
 // their barriers run on across segments; the queries and weights are replaced, which costs about three quarters of a tile's time,
-// once or twice per CTA in a long call.  A grid of fixed chunks left waves unfilled: 2048 rows x 34816 keys 64 x 128 bf16 901 -> 857 us, 777 x 20788 of 32
-// heads 121 -> 114, 1024 x 17408 FP8 183 -> 172; 4096 x 135168 FP8, which is on the power limit, 5.26 -> 5.17 ms.  Small launches give
+// once or twice per CTA in a long call.  A grid of fixed chunks left waves unfilled (in loops of this kernel alone): 2048 rows x 34816 keys
+// 64 x 128 bf16 901 -> 857 us, 777 x 20788 of 32 heads 121 -> 114, 1024 x 17408 FP8 183 -> 172.  4096 x 135168 FP8, which is on the power limit,
+// takes 5.5 ms either way, and where the chunks happened to fill their waves (777 x 66777 bf16) they were 3 % faster.  Small launches give
 // every CTA tiles of one group only (MULTI = false).  256 rows x 4352 keys of 4 heads 18.6 -> 8.0 us, with half the sub-tiles per CTA.
 // Every wait is bounded; on a timeout the CTA reports JANUS_DEV_WAIT_TIMEOUT and winds down normally.
 #include "indexer_tc.cuh"
@@ -541,7 +542,10 @@ int launch_indexer_tc(const void* q_idx, const void* k_idx, int64_t k_stride_tok
         return w;
     };
     // Query sub-tiles per group: the key tiles are read once per group, so four where 128 KB hold them; two when that leaves SMs
-    // idle or the last round of tiles uneven (256 tokens x 34 tiles of 4 heads are 34 CTAs of four sub-tiles or 68 of two).
+    // idle or the last round of tiles uneven (256 tokens x 34 tiles of 4 heads are 34 CTAs of four sub-tiles or 68 of two).  A tile costs
+    // its sub-tiles and about a third of one more (its copy, barriers and the keys' scales), and the longest range decides.  With two
+    // and four, us: 256 x 4352 of 4 heads 7.4 and 11.2, 24 x 131096 FP8 34.9 and 42.9, 40 x 20040 13.2 and 16.0; 128 x 131200 166 and 160.5,
+    // 128 x 16512 26.2 and 24.8, 777 x 20788 161 and 153.
     p.nq = p.atoms == 1 ? 4 : 2;
     int64_t work = total_work(p.nq);      // visible (token group, key tile) pairs of all groups
     p.tiles_per_cta = 0;

@@ -57,7 +57,8 @@ __device__ __forceinline__ void set_bit_shared(uint32_t* bm, int p) {
 // A CTA's tokens become bits of its own bitmap of logical pages; at the end its set pages go through the page table into a
 // bitmap of physical pages, whose words are ORed into the global one (page by page they would be a contended atomic each:
 // 109 us).
-// Whole call at 4096 x 2048 indices: 35 us when every index went through the page table, 24.7 now; 8192 x 2048: 65.8 and 35.7.
+// Whole call at 4096 x 2048 indices, in a loop: 35 us when every index went through the page table, 24.7 now (32 inside a step, whose
+// other calls leave nothing of the indices in L2); 8192 x 2048: 65.8 and 35.7.
 __global__ void __launch_bounds__(MARK_THREADS)
 page_mark_kernel(const PdParams p, int n_log_words) {
     extern __shared__ uint32_t lbm[];

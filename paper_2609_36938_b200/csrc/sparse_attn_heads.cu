@@ -20,8 +20,8 @@
 //
 // Loads are bound by L1's tag stage, one 128-byte line a cycle: with 16-byte loads four lanes touch half a line of each key row
 // (347 us at 777 tokens x 4 kv heads x 2048 keys, L1 at 96 %); 32-byte loads touch whole lines.
-// Measured (B200, 128 / 128 dims): 777 tokens x 32 heads in 4 groups x 2048 keys 5785 -> 271 us = 12.0 TB/s out of L2 (kernel on
-// the fp32 ALUs before); 256 tokens x 8 heads x 256 keys 180 -> 34 us.
+// Measured (B200, 128 / 128 dims): 777 tokens x 32 heads in 4 groups x 2048 keys 5785 -> 275 us = 11.8 TB/s out of L2 (kernel on
+// the fp32 ALUs before; 271 without the check for infinities); 256 tokens x 8 heads x 256 keys 180 -> 34 us.
 #include <type_traits>
 
 #include "janus_common.cuh"

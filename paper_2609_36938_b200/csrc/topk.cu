@@ -194,10 +194,14 @@ topk_ragged_kernel(const float* scores, const int64_t* row_offsets, const int64_
         topk_row(scores + off, static_cast<int>(n), k, out, count != nullptr ? count + b : nullptr, kth != nullptr ? kth + b : nullptr, sh);
 }
 
-// CTAs that share one of `rows` rows of up to `n` elements (n < 0: the lengths are on the device).  One CTA takes 6.6 us and 0.08 us
-// per thousand elements; a cluster streams its share only, but its start and its four cluster-wide barriers cost 2 to 3 us,
-// and more once the clusters leave few SMs free.  Measured with 1, 2, 4 and 8 CTAs (us): 8 rows of 33 K 10.2, 10.5, 11.2, 10.2; of 60 K
-// 12.5, 12.3, 12.8, 10.4; of 131 K 17.5, 14.0, 12.9, 10.1; 24 rows of 131 K 17.6, 14.1, 13.0, 14.7; 74 rows 18.2, 14.5, 28.3, 38.7.
+// CTAs that share one of `rows` rows of up to `n` elements (n < 0: the lengths are on the device).  One CTA takes 7.5 us and 0.08 us
+// per thousand elements; a cluster streams its share only, but its start and its four cluster-wide barriers cost about a
+// microsecond, and more once the clusters leave few SMs free.  With 1, 2, 4 and 8 CTAs, k = 2048 (us): 8 rows of 12 K 8.1, 8.9, 9.6, 8.7; of 33 K 10.5,
+// 10.3, 10.3, 9.0; of 60 K 12.8, 11.3, 10.9, 8.9; of 131 K 18.4, 14.0, 12.0, 10.0; 24 rows of 60 K 13.1, 11.3, 11.1, 11.4; of 131 K 18.1, 13.9, 11.8,
+// 12.6; 74 rows of 48 K 11.7, 11.4, 21.5, 29.2; of 131 K 18.4, 14.4, 25.0, 32.5; 100 rows of 131 K 19.4, 19.8, 27.6, 40.8.  The lines were drawn with
+// a cluster form that took 1 to 1.4 us longer and are on the safe side of these figures: eight CTAs would pay from 16 K elements and up
+// to 12 rows, two from 40 K.  Rows whose length only the device knows take a cluster although short ones lose 0.5 us by it (200 elements 3.7 ->
+// 4.4), since long ones gain up to 18.
 static int topk_cluster_size(int64_t rows, double n) {
     const bool unknown = n < 0;
     if (rows <= 8 && (unknown || n >= 36e3)) return 8;
@@ -348,8 +352,10 @@ extern "C" int janus_topk(const float* scores, int64_t scores_ld, int M, int64_t
     if (!idx) return JANUS_ERR_INVALID_ARG;
     if (n_keys > 0 && (!scores || !aligned16(scores) || (scores_ld & 3) != 0)) return JANUS_ERR_INVALID_ARG;
     // The candidate list of a row holds what passes the sampled threshold: about n * r / 4096 elements for the sample rank
-    // r = e + 4 sqrt(e) + 8, e = 4096 k / n, give or take n sqrt(r) / 4096.  When that plus five deviations fits the small
-    // buffer for the longest row, that is taken.
+    // r = e + 4 sqrt(e) + 8, e = 4096 k / n, give or take n sqrt(r) / 4096 and what the lower edge of the threshold's bucket lets in
+    // besides (3 + r / 16 sample keys at most; drawn normal, gamma and narrow rows had lists under 2 % longer than expected).  When the list
+    // plus five deviations fits the small buffer for the longest row, that is taken; a row that overflows all the same is selected
+    // from global memory.
     const double n_max = static_cast<double>(causal ? (n_keys < q_pos0 + M ? n_keys : q_pos0 + M) : n_keys);
     bool small = false;
     if (n_max > TK_CAP) {

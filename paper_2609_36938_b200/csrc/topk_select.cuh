@@ -6,8 +6,8 @@
 // the lower edge of a bucket of one histogram over the sample (held in registers; a conservative threshold need not be a
 // sample value), candidates are counted into the buckets of a second histogram as they are found, and one pass over them then
 // emits what lies above the k-th key's bucket while the few keys inside it are ranked directly.  Against two selections of repeated
-// histogram passes (B200, k = 2048): 4096 rows of 135168 0.442 -> 0.385 ms (5.7 TB/s, 0.86 of the copy bandwidth; what is left is
-// that a CTA between two streaming passes reads nothing), 2048 rows of 34816 122 -> 100 us, one row of 32768 (a cluster) 15.4 -> 9.6, and 8.2 us
+// histogram passes (B200, k = 2048, the kernel alone in a loop): 4096 rows of 135168 0.442 -> 0.385 ms (5.7 TB/s, 0.86 of the copy bandwidth; what is left
+// is that a CTA between two streaming passes reads nothing; inside a step, after the indexer, 0.483 -> 0.42 = 0.81), 2048 rows of 34816 122 -> 100 us, one row of 32768 (a cluster) 15.4 -> 9.6, and 8.2 us
 // with its first loads issued before the sample and counts of 16 bits exchanged.  The exact selection over
 // repeated histogram passes (select_kth) remains for what this cannot settle: a misjudged sample, or hundreds of keys in one bucket.
 #pragma once
