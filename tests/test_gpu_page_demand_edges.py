@@ -106,3 +106,24 @@ def test_runs_across_the_clusters_of_a_large_pool():
         assert counts[n] == len(pages) and counts[n_runs] == len(first)
         assert np.array_equal(pd[ids][:len(pages)].cpu().numpy(), pages)
         assert np.array_equal(pd[runs][:len(first)].cpu().numpy(), np.stack([pages[first], pages[last] - pages[first] + 1], 1))
+
+
+def test_a_pool_beyond_one_chunk_per_cta():
+    """40 million pages: the clusters' CTAs take their words in several chunks; one run across every cluster boundary and single pages between."""
+    n_phys, words = 40_000_000, 1_250_000
+    step = 16 * -(-words // (64 * 16)) * 32            # pages of a cluster
+    here = np.concatenate([np.arange(i * step - 40, i * step + 40) for i in range(1, -(-n_phys // step))] + [np.arange(0, n_phys, 99_991), [n_phys - 1]])
+    want = np.unique(here)
+    idx = np.random.default_rng(0).permutation(here).astype(np.int32)
+    idx = np.concatenate([idx, np.full(-len(idx) % 64, -1, np.int32)]).reshape(-1, 64)
+    known = want[::7]
+    bits = torch.zeros((words,), dtype=torch.int64, device="cuda").index_add_(0, torch.from_numpy(known // 32).cuda(), torch.from_numpy(1 << (known % 32)).cuda())
+    pd = B.janus_page_demand(dev32(idx), demand_limit=n_phys, page_size=1, page_table=torch.arange(n_phys, dtype=torch.int32, device="cuda"), n_phys_pages=n_phys,
+                             predicted_bitmap=bits.to(torch.int32), capacity=20_000)
+    B.check_dev_status()
+    got = Hp.page_lists_from_device(pd)
+    miss = np.setdiff1d(want, known)
+    for pages, ids, runs in ((want, "pages", "runs"), (miss, "miss", "miss_runs")):
+        cut = np.flatnonzero(np.diff(pages) > 1)
+        first, last = np.concatenate([[0], cut + 1]), np.concatenate([cut, [len(pages) - 1]])
+        assert got[ids] == pages.tolist() and got[runs] == list(zip(pages[first].tolist(), (pages[last] - pages[first] + 1).tolist()))
