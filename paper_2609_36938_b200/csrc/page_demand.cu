@@ -5,7 +5,8 @@
 // Latency bounds all of it: a few hundred kilobytes in, a few kilobytes out, but several dependent steps.  Up to 128 K
 // indices one launch of one cluster does everything (page_demand_kernel): every CTA marks its share of the indices in a private
 // bitmap in shared memory, the cluster ORs the bitmaps slice by slice through distributed shared memory, and each CTA
-// turns its slice of the set into its part of the lists, offsets coming from one exchange of the CTAs' counts.  Larger blocks of
+// turns its slice of the set into its part of the lists, offsets coming from one exchange of the CTAs' counts (page_demand_few_kernel: a
+// small pool's lists come from one CTA, without the exchange).  Larger blocks of
 // indices are marked by the whole chip first (page_mark_kernel, one bitmap of *logical* pages per CTA, so that an index costs
 // one shared-memory test and the page table is read once per page and CTA), and the same kernel then only makes the lists, for large pools
 // in several clusters.  Which of them, and how many CTAs: page_demand_plan.h.
@@ -197,6 +198,166 @@ __device__ __forceinline__ void block_scan2_u64(uint64_t (&v)[2], uint64_t (*war
     }
 }
 
+// Marks the pages of CTA `rank`'s share of the indices in its bitmap in shared memory.  False: something was out of range.
+template <int MODE>
+__device__ __forceinline__ bool mark_share(const PdParams& p, uint32_t* bm, int rank, int n_cta) {
+    const int tid = threadIdx.x;
+            const PageDiv page{p.page_size, p.page_shift};
+            bool bad = false;
+            // Eight indices per thread at a time, in rounds of loads that are all in flight together: indices and their rows' table and
+            // limit, then page table entries (one index after the other: 24.2 us instead of 21.9 for 64 decode rows of 2048, when the rest took 5 us longer)
+            constexpr int U = 8;
+            const int stride = n_cta * PD_THREADS, n_idx = static_cast<int>(p.n_idx);
+            for (int base = rank * PD_THREADS + tid; base < n_idx; base += U * stride) {
+                int s[U];
+                int32_t q[U];
+                const int32_t* entry[U];
+    #pragma unroll
+                for (int u = 0; u < U; ++u) s[u] = base + u * stride < n_idx ? ld_input(p.idx + base + u * stride) : -1;
+                if constexpr (MODE == PD_MARK_ROWS) {
+                    int64_t off[U], end[U], limit[U];
+    #pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        off[u] = end[u] = limit[u] = 0;
+                        if (base + u * stride >= n_idx) continue;
+                        const int r = (base + u * stride) / p.k;
+                        off[u] = ld_input(p.table_offsets + r);
+                        end[u] = ld_input(p.table_offsets + r + 1);
+                        limit[u] = ld_input(p.demand_limits + r);
+                    }
+    #pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        entry[u] = nullptr;
+                        if (s[u] >= 0 && s[u] < limit[u]) {       // a table that starts before the array has no pages
+                            const int64_t lp = page(s[u]);
+                            if (off[u] >= 0 && lp < end[u] - off[u]) entry[u] = p.page_table + off[u] + lp;
+                            else bad = true;
+                        }
+                    }
+                } else {
+    #pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        entry[u] = nullptr;
+                        if (s[u] >= 0 && s[u] < p.demand_limit) {
+                            const int64_t lp = page(s[u]);
+                            if (lp < p.n_logical_pages) entry[u] = p.page_table + lp;
+                            else bad = true;
+                        }
+                    }
+                }
+    #pragma unroll
+                for (int u = 0; u < U; ++u) q[u] = entry[u] != nullptr ? ld_input(entry[u]) : -1;
+    #pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (entry[u] == nullptr) continue;
+                    if (q[u] < 0 || q[u] >= p.n_phys_pages) bad = true;
+                    else set_bit_shared(bm, q[u]);
+                }
+            }
+    return !bad;
+}
+
+// ---- one cluster, a pool of few words --------------------------------------------------------------------------------------------
+// The sets of all CTAs are ORed into CTA 0's shared memory, which then makes the lists alone: a thread has a word, counts are 16 bits
+// each, runs are put together in shared memory.  One cluster-wide barrier on the way instead of four, and no exchange of counts: 7-8 -> 5 us.
+constexpr int PD_FEW_RUNS = PD_FEW_WORDS * 16;
+struct PdFewShared {
+    uint32_t own[PD_FEW_WORDS];
+    uint32_t word[2][PD_FEW_WORDS + 2];       // CTA 0: the set, the miss set, with an empty word on either side
+    uint32_t at[2][PD_FEW_WORDS];             // ids before a word << 16 | run starts before it
+    uint32_t warp_sum[2][PD_FEW_WORDS / 32];
+    uint16_t start[2][PD_FEW_RUNS], end[2][PD_FEW_RUNS];
+};
+static_assert(PD_FEW_WORDS * 32 <= 0xffff && PD_FEW_WORDS <= PD_THREADS, "counts and pages of 16 bits");
+
+template <int MODE>
+__global__ void __launch_bounds__(PD_THREADS)
+page_demand_few_kernel(const PdParams p) {
+    __shared__ PdFewShared sh;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = static_cast<int>(cluster_ctarank()), n_cta = static_cast<int>(cluster_nctarank());
+    const bool want_miss = p.miss_pages != nullptr;
+    grid_launch_next();
+    if (tid < PD_FEW_WORDS) sh.own[tid] = 0u;
+    if (tid < PD_FEW_WORDS + 2) sh.word[0][tid] = sh.word[1][tid] = 0u;
+    cluster_arrive_release();             // (CTA 0's set is empty; waited for before it is written to)
+    grid_wait();
+    uint32_t predicted = 0u;              // on its way while the indices are marked
+    if (rank == 0 && tid < p.n_words && p.predicted != nullptr) predicted = __ldcg(p.predicted + tid);
+    __syncthreads();
+    if (!mark_share<MODE>(p, sh.own, rank, n_cta)) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
+    __syncthreads();
+    cluster_wait();
+    if (tid < p.n_words && sh.own[tid] != 0u) red_or_cluster_u32(mapa_shared(smem_u32(&sh.word[0][tid + 1]), 0), sh.own[tid]);
+    cluster_sync_all();
+    if (rank != 0) return;
+    if (tid < PD_FEW_WORDS) {
+        const uint32_t v = sh.word[0][tid + 1];
+        if (tid < p.n_words) p.bitmap[tid] = v;
+        if (want_miss) sh.word[1][tid + 1] = v & ~predicted;
+    }
+    __syncthreads();
+    uint32_t incl[2] = {0u, 0u}, mine[2] = {0u, 0u};
+    if (tid < PD_FEW_WORDS) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const uint32_t v = sh.word[q][tid + 1], starts = v & ~((v << 1) | (sh.word[q][tid] >> 31));
+            mine[q] = incl[q] = static_cast<uint32_t>(__popc(v)) << 16 | static_cast<uint32_t>(__popc(starts));
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl[q], d);
+                if (lane >= d) incl[q] += y;
+            }
+            if (lane == 31) sh.warp_sum[q][warp] = incl[q];
+        }
+    }
+    __syncthreads();
+    uint32_t total[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const uint32_t x = lane < PD_FEW_WORDS / 32 ? sh.warp_sum[q][lane] : 0u;
+        total[q] = __reduce_add_sync(0xffffffffu, x);
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? x : 0u);
+        if (tid < PD_FEW_WORDS) sh.at[q][tid] = before + incl[q] - mine[q];
+    }
+    __syncthreads();
+    const int cap = static_cast<int>(min(p.capacity, static_cast<int64_t>(0x7fffffff)));
+    const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {         // a warp per word, a lane per page
+        if (q == 1 && !want_miss) break;
+        int32_t* ids = q ? p.miss_pages : p.pages;
+        for (int j = warp; j < p.n_words; j += PD_THREADS / 32) {
+            const uint32_t w = sh.word[q][j + 1];
+            if (((w >> lane) & 1u) == 0u) continue;
+            const uint32_t starts = w & ~((w << 1) | (sh.word[q][j] >> 31)), ends = w & ~((w >> 1) | (sh.word[q][j + 2] << 31));
+            const uint32_t o = sh.at[q][j];
+            const int o_id = static_cast<int>(o >> 16) + __popc(w & below);
+            const int run = static_cast<int>(o & 0xffffu) + __popc(starts & (below | (1u << lane))) - 1;      // the page's run
+            const int page = j * 32 + lane;
+            if (o_id < cap) ids[o_id] = page;
+            if ((starts >> lane) & 1u) sh.start[q][run] = static_cast<uint16_t>(page);
+            if ((ends >> lane) & 1u) sh.end[q][run] = static_cast<uint16_t>(page);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        if (q == 1 && !want_miss) break;
+        int32_t* runs = q ? p.miss_runs : p.runs;
+        const int n_runs = static_cast<int>(total[q] & 0xffffu), n_ids = static_cast<int>(total[q] >> 16);
+        for (int j = tid; j < min(n_runs, cap); j += PD_THREADS) {
+            runs[2 * j] = sh.start[q][j];
+            runs[2 * j + 1] = sh.end[q][j] - sh.start[q][j] + 1;
+        }
+        if (tid == 0) {
+            *(q ? p.n_miss : p.n_pages) = n_ids;
+            *(q ? p.n_miss_runs : p.n_runs) = n_runs;
+            if (n_ids > p.capacity || n_runs > p.capacity) report(p.dev_status, JANUS_DEV_CAPACITY_EXCEEDED);
+        }
+    }
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(PD_THREADS)
 page_demand_kernel(const PdParams p) {
@@ -217,59 +378,7 @@ page_demand_kernel(const PdParams p) {
         for (int i = tid; i < p.n_words; i += PD_THREADS) bm[i] = 0u;
         grid_wait();
         __syncthreads();
-        const PageDiv page{p.page_size, p.page_shift};
-        bool bad = false;
-        // Eight indices per thread at a time, in rounds of loads that are all in flight together: indices and their rows' table and
-        // limit, then page table entries (one index after the other: 24.2 us instead of 21.9 for 64 decode rows of 2048, when the rest took 5 us longer)
-        constexpr int U = 8;
-        const int stride = n_cta * PD_THREADS, n_idx = static_cast<int>(p.n_idx);
-        for (int base = rank * PD_THREADS + tid; base < n_idx; base += U * stride) {
-            int s[U];
-            int32_t q[U];
-            const int32_t* entry[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) s[u] = base + u * stride < n_idx ? ld_input(p.idx + base + u * stride) : -1;
-            if constexpr (MODE == PD_MARK_ROWS) {
-                int64_t off[U], end[U], limit[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    off[u] = end[u] = limit[u] = 0;
-                    if (base + u * stride >= n_idx) continue;
-                    const int r = (base + u * stride) / p.k;
-                    off[u] = ld_input(p.table_offsets + r);
-                    end[u] = ld_input(p.table_offsets + r + 1);
-                    limit[u] = ld_input(p.demand_limits + r);
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    entry[u] = nullptr;
-                    if (s[u] >= 0 && s[u] < limit[u]) {       // a table that starts before the array has no pages
-                        const int64_t lp = page(s[u]);
-                        if (off[u] >= 0 && lp < end[u] - off[u]) entry[u] = p.page_table + off[u] + lp;
-                        else bad = true;
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    entry[u] = nullptr;
-                    if (s[u] >= 0 && s[u] < p.demand_limit) {
-                        const int64_t lp = page(s[u]);
-                        if (lp < p.n_logical_pages) entry[u] = p.page_table + lp;
-                        else bad = true;
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) q[u] = entry[u] != nullptr ? ld_input(entry[u]) : -1;
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (entry[u] == nullptr) continue;
-                if (q[u] < 0 || q[u] >= p.n_phys_pages) bad = true;
-                else set_bit_shared(bm, q[u]);
-            }
-        }
-        if (bad) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
+        if (!mark_share<MODE>(p, bm, rank, n_cta)) report(p.dev_status, JANUS_DEV_INDEX_OUT_OF_RANGE);
         cluster_sync_all();               // every private bitmap is complete
     }
 
@@ -514,6 +623,12 @@ static int run_page_demand(const PdParams& p, cudaStream_t stream) {
     int largest = 0;
     JANUS_CUDA_CHECK(largest_cluster(largest));
     const PdPlan plan = page_demand_plan(p.n_idx, p.n_words, largest);
+    if (plan.few) {
+        static once_per_context attributes;
+        JANUS_CUDA_CHECK(attributes.run([] { return cudaFuncSetAttribute(page_demand_few_kernel<MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); }));
+        JANUS_CUDA_CHECK(launch_kernel(page_demand_few_kernel<MODE>, dim3(plan.cluster), PD_THREADS, 0, stream, plan.cluster, p));
+        return JANUS_OK;
+    }
     if (plan.one_launch) return launch_page_demand<MODE>(p, plan, stream);
     JANUS_CUDA_CHECK(cudaMemsetAsync(p.bitmap, 0, sizeof(uint32_t) * p.n_words, stream));
     const int64_t n_log_words = (p.n_logical_pages + 31) / 32;

@@ -18,6 +18,7 @@ constexpr int PD_FEW_WORDS = 256;
 constexpr int64_t PD_ONE_LAUNCH_INDICES = 1 << 17;
 
 struct PdPlan {
+    bool few;             // marking and lists by one cluster, the lists by one of its CTAs
     bool one_launch;      // marking and lists by one cluster; otherwise the whole chip marks first
     int cluster;          // CTAs of a cluster of page_demand_kernel
     int clusters;         // of the lists
@@ -25,20 +26,22 @@ struct PdPlan {
 
 // `largest`: CTAs of the largest cluster that the device takes (8 always, 16 on a whole B200).
 inline PdPlan page_demand_plan(int64_t n_idx, int n_words, int largest) {
-    // A CTA's slice of the set is one chunk, PD_THREADS words.  Four CTAs for few indices in a small pool (2048 indices of 512 pages 7.4 us, of
-    // 4096 pages 7.7; eight and sixteen cost 0.1 and 0.3 us more), all the device takes beyond: 256 x 256 indices 8.0 us against 10.7 with four
-    // and 8.6 with eight; 2048 indices of 16384 pages 8.2 against 9.6 with four, of 131072 pages 11.8 against 19.1.
+    // A CTA's slice of the set is one chunk, PD_THREADS words, and up to PD_FEW_WORDS words one CTA makes the lists (2048 indices of 513 pages
+    // 6.8 -> 5.0 us, 19 x 2048 of 142 pages 7.7 -> 4.9, 256 x 256 of 68 pages 7.8 -> 5.0, twelve rows of 2048 over 6000 pages 8.4 -> 6.7; at 256 words
+    // 7.7 -> 6.7, and 1.7 us more with every 240 words, so that the lists of a whole cluster catch up at 512).  Four CTAs for few indices in
+    // such a pool (four and eight alike up to three rows of 2048; nineteen rows 7.1 with four, 5.2 with eight, 4.9 with sixteen), all the
+    // device takes beyond: 2048 indices of 16384 pages 8.2 against 9.6 with four, of 131072 pages 11.8 against 19.1.
     if (n_idx <= PD_ONE_LAUNCH_INDICES && n_words <= PD_SMEM_WORDS)
-        return {true, n_idx <= 8192 && n_words <= PD_FEW_WORDS ? 4 : largest, 1};
+        return {n_words <= PD_FEW_WORDS, true, n_idx <= 8192 && n_words <= PD_FEW_WORDS ? 4 : largest, 1};
     // Lists alone: 2112 pages 14.4 us with a cluster of 8, 16.5 with 16; larger pools are shared by clusters, which count what lies before
     // them: up to four while each CTA has 256 words, then as many as give each one chunk.  524288 indices of 500000 pages 43.2 us with one
     // cluster, 30.0 with four; 131072 of 1048576 pages 55.6, 31.8, 23.5 and 29.3 with one, two, four and eight; of 2097152 pages 88 with one,
     // 29.3 with four and 35.7 with eight.
-    if (n_words <= PD_FEW_WORDS) return {false, PD_PORTABLE_CLUSTER, 1};
+    if (n_words <= PD_FEW_WORDS) return {false, false, PD_PORTABLE_CLUSTER, 1};
     const auto shares = [&](int64_t words) { return (n_words + words * largest - 1) / (words * largest); };
     int64_t n = shares(256) < 4 ? shares(256) : 4;
     if (n < shares(PD_THREADS)) n = shares(PD_THREADS);
-    return {false, largest, n < PD_MAX_CLUSTERS ? static_cast<int>(n) : PD_MAX_CLUSTERS};
+    return {false, false, largest, n < PD_MAX_CLUSTERS ? static_cast<int>(n) : PD_MAX_CLUSTERS};
 }
 
 }  // namespace janus

@@ -246,6 +246,7 @@ __device__ __forceinline__ void cluster_sync_all() {   // every thread of every 
 }
 // The two halves of a cluster barrier, without ordering of memory: after the wait every CTA of the cluster is running.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;"); }
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 // Address of the same shared-memory location in CTA `rank` of this cluster.
 __device__ __forceinline__ uint32_t mapa_shared(uint32_t local_addr, uint32_t rank) {
@@ -265,6 +266,9 @@ __device__ __forceinline__ uint64_t ld_cluster_u64(uint32_t cluster_addr) {
     uint64_t v;
     asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(cluster_addr) : "memory");
     return v;
+}
+__device__ __forceinline__ void red_or_cluster_u32(uint32_t cluster_addr, uint32_t v) {
+    asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ int atomic_add_cluster_s32(uint32_t cluster_addr, int v) {
     int old;

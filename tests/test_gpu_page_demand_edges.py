@@ -127,3 +127,28 @@ def test_a_pool_beyond_one_chunk_per_cta():
         cut = np.flatnonzero(np.diff(pages) > 1)
         first, last = np.concatenate([[0], cut + 1]), np.concatenate([cut, [len(pages) - 1]])
         assert got[ids] == pages.tolist() and got[runs] == list(zip(pages[first].tolist(), (pages[last] - pages[first] + 1).tolist()))
+
+
+@pytest.mark.parametrize("n_phys", [1, 32, 250, 8160, 8191, 8192, 8193])
+@pytest.mark.parametrize("which", ["all", "every other", "blocks", "none"])
+def test_pools_of_few_words(n_phys, which):
+    """Around the largest pool whose lists one CTA makes: as many runs as there can be, one run over all words, no page at all; a predicted
+    set and none."""
+    rng = np.random.default_rng(n_phys)
+    pages = {"all": np.arange(n_phys), "every other": np.arange(0, n_phys, 2), "none": np.arange(0),
+             "blocks": np.flatnonzero(np.arange(n_phys) // 37 % 3 > 0)}[which]
+    k = max(4, (len(pages) + 7) // 8 * 4)                       # two rows and more
+    idx = np.full((3, k), -1, np.int32)
+    idx.flat[: len(pages)] = rng.permutation(pages)
+    table = np.arange(n_phys, dtype=np.int32)
+    ref = O.page_demand(idx, n_phys, 1, table)
+    predicted = pages[rng.random(len(pages)) < 0.3]
+    for bits in (torch.from_numpy(bitmap_of(predicted, n_phys)).cuda(), None):
+        pd = B.janus_page_demand(dev32(idx), demand_limit=n_phys, page_size=1, page_table=dev32(table), n_phys_pages=n_phys, predicted_bitmap=bits)
+        B.check_dev_status()
+        got = Hp.page_lists_from_device(pd)
+        assert Hp.bitmap_to_pages(pd["bitmap"], n_phys) == list(ref["pages"]) == pages.tolist()
+        assert got["pages"] == list(ref["pages"]) and got["runs"] == [tuple(r) for r in ref["runs"]]
+        if bits is not None:
+            miss = sorted(set(pages.tolist()) - set(predicted.tolist()))
+            assert got["miss"] == miss and got["miss_runs"] == [tuple(r) for r in O.maximal_runs(miss)]
