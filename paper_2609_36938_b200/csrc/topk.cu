@@ -21,7 +21,6 @@ namespace janus {
 // streaming loads pass, with 54 KB a third: 4096 rows of 135168 390 us against 498, 1024 of 16384 28 against 35.  (Four CTAs of 54 KB and
 // 32 registers: 497.)
 constexpr int TK_CAP = 8192;
-constexpr int TK_CAP_SMALL = 5632;  // for rows whose candidate list is sure to fit
 
 template <int CAP>
 __global__ void __launch_bounds__(TK_THREADS)
@@ -210,36 +209,47 @@ static int topk_cluster_size(int64_t rows, double n) {
     return 1;
 }
 
+// The forms of topk_rows_kernel, by candidate slots.
+struct TopkForm {
+    void (*kernel)(const float*, int64_t, int, int64_t, int64_t, int, int, int32_t*, int32_t*, float*);
+    int cap, smem;
+};
+template <int CAP>
+constexpr TopkForm topk_form() { return {topk_rows_kernel<CAP>, CAP, static_cast<int>(sizeof(TopkSharedT<CAP>))}; }
+constexpr int TK_FORMS = 3;
+static const TopkForm topk_forms[TK_FORMS] = {topk_form<3840>(), topk_form<5632>(), topk_form<TK_CAP>()};
+
 // Kernel attributes, set once in every context, and the number of resident CTAs, a property of the device.
 struct TopkDevice {
-    int resident = 0, resident_small = 0;
+    int n_sm, resident[TK_FORMS];
 };
 static cudaError_t topk_device(TopkDevice& d) {
     static once_per_context once;
-    static std::atomic<int> resident[64], resident_small[64];
+    static std::atomic<int> sms[64], resident[64][TK_FORMS];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     e = once.run([&] {
-        const int smem = static_cast<int>(sizeof(TopkSharedT<TK_CAP>)), smem_small = static_cast<int>(sizeof(TopkSharedT<TK_CAP_SMALL>));
-        int n_sm = 0, per = 0, per_small = 0;
+        const int smem = static_cast<int>(sizeof(TopkSharedT<TK_CAP>));
+        int n_sm = 0;
         cudaError_t r = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         auto limit = [&](const void* f, int bytes) { if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
-        limit(reinterpret_cast<const void*>(topk_rows_kernel<TK_CAP>), smem);
-        limit(reinterpret_cast<const void*>(topk_rows_kernel<TK_CAP_SMALL>), smem_small);
         limit(reinterpret_cast<const void*>(topk_rows_cluster_kernel), smem);
         limit(reinterpret_cast<const void*>(topk_entries_kernel<TK_CAP>), smem);
         limit(reinterpret_cast<const void*>(topk_ragged_kernel<true>), smem);
         limit(reinterpret_cast<const void*>(topk_ragged_kernel<false>), smem);
-        if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, topk_rows_kernel<TK_CAP>, TK_THREADS, smem);
-        if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_small, topk_rows_kernel<TK_CAP_SMALL>, TK_THREADS, smem_small);
-        resident[dev] = std::max(1, per) * n_sm;
-        resident_small[dev] = std::max(1, per_small) * n_sm;
+        sms[dev] = n_sm;
+        for (int f = 0; f < TK_FORMS; ++f) {
+            int per = 0;
+            limit(reinterpret_cast<const void*>(topk_forms[f].kernel), topk_forms[f].smem);
+            if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, topk_forms[f].kernel, TK_THREADS, topk_forms[f].smem);
+            resident[dev][f] = std::max(1, per) * n_sm;
+        }
         return r;
     });
-    d.resident = resident[dev];
-    d.resident_small = resident_small[dev];
+    d.n_sm = sms[dev];
+    for (int f = 0; f < TK_FORMS; ++f) d.resident[f] = resident[dev][f];
     return e;
 }
 
@@ -353,29 +363,28 @@ extern "C" int janus_topk(const float* scores, int64_t scores_ld, int M, int64_t
     if (n_keys > 0 && (!scores || !aligned16(scores) || (scores_ld & 3) != 0)) return JANUS_ERR_INVALID_ARG;
     // The candidate list of a row holds what passes the sampled threshold: about n * r / 4096 elements for the sample rank
     // r = e + 4 sqrt(e) + 8, e = 4096 k / n, give or take n sqrt(r) / 4096 and what the lower edge of the threshold's bucket lets in
-    // besides (3 + r / 16 sample keys at most; drawn normal, gamma and narrow rows had lists under 2 % longer than expected).  When the list
-    // plus five deviations fits the small buffer for the longest row, that is taken; a row that overflows all the same is selected
-    // from global memory.
+    // besides (3 + r / 16 sample keys at most; drawn normal, gamma and narrow rows had lists under 2 % longer than expected).  The smallest
+    // form is taken into which the list plus five deviations fits for the longest row, since less shared memory leaves more of it to L1
+    // (2048 rows of 34816 102.7 us with 5632 slots, 96.7 with 3840; 777 of 20788 34.7 and 32.3; 4096 of 135168 498 with 8192 and 396 with
+    // 5632); a row that overflows all the same is selected from global memory.  Rows that fit a form whole are taken whole where CTAs have
+    // an SM each or half of the row is on the list anyway (256 of 4000, k = 2048, 8.9 us, 11.3 through the sample; 256 of 8000 13.9 and 11.9;
+    // 4000 of 6000, k = 512, 88 and 76).
     const double n_max = static_cast<double>(causal ? (n_keys < q_pos0 + M ? n_keys : q_pos0 + M) : n_keys);
-    bool small = false;
-    if (n_max > TK_CAP) {
-        const double e = 4096.0 * k / n_max, r = e + 4.0 * sqrt(e) + 8.0;
-        small = n_max * (r + 5.0 * sqrt(r)) / 4096.0 <= TK_CAP_SMALL && k <= TK_CAP_SMALL / 2;
-    }
+    const double e = n_max > 0. ? 4096.0 * k / n_max : 0., r = e + 4.0 * sqrt(e) + 8.0, list = n_max * (r + 5.0 * sqrt(r)) / 4096.0;
     TopkDevice d;
     JANUS_CUDA_CHECK(topk_device(d));
+    const bool share = M > d.n_sm, whole = n_max <= TK_CAP && (!share || list > n_max / 2);
+    const double slots = whole ? n_max : list;
+    int form = share ? 0 : 1;
+    while (form < TK_FORMS - 1 && (slots > topk_forms[form].cap || (!whole && k > topk_forms[form].cap / 2 + 256))) ++form;
     const int cluster = topk_cluster_size(M, n_max);
     if (cluster > 1) {
         JANUS_CUDA_CHECK(launch_kernel(topk_rows_cluster_kernel, dim3(M * cluster), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream, cluster, scores,
                                        scores_ld, n_keys, q_pos0, causal, k, idx, count, kth));
         return JANUS_OK;
     }
-    if (small)
-        JANUS_CUDA_CHECK(launch_kernel(topk_rows_kernel<TK_CAP_SMALL>, dim3(std::min(M, d.resident_small)), TK_THREADS,
-                                       sizeof(TopkSharedT<TK_CAP_SMALL>), stream, 1, scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count,
-                                       kth));
-    else
-        JANUS_CUDA_CHECK(launch_kernel(topk_rows_kernel<TK_CAP>, dim3(std::min(M, d.resident)), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream, 1,
-                                       scores, scores_ld, M, n_keys, q_pos0, causal, k, idx, count, kth));
+    const TopkForm& f = topk_forms[form];
+    JANUS_CUDA_CHECK(launch_kernel(f.kernel, dim3(std::min(M, d.resident[form])), TK_THREADS, f.smem, stream, 1, scores, scores_ld, M, n_keys, q_pos0, causal, k,
+                                   idx, count, kth));
     return JANUS_OK;
 }
