@@ -18,9 +18,9 @@ constexpr int PD_FEW_WORDS = 256;
 constexpr int64_t PD_ONE_LAUNCH_INDICES = 1 << 17;
 
 struct PdPlan {
-    bool few;             // marking and lists by one cluster, the lists by one of its CTAs
+    bool few;             // the lists by one CTA, of one cluster that marks as well or alone
     bool one_launch;      // marking and lists by one cluster; otherwise the whole chip marks first
-    int cluster;          // CTAs of a cluster of page_demand_kernel
+    int cluster;          // CTAs of a cluster (few lists alone need one CTA)
     int clusters;         // of the lists
 };
 
@@ -33,11 +33,11 @@ inline PdPlan page_demand_plan(int64_t n_idx, int n_words, int largest) {
     // device takes beyond: 2048 indices of 16384 pages 8.2 against 9.6 with four, of 131072 pages 11.8 against 19.1.
     if (n_idx <= PD_ONE_LAUNCH_INDICES && n_words <= PD_SMEM_WORDS)
         return {n_words <= PD_FEW_WORDS, true, n_idx <= 8192 && n_words <= PD_FEW_WORDS ? 4 : largest, 1};
-    // Lists alone: 2112 pages 14.4 us with a cluster of 8, 16.5 with 16; larger pools are shared by clusters, which count what lies before
-    // them: up to four while each CTA has 256 words, then as many as give each one chunk.  524288 indices of 500000 pages 43.2 us with one
-    // cluster, 30.0 with four; 131072 of 1048576 pages 55.6, 31.8, 23.5 and 29.3 with one, two, four and eight; of 2097152 pages 88 with one,
-    // 29.3 with four and 35.7 with eight.
-    if (n_words <= PD_FEW_WORDS) return {false, false, PD_PORTABLE_CLUSTER, 1};
+    // Lists alone: one CTA for a small pool (whole call of 4096 x 2048 indices of 2112 pages 26.3 us with a cluster of 8, 22.7 with one CTA; 2048 x 2048 of 544 18.5 and 14.6); larger pools are shared by clusters, which
+    // count what lies before them: up to four while each CTA has 256 words, then as many as give each one chunk.  524288 indices of 500000
+    // pages 43.2 us with one cluster, 30.0 with four; 131072 of 1048576 pages 55.6, 31.8, 23.5 and 29.3 with one, two, four and eight; of
+    // 2097152 pages 88 with one, 29.3 with four and 35.7 with eight.
+    if (n_words <= PD_FEW_WORDS) return {true, false, PD_PORTABLE_CLUSTER, 1};
     const auto shares = [&](int64_t words) { return (n_words + words * largest - 1) / (words * largest); };
     int64_t n = shares(256) < 4 ? shares(256) : 4;
     if (n < shares(PD_THREADS)) n = shares(PD_THREADS);
