@@ -43,13 +43,14 @@ def sharded_predicted_pages(q_pred, k_idx, w, *, L: int, k: int, n_shards: int, 
     k_shard = max(1, k // n_shards)
     union: Optional[torch.Tensor] = None
     bitmaps, indices = [], []
+    lists = B.page_demand_buffers(n_phys_pages, want_miss=False, device=q_pred.device)      # only the bitmaps are handed out
     for a, b in shard_bounds(L, n_shards, page_size):
         sc = B.janus_indexer_scores(q_pred, k_idx[a:b], w, q_scale=q_scale, k_scale=None if k_scale is None else k_scale[a:b],
                                     q_pos0=L, causal=False)
         idx, _, _ = B.janus_topk(sc, b - a, k_shard, q_pos0=L, causal=False, want_count=False, want_kth=False)
         # indices are local to the shard; the shard starts on a page boundary, so its pages are a slice of the page table
         pd = B.janus_page_demand(idx, demand_limit=b - a, page_size=page_size, page_table=page_table[a // page_size:],
-                                 n_phys_pages=n_phys_pages, want_miss=False)
+                                 n_phys_pages=n_phys_pages, want_miss=False, out={**lists, "bitmap": torch.empty_like(lists["bitmap"])})
         bitmaps.append(pd["bitmap"])
         indices.append(idx)
         union = pd["bitmap"].clone() if union is None else B.janus_page_union(union, pd["bitmap"], n_phys_pages)
