@@ -152,3 +152,24 @@ def test_pools_of_few_words(n_phys, which):
         if bits is not None:
             miss = sorted(set(pages.tolist()) - set(predicted.tolist()))
             assert got["miss"] == miss and got["miss_runs"] == [tuple(r) for r in O.maximal_runs(miss)]
+
+
+@pytest.mark.parametrize("n_phys", [1, 250, 8192, 8193])
+def test_large_blocks_over_few_words(n_phys):
+    """More indices than one cluster marks, around the largest pool whose lists one CTA makes; buffers that still hold another block's set."""
+    rng = np.random.default_rng(n_phys)
+    out = B.page_demand_buffers(n_phys)
+    table = rng.permutation(n_phys).astype(np.int32)
+    for rows, k, share in ((65, 2048, 1.0), (800, 168, 0.2), (130, 1024, 0.0)):
+        some = np.flatnonzero(rng.random(n_phys) < share)
+        idx = (rng.choice(some, (rows, k)) * 16 + 5 if len(some) else np.full((rows, k), -1)).astype(np.int32)
+        ref = O.page_demand(idx, n_phys * 16, 16, table)
+        predicted = np.flatnonzero(rng.random(n_phys) < 0.3)
+        B.janus_page_demand(dev32(idx), demand_limit=n_phys * 16, page_size=16, page_table=dev32(table), n_phys_pages=n_phys,
+                            predicted_bitmap=torch.from_numpy(bitmap_of(predicted, n_phys)).cuda(), out=out)
+        B.check_dev_status()
+        got = Hp.page_lists_from_device(out)
+        miss = sorted(set(ref["pages"]) - set(predicted.tolist()))
+        assert Hp.bitmap_to_pages(out["bitmap"], n_phys) == list(ref["pages"])
+        assert got["pages"] == list(ref["pages"]) and got["runs"] == [tuple(r) for r in ref["runs"]]
+        assert got["miss"] == miss and got["miss_runs"] == [tuple(r) for r in O.maximal_runs(miss)]

@@ -1,4 +1,4 @@
-"""Top-k where its routes change: rows around the candidate buffers (5632 and 8192 elements), the cluster sizes with their shares of a row,
+"""Top-k where its routes change: rows around the candidate buffers (3840, 5632 and 8192 elements), the cluster sizes with their shares of a row,
 ragged rows of very different lengths in one launch, and score distributions the sample or the buckets cannot settle (ties by the thousand,
 one value, two far-apart levels, -0 and +0, an outlier that stretches the key range, a row whose large scores hide from the sample).
 A selection is checked against a full sort: the values above the k-th are all there, ties at it are free."""
@@ -65,6 +65,24 @@ def test_topk_rows(kind, rows, n):
         idx, cnt, kth = idx.cpu().numpy(), cnt.cpu().numpy(), kth.cpu().numpy()
         for t in {0, 1, rows // 2, rows - 1}:
             check_row(idx[t], cnt[t], kth[t], sc[t, :n - rows + t + 1], k, f"{kind} row {t} of {rows} x {n}, k {k}")
+
+
+@pytest.mark.parametrize("kind", ["normal", "ties", "zeros", "outlier", "hidden"])
+@pytest.mark.parametrize("rows,n,k", [(148, 8192, 64), (149, 3840, 64), (149, 3841, 64), (300, 4090, 1000), (160, 4500, 2048), (149, 5633, 700),
+                                      (149, 8192, 2048), (149, 8193, 2176), (149, 8193, 2177), (700, 20003, 2048), (160, 20003, 3500)])
+def test_topk_rows_that_share_an_sm(kind, rows, n, k):
+    """Around the slots of the three forms and the rules between them: more rows than SMs and not; rows a little longer than the smallest form
+    (sampled groups overlap there); the longest k of the smallest form and one more; rows of which half is on the list."""
+    rng = np.random.default_rng(n + rows + k)
+    sc = np.stack([draw(kind, n, rng) for _ in range(rows)])
+    dev = torch.full((rows, (n + 3) // 4 * 4), float("nan"), device="cuda")
+    dev[:, :n] = torch.from_numpy(sc)
+    for causal in (False, True):
+        idx, cnt, kth = B.janus_topk(dev, n, k, q_pos0=n - rows, causal=causal)
+        B.check_dev_status()
+        idx, cnt, kth = idx.cpu().numpy(), cnt.cpu().numpy(), kth.cpu().numpy()
+        for t in {0, 1, rows // 2, rows - 2, rows - 1}:
+            check_row(idx[t], cnt[t], kth[t], sc[t, :n - rows + t + 1 if causal else n], k, f"{kind} row {t} of {rows} x {n}, k {k}")
 
 
 @pytest.mark.parametrize("kind", ["normal", "ties", "zeros", "hidden"])
