@@ -269,8 +269,8 @@ __device__ __forceinline__ bool mark_share(const PdParams& p, uint32_t* bm, int 
 }
 
 // ---- one cluster, a pool of few words --------------------------------------------------------------------------------------------
-// The sets of all CTAs are ORed into CTA 0's shared memory (PD_LISTS: there is one CTA, and the set is in global memory), which then makes the lists alone: a thread has a word, counts are 16 bits
-// each, runs are put together in shared memory.  One cluster-wide barrier on the way instead of four, and no exchange of counts: 7-8 -> 5 us.
+// The sets of all CTAs are ORed into CTA 0's shared memory, which then makes the lists alone (PD_LISTS: there is one CTA, and the set is
+// in global memory): a thread has a word, counts are 16 bits each, runs are put together in shared memory.  One cluster-wide barrier on the way instead of four, and no exchange of counts: 7-8 -> 5 us.
 constexpr int PD_FEW_RUNS = PD_FEW_WORDS * 16;
 struct PdFewShared {
     uint32_t own[PD_FEW_WORDS];

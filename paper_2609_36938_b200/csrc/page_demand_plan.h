@@ -12,9 +12,10 @@ constexpr int PD_SMEM_WORDS = PD_PORTABLE_CLUSTER * PD_THREADS;      // private 
 constexpr int PD_MAX_CLUSTERS = 64;
 constexpr int PD_FEW_WORDS = 256;
 
-// One launch of one cluster while it reads the indices as fast as memset, chip-wide marking and lists would (12.4 us up to 512 K
-// indices): 128 K indices in 9.6 us, 256 K in 12.3, 512 K in 17.4; and while its lists are as fast as those of several clusters: 131072
-// indices of 524288 pages 38.0 us in one launch, 20.4 without.
+// One launch of one cluster while it reads the indices as fast as clearing, chip-wide marking and lists would: 128 K indices of 142 pages
+// 5.7 us against 5.8, of 2112 pages 7.0 both, of 16384 pages 10.4 against 13.3, 32 K of 2112 pages 5.3 against 6.9; 64 rows with tables of their
+// own over 131136 pages 16.6 against 22.0; and while its lists are as fast as those of several clusters: 131072 indices of 524288 pages
+// 38.0 us in one launch, 20.4 without.
 constexpr int64_t PD_ONE_LAUNCH_INDICES = 1 << 17;
 
 struct PdPlan {
@@ -33,10 +34,11 @@ inline PdPlan page_demand_plan(int64_t n_idx, int n_words, int largest) {
     // device takes beyond: 2048 indices of 16384 pages 8.2 against 9.6 with four, of 131072 pages 11.8 against 19.1.
     if (n_idx <= PD_ONE_LAUNCH_INDICES && n_words <= PD_SMEM_WORDS)
         return {n_words <= PD_FEW_WORDS, true, n_idx <= 8192 && n_words <= PD_FEW_WORDS ? 4 : largest, 1};
-    // Lists alone: one CTA for a small pool (whole call of 4096 x 2048 indices of 2112 pages 26.3 us with a cluster of 8, 22.7 with one CTA; 2048 x 2048 of 544 18.5 and 14.6); larger pools are shared by clusters, which
-    // count what lies before them: up to four while each CTA has 256 words, then as many as give each one chunk.  524288 indices of 500000
-    // pages 43.2 us with one cluster, 30.0 with four; 131072 of 1048576 pages 55.6, 31.8, 23.5 and 29.3 with one, two, four and eight; of
-    // 2097152 pages 88 with one, 29.3 with four and 35.7 with eight.
+    // Lists alone: one CTA for a small pool (whole call of 4096 x 2048 indices of 2112 pages 26.3 us with a cluster of 8, 22.7 with one CTA;
+    // 2048 x 2048 of 544 pages 18.5 and 14.6); larger pools are shared by clusters, which count what lies before them: up to four while
+    // each CTA has 256 words, then as many as give each one chunk.  524288 indices of 500000 pages 43.2 us with one cluster, 30.0 with
+    // four; 131072 of 1048576 pages 55.6, 31.8, 23.5 and 29.3 with one, two, four and eight; of 2097152 pages 88 with one, 29.3 with four
+    // and 35.7 with eight.
     if (n_words <= PD_FEW_WORDS) return {true, false, PD_PORTABLE_CLUSTER, 1};
     const auto shares = [&](int64_t words) { return (n_words + words * largest - 1) / (words * largest); };
     int64_t n = shares(256) < 4 ? shares(256) : 4;

@@ -545,7 +545,9 @@ __global__ void __launch_bounds__(LP_THREADS, 1) sparse_attn_latent_pair_kernel(
             if (lane == 0) mbar_arrive(smem_u32(&sh->r_empty[slot]));
             if (++tile == n_tiles) { tile = 0; ++tok; }
         }
-        cp_async_wait<0>();              // (none in flight unless a wait gave up)
+        // None in flight unless a wait gave up.  Rows on their way by the TMA unit need no wait: a unit is asked for once the MMAs have
+        // freed its place, and a CTA leaves a wait's limit, a quarter of a second, after the last MMAs at the earliest.
+        cp_async_wait<0>();
     } else {
         // ================================================================== heads: softmax, output
         // Thread = head, half of the tile's keys (the lane's half of tensor memory) and one of its two quarters; of O, half of the lane's
