@@ -58,6 +58,7 @@ constexpr int LP_ATOM_BYTES = LP_OWN * 128;                      // 8 KB: 64 row
 constexpr int LP_KPARTS = 3;                // K units of a tile: atoms 6-8 (their queries lie in shared memory), 0-2, 3-5
 constexpr int LP_QPARTS = 2;                // units of a token that bring query atoms 0-2, 3-5 through the ring of K units
 constexpr int LP_KU = 4;                    // K units in the ring
+static_assert(LP_KU - LP_QPARTS >= 1 && LP_KU - LP_QPARTS <= LP_KPARTS, "a copy warp passes over the query units' places without a wait");
 constexpr int LP_K_BYTES = 3 * LP_ATOM_BYTES;
 constexpr int LP_VROWS = 32;                // keys of a V unit
 constexpr int LP_VPARTS = LP_TILE / LP_VROWS;
@@ -507,7 +508,10 @@ __global__ void __launch_bounds__(LP_THREADS, 1) sparse_attn_latent_pair_kernel(
             const int y = (cid + it * n_clusters) * LP_HEADS + LP_OWN * static_cast<int>(c);
             for (int a = 0; a < LP_QPARTS; ++a) {
                 uint64_t *const full = &sh->k_full[unit_slot], *const empty = &sh->k_empty[unit_slot];
-                ok = wait_warp(empty, unit_ph);
+                // ROWS: only the warp that fills the unit waits for its place.  The unit lands and its place is freed again without the others, so that
+                // one of them that looked late would meet the parity of the phase before and wait for good.  They need no wait: the places of the
+                // next two units were freed after this one, and they wait for those.
+                if (!ROWS || w == 0) ok = wait_warp(empty, unit_ph);
                 if (!ok) return;
                 if (w == 0 && elect_one()) {
                     if constexpr (!ROWS) mbar_expect_only(smem_u32(full), LP_K_BYTES);
