@@ -195,16 +195,18 @@ topk_ragged_kernel(const float* scores, const int64_t* row_offsets, const int64_
 
 // CTAs that share one of `rows` rows of up to `n` elements (n < 0: the lengths are on the device).  One CTA takes 7.5 us and 0.08 us
 // per thousand elements; a cluster streams its share only, but its start and its four cluster-wide barriers cost about a
-// microsecond, and more once the clusters leave few SMs free.  With 1, 2, 4 and 8 CTAs, k = 2048 (us): 8 rows of 12 K 8.1, 8.9, 9.6, 8.7; of 33 K 10.5,
-// 10.3, 10.3, 9.0; of 60 K 12.8, 11.3, 10.9, 8.9; of 131 K 18.4, 14.0, 12.0, 10.0; 24 rows of 60 K 13.1, 11.3, 11.1, 11.4; of 131 K 18.1, 13.9, 11.8,
-// 12.6; 74 rows of 48 K 11.7, 11.4, 21.5, 29.2; of 131 K 18.4, 14.4, 25.0, 32.5; 100 rows of 131 K 19.4, 19.8, 27.6, 40.8.  The lines were drawn with
-// a cluster form that took 1 to 1.4 us longer and are on the safe side of these figures: eight CTAs would pay from 16 K elements and up
-// to 12 rows, two from 40 K.  Rows whose length only the device knows take a cluster although short ones lose 0.5 us by it (200 elements 3.7 ->
-// 4.4), since long ones gain up to 18.
+// microsecond, and more once the clusters leave few SMs free.  With 1, 2, 4 and 8 CTAs, k = 2048 (us): 8 rows of 16 K 8.2, 8.7, 9.4, 9.1;
+// of 24 K 9.5, 9.3, 9.3, 9.2; of 50 K 11.7, 10.7, 10.1, 9.2; of 131 K 18.2, 13.6, 11.5, 10.1; 12 rows of 33 K 10.4, 10.1, 10.0, 10.9; of 50 K
+// 11.7, 10.8, 10.3, 11.0; of 131 K 17.9, 13.6, 12.1, 12.0; 24 rows of 33 K 10.4, 10.1, 12.1, 11.7; of 96 K 15.5, 12.4, 13.9, 12.8; of 131 K 18.3, 13.9, 14.2,
+// 12.9; 64 rows of 50 K 12.4, 13.7, 14.5, 22.5; of 96 K 19.4, 17.2, 16.6, 25.1; 74 rows of 64 K 14.2, 11.6, 21.3, 28.9.  Rows whose length only
+// the device knows take a cluster although short ones lose by it (12 rows of 200 elements 1.3 -> 1.8, of 9 K 7.5 -> 9.7, where two CTAs
+// take 8.8), since long ones gain up to 8.
 static int topk_cluster_size(int64_t rows, double n) {
     const bool unknown = n < 0;
-    if (rows <= 8 && (unknown || n >= 36e3)) return 8;
-    if (rows <= 24 && n >= 96e3) return 4;
+    if (rows <= 8 && (unknown || n >= 22e3)) return 8;
+    if (rows <= 14 && (unknown || n >= 36e3)) return 4;
+    if (rows > 14 && rows <= 30 && n >= 112e3) return 8;
+    if (rows <= 37 && n >= 32e3) return 2;
     if (rows <= 74 && (unknown || n >= 64e3)) return 2;
     return 1;
 }
