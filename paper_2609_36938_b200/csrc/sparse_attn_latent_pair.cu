@@ -250,7 +250,6 @@ __global__ void __launch_bounds__(LP_THREADS, 1) sparse_attn_latent_pair_kernel(
         for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&sh->drain[i]), 1);
         fence_mbar_init();
     }
-    __syncwarp();
     grid_wait();
     cluster_wait();                                // every CTA of the cluster runs: its shared memory may be written
     if (threadIdx.x == 0) {
