@@ -175,8 +175,8 @@ __device__ __forceinline__ void st_global_v8(void* p, uint32_t a, uint32_t b, ui
                  "r"(h)
                  : "memory");
 }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+// Waits for every cp.async copy of this thread, whether it was made part of a group or not.
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 
 // Split form of the TMEM load: tmem_ld32_issue starts the load, tmem_ld_wait(r) waits for it.  The wait takes the

@@ -548,9 +548,11 @@ __global__ void __launch_bounds__(LP_THREADS, 1) sparse_attn_latent_pair_kernel(
             if (lane == 0) mbar_arrive(smem_u32(&sh->r_empty[slot]));
             if (++tile == n_tiles) { tile = 0; ++tok; }
         }
-        // None in flight unless a wait gave up.  Rows on their way by the TMA unit need no wait: a unit is asked for once the MMAs have
-        // freed its place, and a CTA leaves a wait's limit, a quarter of a second, after the last MMAs at the earliest.
-        cp_async_wait<0>();
+        // Nothing may be on its way into shared memory when the CTA leaves, also after a wait somewhere gave up.  Copies of this thread by
+        // cp.async are waited for as such.  Rows and queries by the TMA unit have landed once the MMAs have freed every place that was filled;
+        // where those no longer come, the limit of one such wait, a quarter of a second, has passed since the last was asked for.
+        cp_async_wait_all();
+        for (int u = 0; !is_v && u < LP_KU && wait_warp(&sh->k_empty[unit_slot], unit_ph); ++u) next_place();
     } else {
         // ================================================================== heads: softmax, output
         // Thread = head, half of the tile's keys (the lane's half of tensor memory) and one of its two quarters; of O, half of the lane's

@@ -25,3 +25,14 @@ def test_aligned_cluster_barriers_follow_a_reconvergence():
                 wrappers += 1
                 assert "__syncwarp();" in body[:m.start()], body
     assert wrappers == len(re.findall(r"void cluster_(?:sync_all|arrive|arrive_release|wait)\(", code("sm100_ptx.cuh"))) == 4
+
+
+def test_copies_in_flight_are_waited_for():
+    """cp.async.wait_group waits for committed groups only; copies that are counted on an mbarrier belong to none.  Who issues copies that way
+    ends with cp.async.wait_all."""
+    everything = {name: code(name) for name in os.listdir(build.CSRC)}
+    commits = any("cp.async.commit_group" in text for text in everything.values())
+    assert commits or not any("cp.async.wait_group" in text for text in everything.values())
+    for name, text in everything.items():
+        if "cp_async_arrive(" in text and name != "sm100_ptx.cuh":
+            assert text.rindex("cp_async_wait_all()") > text.rindex("cp_async_arrive("), name
