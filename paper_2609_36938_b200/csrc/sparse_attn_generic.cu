@@ -119,7 +119,11 @@ sparse_attn_generic_kernel(const uint16_t* q, int M, int H_q, int d_qk, const ui
         for (int g = 0; g < G; ++g) {
             const float tile_max = corr[g];
             const float m_new = fmaxf(m_run[g], tile_max);
-            if (m_new == __int_as_float(0xff800000)) continue;   // nothing selected so far
+            if (m_new == __int_as_float(0xff800000)) {            // nothing selected so far, or only logits that are not numbers
+                for (int r = 0; r < AG_KT; ++r)
+                    if (isnan(ps[g * AG_KT + r])) l_run[g] = ps[g * AG_KT + r];
+                continue;
+            }
             const float scale_old = __expf(m_run[g] - m_new);     // exp(-inf) = 0 on the first tile
             float tile_sum = 0.f;
             for (int r = 0; r < AG_KT; ++r) tile_sum += __expf(ps[g * AG_KT + r] - m_new);
@@ -149,7 +153,7 @@ sparse_attn_generic_kernel(const uint16_t* q, int M, int H_q, int d_qk, const ui
 #pragma unroll
     for (int g = 0; g < G; ++g) {
         if (g >= g_count) continue;
-        const float inv = l_run[g] > 0.f ? 1.f / l_run[g] : 0.f;
+        const float inv = l_run[g] != 0.f ? 1.f / l_run[g] : 0.f;      // (a NaN is a sum)
         const int64_t o = (static_cast<int64_t>(t) * H_q + h0 + g) * d_v;
         if (c0 < d_v) {
             __nv_bfloat162 a = __floats2bfloat162_rn(acc[g][0] * inv, acc[g][1] * inv);
@@ -160,7 +164,7 @@ sparse_attn_generic_kernel(const uint16_t* q, int M, int H_q, int d_qk, const ui
             *reinterpret_cast<uint2*>(out + o + c0) = pk;
         }
         if (lse != nullptr && tid == 0)
-            lse[static_cast<int64_t>(t) * H_q + h0 + g] = l_run[g] > 0.f ? m_run[g] + logf(l_run[g]) : __int_as_float(0xff800000);
+            lse[static_cast<int64_t>(t) * H_q + h0 + g] = l_run[g] != 0.f ? m_run[g] + logf(l_run[g]) : __int_as_float(0xff800000);
     }
 }
 

@@ -347,14 +347,14 @@ sparse_attn_heads_kernel(const AhParams p) {
         if (split != 0) return;
     }
     if (h < n_heads) {
-        const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+        const float inv = l_all != 0.f ? 1.f / l_all : 0.f;          // (a NaN is a sum)
         uint32_t* dst = reinterpret_cast<uint32_t*>(p.out + (row * p.H_q + h0 + h) * DV + d0);
 #pragma unroll
         for (int e = 0; e < PER; e += 2) {
             const __nv_bfloat162 v = __floats2bfloat162_rn(acc[e] * inv, acc[e + 1] * inv);
             dst[e / 2] = *reinterpret_cast<const uint32_t*>(&v);
         }
-        if (d0 == 0 && p.lse != nullptr) p.lse[row * p.H_q + h0 + h] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : neg_inf;
+        if (d0 == 0 && p.lse != nullptr) p.lse[row * p.H_q + h0 + h] = l_all != 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : neg_inf;
     }
 }
 

@@ -167,7 +167,7 @@ __device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s,
         f[r] = m_all == neg_inf ? 0.f : lp_exp2(f[r] - m_all);
         l_all = fmaf(f[r], l[r], l_all);
     }
-    const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+    const float inv = l_all != 0.f ? 1.f / l_all : 0.f;        // (a NaN is a sum)
     constexpr int GROUPS = LP_THREADS / LP_TILE;
     if (threadIdx.x < GROUPS * LP_TILE) {
         for (int blk = s + N * (threadIdx.x / LP_TILE); blk < LP_DVH / 16; blk += N * GROUPS) {
@@ -202,7 +202,7 @@ __device__ __forceinline__ void lp_merge_splits(const LpParams& p, int t, int s,
         }
     }
     if (p.lse != nullptr && s == 0 && threadIdx.x < LP_OWN)
-        p.lse[static_cast<int64_t>(t) * LP_HEADS + LP_OWN * c + h] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : neg_inf;
+        p.lse[static_cast<int64_t>(t) * LP_HEADS + LP_OWN * c + h] = l_all != 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : neg_inf;
 }
 
 // SPLIT = false: clusters of two CTAs, persistent over tokens.  SPLIT = true: a cluster of 2 n CTAs takes one token, pair s of it
@@ -576,8 +576,8 @@ __global__ void __launch_bounds__(LP_THREADS, 1) sparse_attn_latent_pair_kernel(
         auto write_out = [&](int it, float m_ref) {
             const float(&l)[4][LP_OWN] = sh->l[it & 1];
             const float l_sum = (l[0][h] + l[1][h]) + (l[2][h] + l[3][h]);
-            const bool have_o = __any_sync(0xffffffffu, l_sum > 0.f);   // some key of one of these heads counts
-            const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
+            const bool have_o = __any_sync(0xffffffffu, l_sum != 0.f);  // some key of one of these heads counts, be it as NaN
+            const float inv = l_sum != 0.f ? 1.f / l_sum : 0.f;
             uint16_t* orow = p.out + lp_out_offset(token(it), c, ln) + ch * 128;
             float* mo = reinterpret_cast<float*>(k_smem);               // SPLIT: nothing reads the rings any more
             if (SPLIT && part == 0) { sh->split_m[h] = m_ref; sh->split_l[h] = l_sum; }
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(LP_THREADS, 1) sparse_attn_latent_pair_kernel(
                 }
             }
             if (!SPLIT && p.lse != nullptr && part == 0)
-                p.lse[static_cast<int64_t>(token(it)) * LP_HEADS + LP_OWN * c + h] = l_sum > 0.f ? (m_ref + log2f(l_sum)) * 0.6931471805599453f : neg_inf;
+                p.lse[static_cast<int64_t>(token(it)) * LP_HEADS + LP_OWN * c + h] = l_sum != 0.f ? (m_ref + log2f(l_sum)) * 0.6931471805599453f : neg_inf;
         };
         int gi = 0;                 // tiles done so far, over all tokens
         float m_ref = neg_inf, m_prev = neg_inf;
