@@ -21,6 +21,7 @@ namespace janus {
 // streaming loads pass, with 54 KB a third: 4096 rows of 135168 390 us against 498, 1024 of 16384 28 against 35.  (Four CTAs of 54 KB and
 // 32 registers: 497.)
 constexpr int TK_CAP = 8192;
+constexpr int TK_CAP_SMALLEST = 3840;
 
 template <int CAP>
 __global__ void __launch_bounds__(TK_THREADS)
@@ -36,7 +37,7 @@ topk_rows_kernel(const float* scores, int64_t ld, int M, int64_t n_keys, int64_t
         const int64_t prefix64 = causal ? min(n_keys, q_pos0 + t + 1) : n_keys;
         const int t_next = t + gridDim.x;
         const int64_t prefix_next = t_next < M ? (causal ? min(n_keys, q_pos0 + t_next + 1) : n_keys) : 0;
-        topk_row(scores + static_cast<int64_t>(t) * ld, static_cast<int>(prefix64), k, idx + static_cast<int64_t>(t) * k,
+        topk_row<CAP == TK_CAP_SMALLEST>(scores + static_cast<int64_t>(t) * ld, static_cast<int>(prefix64), k, idx + static_cast<int64_t>(t) * k,
                  count != nullptr ? count + t : nullptr, kth != nullptr ? kth + t : nullptr, sh, t_next < M ? scores + static_cast<int64_t>(t_next) * ld : nullptr, static_cast<int>(prefix_next));
         __syncthreads();   // the selection state in shared memory is reused by the next row
     }
@@ -219,7 +220,7 @@ struct TopkForm {
 template <int CAP>
 constexpr TopkForm topk_form() { return {topk_rows_kernel<CAP>, CAP, static_cast<int>(sizeof(TopkSharedT<CAP>))}; }
 constexpr int TK_FORMS = 3;
-static const TopkForm topk_forms[TK_FORMS] = {topk_form<3840>(), topk_form<5632>(), topk_form<TK_CAP>()};
+static const TopkForm topk_forms[TK_FORMS] = {topk_form<TK_CAP_SMALLEST>(), topk_form<5632>(), topk_form<TK_CAP>()};
 
 // Kernel attributes, set once in every context, and the number of resident CTAs, a property of the device.
 struct TopkDevice {
@@ -369,16 +370,18 @@ extern "C" int janus_topk(const float* scores, int64_t scores_ld, int M, int64_t
     // form is taken into which the list plus five deviations fits for the longest row, since less shared memory leaves more of it to L1
     // (2048 rows of 34816 102.7 us with 5632 slots, 96.7 with 3840; 777 of 20788 34.7 and 32.3; 4096 of 135168 498 with 8192 and 396 with
     // 5632); a row that overflows all the same is selected from global memory.  Rows that fit a form whole are taken whole where CTAs have
-    // an SM each or half of the row is on the list anyway (256 of 4000, k = 2048, 8.9 us, 11.3 through the sample; 256 of 8000 13.9 and 11.9;
-    // 4000 of 6000, k = 512, 88 and 76).
+    // an SM each, half of the row is on the list anyway or the list needs more than the smallest form, which alone is safe against a crowd at
+    // the threshold (256 of 4000, k = 2048, 8.9 us, 11.3 through the sample; 256 of 8000 17.8 and 12.5; 4000 of 6000, k = 512, 216 and 85;
+    // of values in steps of one half 169 and 156, but with few to select the sample's further passes show: 4000 of 3900, k = 64, 100 and 128).
     const double n_max = static_cast<double>(causal ? (n_keys < q_pos0 + M ? n_keys : q_pos0 + M) : n_keys);
     const double e = n_max > 0. ? 4096.0 * k / n_max : 0., r = e + 4.0 * sqrt(e) + 8.0, list = n_max * (r + 5.0 * sqrt(r)) / 4096.0;
     TopkDevice d;
     JANUS_CUDA_CHECK(topk_device(d));
-    const bool share = M > d.n_sm, whole = n_max <= TK_CAP && (!share || list > n_max / 2);
-    const double slots = whole ? n_max : list;
+    const bool share = M > d.n_sm;
+    auto fits = [&](int f) { return list <= topk_forms[f].cap && k <= topk_forms[f].cap / 2 + 256; };
+    const bool whole = n_max <= TK_CAP && (!share || list > n_max / 2 || !fits(0));
     int form = share ? 0 : 1;
-    while (form < TK_FORMS - 1 && (slots > topk_forms[form].cap || (!whole && k > topk_forms[form].cap / 2 + 256))) ++form;
+    while (form < TK_FORMS - 1 && !(whole ? n_max <= topk_forms[form].cap : fits(form))) ++form;
     const int cluster = topk_cluster_size(M, n_max);
     if (cluster > 1) {
         JANUS_CUDA_CHECK(launch_kernel(topk_rows_cluster_kernel, dim3(M * cluster), TK_THREADS, sizeof(TopkSharedT<TK_CAP>), stream, cluster, scores,

@@ -41,6 +41,7 @@ struct TopkSharedT {
     uint32_t red_lo, red_hi;
     int sel_bucket, sel_above, sel_count;
     int n_small;
+    int crowd;                            // see sample_threshold
     int sel_out;                          // cluster form: next free slot of the row's output
 };
 
@@ -232,7 +233,8 @@ __device__ __forceinline__ int4 own_buckets(const Sh& sh) { return reinterpret_c
 
 // Streaming threshold out of a sample of which every thread holds N keys: the lower edge of the bucket that holds the sample's
 // r-th key, once that bucket holds no more than `slack` keys; a fuller one is split further, up to a width of one key.  `hi` receives
-// the largest sample key.
+// the largest sample key, sh.crowd (after a barrier) zero or, where the threshold is one value of which there are more than `slack`, the
+// number of sample keys from it on.
 template <int N, class Sh>
 __device__ __forceinline__ uint32_t sample_threshold(const uint32_t (&key)[N], int r, int slack, uint32_t& hi, Sh& sh) {
     uint32_t lo = key[0];
@@ -242,16 +244,20 @@ __device__ __forceinline__ uint32_t sample_threshold(const uint32_t (&key)[N], i
     clear_hist(sh);
     block_key_range(lo, hi, sh);
     uint32_t top = hi;
-    for (int pass = 0;; ++pass) {
+    int above = 0;
+    for (;;) {
         const BucketMap map(lo, top);
 #pragma unroll
         for (int j = 0; j < N; ++j)
             if (key[j] >= lo && key[j] <= top) atomicAdd(&sh.hist[map(key[j])], 1);
         __syncthreads();
-        find_bucket(own_buckets(sh), r, sh);
+        find_bucket(own_buckets(sh), r - above, sh);
         const int b = sh.sel_bucket, count = sh.sel_count;
-        if (count <= slack || map.shift == 0 || pass == 2) return map.first(b);
-        r -= sh.sel_above;
+        above += sh.sel_above;
+        if (count <= slack || map.shift == 0) {
+            if (threadIdx.x == 0) sh.crowd = count <= slack ? 0 : above + count;
+            return map.first(b);
+        }
         if (b < TK_BUCKETS - 1) top = min(top, map.last(b));
         lo = map.first(b);
         clear_hist(sh);
@@ -452,12 +458,41 @@ __device__ __noinline__ void topk_exact_row(const float* row, int n, int k, int3
     if (threadIdx.x == 0 && kth != nullptr) *kth = key_to_float(T);
 }
 
+// Positions of `need` elements of the row that equal t to out[0 .. need), whichever come first.  sh.n_small, zero on entry, counts those
+// found; at the end it is below `need` if the row has no more.
+template <class Sh>
+__device__ __noinline__ void topk_copies(const float* row, int n, float t, int need, int32_t* __restrict__ out, Sh& sh) {
+    const float nan = __int_as_float(0x7fffffff);
+    const int n4 = n >> 2;
+    for (int i = threadIdx.x; i <= n4 && *reinterpret_cast<volatile int*>(&sh.n_small) < need; i += TK_THREADS) {
+        float4 x = make_float4(nan, nan, nan, nan);
+        if (i < n4) {
+            x = __ldcg(reinterpret_cast<const float4*>(row) + i);
+        } else {                                   // the n % 4 elements after the last whole group
+            if (4 * n4 < n) x.x = __ldcg(row + 4 * n4);
+            if (4 * n4 + 1 < n) x.y = __ldcg(row + 4 * n4 + 1);
+            if (4 * n4 + 2 < n) x.z = __ldcg(row + 4 * n4 + 2);
+        }
+        const int c = (x.x == t ? 1 : 0) + (x.y == t ? 1 : 0) + (x.z == t ? 1 : 0) + (x.w == t ? 1 : 0);
+        if (c == 0) continue;
+        int o = atomicAdd(&sh.n_small, c);
+        auto put = [&](float v, int e) {
+            if (v == t && o < need) out[o++] = e;
+        };
+        put(x.x, 4 * i); put(x.y, 4 * i + 1); put(x.z, 4 * i + 2); put(x.w, 4 * i + 3);
+    }
+}
+
 // Top-k of one fp32 row of n elements (16-byte aligned) by the whole CTA (TK_THREADS threads): out[0..k) receives the
 // indices (-1 padded), *count / *kth the number selected and the smallest selected value (either may be NULL).
 // `next_row` (may be NULL): the row this CTA takes next.  The sample sectors of that row are requested into L2 once this
 // row's streaming pass is over, so the next sample does not start with a DRAM round trip.  (Requesting the head of the next
 // row as well, 96 to 512 KB, made the kernel slower: 0.49 -> 0.50 .. 0.58 ms at 4096 rows of 135168.)
-template <class Sh>
+// COPIES: a threshold that is one value with more copies than the list holds (scores cut off at zero, coarse ones) is met by a list of what
+// lies above it; if that is less than k, copies are looked for afterwards, as many as are missing.  For the small lists: 4000 rows of 8000,
+// k = 512, of which 7 % above zero 105 us, 270 when the list overflows and the row is selected from global memory, 148 with the row in
+// shared memory.  The larger ones seldom overflow, and the few instructions cost them 1 to 3 %.
+template <bool COPIES = false, class Sh>
 __device__ __forceinline__ void topk_row(const float* row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
                          float* __restrict__ kth, Sh& sh, const float* next_row = nullptr, int next_n = 0) {
     const int tid = threadIdx.x;
@@ -489,12 +524,14 @@ __device__ __forceinline__ void topk_row(const float* row, int n, int k, int32_t
         return;
     }
     uint32_t thr, hi;
-    if (tid == 0) sh.n_cand = 0;
+    if (tid == 0) { sh.n_cand = 0; sh.n_small = 0; }
     const bool sampled = topk_sample(row, n, k, thr, hi, sh);
     if (sampled) {
-        const BucketMap map(thr, max(thr, hi));
         clear_hist(sh);
         __syncthreads();
+        auto tied = [&]() { return COPIES && static_cast<int64_t>(sh.crowd) * n > static_cast<int64_t>(Sh::kCap) * (TK_SAMPLE - TK_SAMPLE / 8); };
+        if (tied()) thr += thr == float_to_key(-0.f) ? 2u : 1u;      // (-0 and +0 are the same value)
+        const BucketMap map(thr, max(thr, hi));
         topk_stream(row, n, 0, n >> 2, true, key_to_float(thr), sh);
         if (next_row != nullptr && next_n > Sh::kCap) topk_prefetch_l2(next_row + sample_offset(next_n));
         __syncthreads();
@@ -504,6 +541,16 @@ __device__ __forceinline__ void topk_row(const float* row, int n, int k, int32_t
             __syncthreads();
             select_and_emit(SmemSource{sh.cand_key, sh.cand_idx, n_cand}, map, k, out, kth, sh);
             return;
+        }
+        if (n_cand < k && n_cand <= Sh::kCap && tied()) {
+            const float t = key_to_float(thr - 1u);
+            topk_copies(row, n, t, k - n_cand, out + n_cand, sh);
+            __syncthreads();
+            if (sh.n_small >= k - n_cand) {
+                for (int i = tid; i < n_cand; i += TK_THREADS) out[i] = sh.cand_idx[i];
+                if (tid == 0 && kth != nullptr) *kth = t;
+                return;
+            }
         }
     }
     __syncthreads();
