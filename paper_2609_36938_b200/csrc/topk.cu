@@ -13,6 +13,7 @@
 // sampling step.
 #include <algorithm>
 
+#include "topk_plan.h"
 #include "topk_select.cuh"
 
 namespace janus {
@@ -192,24 +193,6 @@ topk_ragged_kernel(const float* scores, const int64_t* row_offsets, const int64_
         topk_row_cluster(scores + off, static_cast<int>(n), k, out, count != nullptr ? count + b : nullptr, kth != nullptr ? kth + b : nullptr, sh);
     else
         topk_row(scores + off, static_cast<int>(n), k, out, count != nullptr ? count + b : nullptr, kth != nullptr ? kth + b : nullptr, sh);
-}
-
-// CTAs that share one of `rows` rows of up to `n` elements (n < 0: the lengths are on the device).  One CTA takes 7.5 us and 0.08 us
-// per thousand elements; a cluster streams its share only, but its start and its four cluster-wide barriers cost about a
-// microsecond, and more once the clusters leave few SMs free.  With 1, 2, 4 and 8 CTAs, k = 2048 (us): 8 rows of 16 K 8.2, 8.7, 9.4, 9.1;
-// of 24 K 9.5, 9.3, 9.3, 9.2; of 50 K 11.7, 10.7, 10.1, 9.2; of 131 K 18.2, 13.6, 11.5, 10.1; 12 rows of 33 K 10.4, 10.1, 10.0, 10.9; of 50 K
-// 11.7, 10.8, 10.3, 11.0; of 131 K 17.9, 13.6, 12.1, 12.0; 24 rows of 33 K 10.4, 10.1, 12.1, 11.7; of 96 K 15.5, 12.4, 13.9, 12.8; of 131 K 18.3, 13.9, 14.2,
-// 12.9; 64 rows of 50 K 12.4, 13.7, 14.5, 22.5; of 96 K 19.4, 17.2, 16.6, 25.1; 74 rows of 64 K 14.2, 11.6, 21.3, 28.9.  Rows whose length only
-// the device knows take a cluster although short ones lose by it (12 rows of 200 elements 1.3 -> 1.8, of 9 K 7.5 -> 9.7, where two CTAs
-// take 8.8), since long ones gain up to 8.
-static int topk_cluster_size(int64_t rows, double n) {
-    const bool unknown = n < 0;
-    if (rows <= 8 && (unknown || n >= 22e3)) return 8;
-    if (rows <= 14 && (unknown || n >= 36e3)) return 4;
-    if (rows > 14 && rows <= 30 && n >= 112e3) return 8;
-    if (rows <= 37 && n >= 32e3) return 2;
-    if (rows <= 74 && (unknown || n >= 64e3)) return 2;
-    return 1;
 }
 
 // The forms of topk_rows_kernel, by candidate slots.

@@ -14,6 +14,7 @@
 
 #include "janus_common.cuh"
 #include "sm100_ptx.cuh"
+#include "topk_plan.h"
 
 namespace janus {
 
@@ -559,7 +560,7 @@ __device__ __forceinline__ void topk_row(const float* row, int n, int k, int32_t
 
 // The same by a cluster of CTAs (few rows): each CTA samples alike, streams its share of the row into its own candidates and
 // histogram, the histograms are added through distributed shared memory, every CTA emits its own keys above the k-th key's
-// bucket, and CTA 0 ranks the bucket's keys of all of them.
+// bucket, and CTA 0 ranks the bucket's keys of all of them.  CTA 0 takes a short row alone.
 template <class Sh>
 __device__ __forceinline__ void topk_row_cluster(const float* row, int n, int k, int32_t* __restrict__ out, int32_t* __restrict__ count,
                                  float* __restrict__ kth, Sh& sh) {
@@ -572,7 +573,7 @@ __device__ __forceinline__ void topk_row_cluster(const float* row, int n, int k,
     const int64_t n4 = n >> 2;
     const int f4_begin = static_cast<int>(n4 * rank / n_cta), f4_end = static_cast<int>(n4 * (rank + 1) / n_cta);
     float4 x[4];
-    bool split = n > Sh::kCap && n > k;            // the same answer in every CTA
+    bool split = n >= topk_split_from(n_cta) && n > k;      // the same answer in every CTA
     if (split) {
         load_groups(reinterpret_cast<const float4*>(row), f4_begin + tid, f4_end, x);
         split = topk_sample(row, n, k, thr, hi, sh);

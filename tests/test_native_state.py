@@ -112,3 +112,30 @@ def test_page_demand_plan_keeps_to_the_clusters_of_the_device(tmp_path):
     exe = tmp_path / "plan"
     subprocess.check_call(["g++", "-std=c++17", "-I", build.CSRC, str(src), "-o", str(exe)])
     assert subprocess.run([str(exe)]).returncode == 0
+
+
+def test_topk_clusters_split_the_rows_they_are_launched_for(tmp_path):
+    """The rules that share rows out: cluster sizes that the device's kernels take, no cluster for rows that it would leave to its first CTA, and
+    rows of a length that only the device knows are split under the same sizes as the others."""
+    src = tmp_path / "plan.cpp"
+    src.write_text(textwrap.dedent("""
+        #include "topk_plan.h"
+        using namespace janus;
+        int main() {
+            for (int64_t rows = 1; rows <= 200; ++rows) {
+                const int unknown = topk_cluster_size(rows, -1.);
+                if (unknown != 1 && unknown != 2 && unknown != 4 && unknown != 8) return 1;
+                if (topk_split_from(unknown) <= 8192) return 2;
+                for (double n = 0; n < 300e3; n += 500) {
+                    const int c = topk_cluster_size(rows, n);
+                    if (c != 1 && c != 2 && c != 4 && c != 8) return 3;
+                    if (c > 1 && n < topk_split_from(c)) return 4;
+                    if (c > 1 && unknown == 1) return 5;
+                }
+            }
+            return 0;
+        }
+    """))
+    exe = tmp_path / "plan"
+    subprocess.check_call(["g++", "-std=c++17", "-I", build.CSRC, str(src), "-o", str(exe)])
+    assert subprocess.run([str(exe)]).returncode == 0
