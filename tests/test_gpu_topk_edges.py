@@ -72,7 +72,8 @@ def test_topk_rows(kind, rows, n):
 @pytest.mark.parametrize("kind", ["normal", "ties", "cut", "zeros", "outlier", "hidden"])
 @pytest.mark.parametrize("rows,n,k", [(148, 8192, 64), (149, 3840, 64), (149, 3841, 64), (300, 4090, 1000), (160, 4500, 2048), (149, 5633, 700),
                                       (149, 8192, 2048), (149, 8193, 2176), (149, 8193, 2177), (700, 20003, 2048), (160, 20003, 3500),
-                                      (8, 22004, 2048), (14, 36003, 2048), (15, 36003, 2048), (30, 112007, 2048), (37, 32009, 1000)])
+                                      (8, 22004, 2048), (14, 36003, 2048), (15, 36003, 2048), (30, 112007, 2048), (37, 32009, 1000),
+                                      (14, 45003, 2048), (30, 32009, 1000), (33, 112007, 2048), (34, 112007, 2048)])
 def test_topk_rows_that_share_an_sm(kind, rows, n, k):
     """Around the slots of the three forms and the rules between them: more rows than SMs and not; rows a little longer than the smallest form
     (sampled groups overlap there); the longest k of the smallest form and one more; rows of which half is on the list; the lines between cluster sizes."""

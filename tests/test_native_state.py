@@ -133,6 +133,11 @@ def test_topk_clusters_split_the_rows_they_are_launched_for(tmp_path):
                     if (c > 1 && unknown == 1) return 5;
                 }
             }
+            // on both sides of the lines in rows: what measured faster there
+            const struct { int rows; double n; int cluster; } at[] = {{8, 40e3, 8}, {9, 40e3, 2}, {9, 50e3, 4}, {14, 50e3, 4}, {15, 50e3, 2}, {30, 40e3, 2},
+                                                                      {31, 40e3, 1}, {36, 40e3, 1}, {33, 112e3, 8}, {34, 112e3, 2}, {74, 64e3, 2}, {75, 64e3, 1}};
+            for (const auto& a : at)
+                if (topk_cluster_size(a.rows, a.n) != a.cluster) return 6;
             return 0;
         }
     """))
