@@ -30,6 +30,17 @@ def upload_session(sess, device="cuda"):
     return d
 
 
+def strided_pool(bits, tok_pad, page_pad):
+    """bits [n_pages, page, 1, 576] as a device tensor whose rows are 576 + tok_pad apart and whose pages have page_pad elements behind them;
+    everything between is NaN."""
+    n, page = bits.shape[:2]
+    tok = 576 + tok_pad
+    buf = torch.full((n * (page * tok + page_pad),), float("nan"), dtype=torch.bfloat16, device="cuda")
+    view = buf.as_strided((n, page, 1, 576), (page * tok + page_pad, tok, 576, 1))
+    view.copy_(B.to_device(bits, "bf16"))
+    return view
+
+
 def bf16_tensor_to_f64(t: torch.Tensor) -> np.ndarray:
     return t.detach().to(torch.float64).cpu().numpy()
 

@@ -22,17 +22,6 @@ def _lib():
     B.check_dev_status()
 
 
-def strided_pool(bits, tok_pad, page_pad):
-    """bits [n_pages, page, 1, 576] as a device tensor whose rows are 576 + tok_pad apart and whose pages have page_pad elements behind them;
-    everything between is NaN."""
-    n, page = bits.shape[:2]
-    tok = 576 + tok_pad
-    buf = torch.full((n * (page * tok + page_pad),), float("nan"), dtype=torch.bfloat16, device="cuda")
-    view = buf.as_strided((n, page, 1, 576), (page * tok + page_pad, tok, 576, 1))
-    view.copy_(B.to_device(bits, "bf16"))
-    return view
-
-
 @pytest.mark.parametrize("tok_pad,page_pad", [(0, 0), (64, 0), (0, 576), (0, 8), (64, 72)])
 @pytest.mark.parametrize("M,k,page", [(1, 1, 64), (3, 300, 16), (160, 128, 64), (160, 129, 64), (230, 37, 48), (230, 383, 16)])
 def test_tokens_strides_and_tails(M, k, page, tok_pad, page_pad):
@@ -51,7 +40,7 @@ def test_tokens_strides_and_tails(M, k, page, tok_pad, page_pad):
     sel = idx[idx >= 0]
     used[table[sel // page], sel % page] = True
     pool[~used] = 0x7fc0
-    kd = strided_pool(pool, tok_pad, page_pad)
+    kd = Hp.strided_pool(pool, tok_pad, page_pad)
     scale = 1.0 / 24.0
     out, lse = B.janus_sparse_attn_prefill(B.to_device(Q, "bf16"), kd, kd, B.to_device(idx, "i32"), page_table=B.to_device(table, "i32"), page_size=page,
                                            softmax_scale=scale, d_v=512)
