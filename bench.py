@@ -151,6 +151,11 @@ def captured_traffic(kernel_key: str, rows: int):
     return None if e is None else e["bytes"] * rows / e["rows"]
 
 
+def page_demand_launches(n_idx: int, n_phys_pages: int) -> int:
+    """Kernels of one janus_page_demand call: one up to 128 K indices of a pool of up to 262144 pages, else clearing, marking and lists."""
+    return 1 if n_idx <= 1 << 17 and n_phys_pages <= 1 << 18 else 3
+
+
 def workload_numbers(shp):
     """Algorithmic work of one step (exact pass): flops and bytes each call must do at least, from the shapes alone."""
     L, M, S = shp.L, shp.M, shp.S
@@ -364,7 +369,8 @@ def run_sharded_prediction(args, rank, world, local_rank):
                 "config": {"workload": f"key-sharded prediction pass (Eq. 3): L={shp.L} M={shp.M} k={shp.k} -> top-{k_shard} per shard, {world} page-aligned "
                                        f"history shards, indexer {shp.H_I}x{shp.D_I} {kind}, page {shp.page_size}, shuffled page table",
                            "exchange": "one all-gather of the page bitmaps + local union (janus_page_union) per step"},
-                "gpu_launches": 6 * args.steps, "page_report_vs_exact": rep}
+                # of this rank: indexer, top-k, page demand, a union with every other rank's bitmap
+                "gpu_launches": (2 + page_demand_launches(shp.M * k_shard, n_phys) + world - 1) * args.steps, "page_report_vs_exact": rep}
         print(json.dumps(line))
     if world > 1:
         dist.destroy_process_group()
@@ -450,7 +456,8 @@ def run_query_sharded(args, rank, world, local_rank):
                 "config": {"workload": f"query-sharded exact pass: L={shp.L} M={shp.M} k={shp.k} split into {world} contiguous row slices, keys and KV pool "
                                        f"replicated, indexer {shp.H_I}x{shp.D_I} {kind}, latent attention, page {shp.page_size}",
                            "exchange": "one all-gather of the page bitmaps + local union (janus_page_union) per step"},
-                "gpu_launches": 6 * args.steps, "union_pages": R.popcount(union)}
+                # of this rank: indexer, top-k, page demand, attention (no rows, none of them), a union with every other rank's bitmap
+                "gpu_launches": ((3 + page_demand_launches(m * shp.k, n_phys) if m > 0 else 0) + world - 1) * args.steps, "union_pages": R.popcount(union)}
         print(json.dumps(line))
     if world > 1:
         dist.destroy_process_group()
@@ -878,8 +885,9 @@ def main():
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "fp8_e4m3+bf16" if fp8 else "bf16", "data": "synthetic",
         "config": config, "clocks": clocks, "e2e": e2e,
-        # kernels of this library per session pass: indexer, top-k, page mark, page lists, attention (plus one cudaMemsetAsync of the bitmap)
-        "gpu_launches": 6 * args.steps * n_sessions, "roofline": roofline, "cpu_baseline": cpu_baseline, "fp8_peak_probe": fp8_probe,
+        # kernels of this library: indexer, top-k, page demand and attention of every session
+        "gpu_launches": sum(3 + page_demand_launches(x.M * x.k, n_phys) for x in shapes) * args.steps,
+        "roofline": roofline, "cpu_baseline": cpu_baseline, "fp8_peak_probe": fp8_probe,
         "kernels": {k: {kk: (round(float(vv), 4)) for kk, vv in v.items()} for k, v in kernels.items()},
         "indexer_topk_one_call": fused,
         "page_demand": {"n_pages": int(counts[0]), "n_runs": int(counts[1]), "n_miss": int(counts[2]), "n_miss_runs": int(counts[3])},
