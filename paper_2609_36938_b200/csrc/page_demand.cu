@@ -213,64 +213,65 @@ __device__ __forceinline__ void block_scan2_u64(uint64_t (&v)[2], uint64_t (*war
 template <int MODE>
 __device__ __forceinline__ bool mark_share(const PdParams& p, uint32_t* bm, int rank, int n_cta) {
     const int tid = threadIdx.x;
-            const PageDiv page{p.page_size, p.page_shift};
-            bool bad = false;
-            // Eight indices per thread at a time, in rounds of loads that are all in flight together: indices and their rows' table and
-            // limit, then page table entries (one index after the other: 24.2 us instead of 21.9 for 64 decode rows of 2048, when the rest took 5 us longer)
-            constexpr int U = 8;
-            const int stride = n_cta * PD_THREADS, n_idx = static_cast<int>(p.n_idx);
-            for (int base = rank * PD_THREADS + tid; base < n_idx; base += U * stride) {
-                int s[U];
-                int32_t q[U];
-                const int32_t* entry[U];
-    #pragma unroll
-                for (int u = 0; u < U; ++u) s[u] = base + u * stride < n_idx ? ld_input(p.idx + base + u * stride) : -1;
-                if constexpr (MODE == PD_MARK_ROWS) {
-                    int64_t off[U], end[U], limit[U];
-    #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        off[u] = end[u] = limit[u] = 0;
-                        if (base + u * stride >= n_idx) continue;
-                        const int r = (base + u * stride) / p.k;
-                        off[u] = ld_input(p.table_offsets + r);
-                        end[u] = ld_input(p.table_offsets + r + 1);
-                        limit[u] = ld_input(p.demand_limits + r);
-                    }
-    #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        entry[u] = nullptr;
-                        if (s[u] >= 0 && s[u] < limit[u]) {       // a table that starts before the array has no pages
-                            const int64_t lp = page(s[u]);
-                            if (off[u] >= 0 && lp < end[u] - off[u]) entry[u] = p.page_table + off[u] + lp;
-                            else bad = true;
-                        }
-                    }
-                } else {
-    #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        entry[u] = nullptr;
-                        if (s[u] >= 0 && s[u] < p.demand_limit) {
-                            const int64_t lp = page(s[u]);
-                            if (lp < p.n_logical_pages) entry[u] = p.page_table + lp;
-                            else bad = true;
-                        }
-                    }
-                }
-    #pragma unroll
-                for (int u = 0; u < U; ++u) q[u] = entry[u] != nullptr ? ld_input(entry[u]) : -1;
-    #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (entry[u] == nullptr) continue;
-                    if (q[u] < 0 || q[u] >= p.n_phys_pages) bad = true;
-                    else set_bit_shared(bm, q[u]);
+    const PageDiv page{p.page_size, p.page_shift};
+    bool bad = false;
+    // Eight indices per thread at a time, in rounds of loads that are all in flight together: indices and their rows' table and
+    // limit, then page table entries (one index after the other: 24.2 us instead of 21.9 for 64 decode rows of 2048, when the rest took 5 us longer)
+    constexpr int U = 8;
+    const int stride = n_cta * PD_THREADS, n_idx = static_cast<int>(p.n_idx);
+    for (int base = rank * PD_THREADS + tid; base < n_idx; base += U * stride) {
+        int s[U];
+        int32_t q[U];
+        const int32_t* entry[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) s[u] = base + u * stride < n_idx ? ld_input(p.idx + base + u * stride) : -1;
+        if constexpr (MODE == PD_MARK_ROWS) {
+            int64_t off[U], end[U], limit[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                off[u] = end[u] = limit[u] = 0;
+                if (base + u * stride >= n_idx) continue;
+                const int r = (base + u * stride) / p.k;
+                off[u] = ld_input(p.table_offsets + r);
+                end[u] = ld_input(p.table_offsets + r + 1);
+                limit[u] = ld_input(p.demand_limits + r);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                entry[u] = nullptr;
+                if (s[u] >= 0 && s[u] < limit[u]) {       // a table that starts before the array has no pages
+                    const int64_t lp = page(s[u]);
+                    if (off[u] >= 0 && lp < end[u] - off[u]) entry[u] = p.page_table + off[u] + lp;
+                    else bad = true;
                 }
             }
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                entry[u] = nullptr;
+                if (s[u] >= 0 && s[u] < p.demand_limit) {
+                    const int64_t lp = page(s[u]);
+                    if (lp < p.n_logical_pages) entry[u] = p.page_table + lp;
+                    else bad = true;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) q[u] = entry[u] != nullptr ? ld_input(entry[u]) : -1;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (entry[u] == nullptr) continue;
+            if (q[u] < 0 || q[u] >= p.n_phys_pages) bad = true;
+            else set_bit_shared(bm, q[u]);
+        }
+    }
     return !bad;
 }
 
 // ---- one cluster, a pool of few words --------------------------------------------------------------------------------------------
 // The sets of all CTAs are ORed into CTA 0's shared memory, which then makes the lists alone (PD_LISTS: there is one CTA, and the set is
-// in global memory): a thread has a word, counts are 16 bits each, runs are put together in shared memory.  One cluster-wide barrier on the way instead of four, and no exchange of counts: 7-8 -> 5 us.
+// in global memory): a thread has a word, counts are 16 bits each, runs are put together in shared memory.  One cluster-wide barrier on the
+// way instead of four, and no exchange of counts: 7-8 -> 5 us.
 constexpr int PD_FEW_RUNS = PD_FEW_WORDS * 16;
 struct PdFewShared {
     uint32_t own[PD_FEW_WORDS];

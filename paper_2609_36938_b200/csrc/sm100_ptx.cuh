@@ -322,8 +322,9 @@ __device__ __forceinline__ void umma_pair_bf16_ts(uint32_t tmem_d, uint32_t tmem
         "r"(tmem_a), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(UMMA_DESC_HI_SW128)
         : "memory");
 }
-// Arrive on an mbarrier of another CTA of the cluster (its address from mapa), ordered after this thread's earlier accesses to its own
-// shared memory.
+// Arrive on an mbarrier of another CTA of the cluster (its address from mapa).  The release is of CTA scope, the default: what it publishes
+// here stays in this CTA's shared and tensor memory, behind a proxy or tcgen05 fence, and is read there by MMAs of the pair; nothing is
+// read by the other SM's threads.  (A release of cluster scope costs on the order of a thousand cycles.)
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }

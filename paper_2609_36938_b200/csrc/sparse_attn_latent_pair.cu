@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(LP_THREADS, 1) sparse_attn_latent_pair_kernel(
                                                                               const LpParams p) {
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* k_smem = smem;                                              // units of 3 atoms x [64 keys x 128 B]
-    unsigned char* v_smem = smem + LP_KU * LP_K_BYTES;                         // units of 4 atoms x [64 keys x 128 B]
+    unsigned char* v_smem = smem + LP_KU * LP_K_BYTES;                         // units of 4 atoms x [32 keys x 128 B]
     unsigned char* p_smem = smem + LP_SMEM_TILES;                              // 2 x 2 x [64 heads x 64 keys]
     unsigned char* q_smem = p_smem + 2 * LP_P_BYTES;                               // query atoms 6-8, each [64 heads x 128 B]
     LpShared* sh = reinterpret_cast<LpShared*>(q_smem + LP_Q_BYTES);
