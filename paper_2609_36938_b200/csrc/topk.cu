@@ -9,8 +9,8 @@
 //   3. a 2048-bucket histogram of the candidates (linear in the order-preserving integer key) gives the bucket of the k-th
 //      key; one pass emits everything above it and the keys inside are ranked directly.
 // If the sample misjudges the row (fewer than k candidates, or more than the buffer holds) an exact selection over repeated
-// histograms runs over the row in global memory instead; that path is slower, never wrong.  Rows that fit the buffer skip the
-// sampling step.
+// histograms runs over the row in global memory instead; that path is slower, never wrong.  A threshold with thousands of copies has a
+// way of its own (topk_row).  Rows that fit the buffer may skip the sampling step (janus_topk).
 #include <algorithm>
 
 #include "topk_plan.h"
