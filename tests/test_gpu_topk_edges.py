@@ -123,7 +123,7 @@ def test_a_threshold_with_many_copies_costs_no_second_selection(rows, n, k):
             b.record()
             torch.cuda.synchronize()
             times.append(a.elapsed_time(b))
-        took[name] = sorted(times)[len(times) // 2]
+        took[name] = min(times)
     assert took["cut"] < 2 * took["distinct"], took
 
 
@@ -151,5 +151,5 @@ def test_short_rows_of_a_batch_are_not_split(rows):
             b.record()
             torch.cuda.synchronize()
             times.append(a.elapsed_time(b))
-        took[name] = sorted(times)[len(times) // 2]
+        took[name] = min(times)
     assert took["batch"] < 1.1 * took["rows"], took
